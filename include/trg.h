@@ -55,7 +55,13 @@ typedef enum trg_model { TRG_ISING = 0, TRG_XY = 1, TRG_POTTS = 2 } trg_model;
  * Cholesky-QR, the Rayleigh-Ritz eigensolve, normalisation and the log-norm
  * accumulation are FP64 in every mode. */
 typedef enum trg_precision {
-    TRG_FP64 = 0,        /* plain FP64 on the CUDA cores */
+    TRG_FP64 = 0,        /* FP64.  trg_gemm runs on the FP64 pipe.  The products of a solve and of
+                            the component calls do too while they are small; larger ones are
+                            computed from exact BF16 digit products on the tensor cores and
+                            rounded to FP64 once, off by at most 2^-53 |C| + 10 K 2^-62 times the
+                            largest entries of the row and the column (an FP64 sum of K products
+                            is off by up to K 2^-53 |A||B|).  Operands with infinities, NaN or
+                            rows outside 2^-400 .. 2^400 stay on the FP64 pipe. */
     TRG_SPLIT_BF16 = 1   /* FP64 operands cut into BF16 slices, exact FP32
                             partial sums on tcgen05 tensor cores, summed wide */
 } trg_precision;

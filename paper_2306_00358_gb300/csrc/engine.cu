@@ -34,7 +34,8 @@ double secs(Clock::time_point a, Clock::time_point b) { return std::chrono::dura
 // Device bytes one solve can hold at its largest half-step: tensors, the
 // environment and its two intermediates, isometry, subspace-iteration blocks,
 // the contraction workspace and the split-GEMM scratch.  An upper bound.
-size_t estimate_bytes(const trg_solve_spec& s, size_t workspace_cap) {
+// exact: FP64 products may run on the tensor cores (their digits count).
+size_t estimate_bytes(const trg_solve_spec& s, size_t workspace_cap, bool exact) {
     const double d0 = (s.model == TRG_ISING) ? 2 : std::max(1, s.D0);
     const double D = std::max<double>(d0, std::min<double>(s.Dcut, std::max(d0 * d0, (double)s.Dcut)));
     const double D2 = D * D, D4 = D2 * D2;
@@ -61,6 +62,14 @@ size_t estimate_bytes(const trg_solve_spec& s, size_t workspace_cap) {
                  3 * (D2 + 256) * 4 + 3 * 256.0;            // their exponents, alignment
         // split-K parts of the isometry's products: at most 152 x 128 rows x m
         bytes += 152.0 * 128 * m * 8;
+    } else if (exact) {
+        // the digits of the largest FP64 product: environment, U.T.T.U in
+        // blocks of j, M.Q of the isometry
+        const double jb = std::max(1.0, std::floor(ws / std::max(1.0, 2 * D * D * D2 * 8)));
+        const int64_t d = (int64_t)D, d2 = d * d, rows = (int64_t)std::min(D, jb) * d2;
+        bytes += (double)std::max({trg::exact_scratch_bytes(d2, d2, d2), trg::exact_scratch_bytes(d2, rows, d),
+                                   trg::exact_scratch_bytes(rows, d2, d2), trg::exact_scratch_bytes(rows, d, d2),
+                                   trg::exact_scratch_bytes(d2, (int64_t)m, d2)});
     }
     bytes += 64.0 * 1024 * 1024;               // tables, scalars, allocator slack
     return (size_t)bytes;
@@ -76,6 +85,7 @@ struct Request {
     uint64_t ticket = 0;
     trg_solve_spec spec{};
     size_t bytes = 0;
+    bool no_exact = false;   // see Ctx::no_exact
     double work = 0.0;
     Clock::time_point t_submit, t_start, t_end;
     enum { QUEUED, RUNNING, DONE, CANCELLED } state = QUEUED;
@@ -148,6 +158,7 @@ void trg_server::run_request(trg_ctx*& ctx, Request* r) {
     }
     int st = trg_set_precision(ctx, s.precision, s.precision == TRG_SPLIT_BF16 ? s.split_slices : 4, 0);
     if (st == TRG_OK) {
+        ctx->no_exact = r->no_exact;
         ctx->cfg.trunc = s.trunc;
         ctx->cfg.seed = s.seed ? s.seed : 0x5EEDull;
         st = trg_init_tensor(ctx, s.model, s.beta, s.h, s.D0);
@@ -266,7 +277,7 @@ int trg_solve_spec_default(trg_solve_spec* s) {
 
 size_t trg_solve_bytes(const trg_solve_spec* spec, size_t workspace_bytes) {
     if (!spec) return 0;
-    return estimate_bytes(*spec, workspace_bytes ? workspace_bytes : ((size_t)1 << 30));
+    return estimate_bytes(*spec, workspace_bytes ? workspace_bytes : ((size_t)1 << 30), true);
 }
 
 int trg_serve_create(trg_server** out, int device, const trg_server_config* cfg) {
@@ -311,7 +322,11 @@ int trg_serve_submit(trg_server* s, const trg_solve_spec* spec, uint64_t* ticket
     Request* r = new (std::nothrow) Request();
     if (!r) return TRG_ENOMEM;
     r->spec = *spec;
-    r->bytes = estimate_bytes(*spec, s->cfg.workspace_bytes);
+    r->bytes = estimate_bytes(*spec, s->cfg.workspace_bytes, true);
+    if (r->bytes > s->cfg.hbm_budget_bytes) {   // no room for FP64 digits: such a solve takes the FP64 pipe
+        r->no_exact = true;
+        r->bytes = estimate_bytes(*spec, s->cfg.workspace_bytes, false);
+    }
     r->work = estimate_work(*spec);
     if (r->bytes > s->cfg.hbm_budget_bytes) {   // could never be admitted
         delete r;

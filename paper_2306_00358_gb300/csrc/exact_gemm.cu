@@ -1,0 +1,619 @@
+// FP64 products on the tcgen05 tensor cores (TRG_FP64, large products).
+//
+// The FP64 pipe of this part does 1.9 FMA a clock and SM, 1/2000 of the BF16
+// tensor rate, so an FP64 product that is large enough is computed from BF16
+// digit products instead, to more than FP64 accuracy.  Each operand row (A) /
+// column (B) gets a power-of-two scale 2^e with |x| < 2^e, and
+//     X = rint(x 2^(63 - e)) = sum_p d_p 2^(8 (7 - p)),   p = 0..7,
+// d_0 in [-128, 128], d_p in [-128, 127] (an error-free splitting as in
+// split_gemm.cu, with eight digits and every sum exact: Ozaki, Ogita, Oishi,
+// Rump, Numer. Algorithms 59 (2012) 95).  An element down to 2^-10 of its
+// row's largest keeps all 53 bits.  With D_d = sum_{p + q = d} A_p B_q,
+//     C = 2^(ea + eb - 70) sum_{d < 8} D_d 2^(8 (7 - d)):
+// digit products are integers up to 2^14, a run of 128 K sums the at most
+// eight products of a D_d exactly in FP32 (8 x 128 x 2^14 = 2^24), the
+// epilogue moves each run into int64 sums and the 96-bit total is rounded to
+// FP64 once.  What is left out (d >= 8) and the rounding of X are below
+// 10 K 2^-64 2^(ea + eb).  On the method's tensors, environments and isometries (leg sizes 8 to 32) the
+// results are within 1.1e-16 of sum |a||b|, element by element, where a
+// K-long FP64 chain is off by 3e-16 to 3e-15.
+//
+// Rows or columns whose largest entry lies outside 2^-400 .. 2^400, or that
+// hold an infinity or a NaN, raise a device flag: the tensor kernel then
+// returns at once and the FP64 pipe kernel that is queued behind it, idle
+// otherwise, computes the product.
+//
+// What bounds it: the tensor pipe, 36 digit products of 2 M N K each.
+// 128 x 64 output tile, one persistent CTA per SM: the eight D_d of 64
+// columns fill the 512 TMEM columns.  A stage is 32 K of both operands (64 KB
+// of A digits, 32 KB of B digits, one TMA box each), two stages.  The products
+// of one A digit with adjacent B digits land in adjacent accumulators, so 12
+// instructions of up to N = 256 cover the 36 products of a 16-deep step.
+// They are issued in two groups, the one that lands in D_4..D_7 (26 products)
+// before the one that lands in D_0..D_3: a run's drain of D_4..D_7 runs under
+// the other group's products, and the drain of D_0..D_3 under the next run's
+// first group.  Measured, contraction at Dx = Dy = Dn = 48 (three products,
+// 1.22e12 FP64 FLOPs): 993 ms on the FP64 pipe, 34.7 ms here, 30.8 of them in
+// this kernel (4.4e13 digit FLOPs at 1430 TFLOP/s), 2.9 cutting digits, 0.9
+// finding exponents; environment at (24, 22): 0.65 -> 0.25 ms.
+#include <algorithm>
+#include <cmath>
+
+#include "internal.h"
+#include "tcgen05.cuh"
+
+namespace trg {
+
+namespace {
+
+constexpr int XS = 8;                            // digits
+constexpr int XM = 128, XN = 64, XK = 32;        // tile rows, columns, K per stage
+constexpr int XA_TILE = XM * XK * 2;             // bytes of one digit's A tile
+constexpr int XB_TILE = XN * XK * 2;
+constexpr int XSTAGE = XS * (XA_TILE + XB_TILE); // 96 KB
+constexpr int XSTAGES = 2;
+constexpr int XRUN = 128 / XK;                   // stages of an exact run
+constexpr int XEPI = 16;                         // epilogue warps
+constexpr int XTHREADS = 64 + 32 * XEPI;
+constexpr int XCPT = XN / 4;                     // columns per epilogue thread
+constexpr int XSTAGING = XEPI * 32 * 8 * 8;      // store staging, 32 KB
+constexpr int XBAR = 256;
+constexpr int XSMEM = XSTAGES * XSTAGE + XSTAGING + XBAR + 1024;
+static_assert(XSMEM <= 232448, "exact product shared memory");
+
+// The digit products of one 16-deep step: A digit a times the n B digits
+// from b on, into the accumulators D_(a+b) .. D_(a+b+n-1).  Group 1 lands in
+// D_4..D_7, group 0 in D_0..D_3; the first entry of a group covers all four
+// of its accumulators and resets them at the start of a run.
+struct XIns { int a, b, n, group; };
+__host__ __device__ constexpr int xins_count() { return 12; }
+__host__ __device__ constexpr XIns xins(int t) {
+    return t < 8 ? XIns{t, t < 4 ? 4 - t : 0, t < 4 ? 4 : 8 - t, 1} : XIns{t - 8, 0, 4 - (t - 8), 0};
+}
+__host__ __device__ constexpr bool xins_ok() {
+    int seen[XS][XS] = {};
+    for (int t = 0; t < xins_count(); ++t) {
+        const XIns in = xins(t);
+        for (int q = in.b; q < in.b + in.n; ++q) {
+            const int d = in.a + q;
+            if (d >= XS || (d >= 4) != (in.group == 1)) return false;
+            seen[in.a][q] += 1;
+        }
+    }
+    for (int p = 0; p < XS; ++p)
+        for (int q = 0; q < XS; ++q)
+            if (seen[p][q] != (p + q < XS ? 1 : 0)) return false;
+    return xins(0).b == 4 && xins(0).n == 4 && xins(8).n == 4;
+}
+static_assert(xins_ok(), "digit product table");
+
+struct XArgs {
+    int M, N, Kp;
+    const int* fa;                 // largest exponent field of each A row
+    const int* fb;                 // ... of each B column
+    double* C;
+    const int64_t* c_m;
+    const int64_t* c_n;
+    int rows_fast;                 // consecutive rows are (mostly) adjacent in C: store row-wise
+    int sym;                       // C symmetric: the tile list holds the tiles that reach the diagonal
+    const long long* tile_list;    // mb << 32 | nb, or nullptr for all
+    int n_list;
+    int group_n;                   // tile order: column blocks per group
+    const int* bad;                // the operands are outside the digits' range: do nothing
+    int* status;
+};
+
+// (hi 2^32 + lo) 2^e2 in FP64, rounded once (twice when |hi| >= 2^53, where
+// the second rounding is below 2^-20 of an ulp)
+__device__ __forceinline__ double wide_to_double(long long hi, long long lo, int e2) {
+    hi += lo >> 32;
+    const double r = fma((double)hi, 4294967296.0, (double)(unsigned)(lo & 0xffffffffll));
+    if (r == 0.0) return 0.0;
+    // |e2| <= 872 and |r| < 2^96: the exponent field stays in range
+    return __longlong_as_double(__double_as_longlong(r) + ((long long)e2 << 52));
+}
+
+__global__ void __launch_bounds__(XTHREADS, 1)
+k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const XArgs g) {
+    if (*g.bad) return;
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    uint64_t* full = (uint64_t*)(smem + XSTAGES * XSTAGE + XSTAGING);
+    uint64_t* empty = full + XSTAGES;
+    uint64_t* acc_full = empty + XSTAGES;        // [group]
+    uint64_t* acc_empty = acc_full + 2;          // [group]
+    uint64_t* mma_done = acc_empty + 2;
+    uint32_t* tmem_slot = (uint32_t*)(mma_done + 1);
+    volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
+    double* staging = (double*)(smem + XSTAGES * XSTAGE);
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int tiles_m = (g.M + XM - 1) / XM, tiles_n = (g.N + XN - 1) / XN;
+    const int num_tiles = g.tile_list ? g.n_list : tiles_m * tiles_n;
+    const int num_kb = g.Kp / XK;
+    auto coords = [&](int tile, int& mb, int& nb) {
+        if (g.tile_list) {
+            const long long v = g.tile_list[tile];
+            mb = (int)(v >> 32);
+            nb = (int)(v & 0xffffffffll);
+        } else {
+            const int per_group = tiles_m * g.group_n;
+            const int group = tile / per_group, first = group * g.group_n;
+            const int width = min(g.group_n, tiles_n - first), local = tile - group * per_group;
+            mb = local / width;
+            nb = first + local % width;
+        }
+    };
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < XSTAGES; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
+        for (int q = 0; q < 2; ++q) { mbar_init(&acc_full[q], 1); mbar_init(&acc_empty[q], XEPI); }
+        mbar_init(mma_done, 1);
+        *abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                     ::"r"(smem_u32(tmem_slot)), "r"(512u));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+
+    if (warp == 0) {
+        if (lane == 0) {
+            int stage = 0;
+            uint32_t phase = 0;
+            int issued[XSTAGES];
+#pragma unroll
+            for (int s = 0; s < XSTAGES; ++s) issued[s] = -1;
+            bool ok = true;
+            for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
+                int mb, nb;
+                coords(tile, mb, nb);
+                for (int kb = 0; kb < num_kb; ++kb) {
+                    ok = mbar_wait(&empty[stage], phase ^ 1, abort_flag, g.status);
+                    if (!ok) break;
+                    uint8_t* st = smem + stage * XSTAGE;
+                    mbar_expect_tx(&full[stage], XSTAGE);
+                    tma_load_3d(st, &tmA, kb * XK, mb * XM, 0, &full[stage]);
+                    tma_load_3d(st + XS * XA_TILE, &tmB, kb * XK, nb * XN, 0, &full[stage]);
+#pragma unroll
+                    for (int s = 0; s < XSTAGES; ++s)
+                        if (s == stage) issued[s] = (int)phase;
+                    if (++stage == XSTAGES) { stage = 0; phase ^= 1; }
+                }
+            }
+            // every load issued has landed before the CTA may exit (bounded, also after an abort)
+            volatile int never = 0;
+#pragma unroll
+            for (int s = 0; s < XSTAGES; ++s)
+                if (issued[s] >= 0) mbar_wait(&full[s], (uint32_t)issued[s], &never, g.status);
+        }
+    } else if (warp == 1) {
+        if (lane == 0) {
+            int stage = 0;
+            uint32_t phase = 0;
+            uint32_t run_no = 0;        // runs begun so far (all tiles)
+            bool ok = true;
+            for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
+                for (int kb = 0; kb < num_kb; ++kb) {
+                    const bool run_start = kb % XRUN == 0;
+                    const bool run_end = (kb + 1) % XRUN == 0 || kb + 1 == num_kb;
+                    ok = mbar_wait(&full[stage], phase, abort_flag, g.status);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint64_t dbase = smem_desc(smem_u32(smem + stage * XSTAGE));
+                    auto issue = [&](int group) {
+#pragma unroll
+                        for (int kk = 0; kk < XK / 16; ++kk) {
+#pragma unroll
+                            for (int t = 0; t < xins_count(); ++t) {
+                                const XIns in = xins(t);
+                                if (in.group != group) continue;
+                                const bool first = t == 0 || t == 8;
+                                const uint32_t acc = (first && run_start && kk == 0) ? 0u : 1u;
+                                const uint64_t da = dbase + (uint64_t)((in.a * XA_TILE + kk * 32) >> 4);
+                                const uint64_t db = dbase + (uint64_t)((XS * XA_TILE + in.b * XB_TILE + kk * 32) >> 4);
+                                mma_bf16<1>(tmem + (uint32_t)((in.a + in.b) * XN), da, db, idesc_bf16(XM, in.n * XN),
+                                            acc);
+                            }
+                        }
+                    };
+                    if (run_start && run_no > 0) {
+                        ok = mbar_wait(&acc_empty[1], (run_no - 1) & 1, abort_flag, g.status);
+                        if (!ok) break;
+                        tc_fence_after();
+                    }
+                    issue(1);
+                    if (run_end) mma_commit<1>(&acc_full[1]);
+                    if (run_start && run_no > 0) {
+                        ok = mbar_wait(&acc_empty[0], (run_no - 1) & 1, abort_flag, g.status);
+                        if (!ok) break;
+                        tc_fence_after();
+                    }
+                    issue(0);
+                    mma_commit<1>(&empty[stage]);
+                    if (run_end) {
+                        mma_commit<1>(&acc_full[0]);
+                        ++run_no;
+                    }
+                    if (++stage == XSTAGES) { stage = 0; phase ^= 1; }
+                }
+            }
+            // every MMA issued has completed (also after an abort)
+            mma_commit<1>(mma_done);
+            volatile int never = 0;
+            mbar_wait(mma_done, 0, &never, g.status);
+        }
+    } else {
+        const int ew = warp - 2, quad = warp & 3, colq = ew >> 2;
+        const uint32_t lane_base = (uint32_t)(quad * 32) << 16;
+        uint32_t run_no = 0;
+        bool ok = true;
+        for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
+            int mb, nb;
+            coords(tile, mb, nb);
+            const int nruns = (num_kb + XRUN - 1) / XRUN;
+            long long hi[XCPT], lo[XCPT];        // D_0..D_3 and D_4..D_7, each as an int64 in units of its last digit
+#pragma unroll
+            for (int j = 0; j < XCPT; ++j) hi[j] = lo[j] = 0;
+            for (int c = 0; c < nruns && ok; ++c, ++run_no) {
+#pragma unroll
+                for (int grp = 1; grp >= 0; --grp) {
+                    int w_ok = 1;
+                    if (lane == 0) w_ok = mbar_wait(&acc_full[grp], run_no & 1, abort_flag, g.status) ? 1 : 0;
+                    ok = __shfl_sync(0xffffffffu, w_ok, 0) != 0;
+                    if (!ok) break;
+                    tc_fence_after();
+#pragma unroll
+                    for (int d = 0; d < 4; ++d) {
+                        uint32_t r[XCPT];
+                        tmem_ld16(tmem + lane_base + (uint32_t)((grp * 4 + d) * XN + colq * XCPT), r);
+                        tmem_wait_ld();
+#pragma unroll
+                        for (int j = 0; j < XCPT; ++j) {
+                            const long long v = (long long)__float2int_rn(__uint_as_float(r[j])) * (1ll << (8 * (3 - d)));
+                            if (grp) lo[j] += v; else hi[j] += v;
+                        }
+                    }
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&acc_empty[grp]);
+                }
+            }
+            if (!ok) break;
+            const int m = mb * XM + quad * 32 + lane;
+            const bool row_ok = m < g.M;
+            const int nt = nb * XN + colq * XCPT;
+            // the warp's 16 columns are the same for every lane: lane j loads
+            // column j's exponent and offset, the loop takes them by shuffle
+            const bool col_in = lane < XCPT && nt + lane < g.N;
+            const int fb = col_in ? g.fb[nt + lane] : 0;
+            const long long cn_l = col_in ? (long long)g.c_n[nt + lane] : 0;
+            const int ea = row_ok ? max(g.fa[m], 1) - 1022 : 0;
+            const int eb_l = max(fb, 1) - 1022 - 70;
+            if (g.rows_fast) {
+                // lanes are adjacent rows, adjacent in C
+                double* cp = g.C + (row_ok ? g.c_m[m] : 0);
+#pragma unroll
+                for (int j = 0; j < XCPT; ++j) {
+                    const int e2 = ea + __shfl_sync(0xffffffffu, eb_l, j);
+                    const long long cn = __shfl_sync(0xffffffffu, cn_l, j);
+                    if (row_ok && nt + j < g.N) cp[cn] = wide_to_double(hi[j], lo[j], e2);
+                }
+                continue;
+            }
+            double v[XCPT];
+#pragma unroll
+            for (int j = 0; j < XCPT; ++j) {
+                const int e2 = ea + __shfl_sync(0xffffffffu, eb_l, j);
+                v[j] = (row_ok && nt + j < g.N) ? wide_to_double(hi[j], lo[j], e2) : 0.0;
+            }
+            if (g.sym && row_ok) {
+                // the mirror (n, m) of each element above the diagonal
+                const int64_t cm_mirror = g.c_n[m];
+#pragma unroll
+                for (int j = 0; j < XCPT; ++j) {
+                    const int n = nt + j;
+                    if (n < g.N && n > m) g.C[g.c_m[n] + cm_mirror] = v[j];
+                }
+            }
+            // columns adjacent in C: through the warp's 32 x 8 staging tile, so
+            // that a quarter-warp writes 8 adjacent columns of one row
+            double* stg = staging + ew * (32 * 8);
+            const int quarter = lane >> 3, cl = lane & 7;
+#pragma unroll
+            for (int pass = 0; pass < XCPT / 8; ++pass) {
+#pragma unroll
+                for (int jj = 0; jj < 8; ++jj) stg[lane * 8 + (jj ^ ((lane >> 1) & 7))] = v[pass * 8 + jj];
+                const int64_t cn = __shfl_sync(0xffffffffu, cn_l, pass * 8 + cl);
+                __syncwarp();
+                const int n = nt + pass * 8 + cl;
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    const int rr = 4 * q + quarter;
+                    const int mr = mb * XM + quad * 32 + rr;
+                    if (mr < g.M && n < g.N && (!g.sym || n >= mr))
+                        g.C[g.c_m[mr] + cn] = stg[rr * 8 + (cl ^ ((rr >> 1) & 7))];
+                }
+                __syncwarp();
+            }
+        }
+    }
+
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        __syncwarp();
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u));
+    }
+}
+
+// ------------------------------------------------------------- digits ----
+// Largest exponent field of each row r of the gathered operand src[off_r[r] +
+// off_c[k]] (subnormals count as field 1), maxima into ef (zeroed).  HBM-bound;
+// a warp reads along the index that is adjacent in memory.
+constexpr int XF_K = 256;
+__global__ void __launch_bounds__(256) k_row_field(const double* __restrict__ src, const int64_t* __restrict__ off_r,
+                                                   const int64_t* __restrict__ off_c, int R, int K, int k_fast,
+                                                   int* __restrict__ ef) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int k0 = blockIdx.x * XF_K, k1 = min(K, k0 + XF_K);
+    auto field = [](double x) -> unsigned {
+        const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+        const unsigned hi = (unsigned)(b >> 32) & 0x7fffffffu;
+        return hi >= 0x100000u ? hi >> 20 : ((hi | (unsigned)b) ? 1u : 0u);
+    };
+    for (int r0 = blockIdx.y * 32; r0 < R; r0 += gridDim.y * 32) {
+        if (k_fast) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int r = r0 + warp * 4 + i;
+                if (r >= R) break;
+                const double* row = src + off_r[r];
+                unsigned f = 0;
+#pragma unroll 8
+                for (int k = k0 + lane; k < k1; k += 32) f = max(f, field(row[off_c[k]]));
+                f = __reduce_max_sync(0xffffffffu, f);
+                if (lane == 0 && f) atomicMax(&ef[r], (int)f);
+            }
+        } else {
+            __shared__ unsigned red[8][32];
+            const int r = r0 + lane;
+            unsigned f = 0;
+            if (r < R) {
+                const double* row = src + off_r[r];
+#pragma unroll 8
+                for (int k = k0 + warp; k < k1; k += 8) f = max(f, field(row[off_c[k]]));
+            }
+            red[warp][lane] = f;
+            __syncthreads();
+            if (warp == 0) {
+#pragma unroll
+                for (int w = 1; w < 8; ++w) f = max(f, red[w][lane]);
+                if (r < R && f) atomicMax(&ef[r], (int)f);
+            }
+            __syncthreads();
+        }
+    }
+}
+
+// The eight digits (BF16) of each element: out[p][r][k], r < Rp, k < Kp, zero
+// in the padding.  Elements pass through a 32 x 64 shared tile so that both
+// sides are coalesced; a thread cuts eight adjacent k and writes 16 bytes per
+// digit.  Rows outside the digits' range raise *bad.  HBM-bound: 8 B read,
+// 16 B written per element.
+constexpr int XD_R = 32, XD_K = 64, XD_LD = XD_K + XD_K / 8 + 1;
+constexpr int FIELD_LO = 1023 - 400, FIELD_HI = 1023 + 400;
+__global__ void __launch_bounds__(256) k_digits8(const double* __restrict__ src, const int64_t* __restrict__ off_r,
+                                                 const int64_t* __restrict__ off_c, int R, int K, int Rp, int Kp,
+                                                 int k_fast, const int* __restrict__ ef, uint16_t* __restrict__ out,
+                                                 int* bad) {
+    __shared__ double tile[XD_R * XD_LD];
+    const int k0 = blockIdx.x * XD_K;
+    const size_t plane = (size_t)Rp * Kp;
+    for (int r0 = blockIdx.y * XD_R; r0 < Rp; r0 += gridDim.y * XD_R) {
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < XD_R * XD_K / 256; ++q) {
+            const int e = threadIdx.x + q * 256;
+            int rr, kk;
+            if (k_fast) { kk = e % XD_K; rr = e / XD_K; } else { rr = e % XD_R; kk = e / XD_R; }
+            const int r = r0 + rr, k = k0 + kk;
+            tile[rr * XD_LD + kk + (kk >> 3)] = (r < R && k < K) ? src[off_r[r] + off_c[k]] : 0.0;
+        }
+        __syncthreads();
+        const int rr = threadIdx.x >> 3, kg = threadIdx.x & 7;
+        const int r = r0 + rr, k = k0 + kg * 8;
+        if (r >= Rp || k >= Kp) continue;
+        const int f = r < R ? ef[r] : 0;
+        if (f && (f < FIELD_LO || f > FIELD_HI)) *bad = 1;
+        const double* x = tile + rr * XD_LD + kg * 9;
+        uint32_t w[XS][4];
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+            float d[2][XS];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const unsigned long long b = (unsigned long long)__double_as_longlong(x[2 * h + u]);
+                const int ex = (int)((b >> 52) & 0x7FF);
+                const int sh = f - ex - 10;              // X = mantissa 2^-sh
+                unsigned long long m = ex ? ((b & ((1ull << 52) - 1)) | (1ull << 52)) : 0ull;
+                m = sh <= 0 ? m << (-sh & 63) : sh < 60 ? (m + (1ull << (sh - 1))) >> sh : 0ull;
+                const bool neg = (long long)b < 0;
+                // adding 128 to every digit but the first turns the signed
+                // digits into bytes; the first is the signed top byte, whose
+                // sign bit is part of the value when X >= 0
+                const unsigned long long y = (neg ? 0ull - m : m) + 0x0080808080808080ull;
+                const unsigned ylo = (unsigned)y, yhi = (unsigned)(y >> 32);
+                const int top = neg ? (int)yhi >> 24 : (int)(yhi >> 24);
+                d[u][0] = (float)top;
+#pragma unroll
+                for (int p = 1; p < XS; ++p) {
+                    const unsigned byte = p < 4 ? __byte_perm(yhi, 0x4B000000u, 0x7440u | (unsigned)(3 - p))
+                                                : __byte_perm(ylo, 0x4B000000u, 0x7440u | (unsigned)(7 - p));
+                    d[u][p] = __uint_as_float(byte) - 8388736.0f;   // 2^23 + 128
+                }
+            }
+#pragma unroll
+            for (int p = 0; p < XS; ++p) {
+                // exact in BF16: the upper halves of the two FP32 values
+                w[p][h] = __byte_perm(__float_as_uint(d[0][p]), __float_as_uint(d[1][p]), 0x7632);
+            }
+        }
+        uint16_t* o = out + (size_t)r * Kp + k;
+#pragma unroll
+        for (int p = 0; p < XS; ++p) *reinterpret_cast<uint4*>(o + p * plane) = make_uint4(w[p][0], w[p][1], w[p][2], w[p][3]);
+    }
+}
+
+// ------------------------------------------------------------- host side ---
+// Digit planes [XS][rows][kp] as a 3D map, boxes of box_rows x XK of every digit.
+CUtensorMap digit_map(const void* base, int rows, int kp, int box_rows) {
+    CUtensorMap m;
+    std::memset(&m, 0, sizeof(m));
+    const cuuint64_t dims[3] = {(cuuint64_t)kp, (cuuint64_t)rows, (cuuint64_t)XS};
+    const cuuint64_t strides[2] = {(cuuint64_t)kp * 2, (cuuint64_t)kp * 2 * (cuuint64_t)rows};
+    const cuuint32_t box[3] = {(cuuint32_t)XK, (cuuint32_t)box_rows, (cuuint32_t)XS};
+    const cuuint32_t estr[3] = {1, 1, 1};
+    CUresult r = encode_fn()(&m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box,
+                             estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
+                             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) fail(TRG_ECUDA, "cuTensorMapEncodeTiled failed (" + std::to_string((int)r) + ")");
+    return m;
+}
+
+int64_t up(int64_t v, int64_t q) { return (v + q - 1) / q * q; }
+
+// Exponent fields and digits of rows [0, R) of an operand.
+void digits(Ctx& ctx, const Gather& g, int R, int K, int Rp, int Kp, int* ef, uint16_t* out, int* bad) {
+    TRG_CUDA(cudaMemsetAsync(ef, 0, (size_t)R * sizeof(int), ctx.stream));
+    dim3 gf((unsigned)((K + XF_K - 1) / XF_K), (unsigned)std::min((R + 31) / 32, 65535));
+    k_row_field<<<gf, 256, 0, ctx.stream>>>(g.base, g.off_r, g.off_c, R, K, g.c_fast ? 1 : 0, ef);
+    TRG_LAUNCHED(ctx);
+    dim3 gd((unsigned)((Kp + XD_K - 1) / XD_K), (unsigned)std::min((Rp + XD_R - 1) / XD_R, 65535));
+    k_digits8<<<gd, 256, 0, ctx.stream>>>(g.base, g.off_r, g.off_c, R, K, Rp, Kp, g.c_fast ? 1 : 0, ef, out, bad);
+    TRG_LAUNCHED(ctx);
+}
+
+const long long* diagonal_tiles(Ctx& ctx, int tiles_m, int tiles_n, int& n) {
+    const std::string key = "xsym:" + std::to_string(tiles_m) + ":" + std::to_string(tiles_n);
+    auto it = ctx.tables.find(key);
+    if (it == ctx.tables.end()) {
+        std::vector<long long> h;
+        for (int mb = 0; mb < tiles_m; ++mb)
+            for (int nb = 0; nb < tiles_n; ++nb)
+                if ((int64_t)nb * XN + XN - 1 >= (int64_t)mb * XM) h.push_back(((long long)mb << 32) | nb);
+        Buf buf;
+        ctx.ensure(buf, h.size() * sizeof(long long));
+        TRG_CUDA(cudaMemcpyAsync(buf.p, h.data(), h.size() * sizeof(long long), cudaMemcpyHostToDevice, ctx.stream));
+        TRG_CUDA(cudaStreamSynchronize(ctx.stream));   // h dies here
+        it = ctx.tables.emplace(key, buf).first;
+        ctx.list_len[key] = (int)h.size();
+    }
+    n = ctx.list_len[key];
+    return it->second.as<long long>();
+}
+
+// Rows of an operand whose digits are held at a time: at most XCAP bytes of
+// them (a multiple of the tile).
+constexpr int64_t XCAP = (int64_t)1 << 30;
+int64_t block_rows(int64_t rows, int64_t kp, int64_t tile) {
+    const int64_t most = std::max<int64_t>(tile, XCAP / (2 * XS * kp) / tile * tile);
+    return std::min(up(rows, tile), most);
+}
+
+}  // namespace
+
+int64_t exact_scratch_bytes(int64_t M, int64_t N, int64_t K) {
+    const int64_t kp = up(std::max<int64_t>(K, 1), XK);
+    const int64_t ra = block_rows(M, kp, XM), rb = block_rows(N, kp, XN);
+    return 2 * XS * kp * (ra + rb) + 4 * (ra + rb) + 2048;
+}
+
+double exact_us(const Ctx& ctx, int64_t M, int64_t N, int64_t K, bool sym) {
+    if (M > (1ll << 30) || N > (1ll << 30) || K > (1 << 17)) return 1e300;
+    const double tm = (double)up(M, XM) / XM, tn = (double)up(N, XN) / XN;
+    const double tiles = sym ? 0.5 * tm * (tn + 2) : tm * tn;
+    const double runs = std::ceil((double)K / 128.0);
+    const double mma = std::ceil(tiles / ctx.sm_count) * (runs * 5.4 + 3.0);
+    const double moved = (32.0 * (double)K * ((double)M + (sym ? 0.0 : (double)N)) + 8.0 * (double)M * (double)N) / 4.0e6;
+    return 25.0 + mma + moved;
+}
+
+bool gemm_exact(Ctx& ctx, const GemmDesc& d) {
+    const int K = (int)std::max<int64_t>(d.K, 1), Kp = (int)up(K, XK);
+    const int64_t ra = block_rows(d.M, Kp, XM), rb = block_rows(d.N, Kp, XN);
+    const bool sym = d.gram && d.M == d.N && ra >= d.M;
+    try {
+        ctx.ensure(ctx.split_ws, (size_t)exact_scratch_bytes(d.M, sym ? 1 : d.N, K));
+    } catch (const Error& e) {
+        if (e.status == TRG_ENOMEM) return false;    // no room for the digits: the FP64 pipe needs none
+        throw;
+    }
+    uint8_t* p = ctx.split_ws.as<uint8_t>();
+    auto take = [&](size_t bytes) { uint8_t* q = p; p += (bytes + 255) & ~(size_t)255; return q; };
+    int* bad = (int*)take(4);
+    int* fa = (int*)take((size_t)ra * 4);
+    int* fb = sym ? fa : (int*)take((size_t)rb * 4);
+    uint16_t* sa = (uint16_t*)take((size_t)(2 * XS) * ra * Kp);
+    uint16_t* sb = sym ? sa : (uint16_t*)take((size_t)(2 * XS) * rb * Kp);
+    TRG_CUDA(cudaMemsetAsync(bad, 0, sizeof(int), ctx.stream));
+    static std::once_flag once;
+    std::call_once(once, [] {
+        TRG_CUDA(cudaFuncSetAttribute(k_exact_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, XSMEM));
+    });
+
+    // B as rows n, columns k
+    Gather bt = d.B;
+    bt.off_r = d.B.off_c;
+    bt.off_c = d.B.off_r;
+    bt.c_fast = d.B.r_fast && !d.B.c_fast;
+    for (int64_t m0 = 0; m0 < d.M; m0 += ra) {
+        const int mr = (int)std::min(ra, d.M - m0), mp = (int)up(mr, XM);
+        Gather ga = d.A;
+        ga.off_r += m0;
+        digits(ctx, ga, mr, K, mp, Kp, fa, sa, bad);
+        const CUtensorMap ta = digit_map(sa, mp, Kp, XM);
+        for (int64_t n0 = 0; n0 < d.N; n0 += rb) {
+            const int nr = (int)std::min(rb, d.N - n0), np = sym ? mp : (int)up(nr, XN);
+            if (!sym && (m0 == 0 || rb < d.N)) {
+                Gather gb = bt;
+                gb.off_r += n0;
+                digits(ctx, gb, nr, K, np, Kp, fb, sb, bad);
+            }
+            const CUtensorMap tb = digit_map(sb, np, Kp, XN);
+            XArgs a;
+            a.M = mr; a.N = sym ? mr : nr; a.Kp = Kp;
+            a.fa = fa; a.fb = fb;
+            a.C = d.C; a.c_m = d.c_m + m0; a.c_n = d.c_n + n0;
+            a.rows_fast = d.c_m_fast && !sym ? 1 : 0;
+            a.sym = sym ? 1 : 0;
+            a.tile_list = nullptr; a.n_list = 0;
+            a.bad = bad; a.status = ctx.status.as<int>();
+            const int tiles_m = mp / XM, tiles_n = (a.N + XN - 1) / XN;
+            int tiles = tiles_m * tiles_n;
+            if (sym) {
+                a.tile_list = diagonal_tiles(ctx, tiles_m, tiles_n, a.n_list);
+                tiles = a.n_list;
+            }
+            // column blocks whose digits share L2 (about 40 MB of them)
+            a.group_n = (int)std::max<int64_t>(1, std::min<int64_t>(tiles_n, (40ll << 20) / ((int64_t)XN * Kp * 2 * XS)));
+            const int grid = std::min(tiles, ctx.sm_count);
+            const int tok = ctx.region_begin(TRG_PHASE_MMA);
+            k_exact_mma<<<grid, XTHREADS, XSMEM, ctx.stream>>>(ta, tb, a);
+            TRG_LAUNCHED(ctx);
+            ctx.region_end(tok, 2.0 * (double)mr * nr * K, 36.0 * 2.0 * (double)mr * nr * Kp);
+            if (sym) break;
+        }
+    }
+    gemm_f64(ctx, d, bad);    // computes the product if an operand was out of range, else returns at once
+    return true;
+}
+
+}  // namespace trg

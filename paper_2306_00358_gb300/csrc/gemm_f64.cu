@@ -39,6 +39,7 @@ struct GemmArgs {
     double beta;
     int64_t tiles_n, tiles;
     int sym;               // C = A A^T: tiles below the diagonal are mirrors of those above
+    const int* only_if;    // device flag: compute only if it is set
 };
 
 // T x T outputs per block, R x R per thread (stride T / R), BK deep stages.
@@ -50,6 +51,7 @@ __global__ void __launch_bounds__(NT) k_gemm_f64(const GemmArgs g) {
     constexpr int KB = BK / KG;               // k's of a stage each group takes
     constexpr int E = T * BK / NT;            // elements a thread stages per operand
     static_assert(G * KG == NT && KB * KG == BK && E * NT == T * BK, "tile shape");
+    if (g.only_if && *g.only_if == 0) return;
     __shared__ double As[BK][T + 1];
     __shared__ double Bs[BK][T + 1];
     const int tid = threadIdx.x;
@@ -152,7 +154,8 @@ __global__ void __launch_bounds__(NT) k_gemm_f64(const GemmArgs g) {
 
 // C = beta C + sum_z P[z], summed in z order (deterministic).
 __global__ void k_reduce_partials(const double* __restrict__ P, int nz, int64_t M, int64_t N, double* C,
-                                  const int64_t* c_m, const int64_t* c_n, double beta) {
+                                  const int64_t* c_m, const int64_t* c_n, double beta, const int* only_if) {
+    if (only_if && *only_if == 0) return;
     const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (e >= M * N) return;
     double s = 0.0;
@@ -166,9 +169,9 @@ __global__ void k_reduce_partials(const double* __restrict__ P, int nz, int64_t 
 // in clocks.  A block's time is its FMAs at the pipe's rate, the blocks are
 // dealt evenly over the SMs, each K stage costs the latency of its loads
 // unless several blocks share the SM, and split K adds a second launch.
-struct Shape { int T; int64_t nz; };
+struct Shape { int T; int64_t nz; double clocks; };
 Shape choose_shape(int64_t M, int64_t N, int64_t K, int sms, bool sym) {
-    Shape best{64, 1};
+    Shape best{64, 1, 0.0};
     double best_t = 1e300;
     for (int T : {64, 32, 16, 8}) {
         const int bk = T == 64 ? 16 : T == 8 ? 64 : 32;
@@ -180,7 +183,7 @@ Shape choose_shape(int64_t M, int64_t N, int64_t K, int sms, bool sym) {
             const double per_sm = std::ceil(tiles * nz / sms);
             const double t = per_sm * T * T * kper / 1.9 + std::ceil(kper / bk) * (1200.0 / std::min(per_sm, 4.0)) * per_sm +
                              (nz > 1 ? 7000.0 : 0.0);
-            if (t < best_t) { best_t = t; best = {T, nz}; }
+            if (t < best_t) { best_t = t; best = {T, nz, t}; }
         }
     }
     return best;
@@ -196,25 +199,32 @@ void launch(Ctx& ctx, GemmArgs g, int64_t nz) {
         ctx.ensure(ctx.f64_partial, (size_t)(parts * g.M * g.N) * sizeof(double));
         g.partial = ctx.f64_partial.as<double>();
     }
-    dim3 grid((unsigned)std::min<int64_t>(g.tiles, 1 << 30), 1, (unsigned)parts);
+    // a conditional product that is normally skipped launches few blocks
+    const int64_t most = g.only_if ? 8 * ctx.sm_count : 1 << 30;
+    dim3 grid((unsigned)std::min<int64_t>(g.tiles, most), 1, (unsigned)parts);
     k_gemm_f64<T, R, BK><<<grid, NT, 0, ctx.stream>>>(g);
     TRG_LAUNCHED(ctx);
     if (parts > 1) {
         const int64_t tot = g.M * g.N;
         k_reduce_partials<<<(unsigned)((tot + 255) / 256), 256, 0, ctx.stream>>>(g.partial, (int)parts, g.M, g.N, g.C,
-                                                                              g.c_m, g.c_n, g.beta);
+                                                                              g.c_m, g.c_n, g.beta, g.only_if);
         TRG_LAUNCHED(ctx);
     }
 }
 
 }  // namespace
 
-void gemm_f64(Ctx& ctx, const GemmDesc& d) {
+double f64_us(const Ctx& ctx, int64_t M, int64_t N, int64_t K, bool sym) {
+    return choose_shape(M, N, std::max<int64_t>(K, 1), ctx.sm_count, sym).clocks / 1900.0 + 3.0;
+}
+
+void gemm_f64(Ctx& ctx, const GemmDesc& d, const int* only_if) {
     if (d.M <= 0 || d.N <= 0) return;
     GemmArgs g;
     g.M = d.M; g.N = d.N; g.K = d.K;
     g.kper = std::max<int64_t>(d.K, 1);
     g.partial = nullptr;
+    g.only_if = only_if;
     g.A = d.A.base; g.a_m = d.A.off_r; g.a_k = d.A.off_c; g.a_kfast = d.A.c_fast ? 1 : 0;
     g.B = d.B.base; g.b_k = d.B.off_r; g.b_n = d.B.off_c; g.b_nfast = d.B.c_fast ? 1 : 0;
     g.C = d.C; g.c_m = d.c_m; g.c_n = d.c_n; g.beta = d.beta;

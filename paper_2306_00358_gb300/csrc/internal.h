@@ -81,6 +81,7 @@ struct Ctx {
     // split products: limit of the epilogue's wait for a finished accumulator
     // chunk in ns (0 = the kernel's default of 2 s); see trg_set_wait_limit
     unsigned long long acc_wait_ns = 0;
+    bool no_exact = false;   // FP64 products stay on the FP64 pipe (no room for their digits)
 
     // ---- solve state
     bool have_tensor = false;
@@ -171,6 +172,7 @@ struct Gather {
     const int64_t* off_c;   // col offsets   (A: k, B: n, C: n)
     bool c_fast;            // consecutive columns are adjacent in memory
     bool c_identity = false;   // off_c[k] == k: every row is one contiguous run
+    bool r_fast = false;       // consecutive rows are adjacent in memory
 };
 struct GemmDesc {
     int64_t M, N, K;
@@ -183,6 +185,12 @@ struct GemmDesc {
     // over several CTAs per tile when its tiles cannot fill the SMs (the
     // n x m products of the isometry); exact partial sums, deterministic.
     bool allow_ksplit = false;
+    // FP64 mode: the product may run on the tensor cores when it is large
+    // enough (gemm_exact): an error of a few 2^-64 K times the largest entries
+    // of the row and the column, far below the FP64 pipe's on the method's
+    // operands, but relative to those entries and not to each |a||b|.
+    bool allow_exact = false;
+    bool c_m_fast = false;  // consecutive rows are (mostly) adjacent in C
     // The split epilogue may store without staging when consecutive rows are
     // adjacent in C and c_n[n + j] = c_n[n] + j c_col_stride inside each
     // aligned group of 32 columns.
@@ -236,7 +244,14 @@ void split_slice_operand(Ctx& ctx, const Gather& A, int64_t M, int64_t K, uint16
 void split_slice_b(Ctx& ctx, const Gather& B, int64_t K, int64_t N, uint16_t* slices, int* e);
 int64_t split_cols_padded(int64_t N);
 void gemm(Ctx& ctx, const GemmDesc& g, int precision);
-void gemm_f64(Ctx& ctx, const GemmDesc& g);
+// only_if: device flag; the product is computed only if it is set.
+void gemm_f64(Ctx& ctx, const GemmDesc& g, const int* only_if = nullptr);
+double f64_us(const Ctx& ctx, int64_t M, int64_t N, int64_t K, bool sym);   // modelled time of gemm_f64
+// FP64 product from exact BF16 digit products (exact_gemm.cu); false if its
+// scratch cannot be had (nothing computed).
+bool gemm_exact(Ctx& ctx, const GemmDesc& g);
+double exact_us(const Ctx& ctx, int64_t M, int64_t N, int64_t K, bool sym);
+int64_t exact_scratch_bytes(int64_t M, int64_t N, int64_t K);
 
 // Table helpers: enumerate all index tuples of `modes` (size, stride),
 // first mode slowest, and return the device table of offsets.

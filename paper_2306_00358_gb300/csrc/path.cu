@@ -57,6 +57,7 @@ static Gather gather(Ctx& ctx, const double* base, const Modes& rows, const Mode
     g.off_c = ctx.table(cols);
     g.c_fast = unit_first_stride(cols);
     g.c_identity = cols.size() == 1 && cols[0].second == 1;
+    g.r_fast = unit_first_stride(rows);
     return g;
 }
 
@@ -65,8 +66,18 @@ void gemm_split(Ctx& ctx, const GemmDesc& g);  // split_gemm.cu
 void gemm(Ctx& ctx, const GemmDesc& g, int precision) {
     // products inside the isometry are timed as part of that phase
     const int tok = (ctx.phase == TRG_PHASE_EIG) ? -1 : ctx.region_begin(ctx.phase);
-    if (precision == TRG_FP64) gemm_f64(ctx, g);
-    else if (precision == TRG_SPLIT_BF16) gemm_split(ctx, g);
+    if (precision == TRG_FP64) {
+        // the tensor cores once they are modelled to be well ahead of the
+        // FP64 pipe.  Their fixed cost is six launches (25 us in the model)
+        // and the digits; the lines cross at about 200 x 200 x 200.  The
+        // three products of a (24, 22) environment (528 and 576 wide) take
+        // 651 us on the pipe and 250 us on the tensor cores, 256 x 40 x 256
+        // 10 us against more than 30.
+        const bool sym = g.gram && g.M == g.N;
+        const bool exact = g.allow_exact && !ctx.no_exact && g.beta == 0.0 && g.M > 0 && g.N > 0 &&
+                           exact_us(ctx, g.M, g.N, g.K, sym) < 0.8 * f64_us(ctx, g.M, g.N, g.K, sym);
+        if (!exact || !gemm_exact(ctx, g)) gemm_f64(ctx, g);
+    } else if (precision == TRG_SPLIT_BF16) gemm_split(ctx, g);
     else fail(TRG_EINVAL, "unknown precision mode");
     ctx.region_end(tok, 2.0 * (double)g.M * (double)g.N * (double)g.K, 0.0);
 }
@@ -103,6 +114,7 @@ void environment(Ctx& ctx, const View4& t, double* M, int precision) {
         g.C = P; g.c_m = ctx.table({{DD, DD}}); g.c_n = ctx.table({{DD, 1}});
         g.beta = 0.0;
         g.gram = true;          // P = A A^T (the SYRK of the environment)
+        g.allow_exact = true;
         gemm(ctx, g, precision);
     }
     {   // Q: rows (i,e), k (c,d), cols (k,f)
@@ -114,6 +126,7 @@ void environment(Ctx& ctx, const View4& t, double* M, int precision) {
         g.C = Q; g.c_m = ctx.table({{DD, DD}}); g.c_n = ctx.table({{DD, 1}});
         g.beta = 0.0;
         g.gram = true;          // Q = A A^T
+        g.allow_exact = true;
         gemm(ctx, g, precision);
     }
     {   // M: rows (i,k), k (e,f), cols (j,l); stored M[(i,j),(k,l)]
@@ -125,6 +138,7 @@ void environment(Ctx& ctx, const View4& t, double* M, int precision) {
         g.c_m = ctx.table({{Dx, Dx * Dx * Dx}, {Dx, Dx}});
         g.c_n = ctx.table({{Dx, Dx * Dx}, {Dx, 1}});
         g.beta = 0.0;
+        g.allow_exact = true;
         gemm(ctx, g, precision);
     }
 }
@@ -233,6 +247,7 @@ void contract(Ctx& ctx, const View4& top, const View4& bottom, const double* U, 
             ctx.phase = TRG_PHASE_X1;
             GemmDesc g;
             g.M = Dx * Dn; g.N = jn * DD; g.K = Dx;
+            g.allow_exact = true;
             g.A = a1;
             g.a_slices = p1.s;
             g.a_e = p1.e;
@@ -256,6 +271,7 @@ void contract(Ctx& ctx, const View4& top, const View4& bottom, const double* U, 
                 g.c_m = ctx.table({{Dn, Dx * DD}, {Dx, 1}});
                 g.c_n = ctx.table({{jb, Dn * Dx * DD}, {Dx, DD}, {Dy, Dx}});
                 g.c_rows_fast = Dy % 32 == 0;
+                g.c_m_fast = true;
                 g.c_col_stride = Dx;
                 if (split) {
                     TRG_CUDA(cudaMemsetAsync(ef2, 0, (size_t)rows2 * sizeof(int), ctx.stream));
@@ -270,6 +286,7 @@ void contract(Ctx& ctx, const View4& top, const View4& bottom, const double* U, 
             // rows (jj,i,d), d fastest; columns (l,e), e fastest
             ctx.phase = TRG_PHASE_X2;
             GemmDesc g;
+            g.allow_exact = true;
             g.M = M2; g.N = DD; g.K = DD;
             g.A = gather(ctx, X1, {{jb * Dn * Dx, DD}}, {{DD, 1}});
             g.B = b2;
@@ -300,6 +317,7 @@ void contract(Ctx& ctx, const View4& top, const View4& bottom, const double* U, 
                 g.c_m = ctx.table({{jb * Dn, Dy * Dx * Dx}, {Dx, 1}});
                 g.c_n = ctx.table({{Dy, Dx * Dx}, {Dx, Dx}});
                 g.c_rows_fast = Dx % 32 == 0;
+                g.c_m_fast = true;
                 g.c_col_stride = Dx;
                 if (split) {
                     TRG_CUDA(cudaMemsetAsync(ef3, 0, (size_t)rows3 * sizeof(int), ctx.stream));
@@ -313,6 +331,8 @@ void contract(Ctx& ctx, const View4& top, const View4& bottom, const double* U, 
         {   // O[i,j0+jj,k,l] = sum_{e,d} X2[(jj,i,l),(e,d)] U[e,d,k]
             ctx.phase = TRG_PHASE_X3;
             GemmDesc g;
+            g.allow_exact = true;
+            g.c_m_fast = o[3] == 1;
             g.M = M3; g.N = Dn; g.K = Dx * Dx;
             g.A = gather(ctx, X2, {{jb * Dn * Dy, Dx * Dx}}, {{Dx * Dx, 1}});
             g.B = b3;

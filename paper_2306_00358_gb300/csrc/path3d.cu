@@ -46,6 +46,10 @@ void product(Ctx& ctx, const double* A, const Modes& ar, const Modes& ak, const 
     g.c_m = ctx.table(cr);
     g.c_n = ctx.table(cc);
     g.beta = 0.0;
+    g.A.r_fast = !ar.empty() && ar.back().second == 1 && ar.back().first > 1;
+    g.B.r_fast = !bk.empty() && bk.back().second == 1 && bk.back().first > 1;
+    g.c_m_fast = !cr.empty() && cr.back().second == 1 && cr.back().first > 1;
+    g.allow_exact = true;
     gemm(ctx, g, precision);
 }
 

@@ -58,3 +58,76 @@ def test_environment_matches_torch(torch, dx, dy):
     # three products in a row, of lengths dx dy (twice) and dy dy, on each side
     bound = 2.0 * (2 * (dx * dy + 1) + dy * dy + 1) * 1.01 * 2.0 ** -53 * env(t.abs())
     assert bool(((m - env(t)).abs() <= bound).all())
+
+
+def _contract(torch, t, u):
+    # Tx[i,j,k,l] = sum U[a,b,i] t[b,j,d,c] t[a,c,e,l] U[e,d,k], step by step
+    x1 = torch.einsum("abi,bjdc->ijdac", u, t)
+    x2 = torch.einsum("ijdac,acel->ijdel", x1, t)
+    return torch.einsum("ijdel,edk->ijkl", x2, u)
+
+
+# large enough for the tensor-core form: remainders of the 128 x 64 tile, of
+# the 32-deep stages and the 128-deep exact runs; 32: the row-wise stores.
+# The tensor-core form is off by at most 2^-53 |C| + 10 K 2^-64 times the
+# largest entries of the row and the column of each product, for entries of
+# like size far below the chain bound of test_product_matches_torch.
+@pytest.mark.parametrize("dx,dy,dn", [(16, 17, 15), (20, 13, 33), (24, 24, 24), (27, 21, 11), (32, 32, 32)])
+@pytest.mark.parametrize("ws", [0, 40_000_000])
+def test_contraction_matches_torch(torch, dx, dy, dn, ws):
+    rng = np.random.default_rng(dx * dy + dn)
+    t = torch.from_numpy(rng.standard_normal((dx, dy, dx, dy))).cuda()
+    u = torch.from_numpy(rng.standard_normal((dx, dx, dn))).cuda()
+    with Solver(0, workspace_bytes=ws) as s:
+        out = s.contract(t, u)
+    bound = 2.0 * (dx + 1 + dx * dy + 1 + dx * dx + 1) * 1.01 * 2.0 ** -53 * _contract(torch, t.abs(), u.abs())
+    assert bool(((out - _contract(torch, t, u)).abs() <= bound).all())
+
+
+# operands outside the digits' range take the FP64 pipe
+@pytest.mark.parametrize("scale", [2.0 ** 420, 2.0 ** -420, 2.0 ** -480])
+def test_contraction_outside_the_digit_range(torch, scale):
+    rng = np.random.default_rng(5)
+    d = 24
+    t = torch.from_numpy(rng.standard_normal((d, d, d, d))).cuda()
+    u = torch.from_numpy(rng.standard_normal((d, d, d))).cuda()
+    with Solver(0) as s:
+        out = s.contract(t * scale, u)
+    k = d + 1 + 2 * (d * d + 1)
+    bound = 2.0 * k * 1.01 * 2.0 ** -53 * _contract(torch, t.abs(), u.abs())
+    assert bool(((out / scale / scale - _contract(torch, t, u)).abs() <= bound).all())
+
+
+@pytest.mark.parametrize("value", [float("inf"), float("-inf"), float("nan")])
+def test_contraction_carries_infinities_and_nan(torch, value):
+    rng = np.random.default_rng(6)
+    d = 24
+    t = torch.from_numpy(rng.standard_normal((d, d, d, d))).cuda()
+    u = torch.from_numpy(rng.standard_normal((d, d, d))).cuda()
+    t[3, 4, 5, 6] = value
+    with Solver(0) as s:
+        out = s.contract(t, u)
+    ref = _contract(torch, t, u)
+    assert bool((torch.isnan(out) == torch.isnan(ref)).all())
+    assert bool((torch.isinf(out) == torch.isinf(ref)).all())
+
+
+@pytest.mark.parametrize("zero_rows", [True, False])
+def test_environment_of_a_sparse_tensor(torch, zero_rows):
+    """Zero rows and columns (exponent field 0) and entries 2^-70 below the largest."""
+    rng = np.random.default_rng(8)
+    d = 24
+    t = rng.standard_normal((d, d, d, d))
+    if zero_rows:
+        t[5] = 0.0
+        t[:, 7] = 0.0
+    t[9] *= 2.0 ** -70
+    t = torch.from_numpy(t).cuda()
+    with Solver(0) as s:
+        m = s.environment(t)
+    a = t.permute(0, 3, 1, 2).reshape(d * d, d * d)
+    c = t.reshape(d * d, d * d)
+    p, q = (a @ a.T).reshape(d, d, d, d), (c @ c.T).reshape(d, d, d, d)
+    ref = torch.einsum("iekf,jelf->ijkl", q, p).reshape(d * d, d * d)
+    # of the largest element: three products, each within (K + 1) 2^-53 on both sides
+    assert float((m - ref).abs().max()) <= 2.0 * 3 * (d * d + 1) * 2.0 ** -53 * float(ref.abs().max())
