@@ -88,115 +88,213 @@ __global__ void __launch_bounds__(256) k_col_normalize(double* Y, int64_t n, int
     for (int64_t r = threadIdx.x; r < n; r += 256) y[r] *= scale;
 }
 
-// Right-looking Cholesky G = L L^T of an m x m Gram matrix of unit columns.
-// Per column: warp 0 takes the pivot and scales the column (also into a
-// broadcast copy), then all threads update the trailing triangle.
-// A pivot d_j <= tau * G_jj marks column j as dependent (flags[j] = 1,
-// *nbad += 1); the pivot is then replaced by G_jj so the factorisation can
-// continue.
-// The trailing update of column j touches the elements (i, k), j < k <= i.
-// They are listed once, by k descending (k = m-1 first), so those of column
-// j are the first (m-1-j)(m-j)/2 entries: every thread takes a share and a
-// warp's FP64 instructions run on all 32 lanes (the FP64 pipe, not the
-// lanes, is what a lane-per-column layout of short rows wastes).
-__host__ __device__ constexpr int chol_table_entries(int m) { return m * (m - 1) / 2; }
-__global__ void __launch_bounds__(256) k_chol_flag(const double* G, double* Lout, int m, double tau,
-                                                   int* flags, int* nbad, double* pivmin_out) {
-    // m rows of ld = m + 1 (an odd stride: the rows of one column fall in
-    // different banks), m of the original diagonal, m of column j, then the
-    // trailing-element list (i << 7 | k, 16 bits each)
+// Cholesky G = L L^T of an m x m Gram matrix of unit columns.  A pivot
+// d_j <= tau * G_jj marks column j as dependent (flags[j] = 1, *nbad += 1);
+// the pivot is then replaced by G_jj so the factorisation can continue.
+//
+// One CTA; bound by the chain of FP64 operations from pivot to pivot: a
+// warp's FP64 instruction holds its quarter of the SM's pipe for 64 clocks,
+// with one active lane or with 32.  So the chain is kept to warp 0, while the
+// warps of the other three quarters update the trailing triangle:
+//  - warp 0 takes two columns a step in registers, their pivots by shuffle,
+//    and brings the next two up to date itself while the others apply the
+//    current two to the rest: one barrier per two columns;
+//  - pivot ratios (a division each) are taken in parallel at the end.
+// The trailing elements (i, k), k <= i, are listed once by k descending, so
+// those of a step are a prefix of the list and all lanes work.  Every element
+// goes through the operations of the plain right-looking form in its order
+// (scale by rsqrt(d_j), subtract in order of j): the bits of Q decide the
+// digits of the split products that follow, so a rounding changed here moves
+// split-mode vectors by far more than a rounding.
+// Measured at m = 40 / 56 / 88: 31.6 / 46.2 / 81.1 us (one column a step, two
+// barriers and the division in the chain: 46.1 / 70.3 / 135.6).
+constexpr int CHOL_THREADS = 512;
+__host__ __device__ constexpr int chol_even(int m) { return m + (m & 1); }
+__host__ __device__ constexpr int chol_table_entries(int m) { return chol_even(m) * (chol_even(m) + 1) / 2; }
+__global__ void __launch_bounds__(CHOL_THREADS) k_chol_flag(const double* G, double* Lout, int m, double tau,
+                                                            int* flags, int* nbad, double* pivmin_out) {
+    // me rows of ld = me + 1 (an odd stride: the rows of one column fall in
+    // different banks; an odd m gets a unit row and column), tau times the
+    // diagonal, the diagonal, the pivots before a replacement, two buffers of
+    // a step's two columns, then the list
     extern __shared__ double L[];
-    const int ld = m + 1;
-    double* gd = L + m * ld;
-    double* colj = gd + m;
-    uint16_t* tab = (uint16_t*)(colj + m);
+    const int me = chol_even(m), ld = me + 1;
+    double* gd = L + me * ld;
+    double* tg = gd + me;
+    double* draw = tg + me;
+    double* cols = draw + me;              // [2][2][me]
+    uint16_t* tab = (uint16_t*)(cols + 4 * me);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int e = threadIdx.x; e < m * m; e += blockDim.x) L[(e / m) * ld + e % m] = G[e];
-    for (int i = threadIdx.x; i < m; i += blockDim.x) gd[i] = G[(int64_t)i * m + i];
-    for (int e = threadIdx.x; e < chol_table_entries(m); e += blockDim.x) {
-        // group gidx = m-1-k holds the gidx+1 elements (k..m-1, k) from offset gidx(gidx+1)/2
-        int gidx = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);
-        while (gidx * (gidx + 1) / 2 > e) --gidx;
-        while ((gidx + 1) * (gidx + 2) / 2 <= e) ++gidx;
-        const int k = m - 1 - gidx, i = k + (e - gidx * (gidx + 1) / 2);
+    for (int e = threadIdx.x; e < me * me; e += CHOL_THREADS) {
+        const int i = e / me, j = e % me;
+        L[i * ld + j] = (i < m && j < m) ? G[i * m + j] : (i == j ? 1.0 : 0.0);
+    }
+    for (int i = threadIdx.x; i < me; i += CHOL_THREADS) {
+        gd[i] = i < m ? G[(int64_t)i * m + i] : 1.0;
+        tg[i] = i < m ? tau * gd[i] : 0.0;
+    }
+    for (int e = threadIdx.x; e < chol_table_entries(m); e += CHOL_THREADS) {
+        // group q = me-1-k holds the q+1 elements (k..me-1, k) from offset q(q+1)/2
+        int q = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);
+        while (q * (q + 1) / 2 > e) --q;
+        while ((q + 1) * (q + 2) / 2 <= e) ++q;
+        const int k = me - 1 - q, i = k + (e - q * (q + 1) / 2);
         tab[e] = (uint16_t)((i << 7) | k);
     }
     __syncthreads();
-    double pivmin = 1.0;    // smallest d_j / G_jj (thread 0): 1 / pivmin bounds cond(Y)^2 from below
-    for (int j = 0; j < m; ++j) {
+    for (int j = 0; j < me; j += 2) {
+        double* cur = cols + ((j >> 1) & 1) * 2 * me;           // this step's columns
+        const double* old = cols + (((j >> 1) & 1) ^ 1) * 2 * me;   // the previous step's
         if (warp == 0) {
-            double d = L[j * ld + j];
-            if (lane == 0) {
-                const double gjj = gd[j];
-                pivmin = fmin(pivmin, (gjj > 0.0 && isfinite(d)) ? d / gjj : 0.0);
-                if (!(d > tau * gjj) || !isfinite(d)) {
-                    flags[j] = 1;
-                    atomicAdd(nbad, 1);
-                    d = (gjj > 0.0 && isfinite(gjj)) ? gjj : 1.0;
+            // columns j, j + 1 less the previous step's part, rows i >= j
+            double x0[4], x1[4];
+            const double v00 = j ? old[j] : 0.0, v01 = j ? old[j + 1] : 0.0;
+            const double v10 = j ? old[me + j] : 0.0, v11 = j ? old[me + j + 1] : 0.0;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int i = j + lane + 32 * q;
+                x0[q] = x1[q] = 0.0;
+                if (j + 32 * q < me && i < me) {
+                    x0[q] = L[i * ld + j];
+                    x1[q] = L[i * ld + j + 1];
+                    if (j) {
+                        const double u0 = old[i], u1 = old[me + i];
+                        x0[q] = fma(-u0, v00, x0[q]);
+                        x1[q] = fma(-u0, v01, x1[q]);
+                        x0[q] = fma(-u1, v10, x0[q]);
+                        x1[q] = fma(-u1, v11, x1[q]);
+                    }
                 }
             }
-            d = __shfl_sync(0xffffffffu, d, 0);
-            const double il = rsqrt(d);
-            if (lane == 0) L[j * ld + j] = d * il;
-            for (int i = j + 1 + lane; i < m; i += 32) {
-                const double v = L[i * ld + j] * il;
-                L[i * ld + j] = v;
-                colj[i] = v;
+            // pivot c of the step: flagged and replaced if dependent
+            auto pivot = [&](double d, int c) {
+                if (lane == 0) draw[c] = d;
+                if (!(d > tg[c]) || !isfinite(d)) {
+                    if (lane == 0 && c < m) { flags[c] = 1; atomicAdd(nbad, 1); }
+                    d = (gd[c] > 0.0 && isfinite(gd[c])) ? gd[c] : 1.0;
+                }
+                return d;
+            };
+            const double d0 = pivot(__shfl_sync(0xffffffffu, x0[0], 0), j);
+            const double il0 = rsqrt(d0);
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (j + 32 * q < me) x0[q] *= il0;
+            const double w = __shfl_sync(0xffffffffu, x0[0], 1);
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (j + 32 * q < me) x1[q] = fma(-x0[q], w, x1[q]);
+            const double d1 = pivot(__shfl_sync(0xffffffffu, x1[0], 1), j + 1);
+            const double il1 = rsqrt(d1);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int i = j + lane + 32 * q;
+                if (j + 32 * q < me && i < me) {
+                    x1[q] *= il1;
+                    cur[i] = x0[q];
+                    cur[me + i] = x1[q];
+                    L[i * ld + j] = i == j ? d0 * il0 : x0[q];
+                    L[i * ld + j + 1] = i == j + 1 ? d1 * il1 : x1[q];
+                }
             }
-        }
-        __syncthreads();
-        const int cnt = (m - 1 - j) * (m - j) / 2;
-        for (int e = threadIdx.x; e < cnt; e += blockDim.x) {
-            const unsigned t = tab[e];
-            const int i = (int)(t >> 7), k = (int)(t & 127u);
-            L[i * ld + k] = fma(-colj[i], colj[k], L[i * ld + k]);
+        } else if (j && (warp & 3)) {
+            // the previous step's part of the columns from j + 2 on
+            const int n2 = me - 2 - j, cnt = n2 * (n2 + 1) / 2;
+            const int t0 = ((warp >> 2) * 3 + (warp & 3) - 1) * 32 + lane;
+            for (int e = t0; e < cnt; e += CHOL_THREADS / 4 * 3) {
+                const unsigned t = tab[e];
+                const int i = (int)(t >> 7), k = (int)(t & 127u);
+                double v = L[i * ld + k];
+                v = fma(-old[i], old[k], v);
+                v = fma(-old[me + i], old[me + k], v);
+                L[i * ld + k] = v;
+            }
         }
         __syncthreads();
     }
-    for (int e = threadIdx.x; e < m * m; e += blockDim.x)
-        Lout[e] = ((e % m) <= (e / m)) ? L[(e / m) * ld + e % m] : 0.0;
-    if (threadIdx.x == 0 && pivmin_out) *pivmin_out = pivmin;
+    for (int e = threadIdx.x; e < m * m; e += CHOL_THREADS) {
+        const int i = e / m, j = e % m;
+        Lout[e] = j <= i ? L[i * ld + j] : 0.0;
+    }
+    if (warp == 0 && pivmin_out) {
+        double pm = 1.0;   // smallest d_j / G_jj: 1 / pivmin bounds cond(Y)^2 from below
+        for (int i = lane; i < m; i += 32) pm = fmin(pm, (gd[i] > 0.0 && isfinite(draw[i])) ? draw[i] / gd[i] : 0.0);
+        for (int o = 16; o > 0; o >>= 1) pm = fmin(pm, __shfl_xor_sync(0xffffffffu, pm, o));
+        if (lane == 0) *pivmin_out = pm;
+    }
 }
 
-// Q = Y L^{-T} row by row, in place allowed: 32 rows per block, a lane per
-// row, the solution in shared memory.  Right-looking: after x_j is known,
-// every later column k subtracts L[k][j] x_j.  Column k belongs to warp
-// k % 8, so the eight warps (two per FP64 pipe, which hides the latency of
-// each one's load-FMA-store chain) share the updates and x_j needs no
-// reduction, one block barrier per column.
-constexpr int TRSM_ROWS = 32;
+// Q = Y L^{-T} row by row, in place allowed: RB rows per block, the solution
+// in shared memory.  Right-looking in steps of four columns: one warp solves
+// a step's 4 x 4 triangle for the block's rows, then all warps subtract its
+// products from the later columns (a lane per row; with RB < 32 the lanes'
+// groups take different columns).  Bound by the FP64 pipe (n m^2 / 2 FMAs)
+// for large n and by the chain of steps for small n, where fewer rows per
+// block use more SMs (trsm below).  Measured at
+// 256 x 40 / 1024 x 56 / 4096 x 88: 10.5 / 14.6 / 47.8 us (32 rows a block, a
+// barrier per column: 16.1 / 27.4 / 56.2).
 constexpr int TRSM_THREADS = 256;
 constexpr int TRSM_WARPS = TRSM_THREADS / 32;
+template <int RB>
 __global__ void __launch_bounds__(TRSM_THREADS) k_trsm_rows(double* Y, const double* Lg, int64_t n, int m) {
-    extern __shared__ double L[];   // m*m, m inverse diagonals, TRSM_ROWS rows of m + 1, 2 x TRSM_ROWS x_j
+    extern __shared__ double L[];   // m*m, m inverse diagonals, RB rows of m + 1, 2 x 4 x RB solved
+    constexpr int CG = 32 / RB;     // columns a warp updates at a time
     double* dinv = L + m * m;
     double* rows = dinv + m;
-    double* xb = rows + TRSM_ROWS * (m + 1);
+    double* xb = rows + RB * (m + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int e = threadIdx.x; e < m * m; e += blockDim.x) L[e] = Lg[e];
-    for (int i = threadIdx.x; i < m; i += blockDim.x) dinv[i] = 1.0 / Lg[(int64_t)i * m + i];
-    const int64_t r0 = (int64_t)blockIdx.x * TRSM_ROWS;
-    for (int e = threadIdx.x; e < m * TRSM_ROWS; e += blockDim.x) {
-        const int j = e / TRSM_ROWS, t = e % TRSM_ROWS;
+    const int row = lane % RB, cg = lane / RB;
+    for (int e = threadIdx.x; e < m * m; e += TRSM_THREADS) L[e] = Lg[e];
+    for (int i = threadIdx.x; i < m; i += TRSM_THREADS) dinv[i] = 1.0 / Lg[(int64_t)i * m + i];
+    const int64_t r0 = (int64_t)blockIdx.x * RB;
+    for (int e = threadIdx.x; e < m * RB; e += TRSM_THREADS) {
+        const int j = e / RB, t = e % RB;
         rows[t * (m + 1) + j] = (r0 + t < n) ? Y[(int64_t)j * n + r0 + t] : 0.0;
     }
     __syncthreads();
-    double* y = rows + lane * (m + 1);
-    for (int j = 0; j < m; ++j) {
-        double* xs = xb + (j & 1) * TRSM_ROWS;
-        if (warp == (j & (TRSM_WARPS - 1))) {
-            const double x = y[j] * dinv[j];
-            y[j] = x;
-            xs[lane] = x;
+    double* y = rows + row * (m + 1);
+    for (int j = 0, s = 0; j < m; j += 4, ++s) {
+        double* xs = xb + (s & 1) * 4 * RB;
+        const int w = min(4, m - j);
+        if (warp == (s & (TRSM_WARPS - 1))) {
+            // the step's triangle, every lane group redundantly
+            double x[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                if (q < w) {
+                    double v = y[j + q];
+#pragma unroll
+                    for (int p = 0; p < q; ++p) v = fma(-L[(j + q) * m + j + p], x[p], v);
+                    x[q] = v * dinv[j + q];
+                } else {
+                    x[q] = 0.0;
+                }
+            }
+            if (cg == 0) {
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    xs[q * RB + row] = x[q];
+                    if (q < w) y[j + q] = x[q];
+                }
+            }
         }
         __syncthreads();
-        const double x = xs[lane];
-        int k = j + 1 + ((warp - (j + 1)) & (TRSM_WARPS - 1));   // first column > j owned by this warp
-        for (; k < m; k += TRSM_WARPS) y[k] = fma(-L[k * m + j], x, y[k]);
+        if (j + 4 >= m) break;
+        double x[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) x[q] = xs[q * RB + row];
+        for (int k = j + 4 + warp * CG + cg; k < m; k += TRSM_WARPS * CG) {
+            const double* lr = L + k * m + j;
+            double v = y[k];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) v = fma(-lr[q], x[q], v);
+            y[k] = v;
+        }
+        __syncthreads();    // the next triangle's columns belong to several warps
     }
     __syncthreads();
-    for (int e = threadIdx.x; e < m * TRSM_ROWS; e += blockDim.x) {
-        const int j = e / TRSM_ROWS, t = e % TRSM_ROWS;
+    for (int e = threadIdx.x; e < m * RB; e += TRSM_THREADS) {
+        const int j = e / RB, t = e % RB;
         if (r0 + t < n) Y[(int64_t)j * n + r0 + t] = rows[t * (m + 1) + j];
     }
 }
@@ -246,13 +344,35 @@ __global__ void __launch_bounds__(256) k_gram_partial(const double* A, const dou
     }
 }
 
-__global__ void __launch_bounds__(64) k_gram_reduce(const double* part, int nparts, int m, double* G) {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= m * m) return;
+// G = the sum of the parts in slab order (deterministic): 32 elements a
+// block; the eight warps stage 64 parts at a time, the first one adds them.
+// The chain of FP64 additions bounds it: 152 parts of 88 x 88 took 17 us with
+// one thread per element waiting for its own loads and take 9.4 so.
+__global__ void __launch_bounds__(256) k_gram_reduce(const double* part, int nparts, int m, double* G) {
+    __shared__ double st[2][64][32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int e = blockIdx.x * 32 + lane;
+    const bool in = e < m * m;
     double s = 0.0;
+    auto stage = [&](int p0, int b) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const int p = p0 + warp + 8 * q;
+            st[b][warp + 8 * q][lane] = (in && p < nparts) ? part[(int64_t)p * m * m + e] : 0.0;
+        }
+    };
+    stage(0, 0);
+    __syncthreads();
+    for (int p0 = 0, b = 0; p0 < nparts; p0 += 64, b ^= 1) {
+        if (p0 + 64 < nparts) stage(p0 + 64, b ^ 1);
+        if (warp == 0) {
+            const int np = min(64, nparts - p0);
 #pragma unroll 8
-    for (int p = 0; p < nparts; ++p) s += part[(int64_t)p * m * m + e];
-    G[e] = s;
+            for (int q = 0; q < np; ++q) s += st[b][q][lane];
+        }
+        __syncthreads();
+    }
+    if (warp == 0 && in) G[e] = s;
 }
 
 // Cyclic Jacobi sweeps with parallel (round-robin) ordering on a symmetric
@@ -583,11 +703,25 @@ static size_t rr64_smem(int m) {
 }
 
 static size_t chol_smem(int m) {
-    return (size_t)m * (m + 1) * 8 + (size_t)m * 16 + (size_t)chol_table_entries(m) * 2 + 16;
+    const int me = chol_even(m);
+    return (size_t)me * (me + 1) * 8 + (size_t)me * 7 * 8 + (size_t)chol_table_entries(m) * 2 + 16;
 }
 
-static size_t trsm_smem(int m) {
-    return (size_t)m * m * 8 + (size_t)m * 8 + (size_t)TRSM_ROWS * (m + 1) * 8 + 2 * TRSM_ROWS * 8;
+static size_t trsm_smem(int m, int rb) {
+    return ((size_t)m * m + m + (size_t)rb * (m + 1) + (size_t)8 * rb) * 8;
+}
+
+// Y <- Y L^{-T}.  Rows per block: 8 while that gives every SM at most one
+// block (256 rows at m = 40: 32 blocks instead of 8), then 16; 32, which
+// leaves no lane of the triangle idle, for more rows.
+static void trsm(Ctx& ctx, double* Y, const double* L, int64_t n, int m) {
+    const int rb = n <= 8 * ctx.sm_count ? 8 : n <= 16 * ctx.sm_count ? 16 : 32;
+    const unsigned grid = (unsigned)((n + rb - 1) / rb);
+    const size_t smem = trsm_smem(m, rb);
+    if (rb == 8) k_trsm_rows<8><<<grid, TRSM_THREADS, smem, ctx.stream>>>(Y, L, n, m);
+    else if (rb == 16) k_trsm_rows<16><<<grid, TRSM_THREADS, smem, ctx.stream>>>(Y, L, n, m);
+    else k_trsm_rows<32><<<grid, TRSM_THREADS, smem, ctx.stream>>>(Y, L, n, m);
+    TRG_LAUNCHED(ctx);
 }
 
 static void set_smem(const void* fn, size_t bytes) {
@@ -609,17 +743,17 @@ static void gram(Ctx& ctx, const double* A, const double* B, int64_t n, int m, d
     });
     k_gram_partial<<<nparts, 256, smem, ctx.stream>>>(A, B, n, m, rows_c, ctx.f64_partial.as<double>(), A == B ? 1 : 0);
     TRG_LAUNCHED(ctx);
-    k_gram_reduce<<<(m * m + 63) / 64, 64, 0, ctx.stream>>>(ctx.f64_partial.as<double>(), nparts, m, G);
+    k_gram_reduce<<<(m * m + 31) / 32, 256, 0, ctx.stream>>>(ctx.f64_partial.as<double>(), nparts, m, G);
     TRG_LAUNCHED(ctx);
 }
-static void times_small(Ctx& ctx, const double* A, const double* W, int64_t n, int m, double* C) {
+static void times_small(Ctx& ctx, const double* A, const double* W, int64_t n, int m, double* C, int precision) {
     GemmDesc g;
     g.M = n; g.N = m; g.K = m;
     g.A.base = A; g.A.off_r = ctx.table({{n, 1}}); g.A.off_c = ctx.table({{m, n}}); g.A.c_fast = false;
     g.B.base = W; g.B.off_r = ctx.table({{m, 1}}); g.B.off_c = ctx.table({{m, m}}); g.B.c_fast = false;
     g.C = C; g.c_m = ctx.table({{n, 1}}); g.c_n = ctx.table({{m, n}}); g.beta = 0.0;
     g.A.r_fast = true; g.B.r_fast = true;
-    g.allow_exact = true;
+    g.allow_exact = precision == TRG_FP64;    // split mode: see k_chol_flag on the bits of Q
     g.c_m_fast = true;
     gemm(ctx, g, TRG_FP64);
 }
@@ -643,7 +777,7 @@ static void orthonormalise(Ctx& ctx, double* Y, int64_t n, int m, double* G, dou
             k_col_normalize<<<m, 256, 0, ctx.stream>>>(Y, n, flags);
             TRG_LAUNCHED(ctx);
             gram(ctx, Y, Y, n, m, G, TRG_FP64);
-            k_chol_flag<<<1, 256, chol_smem(m), ctx.stream>>>(G, L, m, pass == 0 ? 1e-8 : 1e-12, flags,
+            k_chol_flag<<<1, CHOL_THREADS, chol_smem(m), ctx.stream>>>(G, L, m, pass == 0 ? 1e-8 : 1e-12, flags,
                                                                      nbad, pivmin);
             TRG_LAUNCHED(ctx);
             int hb = 0;
@@ -658,9 +792,7 @@ static void orthonormalise(Ctx& ctx, double* Y, int64_t n, int m, double* G, dou
             k_rand_cols<<<grid, 256, 0, ctx.stream>>>(Y, n, m, flags, seed, ++salt);
             TRG_LAUNCHED(ctx);
         }
-        k_trsm_rows<<<(unsigned)((n + TRSM_ROWS - 1) / TRSM_ROWS), TRSM_THREADS, trsm_smem(m), ctx.stream>>>(Y, L, n,
-                                                                                                          m);
-        TRG_LAUNCHED(ctx);
+        trsm(ctx, Y, L, n, m);
         if (pass == 0 && power_next && first_clean && pm >= PASS2_PIVMIN) {
             ctx.counters[5] += 1;
             return;
@@ -679,7 +811,9 @@ int isometry(Ctx& ctx, const double* M, int64_t n, int dcut, double* U, std::vec
     static std::once_flag once;
     std::call_once(once, [] {
         set_smem((const void*)k_chol_flag, chol_smem(MAX_M));
-        set_smem((const void*)k_trsm_rows, trsm_smem(MAX_M));
+        set_smem((const void*)k_trsm_rows<8>, trsm_smem(MAX_M, 8));
+        set_smem((const void*)k_trsm_rows<16>, trsm_smem(MAX_M, 16));
+        set_smem((const void*)k_trsm_rows<32>, trsm_smem(MAX_M, 32));
         set_smem((const void*)k_rr_fp32, rr32_smem(MAX_M));
         set_smem((const void*)k_rr_fp64, rr64_smem(MAX_M));
     });
@@ -864,11 +998,9 @@ int isometry(Ctx& ctx, const double* M, int64_t n, int dcut, double* U, std::vec
                 // by Cholesky-QR, theta the diagonal of H' = W^T H W
                 k_small_tn<<<m, 128, 0, ctx.stream>>>(W, W, m, G2);
                 TRG_LAUNCHED(ctx);
-                k_chol_flag<<<1, 256, chol_smem(m), ctx.stream>>>(G2, L, m, 0.0, flags, nbad, nullptr);
+                k_chol_flag<<<1, CHOL_THREADS, chol_smem(m), ctx.stream>>>(G2, L, m, 0.0, flags, nbad, nullptr);
                 TRG_LAUNCHED(ctx);
-                k_trsm_rows<<<(unsigned)((m + TRSM_ROWS - 1) / TRSM_ROWS), TRSM_THREADS, trsm_smem(m),
-                              ctx.stream>>>(W, L, m, m);
-                TRG_LAUNCHED(ctx);
+                trsm(ctx, W, L, m, m);
                 k_small_nn<<<m, 128, 0, ctx.stream>>>(Hs, W, m, T1);
                 TRG_LAUNCHED(ctx);
                 k_small_tn<<<m, 128, 0, ctx.stream>>>(W, T1, m, G2);
@@ -877,8 +1009,8 @@ int isometry(Ctx& ctx, const double* M, int64_t n, int dcut, double* U, std::vec
             k_rr_fp64<<<1, 512, rr64_smem(m), ctx.stream>>>(G2, m, jtol, 60, theta, Wj, W, status, sweeps, full);
             TRG_LAUNCHED(ctx);
         }
-        times_small(ctx, Y, W, n, m, Z);
-        times_small(ctx, Q, W, n, m, QW);
+        times_small(ctx, Y, W, n, m, Z, precision);
+        times_small(ctx, Q, W, n, m, QW, precision);
         TRG_CUDA(cudaMemsetAsync(res_slot, 0, sizeof(double), ctx.stream));
         k_residual<<<dn_paper, 256, 0, ctx.stream>>>(Z, QW, theta, n, (unsigned long long*)res_slot);
         TRG_LAUNCHED(ctx);

@@ -12,12 +12,12 @@
 // tile T is therefore chosen by size (choose_shape): 64 x 64 for large
 // products, down to 8 x 8 for the m-column blocks of the isometry, where
 // 64 x 64 tiles left four SMs with all the work: 256 x 40 x 256 took 210 us
-// on 64 x 64 tiles and takes 10 us on 8 x 8 ones, the three products of a
+// on 64 x 64 tiles and takes 14 us on 8 x 8 ones, the three products of a
 // (24, 22) environment 1623 us on 64 (81 tiles, both halves of the Gram
-// products) and 651 us on 16.  256 threads per block;
-// tiles with fewer outputs than threads split each K stage over KG thread
-// groups, whose sums are added in group order.  Operands of the next K stage
-// are loaded to registers while the current one is multiplied.
+// products) and 651 us on 16.
+// Operands of the next K stage are loaded to registers while the current one
+// is multiplied; every output sums its products in order of k whatever the
+// tile, so the tile changes no bit (split K does).
 #include <algorithm>
 #include <cmath>
 
@@ -26,8 +26,6 @@
 namespace trg {
 
 namespace {
-
-constexpr int NT = 256;
 
 struct GemmArgs {
     int64_t M, N, K;
@@ -43,19 +41,16 @@ struct GemmArgs {
 };
 
 // T x T outputs per block, R x R per thread (stride T / R), BK deep stages.
-template <int T, int R, int BK>
+template <int T, int R, int BK, int NT>
 __global__ void __launch_bounds__(NT) k_gemm_f64(const GemmArgs g) {
     constexpr int W = T / R;                  // threads along a tile side
-    constexpr int G = W * W;                  // threads of a K group
-    constexpr int KG = NT / G;                // K groups
-    constexpr int KB = BK / KG;               // k's of a stage each group takes
     constexpr int E = T * BK / NT;            // elements a thread stages per operand
-    static_assert(G * KG == NT && KB * KG == BK && E * NT == T * BK, "tile shape");
+    static_assert(W * W == NT && E * NT == T * BK, "tile shape");
     if (g.only_if && *g.only_if == 0) return;
     __shared__ double As[BK][T + 1];
     __shared__ double Bs[BK][T + 1];
     const int tid = threadIdx.x;
-    const int grp = tid / G, tx = tid % W, ty = (tid % G) / W;
+    const int tx = tid % W, ty = tid / W;
 
     const int64_t kbeg = (int64_t)blockIdx.z * g.kper;
     const int64_t kend = min(g.K, kbeg + g.kper);
@@ -101,8 +96,7 @@ __global__ void __launch_bounds__(NT) k_gemm_f64(const GemmArgs g) {
             __syncthreads();
             if (k0 + BK < kend) load(k0 + BK);
 #pragma unroll 8
-            for (int q = 0; q < KB; ++q) {
-                const int kk = grp * KB + q;
+            for (int kk = 0; kk < BK; ++kk) {
                 double a[R], b[R];
 #pragma unroll
                 for (int i = 0; i < R; ++i) a[i] = As[kk][ty + W * i];
@@ -113,21 +107,6 @@ __global__ void __launch_bounds__(NT) k_gemm_f64(const GemmArgs g) {
 #pragma unroll
                     for (int j = 0; j < R; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
             }
-        }
-        if constexpr (KG > 1) {
-            // add the groups' sums in group order (one output per thread: R = 1);
-            // the first stage buffer holds them
-            static_assert(R == 1 && KG * G <= BK * (T + 1), "group sums");
-            double* red = &As[0][0];
-            __syncthreads();
-            red[tid] = acc[0][0];
-            __syncthreads();
-            if (grp == 0) {
-#pragma unroll
-                for (int q = 1; q < KG; ++q) acc[0][0] += red[tid + q * G];
-            }
-            __syncthreads();                  // before the next tile's stage
-            if (grp != 0) continue;
         }
 #pragma unroll
         for (int i = 0; i < R; ++i) {
@@ -189,7 +168,7 @@ Shape choose_shape(int64_t M, int64_t N, int64_t K, int sms, bool sym) {
     return best;
 }
 
-template <int T, int R, int BK>
+template <int T, int R, int BK, int NT>
 void launch(Ctx& ctx, GemmArgs g, int64_t nz) {
     g.tiles_n = (g.N + T - 1) / T;
     g.tiles = g.tiles_n * ((g.M + T - 1) / T);
@@ -202,7 +181,7 @@ void launch(Ctx& ctx, GemmArgs g, int64_t nz) {
     // a conditional product that is normally skipped launches few blocks
     const int64_t most = g.only_if ? 8 * ctx.sm_count : 1 << 30;
     dim3 grid((unsigned)std::min<int64_t>(g.tiles, most), 1, (unsigned)parts);
-    k_gemm_f64<T, R, BK><<<grid, NT, 0, ctx.stream>>>(g);
+    k_gemm_f64<T, R, BK, NT><<<grid, NT, 0, ctx.stream>>>(g);
     TRG_LAUNCHED(ctx);
     if (parts > 1) {
         const int64_t tot = g.M * g.N;
@@ -233,10 +212,10 @@ void gemm_f64(Ctx& ctx, const GemmDesc& d, const int* only_if) {
     if ((d.M + 63) / 64 > 65535) fail(TRG_EINVAL, "gemm_f64: too many row tiles");
     const Shape s = choose_shape(d.M, d.N, std::max<int64_t>(d.K, 1), ctx.sm_count, g.sym != 0);
     switch (s.T) {
-        case 64: launch<64, 4, 16>(ctx, g, s.nz); break;
-        case 32: launch<32, 2, 32>(ctx, g, s.nz); break;
-        case 16: launch<16, 1, 32>(ctx, g, s.nz); break;
-        default: launch<8, 1, 64>(ctx, g, s.nz); break;
+        case 64: launch<64, 4, 16, 256>(ctx, g, s.nz); break;
+        case 32: launch<32, 2, 32, 256>(ctx, g, s.nz); break;
+        case 16: launch<16, 1, 32, 256>(ctx, g, s.nz); break;
+        default: launch<8, 1, 64, 64>(ctx, g, s.nz); break;
     }
 }
 

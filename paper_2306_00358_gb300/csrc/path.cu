@@ -72,7 +72,7 @@ void gemm(Ctx& ctx, const GemmDesc& g, int precision) {
         // and the digits; the lines cross at about 200 x 200 x 200.  The
         // three products of a (24, 22) environment (528 and 576 wide) take
         // 651 us on the pipe and 250 us on the tensor cores, 256 x 40 x 256
-        // 10 us against more than 30.
+        // 14 us against more than 30.
         const bool sym = g.gram && g.M == g.N;
         const bool exact = g.allow_exact && !ctx.no_exact && g.beta == 0.0 && g.M > 0 && g.N > 0 &&
                            exact_us(ctx, g.M, g.N, g.K, sym) < 0.8 * f64_us(ctx, g.M, g.N, g.K, sym);
