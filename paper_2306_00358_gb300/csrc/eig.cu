@@ -17,6 +17,7 @@
 #include <mutex>
 
 #include "internal.h"
+#include "jacobi32.cuh"
 
 namespace trg {
 
@@ -375,25 +376,13 @@ __global__ void __launch_bounds__(256) k_gram_reduce(const double* part, int npa
     if (warp == 0 && in) G[e] = s;
 }
 
-// Cyclic Jacobi sweeps with parallel (round-robin) ordering on a symmetric
-// m x m matrix H (row-major, shared memory), accumulating W <- W J (W
-// column-major).  Rotation (p,q): tau = (h_qq - h_pp)/(2 h_pq),
-// t = sign(tau)/(|tau| + sqrt(1+tau^2)), c = 1/sqrt(1+t^2), s = t c;
-// H <- J^T H J.  Rotations with |h_pq| <= tol sqrt(|h_pp h_qq|) are skipped
-// (relative-accuracy threshold for graded matrices); the loop ends when no
-// pair is above the threshold.  Returns the number of sweeps that rotated
-// (max_sweeps + 1 if the limit was hit).  All threads of the block call it.
-__device__ __forceinline__ void rr_pair(int r, int i, int mp, int& p, int& q) {
-    if (i == 0) { p = mp - 1; q = r; }
-    else { p = (r + i) % (mp - 1); q = (r - i + (mp - 1)) % (mp - 1); }
-    if (p > q) { const int x = p; p = q; q = x; }
-}
-
-template <typename T>
-__device__ __forceinline__ bool jacobi_rotates(T hpq, T hpp, T hqq, T tol) {
-    return fabs(hpq) > tol * sqrt(fabs(hpp * hqq)) && fabs(hpq) > (T)1e-300;
-}
-
+// Cyclic Jacobi sweeps (FP64, and FP32 above JAC_PIPE_M) with the ordering and
+// rotations of jacobi32.cuh on a symmetric m x m matrix H (row-major, shared memory),
+// accumulating W <- W J (W column-major).  Rotations with |h_pq| <= tol
+// sqrt(|h_pp h_qq|) are skipped (relative-accuracy threshold for graded
+// matrices); the loop ends when no pair is above the threshold.  Returns the
+// number of sweeps that rotated (max_sweeps + 1 if the limit was hit).  All
+// threads of the block call it.
 template <typename T>
 __device__ int jacobi_sweeps(T* H, int ld, T* W, int m, T tol, int max_sweeps, T* cs, int* rot, int* pq) {
     const int mp = m + (m & 1);            // even player count (dummy index m when odd)
@@ -494,13 +483,15 @@ __device__ int jacobi_sweeps(T* H, int ld, T* W, int m, T tol, int max_sweeps, T
 __global__ void __launch_bounds__(512) k_rr_fp32(const double* Hg, int m, double* Hsym, double* Wout,
                                                  int* sweeps_out) {
     extern __shared__ double sm[];
-    const int mp = m + (m & 1);
     const int ld = m + 1;
-    float* H32 = (float*)sm;                   // m*ld floats
-    float* W32 = H32 + m * ld;                 // m*m floats
-    float* cs32 = W32 + m * m;                 // mp
+    const bool piped = m <= JAC_PIPE_M;
+    const int mp = m + (m & 1);
+    float* H32 = (float*)sm;                   // m*ld floats, twice when piped
+    float* W32 = H32 + (piped ? 2 : 1) * m * ld;   // m*m floats
+    float* cs32 = W32 + m * m;                 // plain: mp
     int* rot = (int*)(cs32 + mp + (mp & 1));   // 1
     int* pq = rot + 2;                         // mp: the pairs of the current round
+    __shared__ JacShared jac;
     __shared__ double hmax_s;
     if (threadIdx.x == 0) hmax_s = 0.0;
     __syncthreads();
@@ -521,7 +512,8 @@ __global__ void __launch_bounds__(512) k_rr_fp32(const double* Hg, int m, double
         W32[e] = (i == j) ? 1.0f : 0.0f;
     }
     __syncthreads();
-    const int s32 = jacobi_sweeps<float>(H32, ld, W32, m, 1e-6f, 40, cs32, rot, pq);
+    const int s32 = piped ? jacobi_sweeps_f32<512>(H32, H32 + m * ld, ld, W32, m, 1e-6f, 40, jac)
+                          : jacobi_sweeps<float>(H32, ld, W32, m, 1e-6f, 40, cs32, rot, pq);
     for (int e = threadIdx.x; e < m * m; e += blockDim.x) Wout[e] = (double)W32[e];
     if (threadIdx.x == 0 && sweeps_out) atomicAdd(sweeps_out, s32);
 }
@@ -694,7 +686,8 @@ __global__ void k_to_isometry(const double* QW, int64_t n, int dn, double* U) {
 
 static size_t rr32_smem(int m) {
     const int mp = m + (m & 1);
-    return (size_t)m * (m + 1) * 4 + (size_t)m * m * 4 + (size_t)(mp + 2) * 4 + (size_t)(mp + 4) * 4 + 64;
+    return (size_t)(m <= JAC_PIPE_M ? 2 : 1) * m * (m + 1) * 4 + (size_t)m * m * 4 + (size_t)(mp + 2) * 4 +
+           (size_t)(mp + 4) * 4 + 64;
 }
 
 static size_t rr64_smem(int m) {
@@ -814,7 +807,7 @@ int isometry(Ctx& ctx, const double* M, int64_t n, int dcut, double* U, std::vec
         set_smem((const void*)k_trsm_rows<8>, trsm_smem(MAX_M, 8));
         set_smem((const void*)k_trsm_rows<16>, trsm_smem(MAX_M, 16));
         set_smem((const void*)k_trsm_rows<32>, trsm_smem(MAX_M, 32));
-        set_smem((const void*)k_rr_fp32, rr32_smem(MAX_M));
+        set_smem((const void*)k_rr_fp32, std::max(rr32_smem(MAX_M), rr32_smem(JAC_PIPE_M)));
         set_smem((const void*)k_rr_fp64, rr64_smem(MAX_M));
     });
     // buffers: Q, Y, Z, QW (n x m each); G, L, W (m x m); theta (m)
