@@ -348,7 +348,10 @@ int trg_destroy(trg_ctx* ctx) {
         c.release(*b);
     for (trg::Buf& b : c.s3) c.release(b);
     for (auto& kv : c.tables) c.release(kv.second);
+    for (auto& kv : c.lists) c.release(kv.second);
     c.tables.clear();
+    c.lists.clear();
+    if (c.box) cudaFreeHost(c.box);
     try {
         c.collect_timings();   // a context whose stream has failed still frees its resources
     } catch (const trg::Error&) {
@@ -367,7 +370,7 @@ int trg_set_stream(trg_ctx* ctx, void* stream) {
 int trg_set_allocator(trg_ctx* ctx, trg_alloc_fn alloc, trg_free_fn free_fn, void* user) {
     if (!ctx || (!alloc) != (!free_fn)) return TRG_EINVAL;
     // only the two always-present scalar buffers exist at this point: move them
-    if (ctx->T.p || ctx->M.p || !ctx->tables.empty())
+    if (ctx->T.p || ctx->M.p || !ctx->tables.empty() || !ctx->lists.empty())
         return bad(ctx, TRG_ESTATE, "trg_set_allocator must come before any other call");
     TRG_GUARD_BEGIN
     TRG_CUDA(cudaStreamSynchronize(ctx->stream));

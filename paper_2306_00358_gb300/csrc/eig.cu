@@ -13,7 +13,9 @@
 // a fresh seeded random column (this happens when M's spectrum falls below
 // rounding, e.g. in the ordered phase).  All blocks are column-major (n x m).
 #include <algorithm>
+#include <chrono>
 #include <cmath>
+#include <cstring>
 #include <mutex>
 
 #include "internal.h"
@@ -63,6 +65,7 @@ __device__ double block_sum(double v, double* red) {
 __global__ void __launch_bounds__(256) k_col_normalize(double* Y, int64_t n, int* flags) {
     __shared__ double red[32];
     const int c = blockIdx.x;
+    if (threadIdx.x == 0) flags[c] = 0;
     double* y = Y + (int64_t)c * n;
     double mx = 0.0;
     for (int64_t r = threadIdx.x; r < n; r += 256) mx = fmax(mx, fabs(y[r]));
@@ -89,11 +92,32 @@ __global__ void __launch_bounds__(256) k_col_normalize(double* Y, int64_t n, int
     for (int64_t r = threadIdx.x; r < n; r += 256) y[r] *= scale;
 }
 
-// Cholesky G = L L^T of an m x m Gram matrix of unit columns.  A pivot
-// d_j <= tau * G_jj marks column j as dependent (flags[j] = 1, *nbad += 1);
-// the pivot is then replaced by G_jj so the factorisation can continue.
+// What the host reads of a solve while it runs: mapped host memory that the
+// deciding kernels write, `seq` last.
+struct EigBox {
+    unsigned long long seq;
+    int nbad;                 // dependent columns of the last Cholesky-QR pass
+    int status;
+    int sweeps[2];
+    double pivmin;            // its smallest pivot ratio d_j / G_jj
+    double res;
+    double theta[MAX_M];
+};
+__device__ __forceinline__ void box_done(EigBox* box, unsigned long long seq) {
+    __threadfence_system();
+    *(volatile unsigned long long*)&box->seq = seq;
+}
+
+// One Cholesky-QR pass after the Gram product: G = L L^T (m x m, unit
+// columns), then Y <- Y L^{-T} for the block's RB rows.  A pivot d_j <= tau *
+// G_jj marks column j as dependent (flags[j] = 1, counted in box->nbad); the
+// pivot is replaced by G_jj so the factorisation can continue, and Y is left
+// as it is unless `always`.  Every block factors G itself (the same bits), so
+// no launch and no host decision lies between the two parts; block 0 tells
+// the host (box, may be null) as soon as the pivots are known, while the
+// triangular solve still runs.
 //
-// One CTA; bound by the chain of FP64 operations from pivot to pivot: a
+// Factorisation.  Bound by the chain of FP64 operations from pivot to pivot: a
 // warp's FP64 instruction holds its quarter of the SM's pipe for 64 clocks,
 // with one active lane or with 32.  So the chain is kept to warp 0, while the
 // warps of the other three quarters update the trailing triangle:
@@ -107,25 +131,44 @@ __global__ void __launch_bounds__(256) k_col_normalize(double* Y, int64_t n, int
 // (scale by rsqrt(d_j), subtract in order of j): the bits of Q decide the
 // digits of the split products that follow, so a rounding changed here moves
 // split-mode vectors by far more than a rounding.
-// Measured at m = 40 / 56 / 88: 31.6 / 46.2 / 81.1 us (one column a step, two
-// barriers and the division in the chain: 46.1 / 70.3 / 135.6).
+//
+// Triangular solve.  Right-looking in steps of four columns: one warp solves
+// a step's 4 x 4 triangle for the block's rows, then all warps subtract its
+// products from the later columns (a lane per row; with RB < 32 the lanes'
+// groups take different columns).  Bound by the FP64 pipe (n m^2 / 2 FMAs)
+// for large n and by the chain of steps for small n, where fewer rows per
+// block use more SMs (chol_trsm below).
+// Measured, both parts, at 256 x 40 / 1024 x 56 / 4096 x 88: 39.9 / 58.0 / 124.7 us (as
+// two kernels 42 / 61 / 129, with one column a step, two barriers and the
+// division in the chain, 32 rows a block and a barrier per column 62 / 98 / 192).
 constexpr int CHOL_THREADS = 512;
 __host__ __device__ constexpr int chol_even(int m) { return m + (m & 1); }
 __host__ __device__ constexpr int chol_table_entries(int m) { return chol_even(m) * (chol_even(m) + 1) / 2; }
-__global__ void __launch_bounds__(CHOL_THREADS) k_chol_flag(const double* G, double* Lout, int m, double tau,
-                                                            int* flags, int* nbad, double* pivmin_out) {
+template <int RB>
+__global__ void __launch_bounds__(CHOL_THREADS) k_chol_trsm(const double* G, double* Y, int64_t n, int m, double tau,
+                                                            int always, int* flags, EigBox* box,
+                                                            unsigned long long seq) {
     // me rows of ld = me + 1 (an odd stride: the rows of one column fall in
     // different banks; an odd m gets a unit row and column), tau times the
     // diagonal, the diagonal, the pivots before a replacement, two buffers of
-    // a step's two columns, then the list
+    // a step's two columns, RB rows of Y, 2 x 4 x RB solved values, then the list
     extern __shared__ double L[];
+    __shared__ int bad_s;
     const int me = chol_even(m), ld = me + 1;
     double* gd = L + me * ld;
     double* tg = gd + me;
     double* draw = tg + me;
     double* cols = draw + me;              // [2][2][me]
-    uint16_t* tab = (uint16_t*)(cols + 4 * me);
+    double* rows = cols + 4 * me;
+    double* xb = rows + RB * (m + 1);
+    uint16_t* tab = (uint16_t*)(xb + 8 * RB);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t r0 = (int64_t)blockIdx.x * RB;
+    if (threadIdx.x == 0) bad_s = 0;
+    for (int e = threadIdx.x; e < m * RB; e += CHOL_THREADS) {
+        const int j = e / RB, t = e % RB;
+        rows[t * (m + 1) + j] = (r0 + t < n) ? Y[(int64_t)j * n + r0 + t] : 0.0;
+    }
     for (int e = threadIdx.x; e < me * me; e += CHOL_THREADS) {
         const int i = e / me, j = e % me;
         L[i * ld + j] = (i < m && j < m) ? G[i * m + j] : (i == j ? 1.0 : 0.0);
@@ -171,7 +214,10 @@ __global__ void __launch_bounds__(CHOL_THREADS) k_chol_flag(const double* G, dou
             auto pivot = [&](double d, int c) {
                 if (lane == 0) draw[c] = d;
                 if (!(d > tg[c]) || !isfinite(d)) {
-                    if (lane == 0 && c < m) { flags[c] = 1; atomicAdd(nbad, 1); }
+                    if (lane == 0 && c < m) {
+                        ++bad_s;
+                        if (blockIdx.x == 0) flags[c] = 1;
+                    }
                     d = (gd[c] > 0.0 && isfinite(gd[c])) ? gd[c] : 1.0;
                 }
                 return d;
@@ -213,51 +259,30 @@ __global__ void __launch_bounds__(CHOL_THREADS) k_chol_flag(const double* G, dou
         }
         __syncthreads();
     }
-    for (int e = threadIdx.x; e < m * m; e += CHOL_THREADS) {
-        const int i = e / m, j = e % m;
-        Lout[e] = j <= i ? L[i * ld + j] : 0.0;
-    }
-    if (warp == 0 && pivmin_out) {
-        double pm = 1.0;   // smallest d_j / G_jj: 1 / pivmin bounds cond(Y)^2 from below
+    const int bad = bad_s;
+    double* dinv = cols;                   // 1 / L_jj
+    if (blockIdx.x == 0 && box && warp == CHOL_THREADS / 32 - 1) {
+        double pm = 1.0;   // 1 / pivmin bounds cond(Y)^2 from below
         for (int i = lane; i < m; i += 32) pm = fmin(pm, (gd[i] > 0.0 && isfinite(draw[i])) ? draw[i] / gd[i] : 0.0);
         for (int o = 16; o > 0; o >>= 1) pm = fmin(pm, __shfl_xor_sync(0xffffffffu, pm, o));
-        if (lane == 0) *pivmin_out = pm;
+        if (lane == 0) {
+            box->nbad = bad;
+            box->pivmin = pm;
+            box_done(box, seq);
+        }
     }
-}
-
-// Q = Y L^{-T} row by row, in place allowed: RB rows per block, the solution
-// in shared memory.  Right-looking in steps of four columns: one warp solves
-// a step's 4 x 4 triangle for the block's rows, then all warps subtract its
-// products from the later columns (a lane per row; with RB < 32 the lanes'
-// groups take different columns).  Bound by the FP64 pipe (n m^2 / 2 FMAs)
-// for large n and by the chain of steps for small n, where fewer rows per
-// block use more SMs (trsm below).  Measured at
-// 256 x 40 / 1024 x 56 / 4096 x 88: 10.5 / 14.6 / 47.8 us (32 rows a block, a
-// barrier per column: 16.1 / 27.4 / 56.2).
-constexpr int TRSM_THREADS = 256;
-constexpr int TRSM_WARPS = TRSM_THREADS / 32;
-template <int RB>
-__global__ void __launch_bounds__(TRSM_THREADS) k_trsm_rows(double* Y, const double* Lg, int64_t n, int m) {
-    extern __shared__ double L[];   // m*m, m inverse diagonals, RB rows of m + 1, 2 x 4 x RB solved
-    constexpr int CG = 32 / RB;     // columns a warp updates at a time
-    double* dinv = L + m * m;
-    double* rows = dinv + m;
-    double* xb = rows + RB * (m + 1);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int row = lane % RB, cg = lane / RB;
-    for (int e = threadIdx.x; e < m * m; e += TRSM_THREADS) L[e] = Lg[e];
-    for (int i = threadIdx.x; i < m; i += TRSM_THREADS) dinv[i] = 1.0 / Lg[(int64_t)i * m + i];
-    const int64_t r0 = (int64_t)blockIdx.x * RB;
-    for (int e = threadIdx.x; e < m * RB; e += TRSM_THREADS) {
-        const int j = e / RB, t = e % RB;
-        rows[t * (m + 1) + j] = (r0 + t < n) ? Y[(int64_t)j * n + r0 + t] : 0.0;
-    }
+    if (bad && !always) return;
+    for (int i = threadIdx.x; i < m; i += CHOL_THREADS) dinv[i] = 1.0 / L[i * ld + i];
     __syncthreads();
+
+    constexpr int CG = 32 / RB;            // columns a warp updates at a time
+    constexpr int WARPS = CHOL_THREADS / 32;
+    const int row = lane % RB, cg = lane / RB;
     double* y = rows + row * (m + 1);
     for (int j = 0, s = 0; j < m; j += 4, ++s) {
         double* xs = xb + (s & 1) * 4 * RB;
         const int w = min(4, m - j);
-        if (warp == (s & (TRSM_WARPS - 1))) {
+        if (warp == (s & (WARPS - 1))) {
             // the step's triangle, every lane group redundantly
             double x[4];
 #pragma unroll
@@ -265,7 +290,7 @@ __global__ void __launch_bounds__(TRSM_THREADS) k_trsm_rows(double* Y, const dou
                 if (q < w) {
                     double v = y[j + q];
 #pragma unroll
-                    for (int p = 0; p < q; ++p) v = fma(-L[(j + q) * m + j + p], x[p], v);
+                    for (int p = 0; p < q; ++p) v = fma(-L[(j + q) * ld + j + p], x[p], v);
                     x[q] = v * dinv[j + q];
                 } else {
                     x[q] = 0.0;
@@ -284,8 +309,8 @@ __global__ void __launch_bounds__(TRSM_THREADS) k_trsm_rows(double* Y, const dou
         double x[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) x[q] = xs[q * RB + row];
-        for (int k = j + 4 + warp * CG + cg; k < m; k += TRSM_WARPS * CG) {
-            const double* lr = L + k * m + j;
+        for (int k = j + 4 + warp * CG + cg; k < m; k += WARPS * CG) {
+            const double* lr = L + k * ld + j;
             double v = y[k];
 #pragma unroll
             for (int q = 0; q < 4; ++q) v = fma(-lr[q], x[q], v);
@@ -293,8 +318,7 @@ __global__ void __launch_bounds__(TRSM_THREADS) k_trsm_rows(double* Y, const dou
         }
         __syncthreads();    // the next triangle's columns belong to several warps
     }
-    __syncthreads();
-    for (int e = threadIdx.x; e < m * RB; e += TRSM_THREADS) {
+    for (int e = threadIdx.x; e < m * RB; e += CHOL_THREADS) {
         const int j = e / RB, t = e % RB;
         if (r0 + t < n) Y[(int64_t)j * n + r0 + t] = rows[t * (m + 1) + j];
     }
@@ -668,6 +692,21 @@ __global__ void __launch_bounds__(256) k_residual(const double* Z, const double*
     }
 }
 
+// The outcome of a Rayleigh-Ritz step for the host.
+__global__ void __launch_bounds__(128) k_tell(const double* theta, const double* res, const int* sweeps,
+                                              const int* status, int m, EigBox* box, unsigned long long seq) {
+    if (threadIdx.x < m) box->theta[threadIdx.x] = theta[threadIdx.x];
+    if (threadIdx.x == 0) {
+        box->res = *res;
+        box->sweeps[0] = sweeps[0];
+        box->sweeps[1] = sweeps[1];
+        box->status = *status;
+    }
+    __threadfence_system();
+    __syncthreads();
+    if (threadIdx.x == 0) box_done(box, seq);
+}
+
 // Y <- Y - sigma Q (the shift of a power step)
 __global__ void k_shift(double* Y, const double* Q, double sigma, int64_t count) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x)
@@ -695,25 +734,40 @@ static size_t rr64_smem(int m) {
     return (size_t)2 * m * (m + 1) * 8 + (size_t)mp * 8 + (size_t)(m + 4) * 4 + (size_t)mp * 4 + 64;
 }
 
-static size_t chol_smem(int m) {
+static size_t chol_smem(int m, int rb) {
     const int me = chol_even(m);
-    return (size_t)me * (me + 1) * 8 + (size_t)me * 7 * 8 + (size_t)chol_table_entries(m) * 2 + 16;
+    return ((size_t)me * (me + 1) + (size_t)me * 7 + (size_t)rb * (m + 1) + (size_t)8 * rb) * 8 +
+           (size_t)chol_table_entries(m) * 2 + 16;
 }
 
-static size_t trsm_smem(int m, int rb) {
-    return ((size_t)m * m + m + (size_t)rb * (m + 1) + (size_t)8 * rb) * 8;
+// Wait until the kernel that was given `seq` has written the box: the host
+// needs its few numbers to go on, but not the rest of the kernel.  Spins on
+// the mapped word (tens of microseconds as a rule), then waits for the stream.
+static const EigBox& wait_box(Ctx& ctx, unsigned long long seq) {
+    EigBox* box = (EigBox*)ctx.box;
+    const auto t0 = std::chrono::steady_clock::now();
+    for (;;) {
+        for (int i = 0; i < 512; ++i)
+            if (__atomic_load_n(&box->seq, __ATOMIC_ACQUIRE) == seq) return *box;
+        if (std::chrono::steady_clock::now() - t0 > std::chrono::milliseconds(2)) break;
+    }
+    TRG_CUDA(cudaStreamSynchronize(ctx.stream));
+    if (__atomic_load_n(&box->seq, __ATOMIC_ACQUIRE) != seq) fail(TRG_ECUDA, "isometry: no answer from the device");
+    return *box;
 }
 
-// Y <- Y L^{-T}.  Rows per block: 8 while that gives every SM at most one
-// block (256 rows at m = 40: 32 blocks instead of 8), then 16; 32, which
-// leaves no lane of the triangle idle, for more rows.
-static void trsm(Ctx& ctx, double* Y, const double* L, int64_t n, int m) {
+// Factor G and Y <- Y L^{-T}.  Rows per block: 8 while that gives every SM at
+// most one block (256 rows at m = 40: 32 blocks instead of 8), then 16; 32,
+// which leaves no lane of the triangle idle, for more rows.
+static void chol_trsm(Ctx& ctx, const double* G, double* Y, int64_t n, int m, double tau, bool always, int* flags,
+                      EigBox* box, unsigned long long seq) {
     const int rb = n <= 8 * ctx.sm_count ? 8 : n <= 16 * ctx.sm_count ? 16 : 32;
     const unsigned grid = (unsigned)((n + rb - 1) / rb);
-    const size_t smem = trsm_smem(m, rb);
-    if (rb == 8) k_trsm_rows<8><<<grid, TRSM_THREADS, smem, ctx.stream>>>(Y, L, n, m);
-    else if (rb == 16) k_trsm_rows<16><<<grid, TRSM_THREADS, smem, ctx.stream>>>(Y, L, n, m);
-    else k_trsm_rows<32><<<grid, TRSM_THREADS, smem, ctx.stream>>>(Y, L, n, m);
+    const size_t smem = chol_smem(m, rb);
+    const int al = always ? 1 : 0;
+    if (rb == 8) k_chol_trsm<8><<<grid, CHOL_THREADS, smem, ctx.stream>>>(G, Y, n, m, tau, al, flags, box, seq);
+    else if (rb == 16) k_chol_trsm<16><<<grid, CHOL_THREADS, smem, ctx.stream>>>(G, Y, n, m, tau, al, flags, box, seq);
+    else k_chol_trsm<32><<<grid, CHOL_THREADS, smem, ctx.stream>>>(G, Y, n, m, tau, al, flags, box, seq);
     TRG_LAUNCHED(ctx);
 }
 
@@ -758,25 +812,20 @@ static void times_small(Ctx& ctx, const double* A, const double* W, int64_t n, i
 // which needs only a well-conditioned basis, a clean first pass with
 // pivots above PASS2_PIVMIN is enough and the second pass is skipped.
 constexpr double PASS2_PIVMIN = 1e-3;
-static void orthonormalise(Ctx& ctx, double* Y, int64_t n, int m, double* G, double* L, int* flags,
-                           int* nbad, uint64_t seed, uint64_t& salt, bool power_next = false) {
-    double* pivmin = ctx.scal.as<double>() + SC_PIVMIN;
-    double pm = 0.0;
+static void orthonormalise(Ctx& ctx, double* Y, int64_t n, int m, double* G, int* flags, uint64_t seed,
+                           uint64_t& salt, bool power_next = false) {
     bool first_clean = true;    // the first pass needed no column repair
     for (int pass = 0; pass < 2; ++pass) {
-        int attempt = 0;
-        for (;; ++attempt) {
-            TRG_CUDA(cudaMemsetAsync(flags, 0, (size_t)(m + 1) * sizeof(int), ctx.stream));
+        double pm = 0.0;
+        for (int attempt = 0;; ++attempt) {
             k_col_normalize<<<m, 256, 0, ctx.stream>>>(Y, n, flags);
             TRG_LAUNCHED(ctx);
             gram(ctx, Y, Y, n, m, G, TRG_FP64);
-            k_chol_flag<<<1, CHOL_THREADS, chol_smem(m), ctx.stream>>>(G, L, m, pass == 0 ? 1e-8 : 1e-12, flags,
-                                                                     nbad, pivmin);
-            TRG_LAUNCHED(ctx);
-            int hb = 0;
-            TRG_CUDA(cudaMemcpyAsync(&hb, nbad, sizeof(int), cudaMemcpyDeviceToHost, ctx.stream));
-            TRG_CUDA(cudaMemcpyAsync(&pm, pivmin, sizeof(double), cudaMemcpyDeviceToHost, ctx.stream));
-            TRG_CUDA(cudaStreamSynchronize(ctx.stream));
+            const unsigned long long seq = ++ctx.box_seq;
+            chol_trsm(ctx, G, Y, n, m, pass == 0 ? 1e-8 : 1e-12, false, flags, (EigBox*)ctx.box_dev, seq);
+            const EigBox& box = wait_box(ctx, seq);
+            pm = box.pivmin;
+            const int hb = box.nbad;
             if (hb == 0) break;
             if (pass == 0) first_clean = false;
             ctx.counters[4] += (uint64_t)hb;
@@ -785,7 +834,6 @@ static void orthonormalise(Ctx& ctx, double* Y, int64_t n, int m, double* G, dou
             k_rand_cols<<<grid, 256, 0, ctx.stream>>>(Y, n, m, flags, seed, ++salt);
             TRG_LAUNCHED(ctx);
         }
-        trsm(ctx, Y, L, n, m);
         if (pass == 0 && power_next && first_clean && pm >= PASS2_PIVMIN) {
             ctx.counters[5] += 1;
             return;
@@ -803,10 +851,9 @@ int isometry(Ctx& ctx, const double* M, int64_t n, int dcut, double* U, std::vec
     const int m = (int)std::min<int64_t>({n, (int64_t)dn_paper + std::max(1, ctx.cfg.oversample), (int64_t)MAX_M});
     static std::once_flag once;
     std::call_once(once, [] {
-        set_smem((const void*)k_chol_flag, chol_smem(MAX_M));
-        set_smem((const void*)k_trsm_rows<8>, trsm_smem(MAX_M, 8));
-        set_smem((const void*)k_trsm_rows<16>, trsm_smem(MAX_M, 16));
-        set_smem((const void*)k_trsm_rows<32>, trsm_smem(MAX_M, 32));
+        set_smem((const void*)k_chol_trsm<8>, chol_smem(MAX_M, 8));
+        set_smem((const void*)k_chol_trsm<16>, chol_smem(MAX_M, 16));
+        set_smem((const void*)k_chol_trsm<32>, chol_smem(MAX_M, 32));
         set_smem((const void*)k_rr_fp32, std::max(rr32_smem(MAX_M), rr32_smem(JAC_PIPE_M)));
         set_smem((const void*)k_rr_fp64, rr64_smem(MAX_M));
     });
@@ -819,8 +866,7 @@ int isometry(Ctx& ctx, const double* M, int64_t n, int dcut, double* U, std::vec
     double* Z = Y + n * m;
     double* QW = Z + n * m;
     double* G = ctx.eig_small.as<double>();
-    double* L = G + m * m;
-    double* W = L + m * m;
+    double* W = G + m * m;
     double* theta = W + m * m;
     double* Hs = theta + 2 * m + 8;    // Rayleigh-Ritz scratch: symmetrised H, H W, Gram matrices
     double* T1 = Hs + m * m;
@@ -829,9 +875,13 @@ int isometry(Ctx& ctx, const double* M, int64_t n, int dcut, double* U, std::vec
     double* E = Pm + m * m;            // its correction
     double* Xb = E + m * m;            // a second basis buffer
     int* flags = ctx.flags.as<int>();
-    int* nbad = flags + m;
     int* sweeps = flags + m + 2;   // [0] FP32 sweeps, [1] FP64 sweeps of the last Rayleigh-Ritz
 
+    if (!ctx.box) {
+        TRG_CUDA(cudaHostAlloc(&ctx.box, sizeof(EigBox), cudaHostAllocMapped | cudaHostAllocPortable));
+        std::memset(ctx.box, 0, sizeof(EigBox));
+        TRG_CUDA(cudaHostGetDevicePointer(&ctx.box_dev, ctx.box, 0));
+    }
     int* status = ctx.status.as<int>();
     double* res_slot = ctx.scal.as<double>() + SC_RES;
     const uint64_t seed = ctx.cfg.seed ^ (0xA24BAED4963EE407ull * (uint64_t)step);
@@ -900,13 +950,13 @@ int isometry(Ctx& ctx, const double* M, int64_t n, int dcut, double* U, std::vec
     double sigma = (have_hint && hint.theta_m > 0.0) ? 0.5 * hint.theta_m : 0.0;
     // the start block is followed by power steps unless the first step is a
     // Rayleigh-Ritz step (no plan and m = n)
-    orthonormalise(ctx, Q, n, m, G, L, flags, nbad, seed, salt, have_hint || m < n);
+    orthonormalise(ctx, Q, n, m, G, flags, seed, salt, have_hint || m < n);
     int applied = 0;                 // products of M in the span of Q
     if (!have_hint) {
         for (int pre = 0; pre < 2 && m < n; ++pre) {
             apply_m(0.0);
             std::swap(Q, Y);
-            orthonormalise(ctx, Q, n, m, G, L, flags, nbad, seed, salt, pre == 0);
+            orthonormalise(ctx, Q, n, m, G, flags, seed, salt, pre == 0);
             ++applied;
         }
     }
@@ -932,7 +982,7 @@ int isometry(Ctx& ctx, const double* M, int64_t n, int dcut, double* U, std::vec
         if (pending > 0) {
             apply_m(sigma);
             std::swap(Q, Y);
-            orthonormalise(ctx, Q, n, m, G, L, flags, nbad, seed, salt, pending > 1);
+            orthonormalise(ctx, Q, n, m, G, flags, seed, salt, pending > 1);
             --pending;
             ++since_rr;
             ++applied;
@@ -991,9 +1041,7 @@ int isometry(Ctx& ctx, const double* M, int64_t n, int dcut, double* U, std::vec
                 // by Cholesky-QR, theta the diagonal of H' = W^T H W
                 k_small_tn<<<m, 128, 0, ctx.stream>>>(W, W, m, G2);
                 TRG_LAUNCHED(ctx);
-                k_chol_flag<<<1, CHOL_THREADS, chol_smem(m), ctx.stream>>>(G2, L, m, 0.0, flags, nbad, nullptr);
-                TRG_LAUNCHED(ctx);
-                trsm(ctx, W, L, m, m);
+                chol_trsm(ctx, G2, W, m, m, 0.0, true, flags, nullptr, 0);
                 k_small_nn<<<m, 128, 0, ctx.stream>>>(Hs, W, m, T1);
                 TRG_LAUNCHED(ctx);
                 k_small_tn<<<m, 128, 0, ctx.stream>>>(W, T1, m, G2);
@@ -1007,17 +1055,19 @@ int isometry(Ctx& ctx, const double* M, int64_t n, int dcut, double* U, std::vec
         TRG_CUDA(cudaMemsetAsync(res_slot, 0, sizeof(double), ctx.stream));
         k_residual<<<dn_paper, 256, 0, ctx.stream>>>(Z, QW, theta, n, (unsigned long long*)res_slot);
         TRG_LAUNCHED(ctx);
-        double res = 0.0;
-        int hsw[2] = {0, 0};
-        TRG_CUDA(cudaMemcpyAsync(th.data(), theta, (size_t)m * sizeof(double), cudaMemcpyDeviceToHost, ctx.stream));
-        TRG_CUDA(cudaMemcpyAsync(&res, res_slot, sizeof(double), cudaMemcpyDeviceToHost, ctx.stream));
-        TRG_CUDA(cudaMemcpyAsync(hsw, sweeps, 2 * sizeof(int), cudaMemcpyDeviceToHost, ctx.stream));
-        TRG_CUDA(cudaStreamSynchronize(ctx.stream));
+        const unsigned long long seq = ++ctx.box_seq;
+        k_tell<<<1, 128, 0, ctx.stream>>>(theta, res_slot, sweeps, status, m, (EigBox*)ctx.box_dev, seq);
+        TRG_LAUNCHED(ctx);
+        const EigBox& box = wait_box(ctx, seq);
+        std::copy(box.theta, box.theta + m, th.begin());
+        const double res = box.res;
+        const int hsw[2] = {box.sweeps[0], box.sweeps[1]};
+        const int st = box.status;
         ctx.counters[0] += 1;
         ctx.counters[1] += 1;
         ctx.counters[2] += (uint64_t)hsw[0];
         ctx.counters[3] += (uint64_t)hsw[1];
-        if (read_status(ctx) & ST_EIG_NOCONV) fail(TRG_ENUMERIC, "Rayleigh-Ritz Jacobi did not converge");
+        if (st & ST_EIG_NOCONV) fail(TRG_ENUMERIC, "Rayleigh-Ritz Jacobi did not converge");
         if (!(th[0] > 0.0) || !std::isfinite(th[0])) fail(TRG_ENUMERIC, "environment has no positive eigenvalue");
         if ((res <= tol && full) || m == n) {
             {
@@ -1064,7 +1114,7 @@ int isometry(Ctx& ctx, const double* M, int64_t n, int dcut, double* U, std::vec
         // next block: orth(Y W) = orth(M Q W), same span as M Q
         ++applied;
         std::swap(Q, Z);
-        orthonormalise(ctx, Q, n, m, G, L, flags, nbad, seed, salt, pending > 0);
+        orthonormalise(ctx, Q, n, m, G, flags, seed, salt, pending > 0);
     }
     fail(TRG_ENUMERIC, "subspace iteration did not converge");
 }

@@ -240,7 +240,9 @@ void trim_buffers(Ctx& c) {
         c.release(*b);
     for (Buf& b : c.s3) c.release(b);
     for (auto& kv : c.tables) c.release(kv.second);
+    for (auto& kv : c.lists) c.release(kv.second);
     c.tables.clear();
+    c.lists.clear();
     c.have_tensor = false;
 }
 

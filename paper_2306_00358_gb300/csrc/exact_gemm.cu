@@ -503,8 +503,8 @@ void digits(Ctx& ctx, const Gather& g, int R, int K, int Rp, int Kp, int* ef, ui
 
 const long long* diagonal_tiles(Ctx& ctx, int tiles_m, int tiles_n, int& n) {
     const std::string key = "xsym:" + std::to_string(tiles_m) + ":" + std::to_string(tiles_n);
-    auto it = ctx.tables.find(key);
-    if (it == ctx.tables.end()) {
+    auto it = ctx.lists.find(key);
+    if (it == ctx.lists.end()) {
         std::vector<long long> h;
         for (int mb = 0; mb < tiles_m; ++mb)
             for (int nb = 0; nb < tiles_n; ++nb)
@@ -513,7 +513,7 @@ const long long* diagonal_tiles(Ctx& ctx, int tiles_m, int tiles_n, int& n) {
         ctx.ensure(buf, h.size() * sizeof(long long));
         TRG_CUDA(cudaMemcpyAsync(buf.p, h.data(), h.size() * sizeof(long long), cudaMemcpyHostToDevice, ctx.stream));
         TRG_CUDA(cudaStreamSynchronize(ctx.stream));   // h dies here
-        it = ctx.tables.emplace(key, buf).first;
+        it = ctx.lists.emplace(key, buf).first;
         ctx.list_len[key] = (int)h.size();
     }
     n = ctx.list_len[key];

@@ -116,7 +116,8 @@ struct Ctx {
     Buf cons_ef;           // exponent fields recorded by a producing product (two halves)
     Buf eig_slices;        // split mode: M sliced once per isometry solve
     Buf s3[10];            // cubic-lattice step: P1, P2, Ux, Uy, Mx, My, then A, W, C, D of the contraction
-    std::map<std::string, Buf> tables;  // cached offset tables (and tile lists)
+    std::map<std::vector<std::pair<int64_t, int64_t>>, Buf> tables;   // cached offset tables
+    std::map<std::string, Buf> lists;      // cached tile lists
     std::map<std::string, int> list_len;   // entries of the cached tile lists
 
     // ---- phase timing
@@ -137,6 +138,10 @@ struct Ctx {
     // predecessor needed and that solve's smallest Ritz value theta_m
     struct EigHint { int64_t n = -1; int m = -1; int precision = -1; int products = 0; double theta_m = 0.0; };
     EigHint eig_hint[2];
+    // mapped host memory the isometry's kernels answer to (EigBox, eig.cu)
+    void* box = nullptr;
+    void* box_dev = nullptr;
+    unsigned long long box_seq = 0;
     cudaEvent_t get_event();
     // Record the start of a timed region of phase p (no-op unless profiling).
     int region_begin(int p);
@@ -158,7 +163,6 @@ enum : int {
     SC_TRACE = 3,     // last trace
     SC_RES = 4,       // max Ritz residual / lambda_1 (subspace iteration)
     SC_TRACE_IMP = 5, // last trace of the impure tensor
-    SC_PIVMIN = 6,    // smallest pivot ratio d_j / G_jj of the last Cholesky-QR pass
     SC_COUNT = 8
 };
 

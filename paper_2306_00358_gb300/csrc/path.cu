@@ -3,7 +3,6 @@
 // turn the index wiring (and the y-direction rotation) into plain GEMMs.
 #include <algorithm>
 #include <cstring>
-#include <sstream>
 
 #include "internal.h"
 
@@ -28,9 +27,7 @@ std::vector<int64_t> build_table(const std::vector<std::pair<int64_t, int64_t>>&
 }
 
 const int64_t* Ctx::table(const std::vector<std::pair<int64_t, int64_t>>& modes) {
-    std::ostringstream key;
-    for (auto& m : modes) key << m.first << ':' << m.second << ';';
-    auto it = tables.find(key.str());
+    auto it = tables.find(modes);
     if (it != tables.end()) return it->second.as<int64_t>();
     std::vector<int64_t> h = build_table(modes);
     Buf b;
@@ -39,7 +36,7 @@ const int64_t* Ctx::table(const std::vector<std::pair<int64_t, int64_t>>& modes)
         TRG_CUDA(cudaMemcpyAsync(b.p, h.data(), h.size() * sizeof(int64_t), cudaMemcpyHostToDevice, stream));
     // the host vector dies here: wait for the copy (tables are built once per shape)
     TRG_CUDA(cudaStreamSynchronize(stream));
-    tables[key.str()] = b;
+    tables[modes] = b;
     return b.as<int64_t>();
 }
 

@@ -1497,8 +1497,8 @@ void gemm_split(Ctx& ctx, const GemmDesc& d) {
             b.group_n = gn;
             const std::string key = "sym:" + std::to_string(tiles_m) + ":" + std::to_string(tiles_n) + ":" +
                                     std::to_string(gn) + ":" + std::to_string(tile_m);
-            auto it = ctx.tables.find(key);
-            if (it == ctx.tables.end()) {
+            auto it = ctx.lists.find(key);
+            if (it == ctx.lists.end()) {
                 std::vector<long long> h;
                 for (int t = 0; t < tiles_m * tiles_n; ++t) {
                     int mb, nb;
@@ -1510,7 +1510,7 @@ void gemm_split(Ctx& ctx, const GemmDesc& d) {
                 TRG_CUDA(cudaMemcpyAsync(buf.p, h.data(), h.size() * sizeof(long long), cudaMemcpyHostToDevice,
                                          ctx.stream));
                 TRG_CUDA(cudaStreamSynchronize(ctx.stream));   // h dies here
-                it = ctx.tables.emplace(key, buf).first;
+                it = ctx.lists.emplace(key, buf).first;
                 ctx.list_len[key] = (int)h.size();
             }
             b.tile_list = it->second.as<long long>();
