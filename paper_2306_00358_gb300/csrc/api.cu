@@ -343,7 +343,7 @@ int trg_destroy(trg_ctx* ctx) {
     cudaStreamSynchronize(ctx->stream);
     Ctx& c = *ctx;
     for (trg::Buf* b : {&c.T, &c.Tnext, &c.M, &c.U, &c.scal, &c.status, &c.ws, &c.envP, &c.envQ, &c.eig,
-                        &c.eig_small, &c.flags, &c.split_ws, &c.f64_partial, &c.ksplit_ws, &c.bslices, &c.cons_ef, &c.Timp, &c.Timp_next,
+                        &c.eig_small, &c.flags, &c.split_ws, &c.f64_partial, &c.ksplit_ws, &c.bslices, &c.cons_ef, &c.field_ws, &c.Timp, &c.Timp_next,
                         &c.Timp_tmp, &c.eig_slices})
         c.release(*b);
     for (trg::Buf& b : c.s3) c.release(b);
@@ -757,6 +757,7 @@ int trg_gemm(trg_ctx* ctx, int M, int N, int K, const double* A, int lda, const 
     trg::GemmDesc g;
     g.M = M; g.N = N; g.K = K;
     g.A.base = A; g.A.off_r = ctx->table({{M, lda}}); g.A.off_c = ctx->table({{K, 1}}); g.A.c_fast = true;
+    g.A.c_identity = true;
     g.B.base = B; g.B.off_r = ctx->table({{K, ldb}}); g.B.off_c = ctx->table({{N, 1}}); g.B.c_fast = true;
     g.C = C; g.c_m = ctx->table({{M, ldc}}); g.c_n = ctx->table({{N, 1}}); g.beta = 0.0;
     ctx->phase = TRG_PHASE_X2;

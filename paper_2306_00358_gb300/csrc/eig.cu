@@ -799,7 +799,8 @@ static void times_small(Ctx& ctx, const double* A, const double* W, int64_t n, i
     g.A.base = A; g.A.off_r = ctx.table({{n, 1}}); g.A.off_c = ctx.table({{m, n}}); g.A.c_fast = false;
     g.B.base = W; g.B.off_r = ctx.table({{m, 1}}); g.B.off_c = ctx.table({{m, m}}); g.B.c_fast = false;
     g.C = C; g.c_m = ctx.table({{n, 1}}); g.c_n = ctx.table({{m, n}}); g.beta = 0.0;
-    g.A.r_fast = true; g.B.r_fast = true;
+    g.A.r_fast = true; g.A.r_identity = true;
+    g.B.r_fast = true; g.B.r_identity = true;
     g.allow_exact = precision == TRG_FP64;    // split mode: see k_chol_flag on the bits of Q
     g.c_m_fast = true;
     gemm(ctx, g, TRG_FP64);
@@ -917,7 +918,7 @@ int isometry(Ctx& ctx, const double* M, int64_t n, int dcut, double* U, std::vec
         g.a_e = m_e;
         g.B.base = Q; g.B.off_r = ctx.table({{n, 1}}); g.B.off_c = ctx.table({{m, n}}); g.B.c_fast = false;
         g.C = Y; g.c_m = ctx.table({{n, 1}}); g.c_n = ctx.table({{m, n}}); g.beta = 0.0;
-        g.B.r_fast = true;
+        g.B.r_fast = true; g.B.r_identity = true;
         g.allow_exact = true;
         g.c_m_fast = true;
         g.allow_ksplit = true;    // n / 128 tiles of 128 x m: K is split over the idle SMs

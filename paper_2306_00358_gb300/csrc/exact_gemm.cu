@@ -40,6 +40,7 @@
 #include <cmath>
 
 #include "internal.h"
+#include "slicing.cuh"
 #include "tcgen05.cuh"
 
 namespace trg {
@@ -354,124 +355,6 @@ k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     }
 }
 
-// ------------------------------------------------------------- digits ----
-// Largest exponent field of each row r of the gathered operand src[off_r[r] +
-// off_c[k]] (subnormals count as field 1), maxima into ef (zeroed).  HBM-bound;
-// a warp reads along the index that is adjacent in memory.
-constexpr int XF_K = 256;
-__global__ void __launch_bounds__(256) k_row_field(const double* __restrict__ src, const int64_t* __restrict__ off_r,
-                                                   const int64_t* __restrict__ off_c, int R, int K, int k_fast,
-                                                   int* __restrict__ ef) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int k0 = blockIdx.x * XF_K, k1 = min(K, k0 + XF_K);
-    auto field = [](double x) -> unsigned {
-        const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-        const unsigned hi = (unsigned)(b >> 32) & 0x7fffffffu;
-        return hi >= 0x100000u ? hi >> 20 : ((hi | (unsigned)b) ? 1u : 0u);
-    };
-    for (int r0 = blockIdx.y * 32; r0 < R; r0 += gridDim.y * 32) {
-        if (k_fast) {
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int r = r0 + warp * 4 + i;
-                if (r >= R) break;
-                const double* row = src + off_r[r];
-                unsigned f = 0;
-#pragma unroll 8
-                for (int k = k0 + lane; k < k1; k += 32) f = max(f, field(row[off_c[k]]));
-                f = __reduce_max_sync(0xffffffffu, f);
-                if (lane == 0 && f) atomicMax(&ef[r], (int)f);
-            }
-        } else {
-            __shared__ unsigned red[8][32];
-            const int r = r0 + lane;
-            unsigned f = 0;
-            if (r < R) {
-                const double* row = src + off_r[r];
-#pragma unroll 8
-                for (int k = k0 + warp; k < k1; k += 8) f = max(f, field(row[off_c[k]]));
-            }
-            red[warp][lane] = f;
-            __syncthreads();
-            if (warp == 0) {
-#pragma unroll
-                for (int w = 1; w < 8; ++w) f = max(f, red[w][lane]);
-                if (r < R && f) atomicMax(&ef[r], (int)f);
-            }
-            __syncthreads();
-        }
-    }
-}
-
-// The eight digits (BF16) of each element: out[p][r][k], r < Rp, k < Kp, zero
-// in the padding.  Elements pass through a 32 x 64 shared tile so that both
-// sides are coalesced; a thread cuts eight adjacent k and writes 16 bytes per
-// digit.  Rows outside the digits' range raise *bad.  HBM-bound: 8 B read,
-// 16 B written per element.
-constexpr int XD_R = 32, XD_K = 64, XD_LD = XD_K + XD_K / 8 + 1;
-constexpr int FIELD_LO = 1023 - 400, FIELD_HI = 1023 + 400;
-__global__ void __launch_bounds__(256) k_digits8(const double* __restrict__ src, const int64_t* __restrict__ off_r,
-                                                 const int64_t* __restrict__ off_c, int R, int K, int Rp, int Kp,
-                                                 int k_fast, const int* __restrict__ ef, uint16_t* __restrict__ out,
-                                                 int* bad) {
-    __shared__ double tile[XD_R * XD_LD];
-    const int k0 = blockIdx.x * XD_K;
-    const size_t plane = (size_t)Rp * Kp;
-    for (int r0 = blockIdx.y * XD_R; r0 < Rp; r0 += gridDim.y * XD_R) {
-        __syncthreads();
-#pragma unroll
-        for (int q = 0; q < XD_R * XD_K / 256; ++q) {
-            const int e = threadIdx.x + q * 256;
-            int rr, kk;
-            if (k_fast) { kk = e % XD_K; rr = e / XD_K; } else { rr = e % XD_R; kk = e / XD_R; }
-            const int r = r0 + rr, k = k0 + kk;
-            tile[rr * XD_LD + kk + (kk >> 3)] = (r < R && k < K) ? src[off_r[r] + off_c[k]] : 0.0;
-        }
-        __syncthreads();
-        const int rr = threadIdx.x >> 3, kg = threadIdx.x & 7;
-        const int r = r0 + rr, k = k0 + kg * 8;
-        if (r >= Rp || k >= Kp) continue;
-        const int f = r < R ? ef[r] : 0;
-        if (f && (f < FIELD_LO || f > FIELD_HI)) *bad = 1;
-        const double* x = tile + rr * XD_LD + kg * 9;
-        uint32_t w[XS][4];
-#pragma unroll
-        for (int h = 0; h < 4; ++h) {
-            float d[2][XS];
-#pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                const unsigned long long b = (unsigned long long)__double_as_longlong(x[2 * h + u]);
-                const int ex = (int)((b >> 52) & 0x7FF);
-                const int sh = f - ex - 10;              // X = mantissa 2^-sh
-                unsigned long long m = ex ? ((b & ((1ull << 52) - 1)) | (1ull << 52)) : 0ull;
-                m = sh <= 0 ? m << (-sh & 63) : sh < 60 ? (m + (1ull << (sh - 1))) >> sh : 0ull;
-                const bool neg = (long long)b < 0;
-                // adding 128 to every digit but the first turns the signed
-                // digits into bytes; the first is the signed top byte, whose
-                // sign bit is part of the value when X >= 0
-                const unsigned long long y = (neg ? 0ull - m : m) + 0x0080808080808080ull;
-                const unsigned ylo = (unsigned)y, yhi = (unsigned)(y >> 32);
-                const int top = neg ? (int)yhi >> 24 : (int)(yhi >> 24);
-                d[u][0] = (float)top;
-#pragma unroll
-                for (int p = 1; p < XS; ++p) {
-                    const unsigned byte = p < 4 ? __byte_perm(yhi, 0x4B000000u, 0x7440u | (unsigned)(3 - p))
-                                                : __byte_perm(ylo, 0x4B000000u, 0x7440u | (unsigned)(7 - p));
-                    d[u][p] = __uint_as_float(byte) - 8388736.0f;   // 2^23 + 128
-                }
-            }
-#pragma unroll
-            for (int p = 0; p < XS; ++p) {
-                // exact in BF16: the upper halves of the two FP32 values
-                w[p][h] = __byte_perm(__float_as_uint(d[0][p]), __float_as_uint(d[1][p]), 0x7632);
-            }
-        }
-        uint16_t* o = out + (size_t)r * Kp + k;
-#pragma unroll
-        for (int p = 0; p < XS; ++p) *reinterpret_cast<uint4*>(o + p * plane) = make_uint4(w[p][0], w[p][1], w[p][2], w[p][3]);
-    }
-}
-
 // ------------------------------------------------------------- host side ---
 // Digit planes [XS][rows][kp] as a 3D map, boxes of box_rows x XK of every digit.
 CUtensorMap digit_map(const void* base, int rows, int kp, int box_rows) {
@@ -492,12 +375,15 @@ int64_t up(int64_t v, int64_t q) { return (v + q - 1) / q * q; }
 
 // Exponent fields and digits of rows [0, R) of an operand.
 void digits(Ctx& ctx, const Gather& g, int R, int K, int Rp, int Kp, int* ef, uint16_t* out, int* bad) {
+    if (g.c_identity && Kp <= CUT_ROWS_MAX_K) {
+        launch_cut_rows<XS, true>(ctx.stream, g.base, g.off_r, R, K, Rp, Kp, ef, nullptr, out, bad);
+        TRG_LAUNCHED(ctx);
+        return;
+    }
     TRG_CUDA(cudaMemsetAsync(ef, 0, (size_t)R * sizeof(int), ctx.stream));
-    dim3 gf((unsigned)((K + XF_K - 1) / XF_K), (unsigned)std::min((R + 31) / 32, 65535));
-    k_row_field<<<gf, 256, 0, ctx.stream>>>(g.base, g.off_r, g.off_c, R, K, g.c_fast ? 1 : 0, ef);
+    launch_row_field<true>(ctx.stream, g, R, K, ef);
     TRG_LAUNCHED(ctx);
-    dim3 gd((unsigned)((Kp + XD_K - 1) / XD_K), (unsigned)std::min((Rp + XD_R - 1) / XD_R, 65535));
-    k_digits8<<<gd, 256, 0, ctx.stream>>>(g.base, g.off_r, g.off_c, R, K, Rp, Kp, g.c_fast ? 1 : 0, ef, out, bad);
+    launch_cut<XS>(ctx.stream, g, R, K, Rp, Kp, ef, nullptr, out, bad);
     TRG_LAUNCHED(ctx);
 }
 
@@ -570,10 +456,7 @@ bool gemm_exact(Ctx& ctx, const GemmDesc& d) {
     });
 
     // B as rows n, columns k
-    Gather bt = d.B;
-    bt.off_r = d.B.off_c;
-    bt.off_c = d.B.off_r;
-    bt.c_fast = d.B.r_fast && !d.B.c_fast;
+    const Gather bt = transposed(d.B);
     for (int64_t m0 = 0; m0 < d.M; m0 += ra) {
         const int mr = (int)std::min(ra, d.M - m0), mp = (int)up(mr, XM);
         Gather ga = d.A;

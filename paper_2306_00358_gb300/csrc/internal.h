@@ -113,6 +113,7 @@ struct Ctx {
     Buf f64_partial;       // FP64 GEMM: split-K partial sums
     Buf ksplit_ws;         // split GEMM: split-K partial fixed-point sums
     Buf bslices;           // contraction: the D^7 product's B slices, shared by its j-blocks
+    Buf field_ws;          // split / exact products: exponent fields of an operand's rows
     Buf cons_ef;           // exponent fields recorded by a producing product (two halves)
     Buf eig_slices;        // split mode: M sliced once per isometry solve
     Buf s3[10];            // cubic-lattice step: P1, P2, Ux, Uy, Mx, My, then A, W, C, D of the contraction
@@ -177,6 +178,7 @@ struct Gather {
     bool c_fast;            // consecutive columns are adjacent in memory
     bool c_identity = false;   // off_c[k] == k: every row is one contiguous run
     bool r_fast = false;       // consecutive rows are adjacent in memory
+    bool r_identity = false;   // off_r[r] == r
 };
 struct GemmDesc {
     int64_t M, N, K;

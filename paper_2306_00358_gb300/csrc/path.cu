@@ -47,14 +47,25 @@ static bool unit_first_stride(const Modes& m) {
     return !m.empty() && m.back().second == 1 && m.back().first > 1;
 }
 
+// The flat index of the modes is the offset itself.
+static bool identity(const Modes& m) {
+    int64_t stride = 1;
+    for (auto it = m.rbegin(); it != m.rend(); ++it) {
+        if (it->first != 1 && it->second != stride) return false;
+        stride *= it->first;
+    }
+    return true;
+}
+
 static Gather gather(Ctx& ctx, const double* base, const Modes& rows, const Modes& cols) {
     Gather g;
     g.base = base;
     g.off_r = ctx.table(rows);
     g.off_c = ctx.table(cols);
     g.c_fast = unit_first_stride(cols);
-    g.c_identity = cols.size() == 1 && cols[0].second == 1;
+    g.c_identity = identity(cols);
     g.r_fast = unit_first_stride(rows);
+    g.r_identity = identity(rows);
     return g;
 }
 

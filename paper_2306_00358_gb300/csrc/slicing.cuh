@@ -1,0 +1,311 @@
+// Cutting FP64 operands into BF16 digits for the tensor-core products
+// (split_gemm.cu: S = 2..5 slices, exact_gemm.cu: eight digits).
+//
+// An operand is rows r < R of length K, element (r, k) at src[off_r[r] +
+// off_c[k]]; its digits go to out[p][r][k] (r < Rp, k < Kp, zero in the
+// padding).  With f the largest exponent field of a row and e = f - 1022
+// (|x| < 2^e), X = rint(x 2^(F - e)), F = 7 + 8 (S - 1), halves away from
+// zero, is the sum of d_p 2^(8 (S - 1 - p)), d_0 in [-128, 128], d_p in
+// [-128, 127]; slices are stored as d_p 2^(-8p) (S <= 5) or as d_p (S = 8).
+//
+// All of it is bound by HBM: 8 B read (twice where the exponents take a pass
+// of their own) and 2 S B written per element.
+//  - Rows that are contiguous runs of at most 8192 are read once: a warp or a
+//    block holds a row in registers, finds its exponent and cuts it
+//    (k_cut_rows).  16384 x 4096, S = 4: 153 us (1.07 GB, 7.0 TB/s).
+//  - Rows whose exponents the producing product recorded: a warp per row
+//    (k_slice_contig).
+//  - Gathered operands: k_row_field, then k_cut, both reading along the index
+//    that is adjacent in memory.  4096 x 4096 read across, S = 4: 32 + 77 us.
+//    (With a shared-memory atomic per element for the exponents and 2-byte
+//    stores, two passes for every operand, the two above took 757 us.)
+//  - A few gathered rows: one block per row reads it twice (k_slice_rows, in
+//    split_gemm.cu).
+#pragma once
+
+#include <cstdint>
+
+#include "internal.h"
+
+namespace trg {
+
+namespace {
+
+// Biased exponent field; a subnormal counts as field 1 (SUB) or as zero.
+template <bool SUB>
+__device__ __forceinline__ unsigned exponent_field(double x) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+    const unsigned hi = (unsigned)(b >> 32) & 0x7fffffffu;
+    if (!SUB) return hi >> 20;
+    return hi >= 0x100000u ? hi >> 20 : ((hi | (unsigned)b) ? 1u : 0u);
+}
+
+// Scale exponent of a row from its largest field (-1022 for a zero row).
+__device__ __forceinline__ int row_exponent(int f) { return f ? f - 1022 : -1022; }
+
+// The digits of x in a row of largest field f, as the FP32 values to store
+// (exact in BF16: their upper halves).
+template <int S>
+__device__ __forceinline__ void cut(double x, int f, float (&d)[S]) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+    const int ex = (int)((b >> 52) & 0x7FF);
+    const unsigned long long m53 = ex ? ((b & ((1ull << 52) - 1)) | (1ull << 52)) : 0ull;
+    const bool neg = (long long)b < 0;
+    // adding 128 to every digit but the first turns the signed digits into
+    // bytes; a byte under the exponent of 2^23 is the FP32 number 2^23 + byte
+    if constexpr (S == 8) {
+        const int sh = f - ex - 10;              // X = mantissa 2^-sh
+        const unsigned long long m = sh <= 0 ? m53 << (-sh & 63) : sh < 60 ? (m53 + (1ull << (sh - 1))) >> sh : 0ull;
+        const unsigned long long y = (neg ? 0ull - m : m) + 0x0080808080808080ull;
+        const unsigned ylo = (unsigned)y, yhi = (unsigned)(y >> 32);
+        // the first digit is the signed top byte, whose sign bit is part of the value when X >= 0
+        d[0] = (float)(neg ? (int)yhi >> 24 : (int)(yhi >> 24));
+#pragma unroll
+        for (int p = 1; p < 8; ++p) {
+            const unsigned v = p < 4 ? __byte_perm(yhi, 0x4B000000u, 0x7440u | (unsigned)(3 - p))
+                                     : __byte_perm(ylo, 0x4B000000u, 0x7440u | (unsigned)(7 - p));
+            d[p] = __uint_as_float(v) - 8388736.0f;   // 2^23 + 128
+        }
+    } else {
+        constexpr int F = 7 + 8 * (S - 1);
+        constexpr unsigned BIAS = S == 2 ? 0x80u : S == 3 ? 0x8080u : S == 4 ? 0x808080u : 0x80808080u;
+        const int sh = 53 - F + f - ex;          // > 0
+        const long long m = sh < 63 ? (long long)((m53 + (1ull << (sh - 1))) >> sh) : 0ll;
+        const long long y = (neg ? -m : m) + (long long)BIAS;
+        d[0] = (float)(int)(y >> (8 * (S - 1)));
+#pragma unroll
+        for (int p = 1; p < S; ++p) {
+            const unsigned v = __byte_perm((unsigned)y, 0x4B000000u, 0x7440u | (unsigned)(S - 1 - p));
+            const float w = __int_as_float((127 - 8 * p) << 23);
+            d[p] = fmaf(__uint_as_float(v), w, -8388736.0f * w);   // exact
+        }
+    }
+}
+// Two neighbours' digits as packed BF16.
+template <int S>
+__device__ __forceinline__ void cut2(double x0, double x1, int f, uint32_t (&w)[S]) {
+    float a[S], b[S];
+    cut<S>(x0, f, a);
+    cut<S>(x1, f, b);
+#pragma unroll
+    for (int p = 0; p < S; ++p) w[p] = __byte_perm(__float_as_uint(a[p]), __float_as_uint(b[p]), 0x7632);
+}
+
+// Rows of an exact product whose largest entry lies outside this range make
+// it take the FP64 pipe instead (exact_gemm.cu).
+constexpr int FIELD_LO = 1023 - 400, FIELD_HI = 1023 + 400;
+__device__ __forceinline__ void check_range(int f, int* bad) {
+    if (bad && f && (f < FIELD_LO || f > FIELD_HI)) *bad = 1;
+}
+
+// Largest exponent field of each row, maxima into ef (zeroed).
+constexpr int XF_K = 256;
+template <bool SUB>
+__global__ void __launch_bounds__(256) k_row_field(const double* __restrict__ src, const int64_t* __restrict__ off_r,
+                                                   const int64_t* __restrict__ off_c, int R, int K, int k_fast,
+                                                   int* __restrict__ ef) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int k0 = blockIdx.x * XF_K, k1 = min(K, k0 + XF_K);
+    const int nby = (R + 31) / 32;      // row blocks, strided over grid.y (at most 65535)
+    for (int by = blockIdx.y; by < nby; by += gridDim.y) {
+        const int r0 = by * 32;
+        if (k_fast) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int r = r0 + warp * 4 + i;
+                if (r >= R) break;
+                const double* row = src + off_r[r];
+                unsigned f = 0;
+#pragma unroll 8
+                for (int k = k0 + lane; k < k1; k += 32) f = max(f, exponent_field<SUB>(row[off_c[k]]));
+                f = __reduce_max_sync(0xffffffffu, f);
+                if (lane == 0 && f) atomicMax(&ef[r], (int)f);
+            }
+        } else {
+            __shared__ unsigned red[8][32];
+            const int r = r0 + lane;
+            unsigned f = 0;
+            if (r < R) {
+                const double* row = src + off_r[r];
+#pragma unroll 8
+                for (int k = k0 + warp; k < k1; k += 8) f = max(f, exponent_field<SUB>(row[off_c[k]]));
+            }
+            red[warp][lane] = f;
+            __syncthreads();
+            if (warp == 0) {
+#pragma unroll
+                for (int w = 1; w < 8; ++w) f = max(f, red[w][lane]);
+                if (r < R && f) atomicMax(&ef[r], (int)f);
+            }
+            __syncthreads();
+        }
+    }
+}
+
+// Digits of a gathered operand with known fields ef.  Elements pass through a
+// 32 x 64 shared tile so that both sides are coalesced; a thread cuts eight
+// adjacent k and writes 16 bytes per digit.
+constexpr int XD_R = 32, XD_K = 64, XD_LD = XD_K + XD_K / 8 + 1;
+template <int S>
+__global__ void __launch_bounds__(256) k_cut(const double* __restrict__ src, const int64_t* __restrict__ off_r,
+                                             const int64_t* __restrict__ off_c, int R, int K, int Rp, int Kp,
+                                             int k_fast, const int* __restrict__ ef, int* __restrict__ e_out,
+                                             uint16_t* __restrict__ out, int* bad) {
+    __shared__ double tile[XD_R * XD_LD];
+    const int k0 = blockIdx.x * XD_K;
+    const size_t plane = (size_t)Rp * Kp;
+    const int nby = (Rp + XD_R - 1) / XD_R;
+    for (int by = blockIdx.y; by < nby; by += gridDim.y) {
+        const int r0 = by * XD_R;
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < XD_R * XD_K / 256; ++q) {
+            const int e = threadIdx.x + q * 256;
+            int rr, kk;
+            if (k_fast) { kk = e % XD_K; rr = e / XD_K; } else { rr = e % XD_R; kk = e / XD_R; }
+            const int r = r0 + rr, k = k0 + kk;
+            tile[rr * XD_LD + kk + (kk >> 3)] = (r < R && k < K) ? src[off_r[r] + off_c[k]] : 0.0;
+        }
+        __syncthreads();
+        const int rr = threadIdx.x >> 3, kg = threadIdx.x & 7;
+        const int r = r0 + rr, k = k0 + kg * 8;
+        if (r >= Rp || k >= Kp) continue;
+        const int f = r < R ? ef[r] : 0;
+        check_range(f, bad);
+        if (e_out && blockIdx.x == 0 && kg == 0 && r < R) e_out[r] = row_exponent(f);
+        const double* x = tile + rr * XD_LD + kg * 9;
+        uint32_t w[4][S];
+#pragma unroll
+        for (int h = 0; h < 4; ++h) cut2<S>(x[2 * h], x[2 * h + 1], f, w[h]);
+        uint16_t* o = out + (size_t)r * Kp + k;
+#pragma unroll
+        for (int p = 0; p < S; ++p) *reinterpret_cast<uint4*>(o + p * plane) = make_uint4(w[0][p], w[1][p], w[2][p], w[3][p]);
+    }
+}
+
+// Four adjacent elements of a contiguous row (zero past K).
+__device__ __forceinline__ void load4(const double* row, int k, int K, bool vec, double (&v)[4]) {
+    v[0] = v[1] = v[2] = v[3] = 0.0;
+    if (vec && k + 3 < K) {
+        const double2 a = *reinterpret_cast<const double2*>(row + k);
+        const double2 b = *reinterpret_cast<const double2*>(row + k + 2);
+        v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
+    } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (k + j < K) v[j] = row[k + j];
+    }
+}
+template <int S>
+__device__ __forceinline__ void store4(const double (&v)[4], int f, uint16_t* o, size_t plane) {
+    uint32_t a[S], b[S];
+    cut2<S>(v[0], v[1], f, a);
+    cut2<S>(v[2], v[3], f, b);
+#pragma unroll
+    for (int p = 0; p < S; ++p) *reinterpret_cast<uint2*>(o + p * plane) = make_uint2(a[p], b[p]);
+}
+
+// Contiguous rows with known fields: a warp per row, four columns per lane.
+template <int S>
+__global__ void __launch_bounds__(256) k_slice_contig(const double* __restrict__ src, const int64_t* __restrict__ off_r,
+                                                      int R, int K, int Rp, int Kp, const int* __restrict__ ef,
+                                                      int* __restrict__ e_out, uint16_t* __restrict__ out, int* bad) {
+    const int lane = threadIdx.x & 31;
+    const int r = blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (r >= Rp) return;
+    const size_t plane = (size_t)Rp * Kp;
+    const bool real = r < R;
+    const double* row = real ? src + off_r[r] : nullptr;
+    const bool vec = real && ((reinterpret_cast<uintptr_t>(row) & 15) == 0);
+    const int f = real ? ef[r] : 0;
+    check_range(f, bad);
+    if (e_out && lane == 0 && real) e_out[r] = row_exponent(f);
+    for (int k = lane * 4; k < Kp; k += 128) {
+        double v[4];
+        load4(row, k, real ? K : 0, vec, v);
+        store4<S>(v, f, out + (size_t)r * Kp + k, plane);
+    }
+}
+
+// Contiguous rows with unknown fields, K <= 4 TPR NCH: TPR threads (a warp or
+// the block) hold a row in registers, so it is read once.
+template <int S, int TPR, int NCH, bool SUB>
+__global__ void __launch_bounds__(256) k_cut_rows(const double* __restrict__ src, const int64_t* __restrict__ off_r,
+                                                  int R, int K, int Rp, int Kp, int* __restrict__ ef_out,
+                                                  int* __restrict__ e_out, uint16_t* __restrict__ out, int* bad) {
+    __shared__ unsigned wmax[8];
+    const int t = threadIdx.x % TPR;
+    const int r = blockIdx.x * (256 / TPR) + threadIdx.x / TPR;
+    if (TPR == 32 && r >= Rp) return;
+    const size_t plane = (size_t)Rp * Kp;
+    const bool real = r < R;
+    const double* row = real ? src + off_r[r] : nullptr;
+    const bool vec = real && ((reinterpret_cast<uintptr_t>(row) & 15) == 0);
+    double v[NCH][4];
+    unsigned fm = 0;
+#pragma unroll
+    for (int c = 0; c < NCH; ++c) load4(row, (c * TPR + t) * 4, real ? K : 0, vec, v[c]);
+#pragma unroll
+    for (int c = 0; c < NCH; ++c)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) fm = max(fm, exponent_field<SUB>(v[c][j]));
+    fm = __reduce_max_sync(0xffffffffu, fm);
+    if (TPR == 256) {
+        if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = fm;
+        __syncthreads();
+#pragma unroll
+        for (int w = 0; w < 8; ++w) fm = max(fm, wmax[w]);
+    }
+    const int f = (int)fm;
+    check_range(f, bad);
+    if (t == 0 && real) {
+        if (ef_out) ef_out[r] = f;
+        if (e_out) e_out[r] = row_exponent(f);
+    }
+#pragma unroll
+    for (int c = 0; c < NCH; ++c) {
+        const int k = (c * TPR + t) * 4;
+        if (k < Kp) store4<S>(v[c], f, out + (size_t)r * Kp + k, plane);
+    }
+}
+
+constexpr int CUT_ROWS_MAX_K = 8192;
+template <int S, bool SUB>
+void launch_cut_rows(cudaStream_t stream, const double* src, const int64_t* off_r, int R, int K, int Rp, int Kp,
+                     int* ef_out, int* e_out, uint16_t* out, int* bad) {
+    const unsigned gw = (unsigned)((Rp + 7) / 8), gb = (unsigned)Rp;
+    if (Kp <= 128) k_cut_rows<S, 32, 1, SUB><<<gw, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, e_out, out, bad);
+    else if (Kp <= 512) k_cut_rows<S, 32, 4, SUB><<<gw, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, e_out, out, bad);
+    else if (Kp <= 2048) k_cut_rows<S, 256, 2, SUB><<<gb, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, e_out, out, bad);
+    else if (Kp <= 4096) k_cut_rows<S, 256, 4, SUB><<<gb, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, e_out, out, bad);
+    else k_cut_rows<S, 256, 8, SUB><<<gb, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, e_out, out, bad);
+}
+
+template <bool SUB>
+void launch_row_field(cudaStream_t stream, const Gather& g, int R, int K, int* ef) {
+    dim3 grid((unsigned)((K + XF_K - 1) / XF_K), (unsigned)std::min((R + 31) / 32, 65535));
+    k_row_field<SUB><<<grid, 256, 0, stream>>>(g.base, g.off_r, g.off_c, R, K, g.c_fast ? 1 : 0, ef);
+}
+
+template <int S>
+void launch_cut(cudaStream_t stream, const Gather& g, int R, int K, int Rp, int Kp, const int* ef, int* e_out,
+                uint16_t* out, int* bad) {
+    dim3 grid((unsigned)((Kp + XD_K - 1) / XD_K), (unsigned)std::min((Rp + XD_R - 1) / XD_R, 65535));
+    k_cut<S><<<grid, 256, 0, stream>>>(g.base, g.off_r, g.off_c, R, K, Rp, Kp, g.c_fast ? 1 : 0, ef, e_out, out, bad);
+}
+
+// B operand as rows n, columns k: the roles of its two tables swapped.
+inline Gather transposed(const Gather& b) {
+    Gather t = b;
+    t.off_r = b.off_c;
+    t.off_c = b.off_r;
+    t.c_fast = b.r_fast && !b.c_fast;
+    t.r_fast = b.c_fast;
+    t.c_identity = b.r_identity;
+    t.r_identity = b.c_identity;
+    return t;
+}
+
+}  // namespace
+
+}  // namespace trg

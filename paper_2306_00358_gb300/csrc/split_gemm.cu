@@ -55,6 +55,7 @@
 #include <vector>
 
 #include "internal.h"
+#include "slicing.cuh"
 #include "tcgen05.cuh"
 
 namespace trg {
@@ -869,37 +870,6 @@ k_split_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
 }
 
 // ------------------------------------------------------------- slicing ----
-// Per-row maximum of the biased FP64 exponent field (0 for an all-zero row).
-// Source element (r, k) at src[off_r[r] + off_c[k]].
-constexpr int SL_R = 32, SL_K = 64;
-
-__global__ void __launch_bounds__(256) k_row_exponent(const double* __restrict__ src, const int64_t* __restrict__ off_r,
-                                                      const int64_t* __restrict__ off_c, int R, int K, int k_fast,
-                                                      int* __restrict__ ef_out) {
-    __shared__ int rmax[SL_R];
-    const int k0 = blockIdx.x * SL_K;
-    const int nby = (R + SL_R - 1) / SL_R;   // row blocks, strided over grid.y (at most 65535)
-    for (int by = blockIdx.y; by < nby; by += gridDim.y) {
-        const int r0 = by * SL_R;
-        if (threadIdx.x < SL_R) rmax[threadIdx.x] = 0;
-        __syncthreads();
-        for (int e = threadIdx.x; e < SL_R * SL_K; e += 256) {
-            int rr, kk;
-            if (k_fast) { kk = e % SL_K; rr = e / SL_K; } else { rr = e % SL_R; kk = e / SL_R; }
-            const int r = r0 + rr, k = k0 + kk;
-            if (r < R && k < K) {
-                const unsigned long long b = (unsigned long long)__double_as_longlong(src[off_r[r] + off_c[k]]);
-                const int ef = (int)((b >> 52) & 0x7FF);
-                if (ef) atomicMax(&rmax[rr], ef);
-            }
-        }
-        __syncthreads();
-        if (threadIdx.x < SL_R && r0 + (int)threadIdx.x < R && rmax[threadIdx.x])
-            atomicMax(&ef_out[r0 + threadIdx.x], rmax[threadIdx.x]);
-        __syncthreads();
-    }
-}
-
 // Split K: C(m, n) = the sum over the parts, in part order, of their exact
 // fixed-point sums V (kpart[(p N + n) M + m]), scaled by 2^(ea_m + eb_n - 36)
 // as the staged epilogue scales an unsplit V.
@@ -921,168 +891,9 @@ __global__ void k_exponent_finish(int* ef, int R) {
     if (r < R) ef[r] = ef[r] ? ef[r] - 1022 : -1022;
 }
 
-// Slices: out[p][r][k] (BF16 bits), r < Rp, k < Kp, zero in the padding.
-template <int S>
-__global__ void __launch_bounds__(256) k_slice(const double* __restrict__ src, const int64_t* __restrict__ off_r,
-                                               const int64_t* __restrict__ off_c, int R, int K, int Rp, int Kp,
-                                               int k_fast, const int* __restrict__ e_row,
-                                               uint16_t* __restrict__ out) {
-    __shared__ double tile[SL_R][SL_K + 1];
-    const int k0 = blockIdx.x * SL_K;
-    const int nby = (Rp + SL_R - 1) / SL_R;   // row blocks, strided over grid.y (at most 65535)
-    for (int by = blockIdx.y; by < nby; by += gridDim.y) {
-        const int r0 = by * SL_R;
-        __syncthreads();   // the previous block's tile has been read
-        for (int e = threadIdx.x; e < SL_R * SL_K; e += 256) {
-            int rr, kk;
-            if (k_fast) { kk = e % SL_K; rr = e / SL_K; } else { rr = e % SL_R; kk = e / SL_R; }
-            const int r = r0 + rr, k = k0 + kk;
-            tile[rr][kk] = (r < R && k < K) ? src[off_r[r] + off_c[k]] : 0.0;
-        }
-        __syncthreads();
-        constexpr int F = 7 + 8 * (S - 1);
-        for (int e = threadIdx.x; e < SL_R * SL_K; e += 256) {
-            const int kk = e % SL_K, rr = e / SL_K;
-            const int r = r0 + rr, k = k0 + kk;
-            if (r >= Rp || k >= Kp) continue;
-            long long X = 0;
-            if (r < R) {
-                const unsigned long long b = (unsigned long long)__double_as_longlong(tile[rr][kk]);
-                const int ex = (int)((b >> 52) & 0x7FF);
-                if (ex) {
-                    const int ea = e_row[r];                       // |x| < 2^ea
-                    const int shift = 52 + 1023 + ea - ex - F;     // >= 53 - F > 0
-                    if (shift < 63) {
-                        const unsigned long long m53 = (b & ((1ull << 52) - 1)) | (1ull << 52);
-                        X = (long long)((m53 + (1ull << (shift - 1))) >> shift);
-                        if (b >> 63) X = -X;
-                    }
-                }
-            }
-            int d[S];
-#pragma unroll
-            for (int p = S - 1; p >= 1; --p) {
-                const int lo = (int)(((X + 128) & 255) - 128);
-                d[p] = lo;
-                X = (X - lo) >> 8;
-            }
-            d[0] = (int)X;
-            const size_t plane = (size_t)Rp * Kp;
-#pragma unroll
-            for (int p = 0; p < S; ++p) {
-                // small integer -> FP32 exactly (|d| < 2^22), times 2^-8p, top 16 bits = BF16
-                const float f = (__int_as_float(0x4B400000 + d[p]) - 12582912.0f) * __int_as_float((127 - 8 * p) << 23);
-                out[p * plane + (size_t)r * Kp + k] = (uint16_t)(__float_as_uint(f) >> 16);
-            }
-        }
-    }
-}
-
-// Slices of an operand whose rows are contiguous runs (src + off_r[r] + k):
-// a warp per row, four columns per lane per pass with 16-byte loads and
-// 8-byte stores of four BF16 per slice.  Same arithmetic as k_slice (the
-// slices are bit-identical), without the tile transpose through shared memory.
-template <int S>
-__global__ void __launch_bounds__(256) k_slice_contig(const double* __restrict__ src, const int64_t* __restrict__ off_r,
-                                                      int R, int K, int Rp, int Kp, const int* __restrict__ e_row,
-                                                      uint16_t* __restrict__ out) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int r = blockIdx.x * 8 + warp;
-    if (r >= Rp) return;
-    const size_t plane = (size_t)Rp * Kp;
-    uint16_t* orow = out + (size_t)r * Kp;
-    constexpr int F = 7 + 8 * (S - 1);
-    const bool real = r < R;
-    const double* row = real ? src + off_r[r] : nullptr;
-    const bool vec = real && ((reinterpret_cast<uintptr_t>(row) & 15) == 0);
-    const int ea = real ? e_row[r] : 0;
-    for (int k0 = lane * 4; k0 < Kp; k0 += 128) {
-        double v[4] = {0.0, 0.0, 0.0, 0.0};
-        if (real) {
-            if (vec && k0 + 3 < K) {
-                const double2 a = *reinterpret_cast<const double2*>(row + k0);
-                const double2 b = *reinterpret_cast<const double2*>(row + k0 + 2);
-                v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
-            } else {
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    if (k0 + j < K) v[j] = row[k0 + j];
-            }
-        }
-        uint32_t pk[S][2];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const unsigned long long b = (unsigned long long)__double_as_longlong(v[j]);
-            const int ex = (int)((b >> 52) & 0x7FF);
-            long long X = 0;
-            if (ex) {
-                const int shift = 52 + 1023 + ea - ex - F;     // >= 53 - F > 0
-                if (shift < 63) {
-                    const unsigned long long m53 = (b & ((1ull << 52) - 1)) | (1ull << 52);
-                    X = (long long)((m53 + (1ull << (shift - 1))) >> shift);
-                    if (b >> 63) X = -X;
-                }
-            }
-            int d[S];
-#pragma unroll
-            for (int p = S - 1; p >= 1; --p) {
-                const int lo = (int)(((X + 128) & 255) - 128);
-                d[p] = lo;
-                X = (X - lo) >> 8;
-            }
-            d[0] = (int)X;
-#pragma unroll
-            for (int p = 0; p < S; ++p) {
-                const float f = (__int_as_float(0x4B400000 + d[p]) - 12582912.0f) * __int_as_float((127 - 8 * p) << 23);
-                const uint32_t hb = __float_as_uint(f) >> 16;
-                if (j & 1) pk[p][j >> 1] |= hb << 16;
-                else pk[p][j >> 1] = hb;
-            }
-        }
-#pragma unroll
-        for (int p = 0; p < S; ++p) *reinterpret_cast<uint2*>(orow + p * plane + k0) = make_uint2(pk[p][0], pk[p][1]);
-    }
-}
-
-// The S BF16 slices (bits) of x in a row with |x| < 2^ea: the fixed-point
-// value X = rint(x 2^(F - ea)) (halves away from zero), F = 7 + 8 (S - 1),
-// as S signed base-256 digits, each exact in BF16.  The arithmetic of
-// k_slice and k_slice_contig, element for element.
-template <int S>
-__device__ __forceinline__ void slice_bits(double x, int ea, uint16_t (&h)[S]) {
-    constexpr int F = 7 + 8 * (S - 1);
-    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-    const int ex = (int)((b >> 52) & 0x7FF);
-    long long X = 0;
-    if (ex) {
-        const int shift = 52 + 1023 + ea - ex - F;     // >= 53 - F > 0
-        if (shift < 63) {
-            const unsigned long long m53 = (b & ((1ull << 52) - 1)) | (1ull << 52);
-            X = (long long)((m53 + (1ull << (shift - 1))) >> shift);
-            if (b >> 63) X = -X;
-        }
-    }
-    int d[S];
-#pragma unroll
-    for (int p = S - 1; p >= 1; --p) {
-        const int lo = (int)(((X + 128) & 255) - 128);
-        d[p] = lo;
-        X = (X - lo) >> 8;
-    }
-    d[0] = (int)X;
-#pragma unroll
-    for (int p = 0; p < S; ++p) {
-        const float f = (__int_as_float(0x4B400000 + d[p]) - 12582912.0f) * __int_as_float((127 - 8 * p) << 23);
-        h[p] = (uint16_t)(__float_as_uint(f) >> 16);
-    }
-}
-
-// Exponents and slices of a few rows in one launch (the n x m blocks the
-// isometry multiplies by M: m rows of n as a B operand): a CTA per row r < Rp
-// takes the largest exponent field of its row (e_row[r] = field - 1022,
-// -1022 for a zero row, as row_exponents gives it), then writes the row's
-// slices, reading the row a second time through L1 / L2.  Bit-identical to
-// row_exponents followed by k_slice.
+// Exponents and slices of a few gathered rows in one launch: a CTA per row r
+// < Rp takes the largest exponent field of its row, then writes the row's
+// slices, reading the row a second time through L1 / L2.
 template <int S>
 __global__ void __launch_bounds__(256) k_slice_rows(const double* __restrict__ src, const int64_t* __restrict__ off_r,
                                                     const int64_t* __restrict__ off_c, int R, int K, int Rp, int Kp,
@@ -1102,14 +913,13 @@ __global__ void __launch_bounds__(256) k_slice_rows(const double* __restrict__ s
     int mx = 0;
 #pragma unroll
     for (int w = 0; w < 8; ++w) mx = max(mx, wmax[w]);
-    const int ea = mx ? mx - 1022 : -1022;
-    if (real && threadIdx.x == 0) e_row[r] = ea;
+    if (real && threadIdx.x == 0) e_row[r] = row_exponent(mx);
     const size_t plane = (size_t)Rp * Kp;
     for (int k = threadIdx.x; k < Kp; k += 256) {
-        uint16_t h[S];
-        slice_bits<S>((real && k < K) ? row[off_c[k]] : 0.0, ea, h);
+        float d[S];
+        cut<S>((real && k < K) ? row[off_c[k]] : 0.0, mx, d);
 #pragma unroll
-        for (int p = 0; p < S; ++p) out[p * plane + (size_t)r * Kp + k] = h[p];
+        for (int p = 0; p < S; ++p) out[p * plane + (size_t)r * Kp + k] = (uint16_t)(__float_as_uint(d[p]) >> 16);
     }
 }
 
@@ -1231,87 +1041,61 @@ void launch_mma(Ctx& ctx, const CUtensorMap& ta, const CUtensorMap& tb, const CU
     else launch_mma_k<S, CG, EPI_STAGED>(ctx, ta, tb, tbh, a);
 }
 
+// Exponents (e) and slices of an operand (rows r < R of length K, padded to
+// Rp x Kp); `known` holds the rows' exponent fields if the producing product
+// recorded them.  See slicing.cuh for the forms.  At most SLICE_ROWS_MAX
+// gathered rows of moderate length take one launch (the isometry's blocks, U
+// as an operand), where two launches cost more than the second read.
+constexpr int SLICE_ROWS_MAX = 256, SLICE_ROWS_MAX_K = 16384;
 template <int S>
-void launch_slice(Ctx& ctx, const Gather& g, int R, int K, int Rp, int Kp, const int* e, uint16_t* out) {
-    if (g.c_identity) {
-        k_slice_contig<S><<<(unsigned)((Rp + 7) / 8), 256, 0, ctx.stream>>>(g.base, g.off_r, R, K, Rp, Kp, e, out);
-        TRG_LAUNCHED(ctx);
-        return;
-    }
-    dim3 grid((unsigned)((Kp + SL_K - 1) / SL_K), (unsigned)std::min<int64_t>((Rp + SL_R - 1) / SL_R, 65535));
-    k_slice<S><<<grid, 256, 0, ctx.stream>>>(g.base, g.off_r, g.off_c, R, K, Rp, Kp, g.c_fast ? 1 : 0, e, out);
-    TRG_LAUNCHED(ctx);
-}
-
-void row_exponents(Ctx& ctx, const Gather& g, int R, int K, int* e);
-
-// Exponents and slices of an operand (rows r < R of length K, padded to Rp x
-// Kp): one launch for at most SLICE_ROWS_MAX rows, else the two passes.
-constexpr int SLICE_ROWS_MAX = 256;
-template <int S>
-void exponents_and_slices(Ctx& ctx, const Gather& g, int R, int K, int Rp, int Kp, int* e, uint16_t* out) {
-    if (Rp <= SLICE_ROWS_MAX) {
+void slice_operand(Ctx& ctx, const Gather& g, int R, int K, int Rp, int Kp, const int* known, int* e, uint16_t* out) {
+    if (g.c_identity && known) {
+        k_slice_contig<S><<<(unsigned)((Rp + 7) / 8), 256, 0, ctx.stream>>>(g.base, g.off_r, R, K, Rp, Kp, known, e, out,
+                                                                            nullptr);
+    } else if (g.c_identity && Kp <= CUT_ROWS_MAX_K) {
+        launch_cut_rows<S, false>(ctx.stream, g.base, g.off_r, R, K, Rp, Kp, nullptr, e, out, nullptr);
+    } else if (!known && Rp <= SLICE_ROWS_MAX && K <= SLICE_ROWS_MAX_K) {
         k_slice_rows<S><<<(unsigned)Rp, 256, 0, ctx.stream>>>(g.base, g.off_r, g.off_c, R, K, Rp, Kp, e, out);
-        TRG_LAUNCHED(ctx);
-        return;
+    } else {
+        if (!known) {
+            ctx.ensure(ctx.field_ws, (size_t)R * sizeof(int));
+            int* f = ctx.field_ws.as<int>();
+            TRG_CUDA(cudaMemsetAsync(f, 0, (size_t)R * sizeof(int), ctx.stream));
+            launch_row_field<false>(ctx.stream, g, R, K, f);
+            TRG_LAUNCHED(ctx);
+            known = f;
+        }
+        launch_cut<S>(ctx.stream, g, R, K, Rp, Kp, known, e, out, nullptr);
     }
-    row_exponents(ctx, g, R, K, e);
-    launch_slice<S>(ctx, g, R, K, Rp, Kp, e, out);
+    TRG_LAUNCHED(ctx);
 }
 
-void row_exponents(Ctx& ctx, const Gather& g, int R, int K, int* e) {
-    TRG_CUDA(cudaMemsetAsync(e, 0, (size_t)R * sizeof(int), ctx.stream));
-    dim3 grid((unsigned)((K + SL_K - 1) / SL_K), (unsigned)std::min<int64_t>((R + SL_R - 1) / SL_R, 65535));
-    k_row_exponent<<<grid, 256, 0, ctx.stream>>>(g.base, g.off_r, g.off_c, R, K, g.c_fast ? 1 : 0, e);
-    TRG_LAUNCHED(ctx);
-    k_exponent_finish<<<(unsigned)((R + 255) / 256), 256, 0, ctx.stream>>>(e, R);
-    TRG_LAUNCHED(ctx);
+void slice_operand(Ctx& ctx, int S, const Gather& g, int R, int K, int Rp, int Kp, const int* known, int* e,
+                   uint16_t* out) {
+    switch (S) {
+        case 2: slice_operand<2>(ctx, g, R, K, Rp, Kp, known, e, out); break;
+        case 3: slice_operand<3>(ctx, g, R, K, Rp, Kp, known, e, out); break;
+        case 4: slice_operand<4>(ctx, g, R, K, Rp, Kp, known, e, out); break;
+        case 5: slice_operand<5>(ctx, g, R, K, Rp, Kp, known, e, out); break;
+        default: fail(TRG_EINVAL, "split_slices must be 2..5");
+    }
 }
 
 }  // namespace
-
-// B operand as (n, k): swap the roles of its two tables.
-static Gather transpose_gather(const Gather& b, const int64_t* off_k, const int64_t* off_n) {
-    Gather t = b;
-    t.off_r = off_n;
-    t.off_c = off_k;
-    t.c_fast = false;
-    t.c_identity = false;
-    return t;
-}
 
 // Exponents and BF16 slices of an A operand in the layout a split product
 // reads (rows padded per split_rows_padded, K per split_k_padded), for a
 // caller that reuses one A across several products.
 void split_slice_operand(Ctx& ctx, const Gather& A, int64_t M, int64_t K, uint16_t* slices, int* e) {
-    const int S = slices_now(ctx);
-    const int Mi = (int)M, Ki = (int)std::max<int64_t>(K, 1);
-    const int Mp = (int)split_rows_padded(ctx, M), Kp = (int)split_k_padded(K);
-    row_exponents(ctx, A, Mi, Ki, e);
-    switch (S) {
-        case 2: launch_slice<2>(ctx, A, Mi, Ki, Mp, Kp, e, slices); break;
-        case 3: launch_slice<3>(ctx, A, Mi, Ki, Mp, Kp, e, slices); break;
-        case 4: launch_slice<4>(ctx, A, Mi, Ki, Mp, Kp, e, slices); break;
-        case 5: launch_slice<5>(ctx, A, Mi, Ki, Mp, Kp, e, slices); break;
-        default: fail(TRG_EINVAL, "split_slices must be 2..5");
-    }
+    slice_operand(ctx, slices_now(ctx), A, (int)M, (int)std::max<int64_t>(K, 1), (int)split_rows_padded(ctx, M),
+                  (int)split_k_padded(K), nullptr, e, slices);
 }
 
 // Exponents and BF16 slices of a B operand (K x N) as a split product reads
 // it: rows n of B^T, padded to the 128-column tile.
 void split_slice_b(Ctx& ctx, const Gather& B, int64_t K, int64_t N, uint16_t* slices, int* e) {
-    const int S = slices_now(ctx);
-    const int Ni = (int)N, Ki = (int)std::max<int64_t>(K, 1);
-    const int Np = (int)split_cols_padded(N), Kp = (int)split_k_padded(K);
-    const Gather bt = transpose_gather(B, B.off_r, B.off_c);
-    row_exponents(ctx, bt, Ni, Ki, e);
-    switch (S) {
-        case 2: launch_slice<2>(ctx, bt, Ni, Ki, Np, Kp, e, slices); break;
-        case 3: launch_slice<3>(ctx, bt, Ni, Ki, Np, Kp, e, slices); break;
-        case 4: launch_slice<4>(ctx, bt, Ni, Ki, Np, Kp, e, slices); break;
-        case 5: launch_slice<5>(ctx, bt, Ni, Ki, Np, Kp, e, slices); break;
-        default: fail(TRG_EINVAL, "split_slices must be 2..5");
-    }
+    slice_operand(ctx, slices_now(ctx), transposed(B), (int)N, (int)std::max<int64_t>(K, 1), (int)split_cols_padded(N),
+                  (int)split_k_padded(K), nullptr, e, slices);
 }
 int64_t split_cols_padded(int64_t N) { return (N + BN - 1) / BN * BN; }
 
@@ -1415,32 +1199,10 @@ void gemm_split(Ctx& ctx, const GemmDesc& d) {
                  : pre_b ? const_cast<uint16_t*>(d.b_slices)
                          : (uint16_t*)(base + ((bytes_e + 255) & ~(size_t)255)) + (pre_a ? 0 : (size_t)S * Mp * Kp);
 
+    // (a_ef: the producing product already recorded A's exponent fields)
+    if (!pre_a) slice_operand(ctx, S, d.A, M, K, Mp, Kp, d.a_ef, ea, sa);
     // B as rows n, columns k: element (n, k) at B[b_k[k] + b_n[n]]
-    const Gather bt = transpose_gather(d.B, d.B.off_r, d.B.off_c);
-    Gather bt2 = bt;
-    bt2.c_fast = false;
-    // contiguous along k in memory?  (the k-table of B is B.off_r)
-    if (pre_a) {
-        // slices and exponents of A were written by the producing product
-    } else if (d.a_ef) {
-        // the producing product already recorded A's exponent fields
-        TRG_CUDA(cudaMemcpyAsync(ea, d.a_ef, (size_t)M * sizeof(int), cudaMemcpyDeviceToDevice, ctx.stream));
-        k_exponent_finish<<<(unsigned)((M + 255) / 256), 256, 0, ctx.stream>>>(ea, M);
-        TRG_LAUNCHED(ctx);
-    } else {
-        row_exponents(ctx, d.A, M, K, ea);
-    }
-    switch (S) {
-        case 2: if (!pre_a) launch_slice<2>(ctx, d.A, M, K, Mp, Kp, ea, sa);
-                if (!pre_b) exponents_and_slices<2>(ctx, bt2, N, K, Np, Kp, eb, sb); break;
-        case 3: if (!pre_a) launch_slice<3>(ctx, d.A, M, K, Mp, Kp, ea, sa);
-                if (!pre_b) exponents_and_slices<3>(ctx, bt2, N, K, Np, Kp, eb, sb); break;
-        case 4: if (!pre_a) launch_slice<4>(ctx, d.A, M, K, Mp, Kp, ea, sa);
-                if (!pre_b) exponents_and_slices<4>(ctx, bt2, N, K, Np, Kp, eb, sb); break;
-        case 5: if (!pre_a) launch_slice<5>(ctx, d.A, M, K, Mp, Kp, ea, sa);
-                if (!pre_b) exponents_and_slices<5>(ctx, bt2, N, K, Np, Kp, eb, sb); break;
-        default: fail(TRG_EINVAL, "split_slices must be 2..5");
-    }
+    if (!pre_b) slice_operand(ctx, S, transposed(d.B), N, K, Np, Kp, nullptr, eb, sb);
     const CUtensorMap ta = make_map(sa, S * Mp, Kp);
     const CUtensorMap tb = make_map(sb, S * Np, Kp);
     // a pair also reads B as 64-row half tiles (its narrow products)
@@ -1649,25 +1411,25 @@ extern "C" int trg_gemm_noalloc(int M, int N, int K, const double* A, int lda, c
 
         // row exponents and slices of A (rows m, k contiguous) and of B as (n, k)
         {
-            dim3 ga((unsigned)((K + SL_K - 1) / SL_K), (unsigned)std::min<int64_t>((M + SL_R - 1) / SL_R, 65535));
-            k_row_exponent<<<ga, 256, 0, stream>>>(A, am, ak, M, K, 1, ea);
-            dim3 gb((unsigned)((K + SL_K - 1) / SL_K), (unsigned)std::min<int64_t>((N + SL_R - 1) / SL_R, 65535));
-            k_row_exponent<<<gb, 256, 0, stream>>>(B, bn, bk, N, K, 0, eb);
+            Gather ga, gb;
+            ga.base = A; ga.off_r = am; ga.off_c = ak; ga.c_fast = true;
+            gb.base = B; gb.off_r = bn; gb.off_c = bk; gb.c_fast = false;
+            launch_row_field<false>(stream, ga, M, K, ea);
+            launch_row_field<false>(stream, gb, N, K, eb);
+            TRG_CUDA(cudaGetLastError());
+            switch (S) {
+                case 2: launch_cut<2>(stream, ga, M, K, Mp, Kp, ea, nullptr, sa, nullptr);
+                        launch_cut<2>(stream, gb, N, K, Np, Kp, eb, nullptr, sb, nullptr); break;
+                case 3: launch_cut<3>(stream, ga, M, K, Mp, Kp, ea, nullptr, sa, nullptr);
+                        launch_cut<3>(stream, gb, N, K, Np, Kp, eb, nullptr, sb, nullptr); break;
+                case 4: launch_cut<4>(stream, ga, M, K, Mp, Kp, ea, nullptr, sa, nullptr);
+                        launch_cut<4>(stream, gb, N, K, Np, Kp, eb, nullptr, sb, nullptr); break;
+                default: launch_cut<5>(stream, ga, M, K, Mp, Kp, ea, nullptr, sa, nullptr);
+                         launch_cut<5>(stream, gb, N, K, Np, Kp, eb, nullptr, sb, nullptr); break;
+            }
+            TRG_CUDA(cudaGetLastError());
             k_exponent_finish<<<(unsigned)((M + 255) / 256), 256, 0, stream>>>(ea, M);
             k_exponent_finish<<<(unsigned)((N + 255) / 256), 256, 0, stream>>>(eb, N);
-            TRG_CUDA(cudaGetLastError());
-            dim3 sa_grid((unsigned)((Kp + SL_K - 1) / SL_K), (unsigned)std::min<int64_t>(Mp / SL_R, 65535));
-            dim3 sb_grid((unsigned)((Kp + SL_K - 1) / SL_K), (unsigned)std::min<int64_t>(Np / SL_R, 65535));
-            switch (S) {
-                case 2: k_slice<2><<<sa_grid, 256, 0, stream>>>(A, am, ak, M, K, Mp, Kp, 1, ea, sa);
-                        k_slice<2><<<sb_grid, 256, 0, stream>>>(B, bn, bk, N, K, Np, Kp, 0, eb, sb); break;
-                case 3: k_slice<3><<<sa_grid, 256, 0, stream>>>(A, am, ak, M, K, Mp, Kp, 1, ea, sa);
-                        k_slice<3><<<sb_grid, 256, 0, stream>>>(B, bn, bk, N, K, Np, Kp, 0, eb, sb); break;
-                case 4: k_slice<4><<<sa_grid, 256, 0, stream>>>(A, am, ak, M, K, Mp, Kp, 1, ea, sa);
-                        k_slice<4><<<sb_grid, 256, 0, stream>>>(B, bn, bk, N, K, Np, Kp, 0, eb, sb); break;
-                default: k_slice<5><<<sa_grid, 256, 0, stream>>>(A, am, ak, M, K, Mp, Kp, 1, ea, sa);
-                         k_slice<5><<<sb_grid, 256, 0, stream>>>(B, bn, bk, N, K, Np, Kp, 0, eb, sb); break;
-            }
             TRG_CUDA(cudaGetLastError());
         }
         const CUtensorMap ta = make_map(sa, S * Mp, Kp);
