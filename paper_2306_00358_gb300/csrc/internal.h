@@ -196,12 +196,9 @@ struct GemmDesc {
     // of the row and the column, far below the FP64 pipe's on the method's
     // operands, but relative to those entries and not to each |a||b|.
     bool allow_exact = false;
-    bool c_m_fast = false;  // consecutive rows are (mostly) adjacent in C
-    // The split epilogue may store without staging when consecutive rows are
-    // adjacent in C and c_n[n + j] = c_n[n] + j c_col_stride inside each
-    // aligned group of 32 columns.
-    bool c_rows_fast = false;
-    int64_t c_col_stride = 0;
+    // consecutive rows are (mostly) adjacent in C: the epilogues store row-wise,
+    // without staging.  The consumer rows cons_m + cons_n are below 2^31.
+    bool c_m_fast = false;
     // Split mode only.  Producer side: record, for the product that will
     // consume C as its A operand, the largest FP64 exponent field of each of
     // its rows (row of element (m, n) = cons_m[m] + cons_n[n]) into cons_ef

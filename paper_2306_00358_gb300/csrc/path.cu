@@ -278,9 +278,7 @@ void contract(Ctx& ctx, const View4& top, const View4& bottom, const double* U, 
                 g.C = X1;
                 g.c_m = ctx.table({{Dn, Dx * DD}, {Dx, 1}});
                 g.c_n = ctx.table({{jb, Dn * Dx * DD}, {Dx, DD}, {Dy, Dx}});
-                g.c_rows_fast = Dy % 32 == 0;
                 g.c_m_fast = true;
-                g.c_col_stride = Dx;
                 if (split) {
                     TRG_CUDA(cudaMemsetAsync(ef2, 0, (size_t)rows2 * sizeof(int), ctx.stream));
                     g.cons_ef = ef2;
@@ -324,9 +322,7 @@ void contract(Ctx& ctx, const View4& top, const View4& bottom, const double* U, 
                 g.C = X2;
                 g.c_m = ctx.table({{jb * Dn, Dy * Dx * Dx}, {Dx, 1}});
                 g.c_n = ctx.table({{Dy, Dx * Dx}, {Dx, Dx}});
-                g.c_rows_fast = Dx % 32 == 0;
                 g.c_m_fast = true;
-                g.c_col_stride = Dx;
                 if (split) {
                     TRG_CUDA(cudaMemsetAsync(ef3, 0, (size_t)rows3 * sizeof(int), ctx.stream));
                     g.cons_ef = ef3;

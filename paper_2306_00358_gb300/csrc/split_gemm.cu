@@ -154,17 +154,19 @@ __device__ __forceinline__ double scaled_i64_to_double(long long v, int e2) {
     return __longlong_as_double((long long)bits);
 }
 
-// The same for |v| < 2^53 (the value is exact: no rounding step).
-__device__ __forceinline__ double scaled_i64_to_double_exact(long long v, int e2) {
-    if (v == 0) return 0.0;
-    const unsigned long long sign = v < 0 ? (1ull << 63) : 0ull;
-    const unsigned long long a = v < 0 ? (unsigned long long)(-v) : (unsigned long long)v;
-    const int top = 63 - __clzll((long long)a);
-    const int ex = top + e2;
-    if (ex < -1022) return __longlong_as_double((long long)sign);
-    if (ex > 1023) return __longlong_as_double((long long)(sign | 0x7FF0000000000000ull));
-    const unsigned long long mant = a << (52 - top);
-    return __longlong_as_double((long long)(sign | ((unsigned long long)(ex + 1023) << 52) | (mant & ((1ull << 52) - 1))));
+// The same through the FP64 pipe's conversion (round to nearest even as
+// well), with the exponent field of the result: one instruction on a pipe
+// that has nothing else to do in place of the twenty integer ones, where the
+// integer pipe is the limit (the direct epilogue).
+__device__ __forceinline__ double scaled_i64(long long v, int e2, int& field) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong((double)v);
+    const int f = (int)(b >> 52) & 0x7FF;
+    const int nf = f + e2;
+    const bool zero = f == 0 || nf < 1, inf = nf > 2046;
+    field = zero ? 0 : inf ? 2047 : nf;
+    const unsigned long long body = zero ? 0ull : inf ? 0x7FF0000000000000ull
+                                                     : (b & 0x000FFFFFFFFFFFFFull) | ((unsigned long long)nf << 52);
+    return __longlong_as_double((long long)((f == 0 ? 0ull : b & (1ull << 63)) | body));
 }
 
 // |v| rounded to 53 significant bits (half to even), as the FP64 value of v
@@ -251,8 +253,7 @@ struct MmaArgs {
     int rows_per_crow, cols_per_crow;
     int64_t ck_stride;         // fused: consumer-column step between adjacent producer columns
     int v_exact53;             // fused: every V is below 2^53 in magnitude (K <= 8192)
-    int c_rows_fast;           // C's rows are adjacent: store without staging ...
-    int64_t c_col_stride;      // ... with c_n[n + j] = c_n[n] + j c_col_stride in a 32-column group
+    int c_rows_fast;           // C's rows are adjacent: store without staging
     // limit of the epilogue's wait for a finished accumulator chunk (the
     // other waits keep WAIT_NS); a short one lets tests reach the timeout path
     unsigned long long acc_wait_ns;
@@ -669,42 +670,54 @@ k_split_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                     const int nt = nb * BN + colh * CPT;
                     if constexpr (MODE == EPI_DIRECT) {
                         // rows adjacent in C: form, record and store each result in one
-                        // pass (the lanes, adjacent rows, write 256 contiguous bytes).
+                        // pass (the lanes, adjacent rows, write contiguous runs).
+                        // Bound by the instructions per result where K is short: X1
+                        // at D = 64 (K = 64) takes 1.36 ms a launch (1.50 with integer
+                        // conversion and an atomic per lane), at (45, 43) 0.95 ms
+                        // where the staged form's stores, 8 bytes apart by Dx, took 1.82.
                         // The warp's 32 columns are the same for every lane: lane j
-                        // loads column j's exponent and consumer-row offset once and
-                        // the loop takes them by shuffle, so no global load waits
+                        // loads column j's exponent, offset and consumer-row offset once
+                        // and the loop takes them by shuffle, so no global load waits
                         // inside it.
                         const bool col_in = nt + lane < g.N;
                         const int eb_l = col_in ? g.eb[nt + lane] - 36 : 0;
-                        const long long cn_l = (g.cons_ef && col_in) ? (long long)g.cons_n[nt + lane] : 0;
-                        double* cp = g.C + (row_ok ? g.c_m[m] + g.c_n[nt] : 0);
-                        const int64_t step = g.c_col_stride;
-                        const int64_t cm0 = (g.cons_ef && row_ok) ? g.cons_m[m] : 0;
-                        int64_t cur = -1;
-                        int cur_max = 0;
+                        const long long co_l = col_in ? (long long)g.c_n[nt + lane] : 0;
+                        const int cn_l = (g.cons_ef && col_in) ? (int)g.cons_n[nt + lane] : 0;
+                        double* cp = g.C + (row_ok ? g.c_m[m] : 0);
+                        const int cm0 = (g.cons_ef && row_ok) ? (int)g.cons_m[m] : -1;
+                        // lanes of one consumer row: one atomic for all of them
+                        const bool one_row = __match_any_sync(0xffffffffu, cm0) == 0xffffffffu;
+                        const int ncol = min(CPT, g.N - nt);
+                        int cur = -1, cur_max = 0;
+                        auto record = [&]() {
+                            if (one_row) {
+                                const unsigned mx = __reduce_max_sync(0xffffffffu, (unsigned)cur_max);
+                                if (lane == 0 && mx && cm0 >= 0) atomicMax(&g.cons_ef[cm0 + cur], (int)mx);
+                            } else if (cm0 >= 0 && cur_max) {
+                                atomicMax(&g.cons_ef[cm0 + cur], cur_max);
+                            }
+                        };
 #pragma unroll
                         for (int j = 0; j < CPT; ++j) {
-                            const int e2 = ea + __shfl_sync(0xffffffffu, eb_l, j);
-                            const long long cn = __shfl_sync(0xffffffffu, cn_l, j);
-                            if (row_ok && nt + j < g.N) {
-                                const double v = g.v_exact53 ? scaled_i64_to_double_exact(J[j], e2)
-                                                             : scaled_i64_to_double(J[j], e2);
-                                *cp = v;
+                            if (j < ncol) {
+                                const int e2 = ea + __shfl_sync(0xffffffffu, eb_l, j);
+                                const long long co = __shfl_sync(0xffffffffu, co_l, j);
+                                int field;
+                                const double v = scaled_i64(J[j], e2, field);
+                                if (row_ok) cp[co] = v;
                                 if (g.cons_ef) {
-                                    const int64_t crow = cm0 + cn;
-                                    const int ef = (int)(((unsigned long long)__double_as_longlong(v) >> 52) & 0x7FF);
-                                    if (crow != cur) {
-                                        if (cur >= 0 && cur_max) atomicMax(&g.cons_ef[cur], cur_max);
-                                        cur = crow;
-                                        cur_max = ef;
+                                    const int cn = __shfl_sync(0xffffffffu, cn_l, j);   // the same for all lanes
+                                    if (cn != cur) {
+                                        if (j > 0) record();
+                                        cur = cn;
+                                        cur_max = row_ok ? field : 0;
                                     } else {
-                                        cur_max = max(cur_max, ef);
+                                        cur_max = max(cur_max, row_ok ? field : 0);
                                     }
                                 }
                             }
-                            cp += step;
                         }
-                        if (cur >= 0 && cur_max) atomicMax(&g.cons_ef[cur], cur_max);
+                        if (g.cons_ef && ncol > 0) record();
                         continue;
                     }
                     if constexpr (MODE == EPI_KSPLIT) {
@@ -1181,7 +1194,7 @@ void gemm_split(Ctx& ctx, const GemmDesc& d) {
     const int CG = (ctx.cfg.mma_pairs && M > BM) ? 2 : 1;
     const int Mp = (int)split_rows_padded(ctx, M), Np = (N + BN - 1) / BN * BN, Kp = (int)split_k_padded(K);
     const bool pre_a = d.a_slices != nullptr;    // A arrives sliced from its producer
-    if (d.gram && (M != N || d.b_slices || pre_a || d.cs_out || d.cons_ef || d.c_rows_fast))
+    if (d.gram && (M != N || d.b_slices || pre_a || d.cs_out || d.cons_ef || d.c_m_fast))
         fail(TRG_EINVAL, "split GEMM: a Gram product takes a square C and plain operands");
     // a Gram product reads A's slices for B too (same rows, same padding)
     const bool gram_b = d.gram && Mp == Np;
@@ -1215,7 +1228,7 @@ void gemm_split(Ctx& ctx, const GemmDesc& d) {
     a.cons_ef = d.cons_ef; a.cons_m = d.cons_m; a.cons_n = d.cons_n;
     a.cs_out = d.cs_out; a.cs_plane = d.cs_mp * d.cs_kp; a.cs_kp = d.cs_kp; a.cs_e = d.cs_e;
     a.ck_m = d.ck_m; a.ck_n = d.ck_n; a.rows_per_crow = d.rows_per_crow; a.cols_per_crow = d.cols_per_crow;
-    a.ck_stride = d.ck_stride; a.c_rows_fast = d.c_rows_fast ? 1 : 0; a.c_col_stride = d.c_col_stride;
+    a.ck_stride = d.ck_stride; a.c_rows_fast = d.c_m_fast ? 1 : 0;
     // |V| <= (K / 512) (2^32 + 2^24) 2^14 + 2 K 2^20 < 2^53 for K <= 8192
     a.v_exact53 = Kp <= 8192 ? 1 : 0;
     // split K where the tiles leave most SMs idle: a function of the shape
@@ -1223,7 +1236,7 @@ void gemm_split(Ctx& ctx, const GemmDesc& d) {
     // choice still gives the same bits
     a.ksplit = 1; a.kb_per = Kp / BK; a.kpart = nullptr;
     a.tile_list = nullptr; a.n_list = 0; a.sym = d.gram ? 1 : 0;
-    if (d.allow_ksplit && !d.cs_out && !d.c_rows_fast && !d.cons_ef && !d.gram) {
+    if (d.allow_ksplit && !d.cs_out && !d.cons_ef && !d.gram) {
         const int chunks = (Kp / BK + CHUNK_STAGES - 1) / CHUNK_STAGES;
         const int tiles128 = ((M + BM - 1) / BM) * ((N + BN - 1) / BN);
         if (2 * tiles128 <= ctx.sm_count && chunks >= 2) {
@@ -1234,6 +1247,7 @@ void gemm_split(Ctx& ctx, const GemmDesc& d) {
             if (a.ksplit > 1) {
                 ctx.ensure(ctx.ksplit_ws, (size_t)a.ksplit * N * M * sizeof(long long));
                 a.kpart = ctx.ksplit_ws.as<long long>();
+                a.c_rows_fast = 0;    // the parts have their own layout
             } else {
                 a.kb_per = Kp / BK;
             }
@@ -1289,7 +1303,7 @@ void gemm_split(Ctx& ctx, const GemmDesc& d) {
             case 11: launch_mma<5, 2>(ctx, ta, tb, tbh, b); break;
         }
     };
-    const int mode = d.cs_out ? 2 : (d.c_rows_fast ? 1 : (a.ksplit > 1 ? 3 : (d.gram ? 4 : 0)));
+    const int mode = d.cs_out ? 2 : (a.c_rows_fast ? 1 : (a.ksplit > 1 ? 3 : (d.gram ? 4 : 0)));
     const TuneChoice ch = tuned_choice(ctx, M, N, Kp, S, mode, CG, launch);
     const int tok = ctx.region_begin(TRG_PHASE_MMA);
     const int tok_x2 = ctx.phase == TRG_PHASE_X2 ? ctx.region_begin(TRG_PHASE_MMA_X2) : -1;
@@ -1440,7 +1454,7 @@ extern "C" int trg_gemm_noalloc(int M, int N, int K, const double* A, int lda, c
         a.cons_ef = nullptr; a.cons_m = nullptr; a.cons_n = nullptr;
         a.cs_out = nullptr; a.cs_plane = 0; a.cs_kp = 0; a.cs_e = nullptr; a.ck_m = nullptr; a.ck_n = nullptr;
         a.rows_per_crow = a.cols_per_crow = 0;
-        a.ck_stride = 0; a.c_rows_fast = 0; a.c_col_stride = 0; a.v_exact53 = 0;
+        a.ck_stride = 0; a.c_rows_fast = 0; a.v_exact53 = 0;
         a.acc_wait_ns = WAIT_NS;
         a.ksplit = 1; a.kb_per = Kp / BK; a.kpart = nullptr;
         a.tile_list = nullptr; a.n_list = 0; a.sym = 0;
