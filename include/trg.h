@@ -58,7 +58,7 @@ typedef enum trg_precision {
     TRG_FP64 = 0,        /* FP64.  trg_gemm runs on the FP64 pipe.  The products of a solve and of
                             the component calls do too while they are small; larger ones are
                             computed from exact BF16 digit products on the tensor cores and
-                            rounded to FP64 once, off by at most 2^-53 |C| + 10 K 2^-62 times the
+                            brought to FP64, off by at most 2^-51 |C| + 16 K 2^-118 times the
                             largest entries of the row and the column (an FP64 sum of K products
                             is off by up to K 2^-53 |A||B|).  Operands with infinities, NaN or
                             rows outside 2^-400 .. 2^400 stay on the FP64 pipe. */

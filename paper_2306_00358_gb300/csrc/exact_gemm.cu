@@ -4,38 +4,42 @@
 // tensor rate, so an FP64 product that is large enough is computed from BF16
 // digit products instead, to more than FP64 accuracy.  Each operand row (A) /
 // column (B) gets a power-of-two scale 2^e with |x| < 2^e, and
-//     X = rint(x 2^(63 - e)) = sum_p d_p 2^(8 (7 - p)),   p = 0..7,
+//     X = rint(x 2^(119 - e)) = sum_p d_p 2^(8 (14 - p)),   p = 0..14,
 // d_0 in [-128, 128], d_p in [-128, 127] (an error-free splitting as in
-// split_gemm.cu, with eight digits and every sum exact: Ozaki, Ogita, Oishi,
-// Rump, Numer. Algorithms 59 (2012) 95).  An element down to 2^-10 of its
-// row's largest keeps all 53 bits.  With D_d = sum_{p + q = d} A_p B_q,
-//     C = 2^(ea + eb - 70) sum_{d < 8} D_d 2^(8 (7 - d)):
-// digit products are integers up to 2^14, a run of 128 K sums the at most
-// eight products of a D_d exactly in FP32 (8 x 128 x 2^14 = 2^24), the
-// epilogue moves each run into int64 sums and the 96-bit total is rounded to
-// FP64 once.  What is left out (d >= 8) and the rounding of X are below
-// 10 K 2^-64 2^(ea + eb).  On the method's tensors, environments and isometries (leg sizes 8 to 32) the
-// results are within 1.1e-16 of sum |a||b|, element by element, where a
-// K-long FP64 chain is off by 3e-16 to 3e-15.
+// split_gemm.cu, with every sum exact: Ozaki, Ogita, Oishi, Rump, Numer.
+// Algorithms 59 (2012) 95).  With D_d = sum_{p + q = d} A_p B_q,
+//     C = 2^(ea + eb - 126) sum_{d < 15} D_d 2^(8 (14 - d)):
+// digit products are integers up to 2^14, a run of 64 K sums the at most 15
+// products of a D_d exactly in FP32 (15 x 64 x 2^14 < 2^24), the epilogue
+// moves each run into int64 sums and the wide total is turned into FP64.
+//
+// Why 15 digits: what is left out is below 16 K 2^-120 2^(ea + eb), so every
+// element of C is as accurate as an FP64 sum, relative to its own sum |a||b|,
+// down to sums 2^-60 of the largest possible one.  Eight digits are enough for
+// an error far below FP64's relative to the largest elements, and cost a
+// third, but the method needs the small elements too: the couplings between
+// nearly decoupled sectors of a tensor decide how near-degenerate vectors mix.
+// (Critical Ising with a field, Dcut 16, 20 half-steps: <s> varies with the
+// start vectors by 8e-10 with the FP64 pipe, by 9e-8 with eight digits.)
 //
 // Rows or columns whose largest entry lies outside 2^-400 .. 2^400, or that
 // hold an infinity or a NaN, raise a device flag: the tensor kernel then
 // returns at once and the FP64 pipe kernel that is queued behind it, idle
 // otherwise, computes the product.
 //
-// What bounds it: the tensor pipe, 36 digit products of 2 M N K each.
-// 128 x 64 output tile, one persistent CTA per SM: the eight D_d of 64
-// columns fill the 512 TMEM columns.  A stage is 32 K of both operands (64 KB
-// of A digits, 32 KB of B digits, one TMA box each), two stages.  The products
-// of one A digit with adjacent B digits land in adjacent accumulators, so 12
-// instructions of up to N = 256 cover the 36 products of a 16-deep step.
-// They are issued in two groups, the one that lands in D_4..D_7 (26 products)
-// before the one that lands in D_0..D_3: a run's drain of D_4..D_7 runs under
-// the other group's products, and the drain of D_0..D_3 under the next run's
-// first group.  Measured, contraction at Dx = Dy = Dn = 48 (three products,
-// 1.22e12 FP64 FLOPs): 993 ms on the FP64 pipe, 34.7 ms here, 30.8 of them in
-// this kernel (4.4e13 digit FLOPs at 1430 TFLOP/s), 2.9 cutting digits, 0.9
-// finding exponents; environment at (24, 22): 0.65 -> 0.25 ms.
+// What bounds it: the tensor pipe, 120 digit products of 2 M N K each.
+// 128 x 32 output tile, one persistent CTA per SM: the 15 D_d of 32 columns
+// take 480 TMEM columns.  A stage is 16 K of both operands (60 KB of A digits,
+// 15 KB of B digits, one TMA box each), two stages.  The products of one A
+// digit with adjacent B digits land in adjacent accumulators, so 22
+// instructions of up to N = 256 cover the 120 products of a step.  They are
+// issued in two groups, the one that lands in D_7..D_14 (92 products) before
+// the one that lands in D_0..D_6: a run's drain of D_7..D_14 runs under the
+// other group's products, and the drain of D_0..D_6 under the next run's first
+// group.  Measured, contraction at Dx = Dy = Dn = 48 (three products, 1.22e12
+// FP64 FLOPs): 993 ms on the
+// FP64 pipe, 113 here, 110 of them in this kernel (1.5e14 digit FLOPs, 1340
+// TFLOP/s); environment at (24, 22): 0.65 -> 0.28 ms.
 #include <algorithm>
 #include <cmath>
 
@@ -47,13 +51,14 @@ namespace trg {
 
 namespace {
 
-constexpr int XS = 8;                            // digits
-constexpr int XM = 128, XN = 64, XK = 32;        // tile rows, columns, K per stage
+constexpr int XS = 15;                           // digits
+constexpr int XM = 128, XN = 32, XK = 16;        // tile rows, columns, K per stage
+constexpr int XL = 7;                            // D_0 .. D_(XL-1) are group 0, the rest group 1
 constexpr int XA_TILE = XM * XK * 2;             // bytes of one digit's A tile
 constexpr int XB_TILE = XN * XK * 2;
-constexpr int XSTAGE = XS * (XA_TILE + XB_TILE); // 96 KB
+constexpr int XSTAGE = XS * (XA_TILE + XB_TILE); // 75 KB
 constexpr int XSTAGES = 2;
-constexpr int XRUN = 128 / XK;                   // stages of an exact run
+constexpr int XRUN = 64 / XK;                    // stages of an exact run
 constexpr int XEPI = 16;                         // epilogue warps
 constexpr int XTHREADS = 64 + 32 * XEPI;
 constexpr int XCPT = XN / 4;                     // columns per epilogue thread
@@ -62,31 +67,45 @@ constexpr int XBAR = 256;
 constexpr int XSMEM = XSTAGES * XSTAGE + XSTAGING + XBAR + 1024;
 static_assert(XSMEM <= 232448, "exact product shared memory");
 
-// The digit products of one 16-deep step: A digit a times the n B digits
+// The digit products of one 16-deep step: A digit a times the n <= 8 B digits
 // from b on, into the accumulators D_(a+b) .. D_(a+b+n-1).  Group 1 lands in
-// D_4..D_7, group 0 in D_0..D_3; the first entry of a group covers all four
-// of its accumulators and resets them at the start of a run.
+// D_7..D_14, group 0 in D_0..D_6; the first entry of a group covers all of its
+// accumulators and resets them at the start of a run.
 struct XIns { int a, b, n, group; };
-__host__ __device__ constexpr int xins_count() { return 12; }
+__host__ __device__ constexpr int xins_count() { return XS + XL; }
 __host__ __device__ constexpr XIns xins(int t) {
-    return t < 8 ? XIns{t, t < 4 ? 4 - t : 0, t < 4 ? 4 : 8 - t, 1} : XIns{t - 8, 0, 4 - (t - 8), 0};
+    return t < XS ? XIns{t, t < XL ? XL - t : 0, t < XL ? XS - XL : XS - t, 1} : XIns{t - XS, 0, XL - (t - XS), 0};
 }
 __host__ __device__ constexpr bool xins_ok() {
     int seen[XS][XS] = {};
     for (int t = 0; t < xins_count(); ++t) {
         const XIns in = xins(t);
+        if (in.n < 1 || in.n * XN > 256) return false;
         for (int q = in.b; q < in.b + in.n; ++q) {
             const int d = in.a + q;
-            if (d >= XS || (d >= 4) != (in.group == 1)) return false;
+            if (d >= XS || (d >= XL) != (in.group == 1)) return false;
             seen[in.a][q] += 1;
         }
     }
     for (int p = 0; p < XS; ++p)
         for (int q = 0; q < XS; ++q)
             if (seen[p][q] != (p + q < XS ? 1 : 0)) return false;
-    return xins(0).b == 4 && xins(0).n == 4 && xins(8).n == 4;
+    return xins(0).n == XS - XL && xins(XS).n == XL;
 }
 static_assert(xins_ok(), "digit product table");
+static_assert(XS * XN <= 512 && (double)XS * 64 * (1 << 14) <= (1 << 24), "accumulators");
+
+// Shared-memory matrix descriptor: K-major BF16 tile, 32-byte rows, 32-byte
+// swizzle; 8-row groups 256 bytes apart.
+__device__ __forceinline__ uint64_t xsmem_desc(uint32_t addr) {
+    uint64_t d = 0;
+    d |= (uint64_t)((addr >> 4) & 0x3FFF);          // start address
+    d |= (uint64_t)1 << 16;                         // leading byte offset (unused for swizzled K-major)
+    d |= (uint64_t)(256 >> 4) << 32;                // stride byte offset
+    d |= (uint64_t)1 << 46;                         // descriptor version
+    d |= (uint64_t)6 << 61;                         // swizzle: 32 bytes
+    return d;
+}
 
 struct XArgs {
     int M, N, Kp;
@@ -104,13 +123,18 @@ struct XArgs {
     int* status;
 };
 
-// (hi 2^32 + lo) 2^e2 in FP64, rounded once (twice when |hi| >= 2^53, where
-// the second rounding is below 2^-20 of an ulp)
-__device__ __forceinline__ double wide_to_double(long long hi, long long lo, int e2) {
-    hi += lo >> 32;
-    const double r = fma((double)hi, 4294967296.0, (double)(unsigned)(lo & 0xffffffffll));
+// The int64 sums of an element: D_0..D_3, D_4..D_7, D_8..D_11, D_12..D_14, each
+// in units of its last D: V = w0 2^88 + w1 2^56 + w2 2^24 + w3.
+// V 2^e2 in FP64, within 2 units in the last place.
+__device__ __forceinline__ double wide_to_double(const long long (&w)[4], int e2) {
+    long long w2 = w[2] + (w[3] >> 24);
+    long long w1 = w[1] + (w2 >> 32);
+    const long long w0 = w[0] + (w1 >> 32);
+    double r = fma((double)w0, 4294967296.0, (double)(unsigned)(w1 & 0xffffffffll));
+    r = fma(r, 4294967296.0, (double)(unsigned)(w2 & 0xffffffffll));
+    r = fma(r, 16777216.0, (double)(int)(w[3] & 0xffffffll));
     if (r == 0.0) return 0.0;
-    // |e2| <= 872 and |r| < 2^96: the exponent field stays in range
+    // (nonzero rows and columns have -928 <= e2 <= 676 and |r| < 2^150: the field stays in range)
     return __longlong_as_double(__double_as_longlong(r) + ((long long)e2 << 52));
 }
 
@@ -207,21 +231,16 @@ k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                     ok = mbar_wait(&full[stage], phase, abort_flag, g.status);
                     if (!ok) break;
                     tc_fence_after();
-                    const uint64_t dbase = smem_desc(smem_u32(smem + stage * XSTAGE));
+                    const uint64_t dbase = xsmem_desc(smem_u32(smem + stage * XSTAGE));
                     auto issue = [&](int group) {
 #pragma unroll
-                        for (int kk = 0; kk < XK / 16; ++kk) {
-#pragma unroll
-                            for (int t = 0; t < xins_count(); ++t) {
-                                const XIns in = xins(t);
-                                if (in.group != group) continue;
-                                const bool first = t == 0 || t == 8;
-                                const uint32_t acc = (first && run_start && kk == 0) ? 0u : 1u;
-                                const uint64_t da = dbase + (uint64_t)((in.a * XA_TILE + kk * 32) >> 4);
-                                const uint64_t db = dbase + (uint64_t)((XS * XA_TILE + in.b * XB_TILE + kk * 32) >> 4);
-                                mma_bf16<1>(tmem + (uint32_t)((in.a + in.b) * XN), da, db, idesc_bf16(XM, in.n * XN),
-                                            acc);
-                            }
+                        for (int t = 0; t < xins_count(); ++t) {
+                            const XIns in = xins(t);
+                            if (in.group != group) continue;
+                            const uint32_t acc = ((t == 0 || t == XS) && run_start) ? 0u : 1u;
+                            const uint64_t da = dbase + (uint64_t)((in.a * XA_TILE) >> 4);
+                            const uint64_t db = dbase + (uint64_t)((XS * XA_TILE + in.b * XB_TILE) >> 4);
+                            mma_bf16<1>(tmem + (uint32_t)((in.a + in.b) * XN), da, db, idesc_bf16(XM, in.n * XN), acc);
                         }
                     };
                     if (run_start && run_no > 0) {
@@ -259,9 +278,9 @@ k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             int mb, nb;
             coords(tile, mb, nb);
             const int nruns = (num_kb + XRUN - 1) / XRUN;
-            long long hi[XCPT], lo[XCPT];        // D_0..D_3 and D_4..D_7, each as an int64 in units of its last digit
+            long long w[XCPT][4];
 #pragma unroll
-            for (int j = 0; j < XCPT; ++j) hi[j] = lo[j] = 0;
+            for (int j = 0; j < XCPT; ++j) w[j][0] = w[j][1] = w[j][2] = w[j][3] = 0;
             for (int c = 0; c < nruns && ok; ++c, ++run_no) {
 #pragma unroll
                 for (int grp = 1; grp >= 0; --grp) {
@@ -271,15 +290,14 @@ k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                     if (!ok) break;
                     tc_fence_after();
 #pragma unroll
-                    for (int d = 0; d < 4; ++d) {
+                    for (int d = grp ? XL : 0; d < (grp ? XS : XL); ++d) {
                         uint32_t r[XCPT];
-                        tmem_ld16(tmem + lane_base + (uint32_t)((grp * 4 + d) * XN + colq * XCPT), r);
+                        tmem_ld8(tmem + lane_base + (uint32_t)(d * XN + colq * XCPT), r);
                         tmem_wait_ld();
+                        constexpr int last[4] = {3, 7, 11, 14};
+                        const long long unit = 1ll << (8 * (last[d >> 2] - d));
 #pragma unroll
-                        for (int j = 0; j < XCPT; ++j) {
-                            const long long v = (long long)__float2int_rn(__uint_as_float(r[j])) * (1ll << (8 * (3 - d)));
-                            if (grp) lo[j] += v; else hi[j] += v;
-                        }
+                        for (int j = 0; j < XCPT; ++j) w[j][d >> 2] += (long long)__float2int_rn(__uint_as_float(r[j])) * unit;
                     }
                     tc_fence_before();
                     __syncwarp();
@@ -290,13 +308,13 @@ k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             const int m = mb * XM + quad * 32 + lane;
             const bool row_ok = m < g.M;
             const int nt = nb * XN + colq * XCPT;
-            // the warp's 16 columns are the same for every lane: lane j loads
+            // the warp's eight columns are the same for every lane: lane j loads
             // column j's exponent and offset, the loop takes them by shuffle
             const bool col_in = lane < XCPT && nt + lane < g.N;
             const int fb = col_in ? g.fb[nt + lane] : 0;
             const long long cn_l = col_in ? (long long)g.c_n[nt + lane] : 0;
             const int ea = row_ok ? max(g.fa[m], 1) - 1022 : 0;
-            const int eb_l = max(fb, 1) - 1022 - 70;
+            const int eb_l = max(fb, 1) - 1022 - 126;
             if (g.rows_fast) {
                 // lanes are adjacent rows, adjacent in C
                 double* cp = g.C + (row_ok ? g.c_m[m] : 0);
@@ -304,7 +322,7 @@ k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                 for (int j = 0; j < XCPT; ++j) {
                     const int e2 = ea + __shfl_sync(0xffffffffu, eb_l, j);
                     const long long cn = __shfl_sync(0xffffffffu, cn_l, j);
-                    if (row_ok && nt + j < g.N) cp[cn] = wide_to_double(hi[j], lo[j], e2);
+                    if (row_ok && nt + j < g.N) cp[cn] = wide_to_double(w[j], e2);
                 }
                 continue;
             }
@@ -312,7 +330,7 @@ k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
 #pragma unroll
             for (int j = 0; j < XCPT; ++j) {
                 const int e2 = ea + __shfl_sync(0xffffffffu, eb_l, j);
-                v[j] = (row_ok && nt + j < g.N) ? wide_to_double(hi[j], lo[j], e2) : 0.0;
+                v[j] = (row_ok && nt + j < g.N) ? wide_to_double(w[j], e2) : 0.0;
             }
             if (g.sym && row_ok) {
                 // the mirror (n, m) of each element above the diagonal
@@ -365,7 +383,7 @@ CUtensorMap digit_map(const void* base, int rows, int kp, int box_rows) {
     const cuuint32_t box[3] = {(cuuint32_t)XK, (cuuint32_t)box_rows, (cuuint32_t)XS};
     const cuuint32_t estr[3] = {1, 1, 1};
     CUresult r = encode_fn()(&m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box,
-                             estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
+                             estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B,
                              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) fail(TRG_ECUDA, "cuTensorMapEncodeTiled failed (" + std::to_string((int)r) + ")");
     return m;
@@ -425,10 +443,10 @@ int64_t exact_scratch_bytes(int64_t M, int64_t N, int64_t K) {
 double exact_us(const Ctx& ctx, int64_t M, int64_t N, int64_t K, bool sym) {
     if (M > (1ll << 30) || N > (1ll << 30) || K > (1 << 17)) return 1e300;
     const double tm = (double)up(M, XM) / XM, tn = (double)up(N, XN) / XN;
-    const double tiles = sym ? 0.5 * tm * (tn + 2) : tm * tn;
-    const double runs = std::ceil((double)K / 128.0);
-    const double mma = std::ceil(tiles / ctx.sm_count) * (runs * 5.4 + 3.0);
-    const double moved = (32.0 * (double)K * ((double)M + (sym ? 0.0 : (double)N)) + 8.0 * (double)M * (double)N) / 4.0e6;
+    const double tiles = sym ? 0.5 * tm * (tn + 4) : tm * tn;
+    const double runs = std::ceil((double)K / 64.0);
+    const double mma = std::ceil(tiles / ctx.sm_count) * (runs * 4.4 + 3.0);
+    const double moved = (46.0 * (double)K * ((double)M + (sym ? 0.0 : (double)N)) + 8.0 * (double)M * (double)N) / 4.0e6;
     return 25.0 + mma + moved;
 }
 
@@ -491,7 +509,7 @@ bool gemm_exact(Ctx& ctx, const GemmDesc& d) {
             const int tok = ctx.region_begin(TRG_PHASE_MMA);
             k_exact_mma<<<grid, XTHREADS, XSMEM, ctx.stream>>>(ta, tb, a);
             TRG_LAUNCHED(ctx);
-            ctx.region_end(tok, 2.0 * (double)mr * nr * K, 36.0 * 2.0 * (double)mr * nr * Kp);
+            ctx.region_end(tok, 2.0 * (double)mr * nr * K, 120.0 * 2.0 * (double)mr * nr * Kp);
             if (sym) break;
         }
     }

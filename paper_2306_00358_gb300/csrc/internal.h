@@ -192,9 +192,7 @@ struct GemmDesc {
     // n x m products of the isometry); exact partial sums, deterministic.
     bool allow_ksplit = false;
     // FP64 mode: the product may run on the tensor cores when it is large
-    // enough (gemm_exact): an error of a few 2^-64 K times the largest entries
-    // of the row and the column, far below the FP64 pipe's on the method's
-    // operands, but relative to those entries and not to each |a||b|.
+    // enough (gemm_exact).
     bool allow_exact = false;
     // consecutive rows are (mostly) adjacent in C: the epilogues store row-wise,
     // without staging.  The consumer rows cons_m + cons_n are below 2^31.

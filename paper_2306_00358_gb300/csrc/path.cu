@@ -79,7 +79,7 @@ void gemm(Ctx& ctx, const GemmDesc& g, int precision) {
         // FP64 pipe.  Their fixed cost is six launches (25 us in the model)
         // and the digits; the lines cross at about 200 x 200 x 200.  The
         // three products of a (24, 22) environment (528 and 576 wide) take
-        // 651 us on the pipe and 250 us on the tensor cores, 256 x 40 x 256
+        // 651 us on the pipe and 283 us on the tensor cores, 256 x 40 x 256
         // 14 us against more than 30.
         const bool sym = g.gram && g.M == g.N;
         const bool exact = g.allow_exact && !ctx.no_exact && g.beta == 0.0 && g.M > 0 && g.N > 0 &&

@@ -1,12 +1,12 @@
 // Cutting FP64 operands into BF16 digits for the tensor-core products
-// (split_gemm.cu: S = 2..5 slices, exact_gemm.cu: eight digits).
+// (split_gemm.cu: S = 2..5 slices, exact_gemm.cu: 15 digits).
 //
 // An operand is rows r < R of length K, element (r, k) at src[off_r[r] +
 // off_c[k]]; its digits go to out[p][r][k] (r < Rp, k < Kp, zero in the
 // padding).  With f the largest exponent field of a row and e = f - 1022
 // (|x| < 2^e), X = rint(x 2^(F - e)), F = 7 + 8 (S - 1), halves away from
 // zero, is the sum of d_p 2^(8 (S - 1 - p)), d_0 in [-128, 128], d_p in
-// [-128, 127]; slices are stored as d_p 2^(-8p) (S <= 5) or as d_p (S = 8).
+// [-128, 127]; slices are stored as d_p 2^(-8p) (S <= 5) or as d_p (S = 15).
 //
 // All of it is bound by HBM: 8 B read (twice where the exponents take a pass
 // of their own) and 2 S B written per element.
@@ -53,18 +53,19 @@ __device__ __forceinline__ void cut(double x, int f, float (&d)[S]) {
     const bool neg = (long long)b < 0;
     // adding 128 to every digit but the first turns the signed digits into
     // bytes; a byte under the exponent of 2^23 is the FP32 number 2^23 + byte
-    if constexpr (S == 8) {
-        const int sh = f - ex - 10;              // X = mantissa 2^-sh
-        const unsigned long long m = sh <= 0 ? m53 << (-sh & 63) : sh < 60 ? (m53 + (1ull << (sh - 1))) >> sh : 0ull;
-        const unsigned long long y = (neg ? 0ull - m : m) + 0x0080808080808080ull;
-        const unsigned ylo = (unsigned)y, yhi = (unsigned)(y >> 32);
-        // the first digit is the signed top byte, whose sign bit is part of the value when X >= 0
-        d[0] = (float)(neg ? (int)yhi >> 24 : (int)(yhi >> 24));
+    if constexpr (S == 15) {
+        // X = mantissa 2^(66 - (f - ex)), 120 bits
+        const int sh = f - ex - 66;
+        typedef unsigned __int128 u128;
+        const u128 m = sh <= 0 ? (u128)m53 << (-sh & 127) : sh < 60 ? (u128)((m53 + (1ull << (sh - 1))) >> sh) : (u128)0;
+        const u128 y = (neg ? (u128)0 - m : m) + (((u128)0x0000808080808080ull << 64) | 0x8080808080808080ull);
+        const unsigned long long ylo = (unsigned long long)y, yhi = (unsigned long long)(y >> 64);
+        d[0] = (float)(int)((long long)yhi >> 48);
+        const unsigned q[4] = {(unsigned)ylo, (unsigned)(ylo >> 32), (unsigned)yhi, (unsigned)(yhi >> 32)};
 #pragma unroll
-        for (int p = 1; p < 8; ++p) {
-            const unsigned v = p < 4 ? __byte_perm(yhi, 0x4B000000u, 0x7440u | (unsigned)(3 - p))
-                                     : __byte_perm(ylo, 0x4B000000u, 0x7440u | (unsigned)(7 - p));
-            d[p] = __uint_as_float(v) - 8388736.0f;   // 2^23 + 128
+        for (int p = 1; p < 15; ++p) {
+            const int byte = 14 - p;
+            d[p] = __uint_as_float(__byte_perm(q[byte >> 2], 0x4B000000u, 0x7440u | (unsigned)(byte & 3))) - 8388736.0f;   // 2^23 + 128
         }
     } else {
         constexpr int F = 7 + 8 * (S - 1);
