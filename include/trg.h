@@ -91,12 +91,10 @@ typedef struct trg_config {
                                 tensor-core instruction drives two SMs, each staging half
                                 of B); 0 keeps one CTA per 128 x 128 tile.  Results are
                                 identical either way. */
-    int fused_slices;        /* TRG_SPLIT_BF16, bond dimensions 32, 64 or 128: 1 (default)
-                                lets the D^7 contraction product write the last product's
-                                BF16 operand slices directly (no FP64 intermediate, no
-                                slicing pass); 2 also hands the first product over as
-                                slices; 0 always goes through FP64.  Results are identical
-                                in all three. */
+    int fused_slices;        /* 0, 1 (default) or 2.  Once chose how the contraction's products hand
+                                their results on (FP64 or BF16 slices); results never depended on
+                                it, FP64 is the faster form throughout, and every value now takes
+                                it. */
     int fp64_max_dd;         /* TRG_SPLIT_BF16: half-steps on a tensor with Dx*Dy <= fp64_max_dd
                                 (Dx*Dy*Dz on the cubic lattice) run in FP64 (default 16: the
                                 first three half-steps of a model's solve, bond dimensions 2

@@ -201,25 +201,14 @@ struct GemmDesc {
     // consume C as its A operand, the largest FP64 exponent field of each of
     // its rows (row of element (m, n) = cons_m[m] + cons_n[n]) into cons_ef
     // (zeroed beforehand).  Consumer side: a_ef holds those fields for this
-    // product's A rows, so the exponent pass over A is skipped.
+    // product's A rows, so the exponent pass over A is skipped.  The producer
+    // stores row-wise (c_m_fast).
     int* cons_ef = nullptr;
     const int64_t* cons_m = nullptr;
     const int64_t* cons_n = nullptr;
     const int* a_ef = nullptr;
-    // Split mode, fused hand-over: instead of C, the producer writes the
-    // consumer's BF16 A slices ([S][Mp][Kp], element (m, n) at consumer row
-    // cons_m[m] + cons_n[n], column ck_m[m] + ck_n[n]) and their row
-    // exponents (cs_e).  Valid when every consumer row lies in one 128 x 128
-    // tile as rows_per_crow consecutive rows (a multiple of 32) times
-    // cols_per_crow consecutive columns (32, 64 or 128); the consumer then
-    // takes a_slices / a_e and skips slicing A.  Bit-identical to slicing C.
-    uint16_t* cs_out = nullptr;
-    int64_t cs_mp = 0, cs_kp = 0;
-    int* cs_e = nullptr;
-    const int64_t* ck_m = nullptr;
-    const int64_t* ck_n = nullptr;
-    int rows_per_crow = 0, cols_per_crow = 0;
-    int64_t ck_stride = 0;  // consumer column of producer column n + 1 minus that of n, inside a row group
+    // Split mode: A arrives sliced (split_slice_operand), for an A that several
+    // products share.
     const uint16_t* a_slices = nullptr;
     const int* a_e = nullptr;
     // C = A A^T (a Gram product): B is A read the other way (B(k, n) =
@@ -235,7 +224,7 @@ struct GemmDesc {
     const int* b_e = nullptr;
 };
 // Rows and columns of the padded slice arrays a split product of M rows and
-// K columns reads for its A operand (the fused hand-over writes this layout).
+// K columns reads for its A operand.
 int64_t split_rows_padded(const Ctx& ctx, int64_t M);
 int64_t split_k_padded(int64_t K);
 // Slice an A operand once for several split products (GemmDesc::a_slices / a_e).

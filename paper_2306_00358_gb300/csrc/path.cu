@@ -159,9 +159,13 @@ void environment(Ctx& ctx, const View4& t, double* M, int precision) {
 // The summed pair of each product is ordered with the producer's row index
 // fastest ((c,a) and (e,d)), so a producer warp, whose lanes are adjacent
 // rows, writes adjacent elements of its consumer's rows.  In split mode each
-// producer either records the exponent fields of its consumer's rows (the
-// consumer then skips the exponent pass over the D^5 intermediate) or, when
-// the bond dimensions tile (32, 64, 128), writes the consumer's slices.
+// producer records the exponent fields of its consumer's rows, so the consumer
+// skips the exponent pass over the D^5 intermediate.  (Handing the consumer
+// its slices instead of FP64 saves a pass over HBM, 0.65 ms a D^7 launch at
+// D = 64, but forming them takes the epilogue longer than one 512-deep chunk
+// of products, so the next tile's products wait: D^7 launches 13.0 against
+// 11.3 ms, contraction 62.2 against 58.2 ms; at D = 32 1.09 against 1.01 ms,
+// and likewise for 2, 3 and 5 slices.)
 void contract(Ctx& ctx, const View4& top, const View4& bottom, const double* U, int64_t Dn, const View4& out,
               int precision, int64_t j_begin, int64_t j_end, int64_t j_out0) {
     const View4& t = top;
@@ -176,28 +180,12 @@ void contract(Ctx& ctx, const View4& top, const View4& bottom, const double* U, 
     if (j_end < 0) j_end = Dy;
     if (j_begin < 0 || j_begin > j_end || j_end > Dy || j_out0 > j_begin)
         fail(TRG_EINVAL, "contract: bad j range");
-    // Fused hand-over (split mode): when a consumer row of the next product is
-    // Dx x Dx elements of one 128 x 128 output tile, the producer writes the
-    // next product's A slices directly (bit-identical to slicing its FP64
-    // output).  Done for X2 -> O: the D^7 product is tensor-bound, so the
-    // heavier epilogue hides behind its MMAs and the slicing pass over X2
-    // disappears.  X1 (K = Dx) is bound by its epilogue already; it keeps the
-    // FP64 hand-over, whose epilogue is half as long as the slicing one.
-    // fused_slices = 2 hands X1 over as slices too (same results, slower here).
-    auto tiles_ok = [](int64_t v) { return v == 32 || v == 64 || v == 128; };
-    const bool fuse = split && ctx.cfg.fused_slices >= 1 && tiles_ok(Dx);
-    const bool fuse1 = split && ctx.cfg.fused_slices == 2 && tiles_ok(Dx) && tiles_ok(Dy);
     const int S = ctx.cfg.split_slices;
     const size_t ws_cap = ctx.cfg.workspace_bytes ? ctx.cfg.workspace_bytes : ((size_t)4 << 30);
-    // bytes per j of each intermediate: FP64, or S BF16 slices (+ padding rows)
-    const size_t elem = (fuse || fuse1) ? (size_t)std::max(8, 2 * S) : 8;
-    const size_t per_j = (size_t)(2 * Dn * Dx * DD) * elem;
+    const size_t per_j = (size_t)(2 * Dn * Dx * DD) * 8;     // X1 and X2, FP64
     int64_t jb = std::max<int64_t>(1, std::min<int64_t>(std::max<int64_t>(1, j_end - j_begin), (int64_t)(ws_cap / per_j)));
     const int64_t rows2 = jb * Dn * Dx, rows3 = jb * Dn * Dy;   // A rows of the two consumers
-    size_t r1 = (size_t)(rows2 * DD) * 8, r2 = (size_t)(rows3 * Dx * Dx) * 8;
-    if (fuse1) r1 = std::max(r1, (size_t)S * split_rows_padded(ctx, rows2) * split_k_padded(DD) * 2);
-    if (fuse) r2 = std::max(r2, (size_t)S * split_rows_padded(ctx, rows3) * split_k_padded(Dx * Dx) * 2);
-    r1 = (r1 + 255) & ~(size_t)255;
+    const size_t r1 = ((size_t)(rows2 * DD) * 8 + 255) & ~(size_t)255, r2 = (size_t)(rows3 * Dx * Dx) * 8;
     ctx.ensure(ctx.ws, r1 + r2);
     double* X1 = ctx.ws.as<double>();
     double* X2 = (double*)(ctx.ws.as<uint8_t>() + r1);
@@ -263,28 +251,13 @@ void contract(Ctx& ctx, const View4& top, const View4& bottom, const double* U, 
             // consumer row of element ((i,a),(jj,d,c)) is (jj,i,d), its column c Dx + a
             g.cons_m = ctx.table({{Dn, Dx}, {Dx, 0}});
             g.cons_n = ctx.table({{jb, Dn * Dx}, {Dx, 1}, {Dy, 0}});
-            if (fuse1) {
-                g.C = nullptr;
-                g.cs_out = (uint16_t*)X1;
-                g.cs_mp = split_rows_padded(ctx, M2);
-                g.cs_kp = split_k_padded(DD);
-                g.cs_e = ef2;
-                g.ck_m = ctx.table({{Dn, 0}, {Dx, 1}});
-                g.ck_n = ctx.table({{jb, 0}, {Dx, 0}, {Dy, Dx}});
-                g.ck_stride = Dx;
-                g.rows_per_crow = (int)Dx;
-                g.cols_per_crow = (int)Dy;
-            } else {
-                g.C = X1;
-                g.c_m = ctx.table({{Dn, Dx * DD}, {Dx, 1}});
-                g.c_n = ctx.table({{jb, Dn * Dx * DD}, {Dx, DD}, {Dy, Dx}});
-                g.c_m_fast = true;
-                if (split) {
-                    TRG_CUDA(cudaMemsetAsync(ef2, 0, (size_t)rows2 * sizeof(int), ctx.stream));
-                    g.cons_ef = ef2;
-                } else {
-                    g.cons_m = g.cons_n = nullptr;
-                }
+            g.C = X1;
+            g.c_m = ctx.table({{Dn, Dx * DD}, {Dx, 1}});
+            g.c_n = ctx.table({{jb, Dn * Dx * DD}, {Dx, DD}, {Dy, Dx}});
+            g.c_m_fast = true;
+            if (split) {
+                TRG_CUDA(cudaMemsetAsync(ef2, 0, (size_t)rows2 * sizeof(int), ctx.stream));
+                g.cons_ef = ef2;
             }
             gemm(ctx, g, precision);
         }
@@ -301,34 +274,14 @@ void contract(Ctx& ctx, const View4& top, const View4& bottom, const double* U, 
             // consumer row of element ((jj,i,d),(l,e)) is (jj,i,l), its column e Dx + d
             g.cons_m = ctx.table({{jb * Dn, Dy}, {Dx, 0}});
             g.cons_n = ctx.table({{Dy, 1}, {Dx, 0}});
-            if (fuse1) {
-                g.a_slices = (const uint16_t*)X1;
-                g.a_e = ef2;
-            } else if (split) {
+            g.C = X2;
+            g.c_m = ctx.table({{jb * Dn, Dy * Dx * Dx}, {Dx, 1}});
+            g.c_n = ctx.table({{Dy, Dx * Dx}, {Dx, Dx}});
+            g.c_m_fast = true;
+            if (split) {
                 g.a_ef = ef2;
-            }
-            if (fuse) {
-                g.C = nullptr;
-                g.cs_out = (uint16_t*)X2;
-                g.cs_mp = split_rows_padded(ctx, M3);
-                g.cs_kp = split_k_padded(Dx * Dx);
-                g.cs_e = ef3;
-                g.ck_m = ctx.table({{jb * Dn, 0}, {Dx, 1}});
-                g.ck_n = ctx.table({{Dy, 0}, {Dx, Dx}});
-                g.ck_stride = Dx;
-                g.rows_per_crow = (int)Dx;
-                g.cols_per_crow = (int)Dx;
-            } else {
-                g.C = X2;
-                g.c_m = ctx.table({{jb * Dn, Dy * Dx * Dx}, {Dx, 1}});
-                g.c_n = ctx.table({{Dy, Dx * Dx}, {Dx, Dx}});
-                g.c_m_fast = true;
-                if (split) {
-                    TRG_CUDA(cudaMemsetAsync(ef3, 0, (size_t)rows3 * sizeof(int), ctx.stream));
-                    g.cons_ef = ef3;
-                } else {
-                    g.cons_m = g.cons_n = nullptr;
-                }
+                TRG_CUDA(cudaMemsetAsync(ef3, 0, (size_t)rows3 * sizeof(int), ctx.stream));
+                g.cons_ef = ef3;
             }
             gemm(ctx, g, precision);
         }
@@ -345,12 +298,7 @@ void contract(Ctx& ctx, const View4& top, const View4& bottom, const double* U, 
             g.C = out.p + (j0 - j_out0) * o[1];
             g.c_m = ctx.table({{jb, o[1]}, {Dn, o[0]}, {Dy, o[3]}});
             g.c_n = ctx.table({{Dn, o[2]}});
-            if (fuse) {
-                g.a_slices = (const uint16_t*)X2;
-                g.a_e = ef3;
-            } else if (split) {
-                g.a_ef = ef3;
-            }
+            if (split) g.a_ef = ef3;
             gemm(ctx, g, precision);
         }
     }

@@ -74,7 +74,7 @@ constexpr uint32_t TMEM_COLS = 512;
 constexpr int CPT = 32;                        // accumulator columns per epilogue thread
 constexpr int STAGING_BYTES = EPI_WARPS * 32 * 8 * 8;    // epilogue store staging, 32 KB
 constexpr int SMEM_LIMIT = 232448;             // opt-in shared memory per block
-constexpr int BAR_BYTES = 512;                 // mbarriers, TMEM address, flags, row maxima
+constexpr int BAR_BYTES = 512;                 // mbarriers, TMEM address, flags
 
 // CG = CTAs per MMA (1, or a pair with cta_group::2).  A CTA stages its own
 // 128 rows of A (all S slices) per stage, and B as follows.  One CTA: all S
@@ -110,7 +110,7 @@ __host__ __device__ constexpr int smem_bytes_for(int S, int CG, int MODE) {
 constexpr bool smem_fits() {
     for (int S = 2; S <= 5; ++S)
         for (int CG = 1; CG <= 2; ++CG)
-            for (int MODE = 0; MODE <= 3; ++MODE)
+            for (int MODE = 0; MODE <= 2; ++MODE)
                 if (smem_bytes_for(S, CG, MODE) > SMEM_LIMIT || stages_for(S, CG, MODE) < 2) return false;
     return true;
 }
@@ -169,66 +169,6 @@ __device__ __forceinline__ double scaled_i64(long long v, int e2, int& field) {
     return __longlong_as_double((long long)((f == 0 ? 0ull : b & (1ull << 63)) | body));
 }
 
-// |v| rounded to 53 significant bits (half to even), as the FP64 value of v
-// has it, and the position of its leading one afterwards.
-__device__ __forceinline__ unsigned long long round53(unsigned long long a, int& top) {
-    top = 63 - __clzll((long long)a);
-    if (top <= 52) return a;
-    const int sh = top - 52;
-    const unsigned long long half = 1ull << (sh - 1);
-    const unsigned long long rem = a & ((1ull << sh) - 1);
-    unsigned long long mant = a >> sh;
-    if (rem > half || (rem == half && (mant & 1))) {
-        ++mant;
-        if (mant >> 53) { mant >>= 1; ++top; }
-    }
-    return mant << (top - 52);
-}
-// Biased exponent field of the FP64 value v 2^e2 (0 when v = 0 or the value
-// flushes to zero, as in scaled_i64_to_double).
-__device__ __forceinline__ int fp64_exponent_field(long long v, int e2) {
-    if (v == 0) return 0;
-    int top;
-    round53(v < 0 ? (unsigned long long)(-v) : (unsigned long long)v, top);
-    const int ex = top + e2 + 1023;
-    return ex < 1 ? 0 : (ex > 2046 ? 2047 : ex);
-}
-// The fixed-point integer X = rint(x 2^(F - e_row)) (halves away from zero)
-// that slicing the FP64 value x = v 2^e2 produces, computed from v: with
-// V53 = |v| rounded to 53 bits and r = e_row - e2 - F, X = V53 / 2^r rounded
-// (r > 0) or V53 2^-r (r <= 0).
-// The same two for |v| < 2^53, where the FP64 value holds v exactly.
-__device__ __forceinline__ int fp64_exponent_field_exact(long long v, int e2) {
-    if (v == 0) return 0;
-    const int top = 63 - __clzll(v < 0 ? -v : v);
-    const int ex = top + e2 + 1023;
-    return ex < 1 ? 0 : (ex > 2046 ? 2047 : ex);
-}
-template <int S>
-__device__ __forceinline__ long long fused_fixed_point_exact(long long v, int e2, int e_row) {
-    constexpr int F = 7 + 8 * (S - 1);
-    if (v == 0) return 0;
-    const unsigned long long a = (unsigned long long)(v < 0 ? -v : v);
-    if (63 - __clzll((long long)a) + e2 + 1023 < 1) return 0;   // the FP64 value flushes to zero
-    const int r = e_row - e2 - F;
-    const long long X = r >= 63 ? 0 : r > 0 ? (long long)((a + (1ull << (r - 1))) >> r) : (long long)(a << (-r));
-    return v < 0 ? -X : X;
-}
-template <int S>
-__device__ __forceinline__ long long fused_fixed_point(long long v, int e2, int e_row) {
-    constexpr int F = 7 + 8 * (S - 1);
-    if (v == 0) return 0;
-    int top;
-    const unsigned long long a = round53(v < 0 ? (unsigned long long)(-v) : (unsigned long long)v, top);
-    if (top + e2 + 1023 < 1) return 0;           // the FP64 value flushes to zero
-    const int r = e_row - e2 - F;
-    long long X;
-    if (r >= 63) X = 0;
-    else if (r > 0) X = (long long)((a + (1ull << (r - 1))) >> r);
-    else X = (long long)(a << (-r));
-    return v < 0 ? -X : X;
-}
-
 struct MmaArgs {
     int M, N, Kp;                  // logical rows / cols, padded K (multiple of BK)
     int Mp, Np;                    // padded rows of the A / B slice arrays
@@ -243,16 +183,6 @@ struct MmaArgs {
     const int64_t* cons_m;
     const int64_t* cons_n;
     int group_n;               // tile order: column blocks per group (see tile_coords)
-    // optional fused hand-over: the consumer's A slices instead of C
-    uint16_t* cs_out;
-    int64_t cs_plane;          // Mp * Kp of the consumer's slice arrays
-    int64_t cs_kp;
-    int* cs_e;
-    const int64_t* ck_m;
-    const int64_t* ck_n;
-    int rows_per_crow, cols_per_crow;
-    int64_t ck_stride;         // fused: consumer-column step between adjacent producer columns
-    int v_exact53;             // fused: every V is below 2^53 in magnitude (K <= 8192)
     int c_rows_fast;           // C's rows are adjacent: store without staging
     // limit of the epilogue's wait for a finished accumulator chunk (the
     // other waits keep WAIT_NS); a short one lets tests reach the timeout path
@@ -372,10 +302,12 @@ __host__ __device__ constexpr bool pair_table_ok(int S) {
 static_assert(pair_table_ok(2) && pair_table_ok(3) && pair_table_ok(4) && pair_table_ok(5), "pair staging");
 
 // Epilogue kinds: FP64 results stored through a staging tile (columns
-// adjacent in C), stored directly (rows adjacent in C), or the consumer's
-// slices (fused hand-over).  One kernel instance each keeps the register
-// allocation of each epilogue to itself.
-enum EpiMode { EPI_STAGED = 0, EPI_DIRECT = 1, EPI_FUSED = 2, EPI_KSPLIT = 3 };
+// adjacent in C), stored directly (rows adjacent in C), or split-K parts.  One
+// kernel instance each keeps the register allocation of each epilogue to
+// itself.  Forming a tile's results has to take less time than one 512-deep
+// chunk of products (20k clocks a 256-row pair at S = 4): the next tile's
+// first chunk waits in the accumulators until they are formed.
+enum EpiMode { EPI_STAGED = 0, EPI_DIRECT = 1, EPI_KSPLIT = 2 };
 
 template <int S, int CG, int MODE>
 __global__ void __launch_bounds__(THREADS, 1)
@@ -393,10 +325,8 @@ k_split_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     uint64_t* acc_full = empty + STAGES;
     uint64_t* acc_empty = acc_full + 1;
     uint64_t* mma_done = acc_empty + 1;
-    uint64_t* cs_bar = mma_done + 1;             // epilogue warps: consumer-row maxima are complete
-    uint32_t* tmem_slot = (uint32_t*)(cs_bar + 1);
+    uint32_t* tmem_slot = (uint32_t*)(mma_done + 1);
     volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
-    unsigned* cs_slot = (unsigned*)(tmem_slot + 4);   // 2 x 16 consumer-row maxima, tagged by tile
     double* staging = (double*)(smem + STAGES * STAGE_BYTES + BAR_BYTES);   // EPI_WARPS x 32 x 8 doubles
 
     const int warp = threadIdx.x >> 5;
@@ -416,9 +346,7 @@ k_split_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         mbar_init(acc_full, 1);
         mbar_init(acc_empty, EPI_WARPS * CG);
         mbar_init(mma_done, 1);
-        mbar_init(cs_bar, EPI_WARPS);
         *abort_flag = 0;
-        for (int i = 0; i < 32; ++i) cs_slot[i] = 0u;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
@@ -592,7 +520,6 @@ k_split_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         const uint32_t lane_base = (uint32_t)(quad * 32) << 16;
         const int row_in_tile = quad * 32 + lane;
         uint32_t chunk_no = 0;
-        uint32_t tile_iter = 0;                   // tiles done by this CTA (tags the row maxima)
         bool ok = true;
         for (int unit = first_tile; unit < num_units && ok; unit += tile_step) {
             const int tile = unit / g.ksplit;
@@ -601,7 +528,6 @@ k_split_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             const int nchunks = (min(num_kb, kb0 + g.kb_per) - kb0 + CHUNK_STAGES - 1) / CHUNK_STAGES;
             int mb, nb;
             unit_tile(g, tile, tiles_m, tiles_n, mb, nb);
-            ++tile_iter;
             const int row0 = mb * TILE_M + (int)rank * BM;   // this CTA's rows of the tile
             // J = I0 2^8 + I1: the exact ACC0 and ACC1 sums of this tile's
             // columns in one int64 each; at the end J becomes
@@ -742,93 +668,6 @@ k_split_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                             J[j] = __double_as_longlong(v);
                         }
                     }
-                    if constexpr (MODE == EPI_FUSED) {
-                        // fused hand-over: the consumer's rows lie in this tile; a
-                        // warp's lanes and a thread's columns share one of them.  The
-                        // slices follow from V directly, equal to slicing the FP64
-                        // value V 2^(ea + eb - 36) (see fused_fixed_point).
-                        // |V| < 2^53 (K <= 8192) needs no rounding to 53 bits
-                        const bool exact53 = g.v_exact53 != 0;
-                        unsigned tmax = 0;
-#pragma unroll
-                        for (int j = 0; j < CPT; ++j)
-                            if (row_ok && nt + j < g.N)
-                                tmax = max(tmax, (unsigned)(exact53 ? fp64_exponent_field_exact(J[j], ea + g.eb[nt + j] - 36)
-                                                                    : fp64_exponent_field(J[j], ea + g.eb[nt + j] - 36)));
-                        const unsigned wmax = __reduce_max_sync(0xffffffffu, tmax);
-                        // double-buffered by tile parity: a warp may run one tile ahead
-                        const int slot = (int)(tile_iter & 1) * 16 + (row_in_tile / g.rows_per_crow) * (BN / g.cols_per_crow) +
-                                         (colh * CPT) / g.cols_per_crow;
-                        int w_ok = 1;
-                        if (lane == 0) {
-                            atomicMax(&cs_slot[slot], (tile_iter << 11) | wmax);
-                            mbar_arrive(cs_bar);    // release: the maximum above is visible after the wait
-                            w_ok = mbar_wait(cs_bar, (tile_iter - 1) & 1, abort_flag, g.status) ? 1 : 0;
-                        }
-                        ok = __shfl_sync(0xffffffffu, w_ok, 0) != 0;
-                        if (!ok) break;
-                        const unsigned sv = cs_slot[slot];
-                        const int ef = ((sv >> 11) == (tile_iter & 0x1FFFFFu)) ? (int)(sv & 0x7FFu) : 0;
-                        const int e_row = ef ? ef - 1022 : -1022;           // |x| < 2^e_row over the row
-                        if (row_ok && nt < g.N) {
-                            const int64_t crow = g.cons_m[m] + g.cons_n[nt];
-                            if (lane == 0) g.cs_e[crow] = e_row;
-                            // consumer column of this thread's column j: ck_m[m] + ck_n[nt] +
-                            // j ck_stride, with ck_m[m] = the lane's row offset (adjacent
-                            // lanes, adjacent columns): each store writes 64 contiguous bytes
-                            uint16_t* dst = g.cs_out + crow * g.cs_kp + g.ck_m[m] + g.ck_n[nt];
-                            const int64_t step = g.ck_stride, plane = g.cs_plane;
-#pragma unroll
-                            for (int j = 0; j < CPT; ++j) {
-                                const int e2 = ea + g.eb[nt + j] - 36;
-                                long long X = exact53 ? fused_fixed_point_exact<S>(J[j], e2, e_row)
-                                                      : fused_fixed_point<S>(J[j], e2, e_row);
-                                int d[S];
-                                // signed base-256 digits; |X| <= 2^F, so after S - 3 digits
-                                // (S >= 4) the rest fits in 32 bits
-#pragma unroll
-                                for (int p = S - 1; p >= 1; --p) {
-                                    const int lo8 = (int)(((unsigned)X + 128u) & 255u) - 128;   // low bits only
-                                    d[p] = lo8;
-                                    if (p > 2) X = (X - lo8) >> 8;
-                                    else X = ((int)X - lo8) >> 8;
-                                }
-                                d[0] = (int)X;
-#pragma unroll
-                                for (int p = 0; p < S; ++p) {
-                                    // small integer -> FP32 exactly, times 2^-8p; the top half is the BF16
-                                    float f = __int_as_float(0x4B400000 + d[p]) - 12582912.0f;
-                                    if (p > 0) f *= __int_as_float((127 - 8 * p) << 23);
-                                    dst[p * plane] = (uint16_t)(__float_as_uint(f) >> 16);
-                                }
-                                dst += step;
-                            }
-                        }
-                    }
-                    if (MODE == EPI_STAGED && g.cons_ef && row_ok) {
-                        // exponent fields of the consumer's rows: run-length maxima
-                        // over this thread's columns, one atomic per run
-                        const int64_t cm0 = g.cons_m[m];
-                        int64_t cur = -1;
-                        int cur_max = 0;
-#pragma unroll
-                        for (int j = 0; j < CPT; ++j) {
-                            const int n = nt + j;
-                            if (n < g.N) {
-                                const int64_t crow = cm0 + g.cons_n[n];
-                                const int ef = (int)(((unsigned long long)J[j] >> 52) & 0x7FF);
-                                if (crow != cur) {
-                                    if (cur >= 0 && cur_max) atomicMax(&g.cons_ef[cur], cur_max);
-                                    cur = crow;
-                                    cur_max = ef;
-                                } else {
-                                    cur_max = max(cur_max, ef);
-                                }
-                            }
-                        }
-                        if (cur >= 0 && cur_max) atomicMax(&g.cons_ef[cur], cur_max);
-                    }
-                    if (MODE == EPI_FUSED) continue;
                     if (MODE == EPI_STAGED && g.sym && row_ok) {
                         // symmetric C: the mirror (n, m) of each element above the
                         // diagonal (adjacent lanes, adjacent rows m: contiguous in
@@ -1048,8 +887,7 @@ void launch_mma_k(Ctx& ctx, const CUtensorMap& ta, const CUtensorMap& tb, const 
 
 template <int S, int CG>
 void launch_mma(Ctx& ctx, const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& tbh, const MmaArgs& a) {
-    if (a.cs_out) launch_mma_k<S, CG, EPI_FUSED>(ctx, ta, tb, tbh, a);
-    else if (a.c_rows_fast) launch_mma_k<S, CG, EPI_DIRECT>(ctx, ta, tb, tbh, a);
+    if (a.c_rows_fast) launch_mma_k<S, CG, EPI_DIRECT>(ctx, ta, tb, tbh, a);
     else if (a.ksplit > 1) launch_mma_k<S, CG, EPI_KSPLIT>(ctx, ta, tb, tbh, a);
     else launch_mma_k<S, CG, EPI_STAGED>(ctx, ta, tb, tbh, a);
 }
@@ -1194,7 +1032,7 @@ void gemm_split(Ctx& ctx, const GemmDesc& d) {
     const int CG = (ctx.cfg.mma_pairs && M > BM) ? 2 : 1;
     const int Mp = (int)split_rows_padded(ctx, M), Np = (N + BN - 1) / BN * BN, Kp = (int)split_k_padded(K);
     const bool pre_a = d.a_slices != nullptr;    // A arrives sliced from its producer
-    if (d.gram && (M != N || d.b_slices || pre_a || d.cs_out || d.cons_ef || d.c_m_fast))
+    if (d.gram && (M != N || d.b_slices || pre_a || d.cons_ef || d.c_m_fast))
         fail(TRG_EINVAL, "split GEMM: a Gram product takes a square C and plain operands");
     // a Gram product reads A's slices for B too (same rows, same padding)
     const bool gram_b = d.gram && Mp == Np;
@@ -1226,17 +1064,13 @@ void gemm_split(Ctx& ctx, const GemmDesc& d) {
     a.status = ctx.status.as<int>();
     a.acc_wait_ns = ctx.acc_wait_ns ? ctx.acc_wait_ns : WAIT_NS;
     a.cons_ef = d.cons_ef; a.cons_m = d.cons_m; a.cons_n = d.cons_n;
-    a.cs_out = d.cs_out; a.cs_plane = d.cs_mp * d.cs_kp; a.cs_kp = d.cs_kp; a.cs_e = d.cs_e;
-    a.ck_m = d.ck_m; a.ck_n = d.ck_n; a.rows_per_crow = d.rows_per_crow; a.cols_per_crow = d.cols_per_crow;
-    a.ck_stride = d.ck_stride; a.c_rows_fast = d.c_m_fast ? 1 : 0;
-    // |V| <= (K / 512) (2^32 + 2^24) 2^14 + 2 K 2^20 < 2^53 for K <= 8192
-    a.v_exact53 = Kp <= 8192 ? 1 : 0;
+    a.c_rows_fast = d.c_m_fast ? 1 : 0;
     // split K where the tiles leave most SMs idle: a function of the shape
     // and the SM count only (not of the CTA grouping), so every launch
     // choice still gives the same bits
     a.ksplit = 1; a.kb_per = Kp / BK; a.kpart = nullptr;
     a.tile_list = nullptr; a.n_list = 0; a.sym = d.gram ? 1 : 0;
-    if (d.allow_ksplit && !d.cs_out && !d.cons_ef && !d.gram) {
+    if (d.allow_ksplit && !d.cons_ef && !d.gram) {
         const int chunks = (Kp / BK + CHUNK_STAGES - 1) / CHUNK_STAGES;
         const int tiles128 = ((M + BM - 1) / BM) * ((N + BN - 1) / BN);
         if (2 * tiles128 <= ctx.sm_count && chunks >= 2) {
@@ -1252,16 +1086,6 @@ void gemm_split(Ctx& ctx, const GemmDesc& d) {
                 a.kb_per = Kp / BK;
             }
         }
-    }
-    if (d.cs_out) {
-        // a consumer row = rows_per_crow consecutive rows (32, 64 or 128, so a
-        // warp's lanes and the CTA's 128-row tile hold whole groups) times
-        // cols_per_crow consecutive columns (so a thread's 32 hold one group)
-        auto pow2_32_128 = [](int v) { return v == 32 || v == 64 || v == 128; };
-        const bool shape_ok = pow2_32_128(d.rows_per_crow) && pow2_32_128(d.cols_per_crow) &&
-                              M % d.rows_per_crow == 0 && N % d.cols_per_crow == 0 && d.cs_kp % 8 == 0 &&
-                              d.cons_m && d.cons_n && d.ck_m && d.ck_n && d.cs_e;
-        if (!shape_ok) fail(TRG_EINVAL, "fused slice hand-over: consumer rows do not tile");
     }
     auto launch = [&](int cg, int group_n) {
         MmaArgs b = a;
@@ -1303,7 +1127,8 @@ void gemm_split(Ctx& ctx, const GemmDesc& d) {
             case 11: launch_mma<5, 2>(ctx, ta, tb, tbh, b); break;
         }
     };
-    const int mode = d.cs_out ? 2 : (a.c_rows_fast ? 1 : (a.ksplit > 1 ? 3 : (d.gram ? 4 : 0)));
+    const int mode = a.c_rows_fast ? 1 : (a.ksplit > 1 ? 3 : (d.gram ? 4 : 0));
+    if (d.cons_ef && !a.c_rows_fast) fail(TRG_EINVAL, "split GEMM: exponent fields are recorded by the row-wise epilogue");
     const TuneChoice ch = tuned_choice(ctx, M, N, Kp, S, mode, CG, launch);
     const int tok = ctx.region_begin(TRG_PHASE_MMA);
     const int tok_x2 = ctx.phase == TRG_PHASE_X2 ? ctx.region_begin(TRG_PHASE_MMA_X2) : -1;
@@ -1452,9 +1277,7 @@ extern "C" int trg_gemm_noalloc(int M, int N, int K, const double* A, int lda, c
         a.M = M; a.N = N; a.Kp = Kp; a.Mp = Mp; a.Np = Np; a.S = S;
         a.ea = ea; a.eb = eb; a.C = C; a.c_m = cm; a.c_n = cn; a.status = status;
         a.cons_ef = nullptr; a.cons_m = nullptr; a.cons_n = nullptr;
-        a.cs_out = nullptr; a.cs_plane = 0; a.cs_kp = 0; a.cs_e = nullptr; a.ck_m = nullptr; a.ck_n = nullptr;
-        a.rows_per_crow = a.cols_per_crow = 0;
-        a.ck_stride = 0; a.c_rows_fast = 0; a.v_exact53 = 0;
+        a.c_rows_fast = 0;
         a.acc_wait_ns = WAIT_NS;
         a.ksplit = 1; a.kb_per = Kp / BK; a.kpart = nullptr;
         a.tile_list = nullptr; a.n_list = 0; a.sym = 0;
