@@ -7,39 +7,44 @@
 //     X = rint(x 2^(119 - e)) = sum_p d_p 2^(8 (14 - p)),   p = 0..14,
 // d_0 in [-128, 128], d_p in [-128, 127] (an error-free splitting as in
 // split_gemm.cu, with every sum exact: Ozaki, Ogita, Oishi, Rump, Numer.
-// Algorithms 59 (2012) 95).  With D_d = sum_{p + q = d} A_p B_q,
-//     C = 2^(ea + eb - 126) sum_{d < 15} D_d 2^(8 (14 - d)):
-// digit products are integers up to 2^14, a run of 64 K sums the at most 15
-// products of a D_d exactly in FP32 (15 x 64 x 2^14 < 2^24), the epilogue
-// moves each run into int64 sums and the wide total is turned into FP64.
+// Algorithms 59 (2012) 95).  With D_d = sum_{p + q = d} A_p B_q and S digits,
+//     C = 2^(ea + eb - 14) sum_{d < S} D_d 2^(-8 d):
+// digit products are integers up to 2^14, a short run of K (64 for 15 digits,
+// 128 for 8) sums the at most S products of a D_d exactly in FP32, the
+// epilogue moves each run into int64 sums and the wide total is turned into
+// FP64.
 //
-// Why 15 digits: what is left out is below 16 K 2^-120 2^(ea + eb), so every
-// element of C is as accurate as an FP64 sum, relative to its own sum |a||b|,
-// down to sums 2^-60 of the largest possible one.  Eight digits are enough for
-// an error far below FP64's relative to the largest elements, and cost a
-// third, but the method needs the small elements too: the couplings between
-// nearly decoupled sectors of a tensor decide how near-degenerate vectors mix.
-// (Critical Ising with a field, Dcut 16, 20 half-steps: <s> varies with the
-// start vectors by 8e-10 with the FP64 pipe, by 9e-8 with eight digits.)
+// How many digits: S leave out less than (S + 2) K 2^(-8 S) 2^(ea + eb).  The
+// result has to be as accurate as an FP64 sum element by element, relative to
+// its own sum |a||b| (the method feeds the couplings between nearly decoupled
+// sectors of a tensor back, so small elements count):
+//  - 15 digits do that down to sums |a||b| of 2^-60 2^(ea + eb) (120 digit
+//    products); products too small for a choice always take them;
+//  - 9 digits (45 digit products) do if no sum |a||b| lies between 0 and 2^-8
+//    2^(ea + eb): they leave out less than K 2^-60 |a||b| then, which is also
+//    below what the roundings of an FP64 sum amount to when their signs are
+//    random.  A kernel takes |A||B| from one BF16 plane of each operand and
+//    raises a flag where 9 do not suffice; the two product kernels read it,
+//    and the one that is not wanted returns at once.
+// Rows or columns whose largest entry lies outside 2^-400 .. 2^400, or that hold
+// an infinity or a NaN, raise another flag: then the FP64 pipe kernel that is
+// queued last, idle otherwise, computes the product.
 //
-// Rows or columns whose largest entry lies outside 2^-400 .. 2^400, or that
-// hold an infinity or a NaN, raise a device flag: the tensor kernel then
-// returns at once and the FP64 pipe kernel that is queued behind it, idle
-// otherwise, computes the product.
-//
-// What bounds it: the tensor pipe, 120 digit products of 2 M N K each.
-// 128 x 32 output tile, one persistent CTA per SM: the 15 D_d of 32 columns
-// take 480 TMEM columns.  A stage is 16 K of both operands (60 KB of A digits,
-// 15 KB of B digits, one TMA box each), two stages.  The products of one A
-// digit with adjacent B digits land in adjacent accumulators, so 22
-// instructions of up to N = 256 cover the 120 products of a step.  They are
-// issued in two groups, the one that lands in D_7..D_14 (92 products) before
-// the one that lands in D_0..D_6: a run's drain of D_7..D_14 runs under the
-// other group's products, and the drain of D_0..D_6 under the next run's first
-// group.  Measured, contraction at Dx = Dy = Dn = 48 (three products, 1.22e12
-// FP64 FLOPs): 993 ms on the
-// FP64 pipe, 113 here, 110 of them in this kernel (1.5e14 digit FLOPs, 1340
-// TFLOP/s); environment at (24, 22): 0.65 -> 0.28 ms.
+// What bounds it: the tensor pipe (9 digits in a long product: active 70 % of
+// the time, MMA instructions of N = 48 .. 240; 10 % go to drains that nothing
+// covers).  128 x 32 output tile with 15 digits, 128 x 48 with 9, one persistent
+// CTA per SM: the S accumulators D_d of the tile's columns fill tensor memory.
+// A stage is 16 (32) K of both operands, one TMA box each, two stages.  The
+// products of one A digit with adjacent B digits land in adjacent accumulators,
+// so 23 (13) instructions of up to N = 256 cover the products of a 16-deep
+// step.  They are issued in two groups, the one that lands in the higher D_d
+// (84 of 120, 35 of 45 products) before the other: a run's drain of the higher
+// D_d runs under the other group's products, and the drain of the lower ones
+// under the next run's first group.
+// Measured, contraction at Dx = Dy = Dn = 48 (1.22e12 FP64 FLOPs): 993 ms on
+// the FP64 pipe, 113.6 ms with 15 digits always, 45.3 ms with 9 where they
+// suffice (39.5 ms of it in this kernel, 1.6 ms in the |A||B| sums); with
+// operands that need 15, the sums are the only loss.
 #include <algorithm>
 #include <cmath>
 
@@ -51,53 +56,67 @@ namespace trg {
 
 namespace {
 
-constexpr int XS = 15;                           // digits
-constexpr int XM = 128, XN = 32, XK = 16;        // tile rows, columns, K per stage
-constexpr int XL = 7;                            // D_0 .. D_(XL-1) are group 0, the rest group 1
-constexpr int XA_TILE = XM * XK * 2;             // bytes of one digit's A tile
-constexpr int XB_TILE = XN * XK * 2;
-constexpr int XSTAGE = XS * (XA_TILE + XB_TILE); // 75 KB
-constexpr int XSTAGES = 2;
-constexpr int XRUN = 64 / XK;                    // stages of an exact run
-constexpr int XEPI = 16;                         // epilogue warps
-constexpr int XTHREADS = 64 + 32 * XEPI;
-constexpr int XCPT = XN / 4;                     // columns per epilogue thread
-constexpr int XSTAGING = XEPI * 32 * 8 * 8;      // store staging, 32 KB
+constexpr int XM = 128;                          // tile rows
+constexpr int XKP = 32;                          // K is padded to this
+constexpr int XPLANES = planes(15);
 constexpr int XBAR = 256;
-constexpr int XSMEM = XSTAGES * XSTAGE + XSTAGING + XBAR + 1024;
-static_assert(XSMEM <= 232448, "exact product shared memory");
 
-// The digit products of one 16-deep step: A digit a times the n <= 8 B digits
-// from b on, into the accumulators D_(a+b) .. D_(a+b+n-1).  Group 1 lands in
-// D_7..D_14, group 0 in D_0..D_6; the first entry of a group covers all of its
-// accumulators and resets them at the start of a run.
+// Shape of the kernel for S digits; S = 1 is the sum of |a||b|.
+template <int S>
+struct XT {
+    static constexpr int N = S == 15 ? 32 : S == 9 ? 48 : 256;     // tile columns
+    static constexpr int K = S == 15 ? 16 : 32;                    // K per stage
+    static constexpr int L = S == 15 ? 8 : S == 9 ? 4 : 0;         // D_0 .. D_(L-1) are group 0, the rest group 1
+    static constexpr int EPI = S == 9 ? 12 : 16;                   // epilogue warps: 16 columns each with 9 digits
+    static constexpr int THREADS = 64 + 32 * EPI;
+    static constexpr int A_TILE = XM * K * 2, B_TILE = N * K * 2;  // bytes of one digit's tiles
+    static constexpr int STAGE = S * (A_TILE + B_TILE);            // 75, 50 and 24 KB
+    static constexpr int STAGES = S == 1 ? 4 : 2;
+    static constexpr int RUN = S == 1 ? 1 << 30 : S == 9 ? 3 : 4;  // stages of an exact run
+    static constexpr int CPT = N / (EPI / 4);                      // columns per epilogue thread
+    static constexpr int LIMBS = S == 15 ? 4 : 2;
+    static constexpr int STAGING = S == 1 ? 0 : EPI * 32 * 8 * 8;  // store staging
+    // at least 120 KB, so that a second CTA (and its tensor memory) never shares the SM
+    static constexpr int BYTES = STAGES * STAGE + STAGING + XBAR + 1024;
+    static constexpr int SMEM = BYTES > 120 * 1024 ? BYTES : 120 * 1024;
+    static_assert(SMEM <= 232448, "exact product shared memory");
+    static_assert(S * N <= 512 && (S == 1 || (double)S * RUN * K * (1 << 14) <= (1 << 24)), "accumulators");
+};
+
+// The digit products of one 16-deep step: A digit a times the n B digits from
+// b on, into the accumulators D_(a+b) .. D_(a+b+n-1).  The first entry of a
+// group covers all of its accumulators and resets them at the start of a run.
 struct XIns { int a, b, n, group; };
-__host__ __device__ constexpr int xins_count() { return XS + XL; }
+template <int S>
+__host__ __device__ constexpr int xins_count() { return S + XT<S>::L; }
+template <int S>
 __host__ __device__ constexpr XIns xins(int t) {
-    return t < XS ? XIns{t, t < XL ? XL - t : 0, t < XL ? XS - XL : XS - t, 1} : XIns{t - XS, 0, XL - (t - XS), 0};
+    constexpr int L = XT<S>::L;
+    return t < S ? XIns{t, t < L ? L - t : 0, t < L ? S - L : S - t, 1} : XIns{t - S, 0, L - (t - S), 0};
 }
+template <int S>
 __host__ __device__ constexpr bool xins_ok() {
-    int seen[XS][XS] = {};
-    for (int t = 0; t < xins_count(); ++t) {
-        const XIns in = xins(t);
-        if (in.n < 1 || in.n * XN > 256) return false;
+    constexpr int L = XT<S>::L;
+    int seen[S][S] = {};
+    for (int t = 0; t < xins_count<S>(); ++t) {
+        const XIns in = xins<S>(t);
+        if (in.n < 1 || in.n * XT<S>::N > 256) return false;
         for (int q = in.b; q < in.b + in.n; ++q) {
             const int d = in.a + q;
-            if (d >= XS || (d >= XL) != (in.group == 1)) return false;
+            if (d >= S || (d >= L) != (in.group == 1)) return false;
             seen[in.a][q] += 1;
         }
     }
-    for (int p = 0; p < XS; ++p)
-        for (int q = 0; q < XS; ++q)
-            if (seen[p][q] != (p + q < XS ? 1 : 0)) return false;
-    return xins(0).n == XS - XL && xins(XS).n == XL;
+    for (int p = 0; p < S; ++p)
+        for (int q = 0; q < S; ++q)
+            if (seen[p][q] != (p + q < S ? 1 : 0)) return false;
+    return xins<S>(0).n == S - L && (L == 0 || xins<S>(S).n == L);
 }
-static_assert(xins_ok(), "digit product table");
-static_assert(XS * XN <= 512 && (double)XS * 64 * (1 << 14) <= (1 << 24), "accumulators");
+static_assert(xins_ok<15>() && xins_ok<9>() && xins_ok<1>(), "digit product table");
 
 // Shared-memory matrix descriptor: K-major BF16 tile, 32-byte rows, 32-byte
 // swizzle; 8-row groups 256 bytes apart.
-__device__ __forceinline__ uint64_t xsmem_desc(uint32_t addr) {
+__device__ __forceinline__ uint64_t smem_desc32(uint32_t addr) {
     uint64_t d = 0;
     d |= (uint64_t)((addr >> 4) & 0x3FFF);          // start address
     d |= (uint64_t)1 << 16;                         // leading byte offset (unused for swizzled K-major)
@@ -119,13 +138,15 @@ struct XArgs {
     const long long* tile_list;    // mb << 32 | nb, or nullptr for all
     int n_list;
     int group_n;                   // tile order: column blocks per group
-    const int* bad;                // the operands are outside the digits' range: do nothing
+    int* flags;                    // [0] an operand is outside the digits' range, [1] nine digits do not suffice
+    int nine;                      // the nine-digit form has been tried
     int* status;
 };
 
-// The int64 sums of an element: D_0..D_3, D_4..D_7, D_8..D_11, D_12..D_14, each
-// in units of its last D: V = w0 2^88 + w1 2^56 + w2 2^24 + w3.
-// V 2^e2 in FP64, within 2 units in the last place.
+// The int64 sums of an element, each in units of its last D, as FP64 times
+// 2^e2, within 2 units in the last place.  15 digits: D_0..D_3, D_4..D_7,
+// D_8..D_11, D_12..D_14, V = w0 2^88 + w1 2^56 + w2 2^24 + w3; 9 digits:
+// D_0..D_3, D_4..D_8, V = w0 2^40 + w1.
 __device__ __forceinline__ double wide_to_double(const long long (&w)[4], int e2) {
     long long w2 = w[2] + (w[3] >> 24);
     long long w1 = w[1] + (w2 >> 32);
@@ -134,16 +155,38 @@ __device__ __forceinline__ double wide_to_double(const long long (&w)[4], int e2
     r = fma(r, 4294967296.0, (double)(unsigned)(w2 & 0xffffffffll));
     r = fma(r, 16777216.0, (double)(int)(w[3] & 0xffffffll));
     if (r == 0.0) return 0.0;
-    // (nonzero rows and columns have -928 <= e2 <= 676 and |r| < 2^150: the field stays in range)
+    // (nonzero rows and columns have -928 <= e2 <= 732 and |r| < 2^150: the field stays in range)
+    return __longlong_as_double(__double_as_longlong(r) + ((long long)e2 << 52));
+}
+__device__ __forceinline__ double wide_to_double(const long long (&w)[2], int e2) {
+    const long long w0 = w[0] + (w[1] >> 40);
+    const double r = fma((double)w0, 1099511627776.0, (double)(w[1] & 0xffffffffffll));
+    if (r == 0.0) return 0.0;
     return __longlong_as_double(__double_as_longlong(r) + ((long long)e2 << 52));
 }
 
-__global__ void __launch_bounds__(XTHREADS, 1)
+__device__ __forceinline__ void tmem_ldn(uint32_t taddr, uint32_t (&r)[8]) { tmem_ld8(taddr, r); }
+__device__ __forceinline__ void tmem_ldn(uint32_t taddr, uint32_t (&r)[16]) { tmem_ld16(taddr, r); }
+// Keeps the use of loaded registers behind the wait for them.
+template <int N>
+__device__ __forceinline__ void tmem_arrived(uint32_t (&r)[N]) {
+#pragma unroll
+    for (int j = 0; j < N; ++j) asm volatile("" : "+r"(r[j]));
+}
+
+constexpr int XNINE_K = 16384;                    // the nine-digit sums fit in int64 up to this K
+static_assert(5.0 * XNINE_K * (1 << 14) * 4294967296.0 * 1.01 < 9.2e18, "nine-digit sums");
+constexpr float SUM_MIN = 0.00390625f;           // 2^-8
+
+template <int S>
+__global__ void __launch_bounds__(XT<S>::THREADS, 1)
 k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const XArgs g) {
-    if (*g.bad) return;
+    constexpr int XN = XT<S>::N, XK = XT<S>::K, XL = XT<S>::L, XSTAGES = XT<S>::STAGES, XSTAGE = XT<S>::STAGE;
+    constexpr int XA_TILE = XT<S>::A_TILE, XB_TILE = XT<S>::B_TILE, XRUN = XT<S>::RUN, XCPT = XT<S>::CPT;
+    if (g.flags[0] || (S == 9 && g.flags[1]) || (S == 15 && g.nine && !g.flags[1])) return;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    uint64_t* full = (uint64_t*)(smem + XSTAGES * XSTAGE + XSTAGING);
+    uint64_t* full = (uint64_t*)(smem + XSTAGES * XSTAGE + XT<S>::STAGING);
     uint64_t* empty = full + XSTAGES;
     uint64_t* acc_full = empty + XSTAGES;        // [group]
     uint64_t* acc_empty = acc_full + 2;          // [group]
@@ -172,7 +215,7 @@ k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < XSTAGES; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
-        for (int q = 0; q < 2; ++q) { mbar_init(&acc_full[q], 1); mbar_init(&acc_empty[q], XEPI); }
+        for (int q = 0; q < 2; ++q) { mbar_init(&acc_full[q], 1); mbar_init(&acc_empty[q], XT<S>::EPI); }
         mbar_init(mma_done, 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -205,7 +248,7 @@ k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                     uint8_t* st = smem + stage * XSTAGE;
                     mbar_expect_tx(&full[stage], XSTAGE);
                     tma_load_3d(st, &tmA, kb * XK, mb * XM, 0, &full[stage]);
-                    tma_load_3d(st + XS * XA_TILE, &tmB, kb * XK, nb * XN, 0, &full[stage]);
+                    tma_load_3d(st + S * XA_TILE, &tmB, kb * XK, nb * XN, 0, &full[stage]);
 #pragma unroll
                     for (int s = 0; s < XSTAGES; ++s)
                         if (s == stage) issued[s] = (int)phase;
@@ -231,16 +274,21 @@ k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                     ok = mbar_wait(&full[stage], phase, abort_flag, g.status);
                     if (!ok) break;
                     tc_fence_after();
-                    const uint64_t dbase = xsmem_desc(smem_u32(smem + stage * XSTAGE));
+                    const uint32_t sbase = smem_u32(smem + stage * XSTAGE);
+                    const uint64_t dbase = XK == 16 ? smem_desc32(sbase) : smem_desc(sbase);
                     auto issue = [&](int group) {
 #pragma unroll
-                        for (int t = 0; t < xins_count(); ++t) {
-                            const XIns in = xins(t);
-                            if (in.group != group) continue;
-                            const uint32_t acc = ((t == 0 || t == XS) && run_start) ? 0u : 1u;
-                            const uint64_t da = dbase + (uint64_t)((in.a * XA_TILE) >> 4);
-                            const uint64_t db = dbase + (uint64_t)((XS * XA_TILE + in.b * XB_TILE) >> 4);
-                            mma_bf16<1>(tmem + (uint32_t)((in.a + in.b) * XN), da, db, idesc_bf16(XM, in.n * XN), acc);
+                        for (int kk = 0; kk < XK / 16; ++kk) {
+#pragma unroll
+                            for (int t = 0; t < xins_count<S>(); ++t) {
+                                const XIns in = xins<S>(t);
+                                if (in.group != group) continue;
+                                const uint32_t acc = ((t == 0 || t == S) && run_start && kk == 0) ? 0u : 1u;
+                                const uint64_t da = dbase + (uint64_t)((in.a * XA_TILE + kk * 32) >> 4);
+                                const uint64_t db = dbase + (uint64_t)((S * XA_TILE + in.b * XB_TILE + kk * 32) >> 4);
+                                mma_bf16<1>(tmem + (uint32_t)((in.a + in.b) * XN), da, db, idesc_bf16(XM, in.n * XN),
+                                            acc);
+                            }
                         }
                     };
                     if (run_start && run_no > 0) {
@@ -250,17 +298,17 @@ k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                     }
                     issue(1);
                     if (run_end) mma_commit<1>(&acc_full[1]);
-                    if (run_start && run_no > 0) {
-                        ok = mbar_wait(&acc_empty[0], (run_no - 1) & 1, abort_flag, g.status);
-                        if (!ok) break;
-                        tc_fence_after();
+                    if constexpr (XL > 0) {
+                        if (run_start && run_no > 0) {
+                            ok = mbar_wait(&acc_empty[0], (run_no - 1) & 1, abort_flag, g.status);
+                            if (!ok) break;
+                            tc_fence_after();
+                        }
+                        issue(0);
+                        if (run_end) mma_commit<1>(&acc_full[0]);
                     }
-                    issue(0);
                     mma_commit<1>(&empty[stage]);
-                    if (run_end) {
-                        mma_commit<1>(&acc_full[0]);
-                        ++run_no;
-                    }
+                    if (run_end) ++run_no;
                     if (++stage == XSTAGES) { stage = 0; phase ^= 1; }
                 }
             }
@@ -277,10 +325,34 @@ k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
             int mb, nb;
             coords(tile, mb, nb);
-            const int nruns = (num_kb + XRUN - 1) / XRUN;
-            long long w[XCPT][4];
+            if constexpr (S == 1) {
+                // the sums of |a||b|: is any of them small?
+                int w_ok = 1;
+                if (lane == 0) w_ok = mbar_wait(&acc_full[1], run_no & 1, abort_flag, g.status) ? 1 : 0;
+                ok = __shfl_sync(0xffffffffu, w_ok, 0) != 0;
+                if (!ok) break;
+                tc_fence_after();
+                bool small = false;
 #pragma unroll
-            for (int j = 0; j < XCPT; ++j) w[j][0] = w[j][1] = w[j][2] = w[j][3] = 0;
+                for (int h = 0; h < XCPT / 8; ++h) {
+                    uint32_t r[8];
+                    tmem_ld8(tmem + lane_base + (uint32_t)(colq * XCPT + h * 8), r);
+                    tmem_wait_ld();
+                    tmem_arrived(r);
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) small |= __uint_as_float(r[j]) > 0.0f && __uint_as_float(r[j]) < SUM_MIN;
+                }
+                tc_fence_before();
+                if (__any_sync(0xffffffffu, small) && lane == 0) g.flags[1] = 1;
+                if (lane == 0) mbar_arrive(&acc_empty[1]);
+                ++run_no;
+            } else {
+            const int nruns = (num_kb + XRUN - 1) / XRUN;
+            long long w[XCPT][XT<S>::LIMBS];
+#pragma unroll
+            for (int j = 0; j < XCPT; ++j)
+#pragma unroll
+                for (int q = 0; q < XT<S>::LIMBS; ++q) w[j][q] = 0;
             for (int c = 0; c < nruns && ok; ++c, ++run_no) {
 #pragma unroll
                 for (int grp = 1; grp >= 0; --grp) {
@@ -289,15 +361,29 @@ k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                     ok = __shfl_sync(0xffffffffu, w_ok, 0) != 0;
                     if (!ok) break;
                     tc_fence_after();
+                    // two D's at a time
 #pragma unroll
-                    for (int d = grp ? XL : 0; d < (grp ? XS : XL); ++d) {
-                        uint32_t r[XCPT];
-                        tmem_ld8(tmem + lane_base + (uint32_t)(d * XN + colq * XCPT), r);
+                    for (int d = grp ? XL : 0; d < (grp ? S : XL); d += 2) {
+                        uint32_t r[2][XCPT];
+                        const uint32_t src = tmem + lane_base + (uint32_t)(d * XN + colq * XCPT);
+                        tmem_ldn(src, r[0]);
+                        if (d + 1 < S) tmem_ldn(src + XN, r[1]);
                         tmem_wait_ld();
-                        constexpr int last[4] = {3, 7, 11, 14};
-                        const long long unit = 1ll << (8 * (last[d >> 2] - d));
+                        tmem_arrived(r[0]);
+                        if (d + 1 < S) tmem_arrived(r[1]);
+                        constexpr long long TERM = (long long)XRUN * XK << 14;       // |D_d| <= (d + 1) TERM
+                        const int q = S == 9 && d == 8 ? 1 : d >> 2;
+                        const int last = S == 9 && d >= 4 ? 8 : d >= 12 ? 14 : (d | 3);
 #pragma unroll
-                        for (int j = 0; j < XCPT; ++j) w[j][d >> 2] += (long long)__float2int_rn(__uint_as_float(r[j])) * unit;
+                        for (int j = 0; j < XCPT; ++j) {
+                            const int x = __float2int_rn(__uint_as_float(r[0][j]));
+                            const int y = d + 1 < S ? __float2int_rn(__uint_as_float(r[1][j])) : 0;
+                            if (d + 1 == S) w[j][q] += x;
+                            else if ((d + 1) * TERM * 256 + (d + 2) * TERM < (1ll << 31))
+                                w[j][q] += (long long)(x * 256 + y) * (1ll << (8 * (last - d - 1)));
+                            else
+                                w[j][q] += (long long)x * (1ll << (8 * (last - d))) + (long long)y * (1ll << (8 * (last - d - 1)));
+                        }
                     }
                     tc_fence_before();
                     __syncwarp();
@@ -308,13 +394,13 @@ k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             const int m = mb * XM + quad * 32 + lane;
             const bool row_ok = m < g.M;
             const int nt = nb * XN + colq * XCPT;
-            // the warp's eight columns are the same for every lane: lane j loads
+            // the warp's columns are the same for every lane: lane j loads
             // column j's exponent and offset, the loop takes them by shuffle
             const bool col_in = lane < XCPT && nt + lane < g.N;
             const int fb = col_in ? g.fb[nt + lane] : 0;
             const long long cn_l = col_in ? (long long)g.c_n[nt + lane] : 0;
             const int ea = row_ok ? max(g.fa[m], 1) - 1022 : 0;
-            const int eb_l = max(fb, 1) - 1022 - 126;
+            const int eb_l = max(fb, 1) - 1022 - 14 - 8 * (S - 1);
             if (g.rows_fast) {
                 // lanes are adjacent rows, adjacent in C
                 double* cp = g.C + (row_ok ? g.c_m[m] : 0);
@@ -361,6 +447,7 @@ k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                 }
                 __syncwarp();
             }
+            }
         }
     }
 
@@ -374,45 +461,48 @@ k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
 }
 
 // ------------------------------------------------------------- host side ---
-// Digit planes [XS][rows][kp] as a 3D map, boxes of box_rows x XK of every digit.
-CUtensorMap digit_map(const void* base, int rows, int kp, int box_rows) {
+// `count` planes from plane `first` on of [XPLANES][rows][kp], boxes of
+// box_rows x box_k of all of them.
+CUtensorMap digit_map(const uint16_t* base, int first, int count, int64_t rows, int kp, int box_rows, int box_k) {
     CUtensorMap m;
     std::memset(&m, 0, sizeof(m));
-    const cuuint64_t dims[3] = {(cuuint64_t)kp, (cuuint64_t)rows, (cuuint64_t)XS};
+    const cuuint64_t dims[3] = {(cuuint64_t)kp, (cuuint64_t)rows, (cuuint64_t)count};
     const cuuint64_t strides[2] = {(cuuint64_t)kp * 2, (cuuint64_t)kp * 2 * (cuuint64_t)rows};
-    const cuuint32_t box[3] = {(cuuint32_t)XK, (cuuint32_t)box_rows, (cuuint32_t)XS};
+    const cuuint32_t box[3] = {(cuuint32_t)box_k, (cuuint32_t)box_rows, (cuuint32_t)count};
     const cuuint32_t estr[3] = {1, 1, 1};
-    CUresult r = encode_fn()(&m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box,
-                             estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B,
+    CUresult r = encode_fn()(&m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<uint16_t*>(base + (size_t)first * rows * kp),
+                             dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                             box_k == 16 ? CU_TENSOR_MAP_SWIZZLE_32B : CU_TENSOR_MAP_SWIZZLE_64B,
                              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) fail(TRG_ECUDA, "cuTensorMapEncodeTiled failed (" + std::to_string((int)r) + ")");
     return m;
 }
 
-int64_t up(int64_t v, int64_t q) { return (v + q - 1) / q * q; }
+inline int64_t up(int64_t v, int64_t q) { return (v + q - 1) / q * q; }
 
 // Exponent fields and digits of rows [0, R) of an operand.
 void digits(Ctx& ctx, const Gather& g, int R, int K, int Rp, int Kp, int* ef, uint16_t* out, int* bad) {
     if (g.c_identity && Kp <= CUT_ROWS_MAX_K) {
-        launch_cut_rows<XS, true>(ctx.stream, g.base, g.off_r, R, K, Rp, Kp, ef, nullptr, out, bad);
+        launch_cut_rows<15, true>(ctx.stream, g.base, g.off_r, R, K, Rp, Kp, ef, nullptr, out, bad);
         TRG_LAUNCHED(ctx);
         return;
     }
     TRG_CUDA(cudaMemsetAsync(ef, 0, (size_t)R * sizeof(int), ctx.stream));
     launch_row_field<true>(ctx.stream, g, R, K, ef);
     TRG_LAUNCHED(ctx);
-    launch_cut<XS>(ctx.stream, g, R, K, Rp, Kp, ef, nullptr, out, bad);
+    launch_cut<15>(ctx.stream, g, R, K, Rp, Kp, ef, nullptr, out, bad);
     TRG_LAUNCHED(ctx);
 }
 
-const long long* diagonal_tiles(Ctx& ctx, int tiles_m, int tiles_n, int& n) {
-    const std::string key = "xsym:" + std::to_string(tiles_m) + ":" + std::to_string(tiles_n);
+// Tiles (128 rows, xn columns) that reach the diagonal or above it.
+const long long* diagonal_tiles(Ctx& ctx, int tiles_m, int tiles_n, int xn, int& n) {
+    const std::string key = "xsym:" + std::to_string(tiles_m) + ":" + std::to_string(tiles_n) + ":" + std::to_string(xn);
     auto it = ctx.lists.find(key);
     if (it == ctx.lists.end()) {
         std::vector<long long> h;
         for (int mb = 0; mb < tiles_m; ++mb)
             for (int nb = 0; nb < tiles_n; ++nb)
-                if ((int64_t)nb * XN + XN - 1 >= (int64_t)mb * XM) h.push_back(((long long)mb << 32) | nb);
+                if ((int64_t)nb * xn + xn - 1 >= (int64_t)mb * XM) h.push_back(((long long)mb << 32) | nb);
         Buf buf;
         ctx.ensure(buf, h.size() * sizeof(long long));
         TRG_CUDA(cudaMemcpyAsync(buf.p, h.data(), h.size() * sizeof(long long), cudaMemcpyHostToDevice, ctx.stream));
@@ -427,32 +517,75 @@ const long long* diagonal_tiles(Ctx& ctx, int tiles_m, int tiles_n, int& n) {
 // Rows of an operand whose digits are held at a time: at most XCAP bytes of
 // them (a multiple of the tile).
 constexpr int64_t XCAP = (int64_t)1 << 30;
+constexpr int64_t XNP = 64;                      // B's rows are padded to this
 int64_t block_rows(int64_t rows, int64_t kp, int64_t tile) {
-    const int64_t most = std::max<int64_t>(tile, XCAP / (2 * XS * kp) / tile * tile);
+    const int64_t most = std::max<int64_t>(tile, XCAP / (2 * XPLANES * kp) / tile * tile);
     return std::min(up(rows, tile), most);
 }
 
 }  // namespace
 
 int64_t exact_scratch_bytes(int64_t M, int64_t N, int64_t K) {
-    const int64_t kp = up(std::max<int64_t>(K, 1), XK);
-    const int64_t ra = block_rows(M, kp, XM), rb = block_rows(N, kp, XN);
-    return 2 * XS * kp * (ra + rb) + 4 * (ra + rb) + 2048;
+    const int64_t kp = up(std::max<int64_t>(K, 1), XKP);
+    const int64_t ra = block_rows(M, kp, XM), rb = block_rows(N, kp, XNP);
+    return 2 * XPLANES * kp * (ra + rb) + 4 * (ra + rb) + 2048;
 }
+
+namespace {
+double tiles_of(int64_t M, int64_t N, int xn, bool sym) {
+    const double tm = (double)up(M, XM) / XM, tn = (double)up(N, xn) / xn;
+    return sym ? 0.5 * tm * (tn + 128.0 / xn) : tm * tn;
+}
+double us15(const Ctx& ctx, int64_t M, int64_t N, int64_t K, bool sym) {
+    return std::ceil(tiles_of(M, N, XT<15>::N, sym) / ctx.sm_count) * (std::ceil((double)K / 64.0) * 4.4 + 3.0);
+}
+// Whether to look for the nine-digit form: the check and the two more launches
+// have to be made good.
+bool try_nine(const Ctx& ctx, int64_t M, int64_t N, int64_t K, bool sym) {
+    if (K > XNINE_K) return false;
+    const double nine = std::ceil(tiles_of(M, N, XT<9>::N, sym) / ctx.sm_count) * (std::ceil((double)K / 96.0) * 3.8 + 3.0);
+    const double check = std::ceil(tiles_of(M, N, XT<1>::N, sym) / ctx.sm_count) * (std::ceil((double)K / 32.0) * 0.35 + 1.0);
+    return nine + check + 16.0 < us15(ctx, M, N, K, sym);
+}
+}  // namespace
 
 double exact_us(const Ctx& ctx, int64_t M, int64_t N, int64_t K, bool sym) {
     if (M > (1ll << 30) || N > (1ll << 30) || K > (1 << 17)) return 1e300;
-    const double tm = (double)up(M, XM) / XM, tn = (double)up(N, XN) / XN;
-    const double tiles = sym ? 0.5 * tm * (tn + 4) : tm * tn;
-    const double runs = std::ceil((double)K / 64.0);
-    const double mma = std::ceil(tiles / ctx.sm_count) * (runs * 4.4 + 3.0);
     const double moved = (46.0 * (double)K * ((double)M + (sym ? 0.0 : (double)N)) + 8.0 * (double)M * (double)N) / 4.0e6;
-    return 25.0 + mma + moved;
+    return 25.0 + us15(ctx, M, N, K, sym) + moved;
 }
 
+namespace {
+
+// The kernel for S digits (S = 1: the sums of |a||b|) on the cut planes.
+template <int S>
+void launch_exact(Ctx& ctx, const uint16_t* sa, int64_t mp, const uint16_t* sb, int64_t np, XArgs a) {
+    constexpr int first = S == 1 ? 15 : 0;
+    static std::once_flag once;
+    std::call_once(once, [] {
+        TRG_CUDA(cudaFuncSetAttribute(k_exact_mma<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, XT<S>::SMEM));
+    });
+    const CUtensorMap ta = digit_map(sa, first, S, mp, a.Kp, XM, XT<S>::K);
+    const CUtensorMap tb = digit_map(sb, first, S, np, a.Kp, XT<S>::N, XT<S>::K);
+    const int tiles_m = (a.M + XM - 1) / XM, tiles_n = (a.N + XT<S>::N - 1) / XT<S>::N;
+    int tiles = tiles_m * tiles_n;
+    a.tile_list = nullptr;
+    a.n_list = 0;
+    if (a.sym) {
+        a.tile_list = diagonal_tiles(ctx, tiles_m, tiles_n, XT<S>::N, a.n_list);
+        tiles = a.n_list;
+    }
+    // column blocks whose digits share L2 (about 40 MB of them)
+    a.group_n = (int)std::max<int64_t>(1, std::min<int64_t>(tiles_n, (40ll << 20) / ((int64_t)XT<S>::N * a.Kp * 2 * S)));
+    k_exact_mma<S><<<std::min(tiles, ctx.sm_count), XT<S>::THREADS, XT<S>::SMEM, ctx.stream>>>(ta, tb, a);
+    TRG_LAUNCHED(ctx);
+}
+
+}  // namespace
+
 bool gemm_exact(Ctx& ctx, const GemmDesc& d) {
-    const int K = (int)std::max<int64_t>(d.K, 1), Kp = (int)up(K, XK);
-    const int64_t ra = block_rows(d.M, Kp, XM), rb = block_rows(d.N, Kp, XN);
+    const int K = (int)std::max<int64_t>(d.K, 1), Kp = (int)up(K, XKP);
+    const int64_t ra = block_rows(d.M, Kp, XM), rb = block_rows(d.N, Kp, XNP);
     const bool sym = d.gram && d.M == d.N && ra >= d.M;
     try {
         ctx.ensure(ctx.split_ws, (size_t)exact_scratch_bytes(d.M, sym ? 1 : d.N, K));
@@ -462,16 +595,13 @@ bool gemm_exact(Ctx& ctx, const GemmDesc& d) {
     }
     uint8_t* p = ctx.split_ws.as<uint8_t>();
     auto take = [&](size_t bytes) { uint8_t* q = p; p += (bytes + 255) & ~(size_t)255; return q; };
-    int* bad = (int*)take(4);
+    int* flags = (int*)take(2 * sizeof(int));
+    int* bad = flags;
     int* fa = (int*)take((size_t)ra * 4);
     int* fb = sym ? fa : (int*)take((size_t)rb * 4);
-    uint16_t* sa = (uint16_t*)take((size_t)(2 * XS) * ra * Kp);
-    uint16_t* sb = sym ? sa : (uint16_t*)take((size_t)(2 * XS) * rb * Kp);
-    TRG_CUDA(cudaMemsetAsync(bad, 0, sizeof(int), ctx.stream));
-    static std::once_flag once;
-    std::call_once(once, [] {
-        TRG_CUDA(cudaFuncSetAttribute(k_exact_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, XSMEM));
-    });
+    uint16_t* sa = (uint16_t*)take((size_t)(2 * XPLANES) * ra * Kp);
+    uint16_t* sb = sym ? sa : (uint16_t*)take((size_t)(2 * XPLANES) * rb * Kp);
+    TRG_CUDA(cudaMemsetAsync(flags, 0, 2 * sizeof(int), ctx.stream));
 
     // B as rows n, columns k
     const Gather bt = transposed(d.B);
@@ -480,36 +610,31 @@ bool gemm_exact(Ctx& ctx, const GemmDesc& d) {
         Gather ga = d.A;
         ga.off_r += m0;
         digits(ctx, ga, mr, K, mp, Kp, fa, sa, bad);
-        const CUtensorMap ta = digit_map(sa, mp, Kp, XM);
         for (int64_t n0 = 0; n0 < d.N; n0 += rb) {
-            const int nr = (int)std::min(rb, d.N - n0), np = sym ? mp : (int)up(nr, XN);
+            const int nr = (int)std::min(rb, d.N - n0), np = sym ? mp : (int)up(nr, XNP);
             if (!sym && (m0 == 0 || rb < d.N)) {
                 Gather gb = bt;
                 gb.off_r += n0;
                 digits(ctx, gb, nr, K, np, Kp, fb, sb, bad);
             }
-            const CUtensorMap tb = digit_map(sb, np, Kp, XN);
             XArgs a;
             a.M = mr; a.N = sym ? mr : nr; a.Kp = Kp;
             a.fa = fa; a.fb = fb;
             a.C = d.C; a.c_m = d.c_m + m0; a.c_n = d.c_n + n0;
             a.rows_fast = d.c_m_fast && !sym ? 1 : 0;
             a.sym = sym ? 1 : 0;
-            a.tile_list = nullptr; a.n_list = 0;
-            a.bad = bad; a.status = ctx.status.as<int>();
-            const int tiles_m = mp / XM, tiles_n = (a.N + XN - 1) / XN;
-            int tiles = tiles_m * tiles_n;
-            if (sym) {
-                a.tile_list = diagonal_tiles(ctx, tiles_m, tiles_n, a.n_list);
-                tiles = a.n_list;
-            }
-            // column blocks whose digits share L2 (about 40 MB of them)
-            a.group_n = (int)std::max<int64_t>(1, std::min<int64_t>(tiles_n, (40ll << 20) / ((int64_t)XN * Kp * 2 * XS)));
-            const int grid = std::min(tiles, ctx.sm_count);
+            a.flags = flags; a.status = ctx.status.as<int>();
             const int tok = ctx.region_begin(TRG_PHASE_MMA);
-            k_exact_mma<<<grid, XTHREADS, XSMEM, ctx.stream>>>(ta, tb, a);
-            TRG_LAUNCHED(ctx);
-            ctx.region_end(tok, 2.0 * (double)mr * nr * K, 120.0 * 2.0 * (double)mr * nr * Kp);
+            const bool nine = try_nine(ctx, a.M, a.N, K, sym);
+            a.nine = nine ? 1 : 0;
+            if (nine) {
+                // (each block decides for itself; an operand out of range stays so)
+                if (m0 + n0 > 0) TRG_CUDA(cudaMemsetAsync(flags + 1, 0, sizeof(int), ctx.stream));
+                launch_exact<1>(ctx, sa, mp, sb, np, a);
+                launch_exact<9>(ctx, sa, mp, sb, np, a);
+            }
+            launch_exact<15>(ctx, sa, mp, sb, np, a);
+            ctx.region_end(tok, 2.0 * (double)mr * nr * K, (nine ? 45.0 : 120.0) * 2.0 * (double)mr * nr * Kp);   // 120 also if nine do not suffice
             if (sym) break;
         }
     }

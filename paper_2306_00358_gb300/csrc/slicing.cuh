@@ -43,10 +43,14 @@ __device__ __forceinline__ unsigned exponent_field(double x) {
 // Scale exponent of a row from its largest field (-1022 for a zero row).
 __device__ __forceinline__ int row_exponent(int f) { return f ? f - 1022 : -1022; }
 
+// Planes stored for S digits: 15 digits are followed by |x| 2^-e itself, cut off
+// to BF16 (the operands of the product's |A||B|, see exact_gemm.cu).
+__host__ __device__ constexpr int planes(int S) { return S == 15 ? 16 : S; }
+
 // The digits of x in a row of largest field f, as the FP32 values to store
 // (exact in BF16: their upper halves).
 template <int S>
-__device__ __forceinline__ void cut(double x, int f, float (&d)[S]) {
+__device__ __forceinline__ void cut(double x, int f, float (&d)[planes(S)]) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(x);
     const int ex = (int)((b >> 52) & 0x7FF);
     const unsigned long long m53 = ex ? ((b & ((1ull << 52) - 1)) | (1ull << 52)) : 0ull;
@@ -67,6 +71,9 @@ __device__ __forceinline__ void cut(double x, int f, float (&d)[S]) {
             const int byte = 14 - p;
             d[p] = __uint_as_float(__byte_perm(q[byte >> 2], 0x4B000000u, 0x7440u | (unsigned)(byte & 3))) - 8388736.0f;   // 2^23 + 128
         }
+        // FP32 exponent field of |x| 2^-e, not below 2^-60: products stay normal
+        const int ea = max(ex - f + 126, 127 - 60);
+        d[15] = ex ? __uint_as_float(((unsigned)ea << 23) | (((unsigned)(m53 >> 45) & 0x7Fu) << 16)) : 0.0f;
     } else {
         constexpr int F = 7 + 8 * (S - 1);
         constexpr unsigned BIAS = S == 2 ? 0x80u : S == 3 ? 0x8080u : S == 4 ? 0x808080u : 0x80808080u;
@@ -84,12 +91,12 @@ __device__ __forceinline__ void cut(double x, int f, float (&d)[S]) {
 }
 // Two neighbours' digits as packed BF16.
 template <int S>
-__device__ __forceinline__ void cut2(double x0, double x1, int f, uint32_t (&w)[S]) {
-    float a[S], b[S];
+__device__ __forceinline__ void cut2(double x0, double x1, int f, uint32_t (&w)[planes(S)]) {
+    float a[planes(S)], b[planes(S)];
     cut<S>(x0, f, a);
     cut<S>(x1, f, b);
 #pragma unroll
-    for (int p = 0; p < S; ++p) w[p] = __byte_perm(__float_as_uint(a[p]), __float_as_uint(b[p]), 0x7632);
+    for (int p = 0; p < planes(S); ++p) w[p] = __byte_perm(__float_as_uint(a[p]), __float_as_uint(b[p]), 0x7632);
 }
 
 // Rows of an exact product whose largest entry lies outside this range make
@@ -175,12 +182,12 @@ __global__ void __launch_bounds__(256) k_cut(const double* __restrict__ src, con
         check_range(f, bad);
         if (e_out && blockIdx.x == 0 && kg == 0 && r < R) e_out[r] = row_exponent(f);
         const double* x = tile + rr * XD_LD + kg * 9;
-        uint32_t w[4][S];
+        uint32_t w[4][planes(S)];
 #pragma unroll
         for (int h = 0; h < 4; ++h) cut2<S>(x[2 * h], x[2 * h + 1], f, w[h]);
         uint16_t* o = out + (size_t)r * Kp + k;
 #pragma unroll
-        for (int p = 0; p < S; ++p) *reinterpret_cast<uint4*>(o + p * plane) = make_uint4(w[0][p], w[1][p], w[2][p], w[3][p]);
+        for (int p = 0; p < planes(S); ++p) *reinterpret_cast<uint4*>(o + p * plane) = make_uint4(w[0][p], w[1][p], w[2][p], w[3][p]);
     }
 }
 
@@ -199,11 +206,11 @@ __device__ __forceinline__ void load4(const double* row, int k, int K, bool vec,
 }
 template <int S>
 __device__ __forceinline__ void store4(const double (&v)[4], int f, uint16_t* o, size_t plane) {
-    uint32_t a[S], b[S];
+    uint32_t a[planes(S)], b[planes(S)];
     cut2<S>(v[0], v[1], f, a);
     cut2<S>(v[2], v[3], f, b);
 #pragma unroll
-    for (int p = 0; p < S; ++p) *reinterpret_cast<uint2*>(o + p * plane) = make_uint2(a[p], b[p]);
+    for (int p = 0; p < planes(S); ++p) *reinterpret_cast<uint2*>(o + p * plane) = make_uint2(a[p], b[p]);
 }
 
 // Contiguous rows with known fields: a warp per row, four columns per lane.

@@ -84,6 +84,26 @@ def test_contraction_matches_torch(torch, dx, dy, dn, ws):
     assert bool(((out - _contract(torch, t, u)).abs() <= bound).all())
 
 
+# nearly decoupled sectors (even and odd index sums, coupled by eps): sums of
+# products far below the largest ones keep their own accuracy.  0: the odd sums
+# are exact zeros; 2^-4: all sums are of like size.
+@pytest.mark.parametrize("eps", [0.0, 2.0 ** -70, 2.0 ** -30, 2.0 ** -9, 2.0 ** -4])
+@pytest.mark.parametrize("dx,dy,dn", [(16, 16, 16), (24, 24, 24), (27, 22, 31)])
+def test_contraction_of_weakly_coupled_sectors(torch, eps, dx, dy, dn):
+    rng = np.random.default_rng(dx)
+
+    def graded(*shape):
+        odd = np.indices(shape).sum(0) % 2
+        x = rng.uniform(0.5, 1.0, shape) * rng.choice([-1.0, 1.0], shape) * np.where(odd, eps, 1.0)
+        return torch.from_numpy(x).cuda()
+
+    t, u = graded(dx, dy, dx, dy), graded(dx, dx, dn)
+    with Solver(0) as s:
+        out = s.contract(t, u)
+    bound = 2.0 * (dx + 1 + dx * dy + 1 + dx * dx + 1) * 1.01 * 2.0 ** -53 * _contract(torch, t.abs(), u.abs())
+    assert bool(((out - _contract(torch, t, u)).abs() <= bound).all())
+
+
 # operands outside the digits' range take the FP64 pipe
 @pytest.mark.parametrize("scale", [2.0 ** 420, 2.0 ** -420, 2.0 ** -480])
 def test_contraction_outside_the_digit_range(torch, scale):
