@@ -10,7 +10,7 @@
 // Algorithms 59 (2012) 95).  With D_d = sum_{p + q = d} A_p B_q and S digits,
 //     C = 2^(ea + eb - 14) sum_{d < S} D_d 2^(-8 d):
 // digit products are integers up to 2^14, a short run of K (64 for 15 digits,
-// 128 for 8) sums the at most S products of a D_d exactly in FP32, the
+// 96 for 9) sums the at most S products of a D_d exactly in FP32, the
 // epilogue moves each run into int64 sums and the wide total is turned into
 // FP64.
 //
@@ -34,7 +34,11 @@
 // the time, MMA instructions of N = 48 .. 240; 10 % go to drains that nothing
 // covers).  128 x 32 output tile with 15 digits, 128 x 48 with 9, one persistent
 // CTA per SM: the S accumulators D_d of the tile's columns fill tensor memory.
-// A stage is 16 (32) K of both operands, one TMA box each, two stages.  The
+// A stage is 16 (32) K of both operands, one TMA box each, two stages; the cut
+// stores the digits in the order of a stage, so that a box is made of 4 KB
+// pieces (as [p][r][k] planes its rows are pieces of 32 or 64 bytes, and the TMA
+// unit's requests hold the products up: 72 -> 68.6 us a product of an
+// environment at (24, 22)).  The
 // products of one A digit with adjacent B digits land in adjacent accumulators,
 // so 23 (13) instructions of up to N = 256 cover the products of a 16-deep
 // step.  They are issued in two groups, the one that lands in the higher D_d
@@ -43,8 +47,8 @@
 // under the next run's first group.
 // Measured, contraction at Dx = Dy = Dn = 48 (1.22e12 FP64 FLOPs): 993 ms on
 // the FP64 pipe, 113.6 ms with 15 digits always, 45.3 ms with 9 where they
-// suffice (39.5 ms of it in this kernel, 1.6 ms in the |A||B| sums); with
-// operands that need 15, the sums are the only loss.
+// suffice (38.7 ms of it in this kernel, 1.5 ms in the |A||B| sums, 3.8 ms in
+// the cut); with operands that need 15, the sums are the only loss.
 #include <algorithm>
 #include <cmath>
 
@@ -69,8 +73,9 @@ struct XT {
     static constexpr int L = S == 15 ? 8 : S == 9 ? 4 : 0;         // D_0 .. D_(L-1) are group 0, the rest group 1
     static constexpr int EPI = S == 9 ? 12 : 16;                   // epilogue warps: 16 columns each with 9 digits
     static constexpr int THREADS = 64 + 32 * EPI;
-    static constexpr int A_TILE = XM * K * 2, B_TILE = N * K * 2;  // bytes of one digit's tiles
-    static constexpr int STAGE = S * (A_TILE + B_TILE);            // 75, 50 and 24 KB
+    static constexpr int KB = K / 16;
+    static constexpr int A_TILE = XM * 32, B_TILE = N * 32;        // bytes of 16 K of one digit's tiles
+    static constexpr int STAGE = KB * S * (A_TILE + B_TILE);       // 75, 99 and 24 KB
     static constexpr int STAGES = S == 1 ? 4 : 2;
     static constexpr int RUN = S == 1 ? 1 << 30 : S == 9 ? 3 : 4;  // stages of an exact run
     static constexpr int CPT = N / (EPI / 4);                      // columns per epilogue thread
@@ -182,7 +187,7 @@ template <int S>
 __global__ void __launch_bounds__(XT<S>::THREADS, 1)
 k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const XArgs g) {
     constexpr int XN = XT<S>::N, XK = XT<S>::K, XL = XT<S>::L, XSTAGES = XT<S>::STAGES, XSTAGE = XT<S>::STAGE;
-    constexpr int XA_TILE = XT<S>::A_TILE, XB_TILE = XT<S>::B_TILE, XRUN = XT<S>::RUN, XCPT = XT<S>::CPT;
+    constexpr int XA_TILE = XT<S>::A_TILE, XKB = XT<S>::KB, XB_TILE = XT<S>::B_TILE, XRUN = XT<S>::RUN, XCPT = XT<S>::CPT;
     if (g.flags[0] || (S == 9 && g.flags[1]) || (S == 15 && g.nine && !g.flags[1])) return;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -247,8 +252,8 @@ k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                     if (!ok) break;
                     uint8_t* st = smem + stage * XSTAGE;
                     mbar_expect_tx(&full[stage], XSTAGE);
-                    tma_load_3d(st, &tmA, kb * XK, mb * XM, 0, &full[stage]);
-                    tma_load_3d(st + S * XA_TILE, &tmB, kb * XK, nb * XN, 0, &full[stage]);
+                    tma_load_4d(st, &tmA, 0, mb * (XM / 4), 0, kb * XKB, &full[stage]);
+                    tma_load_4d(st + XKB * S * XA_TILE, &tmB, 0, nb * (XN / 4), 0, kb * XKB, &full[stage]);
 #pragma unroll
                     for (int s = 0; s < XSTAGES; ++s)
                         if (s == stage) issued[s] = (int)phase;
@@ -274,18 +279,18 @@ k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                     ok = mbar_wait(&full[stage], phase, abort_flag, g.status);
                     if (!ok) break;
                     tc_fence_after();
-                    const uint32_t sbase = smem_u32(smem + stage * XSTAGE);
-                    const uint64_t dbase = XK == 16 ? smem_desc32(sbase) : smem_desc(sbase);
+                    const uint64_t dbase = smem_desc32(smem_u32(smem + stage * XSTAGE));
                     auto issue = [&](int group) {
 #pragma unroll
-                        for (int kk = 0; kk < XK / 16; ++kk) {
+                        for (int kk = 0; kk < XKB; ++kk) {
 #pragma unroll
                             for (int t = 0; t < xins_count<S>(); ++t) {
                                 const XIns in = xins<S>(t);
                                 if (in.group != group) continue;
                                 const uint32_t acc = ((t == 0 || t == S) && run_start && kk == 0) ? 0u : 1u;
-                                const uint64_t da = dbase + (uint64_t)((in.a * XA_TILE + kk * 32) >> 4);
-                                const uint64_t db = dbase + (uint64_t)((S * XA_TILE + in.b * XB_TILE + kk * 32) >> 4);
+                                const uint64_t da = dbase + (uint64_t)(((kk * S + in.a) * XA_TILE) >> 4);
+                                const uint64_t db =
+                                    dbase + (uint64_t)((XKB * S * XA_TILE + (kk * S + in.b) * XB_TILE) >> 4);
                                 mma_bf16<1>(tmem + (uint32_t)((in.a + in.b) * XN), da, db, idesc_bf16(XM, in.n * XN),
                                             acc);
                             }
@@ -461,18 +466,18 @@ k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
 }
 
 // ------------------------------------------------------------- host side ---
-// `count` planes from plane `first` on of [XPLANES][rows][kp], boxes of
-// box_rows x box_k of all of them.
+// `count` planes from plane `first` on of the digits [kp / 16][XPLANES][rows][16]
+// (their order in a stage: no swizzle here), four rows to a 128-byte line,
+// boxes of box_rows rows and box_k K of all of them.
 CUtensorMap digit_map(const uint16_t* base, int first, int count, int64_t rows, int kp, int box_rows, int box_k) {
     CUtensorMap m;
     std::memset(&m, 0, sizeof(m));
-    const cuuint64_t dims[3] = {(cuuint64_t)kp, (cuuint64_t)rows, (cuuint64_t)count};
-    const cuuint64_t strides[2] = {(cuuint64_t)kp * 2, (cuuint64_t)kp * 2 * (cuuint64_t)rows};
-    const cuuint32_t box[3] = {(cuuint32_t)box_k, (cuuint32_t)box_rows, (cuuint32_t)count};
-    const cuuint32_t estr[3] = {1, 1, 1};
-    CUresult r = encode_fn()(&m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<uint16_t*>(base + (size_t)first * rows * kp),
-                             dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                             box_k == 16 ? CU_TENSOR_MAP_SWIZZLE_32B : CU_TENSOR_MAP_SWIZZLE_64B,
+    const cuuint64_t dims[4] = {64, (cuuint64_t)rows / 4, (cuuint64_t)count, (cuuint64_t)kp / 16};
+    const cuuint64_t strides[3] = {128, (cuuint64_t)rows * 32, (cuuint64_t)rows * 32 * XPLANES};
+    const cuuint32_t box[4] = {64, (cuuint32_t)box_rows / 4, (cuuint32_t)count, (cuuint32_t)box_k / 16};
+    const cuuint32_t estr[4] = {1, 1, 1, 1};
+    CUresult r = encode_fn()(&m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<uint16_t*>(base + (size_t)first * rows * 16),
+                             dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
                              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) fail(TRG_ECUDA, "cuTensorMapEncodeTiled failed (" + std::to_string((int)r) + ")");
     return m;
@@ -482,8 +487,8 @@ inline int64_t up(int64_t v, int64_t q) { return (v + q - 1) / q * q; }
 
 // Exponent fields and digits of rows [0, R) of an operand.
 void digits(Ctx& ctx, const Gather& g, int R, int K, int Rp, int Kp, int* ef, uint16_t* out, int* bad) {
-    if (g.c_identity && Kp <= CUT_ROWS_MAX_K) {
-        launch_cut_rows<15, true>(ctx.stream, g.base, g.off_r, R, K, Rp, Kp, ef, nullptr, out, bad);
+    if (g.c_identity && Kp <= CUT_ROWS4_MAX_K) {
+        launch_cut_rows4(ctx.stream, g.base, g.off_r, R, K, Rp, Kp, ef, out, bad);
         TRG_LAUNCHED(ctx);
         return;
     }

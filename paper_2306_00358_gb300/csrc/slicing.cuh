@@ -3,7 +3,7 @@
 //
 // An operand is rows r < R of length K, element (r, k) at src[off_r[r] +
 // off_c[k]]; its digits go to out[p][r][k] (r < Rp, k < Kp, zero in the
-// padding).  With f the largest exponent field of a row and e = f - 1022
+// padding; digit_at for the order of 15 digits).  With f the largest exponent field of a row and e = f - 1022
 // (|x| < 2^e), X = rint(x 2^(F - e)), F = 7 + 8 (S - 1), halves away from
 // zero, is the sum of d_p 2^(8 (S - 1 - p)), d_0 in [-128, 128], d_p in
 // [-128, 127]; slices are stored as d_p 2^(-8p) (S <= 5) or as d_p (S = 15).
@@ -12,7 +12,7 @@
 // of their own) and 2 S B written per element.
 //  - Rows that are contiguous runs of at most 8192 are read once: a warp or a
 //    block holds a row in registers, finds its exponent and cuts it
-//    (k_cut_rows).  16384 x 4096, S = 4: 153 us (1.07 GB, 7.0 TB/s).
+//    (k_cut_rows; k_cut_rows4 for 15 digits, up to 4096).  16384 x 4096, S = 4: 153 us (1.07 GB, 7.0 TB/s).
 //  - Rows whose exponents the producing product recorded: a warp per row
 //    (k_slice_contig).
 //  - Gathered operands: k_row_field, then k_cut, both reading along the index
@@ -89,6 +89,19 @@ __device__ __forceinline__ void cut(double x, int f, float (&d)[planes(S)]) {
         }
     }
 }
+// Where digit 0 of element (r, k) goes, and how far apart the digits of an
+// element are: [p][r][k], but for 15 digits (and |x| 2^-e) the order in which
+// their product's stages hold them in shared memory, [k / 16][p][r][k % 16] with
+// the two 16-byte halves of a row's 16 k swapped in every other four rows (the
+// 32-byte swizzle): a stage is a few long pieces of memory then.
+template <int S>
+__device__ __forceinline__ size_t digit_at(int r, int k, int Rp, int Kp) {
+    if (S == 15) return ((size_t)(k >> 4) * planes(S) * Rp + r) * 16 + ((((k >> 3) ^ (r >> 2)) & 1) << 3) + (k & 7);
+    return (size_t)r * Kp + k;
+}
+template <int S>
+__device__ __forceinline__ size_t digit_stride(int Rp, int Kp) { return (size_t)Rp * (S == 15 ? 16 : Kp); }
+
 // Two neighbours' digits as packed BF16.
 template <int S>
 __device__ __forceinline__ void cut2(double x0, double x1, int f, uint32_t (&w)[planes(S)]) {
@@ -109,9 +122,8 @@ __device__ __forceinline__ void check_range(int f, int* bad) {
 // Largest exponent field of each row, maxima into ef (zeroed); a block takes 32
 // rows and xf_k of their entries.  It is bound by latency where the operand is
 // small: 256 entries (eight loads in flight per thread, fewest atomics) leave
-// most of the chip idle there, so 64 are taken below four blocks per SM
-// (576 rows of 576:
-// 11.4 -> 4.2 us).
+// most of the chip idle there, so 64 are taken below four blocks per SM (576
+// rows of 576: 11.4 -> 4.2 us).
 constexpr int XF_BLOCKS = 600;
 template <bool SUB>
 __global__ void __launch_bounds__(256) k_row_field(const double* __restrict__ src, const int64_t* __restrict__ off_r,
@@ -166,7 +178,7 @@ __global__ void __launch_bounds__(256) k_cut(const double* __restrict__ src, con
                                              uint16_t* __restrict__ out, int* bad) {
     __shared__ double tile[XD_R * XD_LD];
     const int k0 = blockIdx.x * XD_K;
-    const size_t plane = (size_t)Rp * Kp;
+    const size_t plane = digit_stride<S>(Rp, Kp);
     const int nby = (Rp + XD_R - 1) / XD_R;
     for (int by = blockIdx.y; by < nby; by += gridDim.y) {
         const int r0 = by * XD_R;
@@ -190,7 +202,7 @@ __global__ void __launch_bounds__(256) k_cut(const double* __restrict__ src, con
         uint32_t w[4][planes(S)];
 #pragma unroll
         for (int h = 0; h < 4; ++h) cut2<S>(x[2 * h], x[2 * h + 1], f, w[h]);
-        uint16_t* o = out + (size_t)r * Kp + k;
+        uint16_t* o = out + digit_at<S>(r, k, Rp, Kp);
 #pragma unroll
         for (int p = 0; p < planes(S); ++p) *reinterpret_cast<uint4*>(o + p * plane) = make_uint4(w[0][p], w[1][p], w[2][p], w[3][p]);
     }
@@ -226,7 +238,7 @@ __global__ void __launch_bounds__(256) k_slice_contig(const double* __restrict__
     const int lane = threadIdx.x & 31;
     const int r = blockIdx.x * 8 + (threadIdx.x >> 5);
     if (r >= Rp) return;
-    const size_t plane = (size_t)Rp * Kp;
+    const size_t plane = digit_stride<S>(Rp, Kp);
     const bool real = r < R;
     const double* row = real ? src + off_r[r] : nullptr;
     const bool vec = real && ((reinterpret_cast<uintptr_t>(row) & 15) == 0);
@@ -236,7 +248,7 @@ __global__ void __launch_bounds__(256) k_slice_contig(const double* __restrict__
     for (int k = lane * 4; k < Kp; k += 128) {
         double v[4];
         load4(row, k, real ? K : 0, vec, v);
-        store4<S>(v, f, out + (size_t)r * Kp + k, plane);
+        store4<S>(v, f, out + digit_at<S>(r, k, Rp, Kp), plane);
     }
 }
 
@@ -250,7 +262,7 @@ __global__ void __launch_bounds__(256) k_cut_rows(const double* __restrict__ src
     const int t = threadIdx.x % TPR;
     const int r = blockIdx.x * (256 / TPR) + threadIdx.x / TPR;
     if (TPR == 32 && r >= Rp) return;
-    const size_t plane = (size_t)Rp * Kp;
+    const size_t plane = digit_stride<S>(Rp, Kp);
     const bool real = r < R;
     const double* row = real ? src + off_r[r] : nullptr;
     const bool vec = real && ((reinterpret_cast<uintptr_t>(row) & 15) == 0);
@@ -278,7 +290,7 @@ __global__ void __launch_bounds__(256) k_cut_rows(const double* __restrict__ src
 #pragma unroll
     for (int c = 0; c < NCH; ++c) {
         const int k = (c * TPR + t) * 4;
-        if (k < Kp) store4<S>(v[c], f, out + (size_t)r * Kp + k, plane);
+        if (k < Kp) store4<S>(v[c], f, out + digit_at<S>(r, k, Rp, Kp), plane);
     }
 }
 
@@ -292,6 +304,57 @@ void launch_cut_rows(cudaStream_t stream, const double* src, const int64_t* off_
     else if (Kp <= 2048) k_cut_rows<S, 256, 2, SUB><<<gb, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, e_out, out, bad);
     else if (Kp <= 4096) k_cut_rows<S, 256, 4, SUB><<<gb, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, e_out, out, bad);
     else k_cut_rows<S, 256, 8, SUB><<<gb, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, e_out, out, bad);
+}
+
+// The same for 15 digits, K <= 256 NCH: a block holds four rows, and a warp
+// stores 32 k of all four at a time, so that each digit's 2 x 128 bytes are
+// contiguous (digit_at; a warp per row writes eight pieces of 32 bytes, which
+// takes 564 us where this takes 236: 6912 rows of 2304).
+template <int NCH>
+__global__ void __launch_bounds__(256) k_cut_rows4(const double* __restrict__ src, const int64_t* __restrict__ off_r,
+                                                   int R, int K, int Rp, int Kp, int* __restrict__ ef_out,
+                                                   uint16_t* __restrict__ out, int* bad) {
+    __shared__ unsigned wmax[8][4];
+    const int warp = threadIdx.x >> 5, rr = (threadIdx.x >> 3) & 3, kc = threadIdx.x & 7;
+    const int r = blockIdx.x * 4 + rr;                   // Rp is a multiple of four
+    const size_t plane = digit_stride<15>(Rp, Kp);
+    const bool real = r < R;
+    const double* row = real ? src + off_r[r] : nullptr;
+    const bool vec = real && ((reinterpret_cast<uintptr_t>(row) & 15) == 0);
+    double v[NCH][4];
+    unsigned fm = 0;
+#pragma unroll
+    for (int c = 0; c < NCH; ++c) load4(row, ((c * 8 + warp) * 8 + kc) * 4, real ? K : 0, vec, v[c]);
+#pragma unroll
+    for (int c = 0; c < NCH; ++c)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) fm = max(fm, exponent_field<true>(v[c][j]));
+#pragma unroll
+    for (int m = 1; m < 8; m *= 2) fm = max(fm, __shfl_xor_sync(0xffffffffu, fm, m));
+    if (kc == 0) wmax[warp][rr] = fm;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < 8; ++w) fm = max(fm, wmax[w][rr]);
+    const int f = (int)fm;
+    check_range(f, bad);
+    if (warp == 0 && kc == 0 && real) ef_out[r] = f;
+#pragma unroll
+    for (int c = 0; c < NCH; ++c) {
+        const int k = ((c * 8 + warp) * 8 + kc) * 4;
+        if (k < Kp) store4<15>(v[c], f, out + digit_at<15>(r, k, Rp, Kp), plane);
+    }
+}
+
+constexpr int CUT_ROWS4_MAX_K = 4096;
+inline void launch_cut_rows4(cudaStream_t stream, const double* src, const int64_t* off_r, int R, int K, int Rp, int Kp,
+                             int* ef_out, uint16_t* out, int* bad) {
+    const unsigned grid = (unsigned)(Rp / 4);
+    if (Kp <= 256) k_cut_rows4<1><<<grid, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, out, bad);
+    else if (Kp <= 512) k_cut_rows4<2><<<grid, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, out, bad);
+    else if (Kp <= 1024) k_cut_rows4<4><<<grid, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, out, bad);
+    else if (Kp <= 2048) k_cut_rows4<8><<<grid, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, out, bad);
+    else if (Kp <= 3072) k_cut_rows4<12><<<grid, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, out, bad);
+    else k_cut_rows4<16><<<grid, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, out, bad);
 }
 
 template <bool SUB>
