@@ -68,6 +68,8 @@ size_t estimate_bytes(const trg_solve_spec& s, size_t workspace_cap, bool exact)
         const double jb = std::max(1.0, std::floor(ws / std::max(1.0, 2 * D * D * D2 * 8)));
         const int64_t d = (int64_t)D, d2 = d * d, rows = (int64_t)std::min(D, jb) * d2;
         bytes += (double)std::max({trg::exact_scratch_bytes(d2, d2, d2), trg::exact_scratch_bytes(d2, rows, d),
+                                   // (two Gram products share a launch up to 640 rows)
+                                   trg::exact_pair_scratch_bytes(std::min<int64_t>(d2, 640), d2),
                                    trg::exact_scratch_bytes(rows, d2, d2), trg::exact_scratch_bytes(rows, d, d2),
                                    trg::exact_scratch_bytes(d2, (int64_t)m, d2)});
     }

@@ -145,6 +145,12 @@ struct XArgs {
     int group_n;                   // tile order: column blocks per group
     int* flags;                    // [0] an operand is outside the digits' range, [1] nine digits do not suffice
     int nine;                      // the nine-digit form has been tried
+    // a second Gram product of the same size: its rows are those from half on
+    // (0: none), its tiles are in tile_list too
+    int half;
+    double* C1;
+    const int64_t* c_m1;
+    const int64_t* c_n1;
     int* status;
 };
 
@@ -396,19 +402,24 @@ k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                 }
             }
             if (!ok) break;
-            const int m = mb * XM + quad * 32 + lane;
+            const bool second = g.half && mb * XM >= g.half;
+            const int r0 = second ? g.half : 0;
+            double* const C = second ? g.C1 : g.C;
+            const int64_t* const c_m = second ? g.c_m1 : g.c_m;
+            const int64_t* const c_n = second ? g.c_n1 : g.c_n;
+            const int m = mb * XM + quad * 32 + lane - r0;
             const bool row_ok = m < g.M;
-            const int nt = nb * XN + colq * XCPT;
+            const int nt = nb * XN + colq * XCPT - r0;
             // the warp's columns are the same for every lane: lane j loads
             // column j's exponent and offset, the loop takes them by shuffle
             const bool col_in = lane < XCPT && nt + lane < g.N;
-            const int fb = col_in ? g.fb[nt + lane] : 0;
-            const long long cn_l = col_in ? (long long)g.c_n[nt + lane] : 0;
-            const int ea = row_ok ? max(g.fa[m], 1) - 1022 : 0;
+            const int fb = col_in ? g.fb[nt + lane + r0] : 0;
+            const long long cn_l = col_in ? (long long)c_n[nt + lane] : 0;
+            const int ea = row_ok ? max(g.fa[m + r0], 1) - 1022 : 0;
             const int eb_l = max(fb, 1) - 1022 - 14 - 8 * (S - 1);
             if (g.rows_fast) {
                 // lanes are adjacent rows, adjacent in C
-                double* cp = g.C + (row_ok ? g.c_m[m] : 0);
+                double* cp = C + (row_ok ? c_m[m] : 0);
 #pragma unroll
                 for (int j = 0; j < XCPT; ++j) {
                     const int e2 = ea + __shfl_sync(0xffffffffu, eb_l, j);
@@ -425,11 +436,11 @@ k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             }
             if (g.sym && row_ok) {
                 // the mirror (n, m) of each element above the diagonal
-                const int64_t cm_mirror = g.c_n[m];
+                const int64_t cm_mirror = c_n[m];
 #pragma unroll
                 for (int j = 0; j < XCPT; ++j) {
                     const int n = nt + j;
-                    if (n < g.N && n > m) g.C[g.c_m[n] + cm_mirror] = v[j];
+                    if (n < g.N && n > m) C[c_m[n] + cm_mirror] = v[j];
                 }
             }
             // columns adjacent in C: through the warp's 32 x 8 staging tile, so
@@ -446,9 +457,9 @@ k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
 #pragma unroll
                 for (int q = 0; q < 8; ++q) {
                     const int rr = 4 * q + quarter;
-                    const int mr = mb * XM + quad * 32 + rr;
+                    const int mr = mb * XM + quad * 32 + rr - r0;
                     if (mr < g.M && n < g.N && (!g.sym || n >= mr))
-                        g.C[g.c_m[mr] + cn] = stg[rr * 8 + (cl ^ ((rr >> 1) & 7))];
+                        C[c_m[mr] + cn] = stg[rr * 8 + (cl ^ ((rr >> 1) & 7))];
                 }
                 __syncwarp();
             }
@@ -485,29 +496,34 @@ CUtensorMap digit_map(const uint16_t* base, int first, int count, int64_t rows, 
 
 inline int64_t up(int64_t v, int64_t q) { return (v + q - 1) / q * q; }
 
-// Exponent fields and digits of rows [0, R) of an operand.
-void digits(Ctx& ctx, const Gather& g, int R, int K, int Rp, int Kp, int* ef, uint16_t* out, int* bad) {
+// Exponent fields and digits of rows [0, R) of an operand, as rows of an array
+// of Rs.
+void digits(Ctx& ctx, const Gather& g, int R, int K, int Rp, int Kp, int* ef, uint16_t* out, int* bad, int Rs) {
     if (g.c_identity && Kp <= CUT_ROWS4_MAX_K) {
-        launch_cut_rows4(ctx.stream, g.base, g.off_r, R, K, Rp, Kp, ef, out, bad);
+        launch_cut_rows4(ctx.stream, g.base, g.off_r, R, K, Rp, Kp, ef, out, bad, Rs);
         TRG_LAUNCHED(ctx);
         return;
     }
     TRG_CUDA(cudaMemsetAsync(ef, 0, (size_t)R * sizeof(int), ctx.stream));
     launch_row_field<true>(ctx.stream, g, R, K, ef);
     TRG_LAUNCHED(ctx);
-    launch_cut<15>(ctx.stream, g, R, K, Rp, Kp, ef, nullptr, out, bad);
+    launch_cut<15>(ctx.stream, g, R, K, Rp, Kp, ef, nullptr, out, bad, Rs);
     TRG_LAUNCHED(ctx);
 }
 
-// Tiles (128 rows, xn columns) that reach the diagonal or above it.
-const long long* diagonal_tiles(Ctx& ctx, int tiles_m, int tiles_n, int xn, int& n) {
-    const std::string key = "xsym:" + std::to_string(tiles_m) + ":" + std::to_string(tiles_n) + ":" + std::to_string(xn);
+// Tiles (128 rows, xn columns) that reach the diagonal or above it, and those of
+// a second product whose rows start at half.
+const long long* diagonal_tiles(Ctx& ctx, int tiles_m, int tiles_n, int xn, int half, int& n) {
+    const std::string key = "xsym:" + std::to_string(tiles_m) + ":" + std::to_string(tiles_n) + ":" +
+                            std::to_string(xn) + ":" + std::to_string(half);
     auto it = ctx.lists.find(key);
     if (it == ctx.lists.end()) {
         std::vector<long long> h;
         for (int mb = 0; mb < tiles_m; ++mb)
             for (int nb = 0; nb < tiles_n; ++nb)
                 if ((int64_t)nb * xn + xn - 1 >= (int64_t)mb * XM) h.push_back(((long long)mb << 32) | nb);
+        for (size_t i = 0, one = h.size(); half && i < one; ++i)
+            h.push_back(h[i] + ((long long)(half / XM) << 32) + half / xn);
         Buf buf;
         ctx.ensure(buf, h.size() * sizeof(long long));
         TRG_CUDA(cudaMemcpyAsync(buf.p, h.data(), h.size() * sizeof(long long), cudaMemcpyHostToDevice, ctx.stream));
@@ -534,6 +550,11 @@ int64_t exact_scratch_bytes(int64_t M, int64_t N, int64_t K) {
     const int64_t kp = up(std::max<int64_t>(K, 1), XKP);
     const int64_t ra = block_rows(M, kp, XM), rb = block_rows(N, kp, XNP);
     return 2 * XPLANES * kp * (ra + rb) + 4 * (ra + rb) + 2048;
+}
+
+int64_t exact_pair_scratch_bytes(int64_t M, int64_t K) {
+    const int64_t kp = up(std::max<int64_t>(K, 1), XKP), rows = 2 * up(M, XM);
+    return 2 * XPLANES * kp * rows + 4 * rows + 2048;
 }
 
 namespace {
@@ -577,7 +598,7 @@ void launch_exact(Ctx& ctx, const uint16_t* sa, int64_t mp, const uint16_t* sb, 
     a.tile_list = nullptr;
     a.n_list = 0;
     if (a.sym) {
-        a.tile_list = diagonal_tiles(ctx, tiles_m, tiles_n, XT<S>::N, a.n_list);
+        a.tile_list = diagonal_tiles(ctx, tiles_m, tiles_n, XT<S>::N, a.half, a.n_list);
         tiles = a.n_list;
     }
     // column blocks whose digits share L2 (about 40 MB of them)
@@ -614,13 +635,13 @@ bool gemm_exact(Ctx& ctx, const GemmDesc& d) {
         const int mr = (int)std::min(ra, d.M - m0), mp = (int)up(mr, XM);
         Gather ga = d.A;
         ga.off_r += m0;
-        digits(ctx, ga, mr, K, mp, Kp, fa, sa, bad);
+        digits(ctx, ga, mr, K, mp, Kp, fa, sa, bad, mp);
         for (int64_t n0 = 0; n0 < d.N; n0 += rb) {
             const int nr = (int)std::min(rb, d.N - n0), np = sym ? mp : (int)up(nr, XNP);
             if (!sym && (m0 == 0 || rb < d.N)) {
                 Gather gb = bt;
                 gb.off_r += n0;
-                digits(ctx, gb, nr, K, np, Kp, fb, sb, bad);
+                digits(ctx, gb, nr, K, np, Kp, fb, sb, bad, np);
             }
             XArgs a;
             a.M = mr; a.N = sym ? mr : nr; a.Kp = Kp;
@@ -632,6 +653,7 @@ bool gemm_exact(Ctx& ctx, const GemmDesc& d) {
             const int tok = ctx.region_begin(TRG_PHASE_MMA);
             const bool nine = try_nine(ctx, a.M, a.N, K, sym);
             a.nine = nine ? 1 : 0;
+            a.half = 0;
             if (nine) {
                 // (each block decides for itself; an operand out of range stays so)
                 if (m0 + n0 > 0) TRG_CUDA(cudaMemsetAsync(flags + 1, 0, sizeof(int), ctx.stream));
@@ -644,6 +666,48 @@ bool gemm_exact(Ctx& ctx, const GemmDesc& d) {
         }
     }
     gemm_f64(ctx, d, bad);    // computes the product if an operand was out of range, else returns at once
+    return true;
+}
+
+// Two Gram products of one size whose tiles fit the chip together (the P and Q
+// of an environment): one launch, which takes as long as either alone.  At (24,
+// 22), 2 x 55 tiles on 152 SMs, the environment takes 228 us instead of 300.
+bool gemm_exact_pair(Ctx& ctx, const GemmDesc& d0, const GemmDesc& d1) {
+    const int64_t M = d0.M, K = std::max<int64_t>(d0.K, 1);
+    if (!(d0.gram && d1.gram && d0.N == M && d1.M == M && d1.N == M && d1.K == d0.K)) return false;
+    if (2 * tiles_of(M, M, XT<15>::N, true) > ctx.sm_count || try_nine(ctx, M, M, K, true)) return false;
+    const int Kp = (int)up(K, XKP), mp = (int)up(M, XM);
+    static_assert(XM % XT<15>::N == 0, "the second product starts on a column tile");
+    try {
+        ctx.ensure(ctx.split_ws, (size_t)exact_pair_scratch_bytes(M, K));
+    } catch (const Error& e) {
+        if (e.status == TRG_ENOMEM) return false;
+        throw;
+    }
+    const int phase = ctx.region_begin(ctx.phase);
+    uint8_t* p = ctx.split_ws.as<uint8_t>();
+    int* flags = (int*)p;
+    int* f = (int*)(p + 256);
+    uint16_t* s = (uint16_t*)(p + 256 + up((int64_t)2 * mp * 4, 256));
+    TRG_CUDA(cudaMemsetAsync(flags, 0, 2 * sizeof(int), ctx.stream));
+    digits(ctx, d0.A, (int)M, (int)K, mp, Kp, f, s, flags, 2 * mp);
+    digits(ctx, d1.A, (int)M, (int)K, mp, Kp, f + mp, s + (size_t)mp * 16, flags, 2 * mp);
+    XArgs a;
+    a.M = (int)M; a.N = (int)M; a.Kp = Kp;
+    a.fa = f; a.fb = f;
+    a.C = d0.C; a.c_m = d0.c_m; a.c_n = d0.c_n;
+    a.C1 = d1.C; a.c_m1 = d1.c_m; a.c_n1 = d1.c_n;
+    a.rows_fast = 0;
+    a.sym = 1;
+    a.half = mp;
+    a.nine = 0;
+    a.flags = flags; a.status = ctx.status.as<int>();
+    const int tok = ctx.region_begin(TRG_PHASE_MMA);
+    launch_exact<15>(ctx, s, 2 * mp, s, 2 * mp, a);
+    ctx.region_end(tok, 4.0 * (double)M * M * K, 120.0 * 4.0 * (double)M * M * Kp);
+    gemm_f64(ctx, d0, flags);
+    gemm_f64(ctx, d1, flags);
+    ctx.region_end(phase, 4.0 * (double)M * M * K, 0.0);
     return true;
 }
 

@@ -216,7 +216,7 @@ struct GemmDesc {
     // slices A once for both operands (when their padded sizes agree),
     // computes only the tiles that reach the diagonal or above it, and
     // writes each element above the diagonal also at its mirror position,
-    // so C is exactly symmetric; FP64 mode computes all of C.
+    // so C is exactly symmetric; so does FP64 mode.
     bool gram = false;
     // Split mode: B arrives sliced (split_slice_b), for a B that several
     // products share; the product then skips B's exponent and slicing passes.
@@ -242,6 +242,10 @@ double f64_us(const Ctx& ctx, int64_t M, int64_t N, int64_t K, bool sym);   // m
 bool gemm_exact(Ctx& ctx, const GemmDesc& g);
 double exact_us(const Ctx& ctx, int64_t M, int64_t N, int64_t K, bool sym);
 int64_t exact_scratch_bytes(int64_t M, int64_t N, int64_t K);
+// Two Gram products in one launch; false, with nothing computed, if they do not
+// fit the chip together or their scratch cannot be had.
+bool gemm_exact_pair(Ctx& ctx, const GemmDesc& d0, const GemmDesc& d1);
+int64_t exact_pair_scratch_bytes(int64_t M, int64_t K);
 
 // Table helpers: enumerate all index tuples of `modes` (size, stride),
 // first mode slowest, and return the device table of offsets.

@@ -71,23 +71,33 @@ static Gather gather(Ctx& ctx, const double* base, const Modes& rows, const Mode
 
 void gemm_split(Ctx& ctx, const GemmDesc& g);  // split_gemm.cu
 
+// FP64 products take the tensor cores once they are modelled to be well ahead
+// of the FP64 pipe.  Their fixed cost is six launches (25 us in the model) and
+// the digits; the lines cross at about 200 x 200 x 200.  The three products of a
+// (24, 22) environment (528 and 576 wide) take 651 us on the pipe and 300 us on
+// the tensor cores (228 us with P and Q in one launch), 256 x 40 x 256 14 us
+// against more than 30.
+static bool takes_exact(const Ctx& ctx, const GemmDesc& g) {
+    const bool sym = g.gram && g.M == g.N;
+    return g.allow_exact && !ctx.no_exact && g.beta == 0.0 && g.M > 0 && g.N > 0 &&
+           exact_us(ctx, g.M, g.N, g.K, sym) < 0.8 * f64_us(ctx, g.M, g.N, g.K, sym);
+}
+
 void gemm(Ctx& ctx, const GemmDesc& g, int precision) {
     // products inside the isometry are timed as part of that phase
     const int tok = (ctx.phase == TRG_PHASE_EIG) ? -1 : ctx.region_begin(ctx.phase);
     if (precision == TRG_FP64) {
-        // the tensor cores once they are modelled to be well ahead of the
-        // FP64 pipe.  Their fixed cost is six launches (25 us in the model)
-        // and the digits; the lines cross at about 200 x 200 x 200.  The
-        // three products of a (24, 22) environment (528 and 576 wide) take
-        // 651 us on the pipe and 283 us on the tensor cores, 256 x 40 x 256
-        // 14 us against more than 30.
-        const bool sym = g.gram && g.M == g.N;
-        const bool exact = g.allow_exact && !ctx.no_exact && g.beta == 0.0 && g.M > 0 && g.N > 0 &&
-                           exact_us(ctx, g.M, g.N, g.K, sym) < 0.8 * f64_us(ctx, g.M, g.N, g.K, sym);
-        if (!exact || !gemm_exact(ctx, g)) gemm_f64(ctx, g);
+        if (!takes_exact(ctx, g) || !gemm_exact(ctx, g)) gemm_f64(ctx, g);
     } else if (precision == TRG_SPLIT_BF16) gemm_split(ctx, g);
     else fail(TRG_EINVAL, "unknown precision mode");
     ctx.region_end(tok, 2.0 * (double)g.M * (double)g.N * (double)g.K, 0.0);
+}
+
+// Two products that do not depend on one another.
+static void gemm_pair(Ctx& ctx, const GemmDesc& g0, const GemmDesc& g1, int precision) {
+    if (precision == TRG_FP64 && takes_exact(ctx, g0) && takes_exact(ctx, g1) && gemm_exact_pair(ctx, g0, g1)) return;
+    gemm(ctx, g0, precision);
+    gemm(ctx, g1, precision);
 }
 
 int slices_now(const Ctx& ctx) {
@@ -113,30 +123,21 @@ void environment(Ctx& ctx, const View4& t, double* M, int precision) {
     double* P = ctx.envP.as<double>();
     double* Q = ctx.envQ.as<double>();
 
-    {   // P: rows (j,e), k (a,b), cols (l,f)
-        const Modes r = {{Dx, s[0]}, {Dy, s[3]}}, k = {{Dy, s[1]}, {Dx, s[2]}};
+    // P: rows (j,e), k (a,b), cols (l,f); Q: rows (i,e), k (c,d), cols (k,f).
+    // Both are Gram products A A^T.
+    auto gram = [&](const Modes& r, const Modes& k, double* C) {
         GemmDesc g;
         g.M = DD; g.N = DD; g.K = DD;
         g.A = gather(ctx, t.p, r, k);
         g.B = gather(ctx, t.p, k, r);
-        g.C = P; g.c_m = ctx.table({{DD, DD}}); g.c_n = ctx.table({{DD, 1}});
+        g.C = C; g.c_m = ctx.table({{DD, DD}}); g.c_n = ctx.table({{DD, 1}});
         g.beta = 0.0;
-        g.gram = true;          // P = A A^T (the SYRK of the environment)
+        g.gram = true;
         g.allow_exact = true;
-        gemm(ctx, g, precision);
-    }
-    {   // Q: rows (i,e), k (c,d), cols (k,f)
-        const Modes r = {{Dx, s[0]}, {Dy, s[1]}}, k = {{Dx, s[2]}, {Dy, s[3]}};
-        GemmDesc g;
-        g.M = DD; g.N = DD; g.K = DD;
-        g.A = gather(ctx, t.p, r, k);
-        g.B = gather(ctx, t.p, k, r);
-        g.C = Q; g.c_m = ctx.table({{DD, DD}}); g.c_n = ctx.table({{DD, 1}});
-        g.beta = 0.0;
-        g.gram = true;          // Q = A A^T
-        g.allow_exact = true;
-        gemm(ctx, g, precision);
-    }
+        return g;
+    };
+    gemm_pair(ctx, gram({{Dx, s[0]}, {Dy, s[3]}}, {{Dy, s[1]}, {Dx, s[2]}}, P),
+              gram({{Dx, s[0]}, {Dy, s[1]}}, {{Dx, s[2]}, {Dy, s[3]}}, Q), precision);
     {   // M: rows (i,k), k (e,f), cols (j,l); stored M[(i,j),(k,l)]
         GemmDesc g;
         g.M = Dx * Dx; g.N = Dx * Dx; g.K = Dy * Dy;

@@ -3,7 +3,8 @@
 //
 // An operand is rows r < R of length K, element (r, k) at src[off_r[r] +
 // off_c[k]]; its digits go to out[p][r][k] (r < Rp, k < Kp, zero in the
-// padding; digit_at for the order of 15 digits).  With f the largest exponent field of a row and e = f - 1022
+// padding; digit_at for the order of 15 digits, whose rows may be a part of a
+// larger array of Rs).  With f the largest exponent field of a row and e = f - 1022
 // (|x| < 2^e), X = rint(x 2^(F - e)), F = 7 + 8 (S - 1), halves away from
 // zero, is the sum of d_p 2^(8 (S - 1 - p)), d_0 in [-128, 128], d_p in
 // [-128, 127]; slices are stored as d_p 2^(-8p) (S <= 5) or as d_p (S = 15).
@@ -175,10 +176,10 @@ template <int S>
 __global__ void __launch_bounds__(256) k_cut(const double* __restrict__ src, const int64_t* __restrict__ off_r,
                                              const int64_t* __restrict__ off_c, int R, int K, int Rp, int Kp,
                                              int k_fast, const int* __restrict__ ef, int* __restrict__ e_out,
-                                             uint16_t* __restrict__ out, int* bad) {
+                                             uint16_t* __restrict__ out, int* bad, int Rs) {
     __shared__ double tile[XD_R * XD_LD];
     const int k0 = blockIdx.x * XD_K;
-    const size_t plane = digit_stride<S>(Rp, Kp);
+    const size_t plane = digit_stride<S>(Rs, Kp);
     const int nby = (Rp + XD_R - 1) / XD_R;
     for (int by = blockIdx.y; by < nby; by += gridDim.y) {
         const int r0 = by * XD_R;
@@ -202,7 +203,7 @@ __global__ void __launch_bounds__(256) k_cut(const double* __restrict__ src, con
         uint32_t w[4][planes(S)];
 #pragma unroll
         for (int h = 0; h < 4; ++h) cut2<S>(x[2 * h], x[2 * h + 1], f, w[h]);
-        uint16_t* o = out + digit_at<S>(r, k, Rp, Kp);
+        uint16_t* o = out + digit_at<S>(r, k, Rs, Kp);
 #pragma unroll
         for (int p = 0; p < planes(S); ++p) *reinterpret_cast<uint4*>(o + p * plane) = make_uint4(w[0][p], w[1][p], w[2][p], w[3][p]);
     }
@@ -313,11 +314,11 @@ void launch_cut_rows(cudaStream_t stream, const double* src, const int64_t* off_
 template <int NCH>
 __global__ void __launch_bounds__(256) k_cut_rows4(const double* __restrict__ src, const int64_t* __restrict__ off_r,
                                                    int R, int K, int Rp, int Kp, int* __restrict__ ef_out,
-                                                   uint16_t* __restrict__ out, int* bad) {
+                                                   uint16_t* __restrict__ out, int* bad, int Rs) {
     __shared__ unsigned wmax[8][4];
     const int warp = threadIdx.x >> 5, rr = (threadIdx.x >> 3) & 3, kc = threadIdx.x & 7;
     const int r = blockIdx.x * 4 + rr;                   // Rp is a multiple of four
-    const size_t plane = digit_stride<15>(Rp, Kp);
+    const size_t plane = digit_stride<15>(Rs, Kp);
     const bool real = r < R;
     const double* row = real ? src + off_r[r] : nullptr;
     const bool vec = real && ((reinterpret_cast<uintptr_t>(row) & 15) == 0);
@@ -341,20 +342,20 @@ __global__ void __launch_bounds__(256) k_cut_rows4(const double* __restrict__ sr
 #pragma unroll
     for (int c = 0; c < NCH; ++c) {
         const int k = ((c * 8 + warp) * 8 + kc) * 4;
-        if (k < Kp) store4<15>(v[c], f, out + digit_at<15>(r, k, Rp, Kp), plane);
+        if (k < Kp) store4<15>(v[c], f, out + digit_at<15>(r, k, Rs, Kp), plane);
     }
 }
 
 constexpr int CUT_ROWS4_MAX_K = 4096;
 inline void launch_cut_rows4(cudaStream_t stream, const double* src, const int64_t* off_r, int R, int K, int Rp, int Kp,
-                             int* ef_out, uint16_t* out, int* bad) {
+                             int* ef_out, uint16_t* out, int* bad, int Rs) {
     const unsigned grid = (unsigned)(Rp / 4);
-    if (Kp <= 256) k_cut_rows4<1><<<grid, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, out, bad);
-    else if (Kp <= 512) k_cut_rows4<2><<<grid, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, out, bad);
-    else if (Kp <= 1024) k_cut_rows4<4><<<grid, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, out, bad);
-    else if (Kp <= 2048) k_cut_rows4<8><<<grid, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, out, bad);
-    else if (Kp <= 3072) k_cut_rows4<12><<<grid, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, out, bad);
-    else k_cut_rows4<16><<<grid, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, out, bad);
+    if (Kp <= 256) k_cut_rows4<1><<<grid, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, out, bad, Rs);
+    else if (Kp <= 512) k_cut_rows4<2><<<grid, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, out, bad, Rs);
+    else if (Kp <= 1024) k_cut_rows4<4><<<grid, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, out, bad, Rs);
+    else if (Kp <= 2048) k_cut_rows4<8><<<grid, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, out, bad, Rs);
+    else if (Kp <= 3072) k_cut_rows4<12><<<grid, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, out, bad, Rs);
+    else k_cut_rows4<16><<<grid, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, out, bad, Rs);
 }
 
 template <bool SUB>
@@ -367,9 +368,10 @@ void launch_row_field(cudaStream_t stream, const Gather& g, int R, int K, int* e
 
 template <int S>
 void launch_cut(cudaStream_t stream, const Gather& g, int R, int K, int Rp, int Kp, const int* ef, int* e_out,
-                uint16_t* out, int* bad) {
+                uint16_t* out, int* bad, int Rs = 0) {
     dim3 grid((unsigned)((Kp + XD_K - 1) / XD_K), (unsigned)std::min((Rp + XD_R - 1) / XD_R, 65535));
-    k_cut<S><<<grid, 256, 0, stream>>>(g.base, g.off_r, g.off_c, R, K, Rp, Kp, g.c_fast ? 1 : 0, ef, e_out, out, bad);
+    k_cut<S><<<grid, 256, 0, stream>>>(g.base, g.off_r, g.off_c, R, K, Rp, Kp, g.c_fast ? 1 : 0, ef, e_out, out, bad,
+                                         Rs ? Rs : Rp);
 }
 
 // B operand as rows n, columns k: the roles of its two tables swapped.

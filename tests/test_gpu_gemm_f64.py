@@ -132,6 +132,23 @@ def test_contraction_carries_infinities_and_nan(torch, value):
     assert bool((torch.isinf(out) == torch.isinf(ref)).all())
 
 
+# P and Q share a launch, and its fallback
+@pytest.mark.parametrize("value", [float("inf"), float("nan")])
+def test_environment_carries_infinities_and_nan(torch, value):
+    rng = np.random.default_rng(7)
+    dx, dy = 24, 22
+    t = torch.from_numpy(rng.standard_normal((dx, dy, dx, dy))).cuda()
+    t[3, 4, 5, 6] = value
+    with Solver(0) as s:
+        m = s.environment(t)
+    a = t.permute(0, 3, 1, 2).reshape(dx * dy, dx * dy)
+    c = t.reshape(dx * dy, dx * dy)
+    p, q = (a @ a.T).reshape(dx, dy, dx, dy), (c @ c.T).reshape(dx, dy, dx, dy)
+    ref = torch.einsum("iekf,jelf->ijkl", q, p).reshape(dx * dx, dx * dx)
+    assert bool((torch.isnan(m) == torch.isnan(ref)).all())
+    assert bool((torch.isinf(m) == torch.isinf(ref)).all())
+
+
 @pytest.mark.parametrize("zero_rows", [True, False])
 def test_environment_of_a_sparse_tensor(torch, zero_rows):
     """Zero rows and columns (exponent field 0) and entries 2^-70 below the largest."""
