@@ -110,7 +110,7 @@ __host__ __device__ constexpr int smem_bytes_for(int S, int CG, int MODE) {
 constexpr bool smem_fits() {
     for (int S = 2; S <= 5; ++S)
         for (int CG = 1; CG <= 2; ++CG)
-            for (int MODE = 0; MODE <= 2; ++MODE)
+            for (int MODE = 0; MODE <= 3; ++MODE)
                 if (smem_bytes_for(S, CG, MODE) > SMEM_LIMIT || stages_for(S, CG, MODE) < 2) return false;
     return true;
 }
@@ -307,7 +307,8 @@ static_assert(pair_table_ok(2) && pair_table_ok(3) && pair_table_ok(4) && pair_t
 // itself.  Forming a tile's results has to take less time than one 512-deep
 // chunk of products (20k clocks a 256-row pair at S = 4): the next tile's
 // first chunk waits in the accumulators until they are formed.
-enum EpiMode { EPI_STAGED = 0, EPI_DIRECT = 1, EPI_KSPLIT = 2 };
+// EPI_SHORT: EPI_DIRECT of a product that is one run (K <= 512).
+enum EpiMode { EPI_STAGED = 0, EPI_DIRECT = 1, EPI_KSPLIT = 2, EPI_SHORT = 3 };
 
 template <int S, int CG, int MODE>
 __global__ void __launch_bounds__(THREADS, 1)
@@ -546,39 +547,69 @@ k_split_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                 const int m = row0 + row_in_tile;
                 const bool row_ok = m < g.M;
                 const int ea = (last && row_ok) ? g.ea[m] : 0;
+                if constexpr (MODE == EPI_SHORT) {
+                    // one run: each of the four sums times its weight is an
+                    // integer below 2^31, one 32-bit conversion and one wide
+                    // multiply-add each, where the general form takes six
+                    // conversions, two roundings and 64-bit shifts.
 #pragma unroll
-                for (int h = 0; h < CPT / 8; ++h) {           // 8 columns at a time
-                    const uint32_t col = (uint32_t)(colh * CPT + h * 8);
-                    uint32_t r[8];
-                    tmem_ld8(tmem + lane_base + col, r);
-                    tmem_wait_ld();
+                    for (int h = 0; h < CPT / 8; ++h) {
+                        const uint32_t col = tmem + lane_base + (uint32_t)(colh * CPT + h * 8);
+                        uint32_t r[8], q[8];
+                        tmem_ld8(col, r);
+                        tmem_ld8(col + 128, q);
+                        tmem_wait_ld();
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) J[h * 8 + j] += (long long)__float2int_rn(__uint_as_float(r[j])) << 8;
-                    tmem_ld8(tmem + lane_base + 128 + col, r);
-                    tmem_wait_ld();
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) J[h * 8 + j] += __float2int_rn(__uint_as_float(r[j]) * 256.0f);
-                    if (last) {
-                        // fold in R and R2: J becomes V = J 2^14 + rint(R 2^22) + rint(R2 2^22)
-                        // (with two slices no product lands in R, with three none in R2:
-                        // their columns are never written and read as zero here)
-                        long long rr[8];
-#pragma unroll
-                        for (int j = 0; j < 8; ++j) rr[j] = 0;
+                        for (int j = 0; j < 8; ++j)
+                            J[h * 8 + j] = (long long)__float2int_rn(__uint_as_float(r[j])) * (1ll << 22) +
+                                           (long long)__float2int_rn(__uint_as_float(q[j]) * 256.0f) * (1ll << 14);
                         if (S >= 3) {
-                            tmem_ld8(tmem + lane_base + 256 + col, r);
+                            tmem_ld8(col + 256, r);
+                            if (S >= 4) tmem_ld8(col + 384, q);
                             tmem_wait_ld();
 #pragma unroll
-                            for (int j = 0; j < 8; ++j) rr[j] = rint_f32_to_i64(__uint_as_float(r[j]) * 4194304.0f);
+                            for (int j = 0; j < 8; ++j) {
+                                int rem = __float2int_rn(__uint_as_float(r[j]) * 4194304.0f);
+                                if (S >= 4) rem += __float2int_rn(__uint_as_float(q[j]) * 4194304.0f);
+                                J[h * 8 + j] += rem;
+                            }
                         }
-                        if (S >= 4) {
-                            tmem_ld8(tmem + lane_base + 384 + col, r);
-                            tmem_wait_ld();
+                    }
+                } else {
 #pragma unroll
-                            for (int j = 0; j < 8; ++j) rr[j] += rint_f32_to_i64(__uint_as_float(r[j]) * 4194304.0f);
+                    for (int h = 0; h < CPT / 8; ++h) {           // 8 columns at a time
+                        const uint32_t col = (uint32_t)(colh * CPT + h * 8);
+                        uint32_t r[8];
+                        tmem_ld8(tmem + lane_base + col, r);
+                        tmem_wait_ld();
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) J[h * 8 + j] += (long long)__float2int_rn(__uint_as_float(r[j])) << 8;
+                        tmem_ld8(tmem + lane_base + 128 + col, r);
+                        tmem_wait_ld();
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) J[h * 8 + j] += __float2int_rn(__uint_as_float(r[j]) * 256.0f);
+                        if (last) {
+                            // fold in R and R2: J becomes V = J 2^14 + rint(R 2^22) + rint(R2 2^22)
+                            // (with two slices no product lands in R, with three none in R2:
+                            // their columns are never written and read as zero here)
+                            long long rr[8];
+#pragma unroll
+                            for (int j = 0; j < 8; ++j) rr[j] = 0;
+                            if (S >= 3) {
+                                tmem_ld8(tmem + lane_base + 256 + col, r);
+                                tmem_wait_ld();
+#pragma unroll
+                                for (int j = 0; j < 8; ++j) rr[j] = rint_f32_to_i64(__uint_as_float(r[j]) * 4194304.0f);
+                            }
+                            if (S >= 4) {
+                                tmem_ld8(tmem + lane_base + 384 + col, r);
+                                tmem_wait_ld();
+#pragma unroll
+                                for (int j = 0; j < 8; ++j) rr[j] += rint_f32_to_i64(__uint_as_float(r[j]) * 4194304.0f);
+                            }
+#pragma unroll
+                            for (int j = 0; j < 8; ++j) J[h * 8 + j] = (J[h * 8 + j] << 14) + rr[j];
                         }
-#pragma unroll
-                        for (int j = 0; j < 8; ++j) J[h * 8 + j] = (J[h * 8 + j] << 14) + rr[j];
                     }
                 }
                 // TMEM is free for the next tile before the FP64 results are
@@ -594,13 +625,11 @@ k_split_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                 ++chunk_no;
                 if (last) {
                     const int nt = nb * BN + colh * CPT;
-                    if constexpr (MODE == EPI_DIRECT) {
+                    if constexpr (MODE == EPI_DIRECT || MODE == EPI_SHORT) {
                         // rows adjacent in C: form, record and store each result in one
                         // pass (the lanes, adjacent rows, write contiguous runs).
-                        // Bound by the instructions per result where K is short: X1
-                        // at D = 64 (K = 64) takes 1.36 ms a launch (1.50 with integer
-                        // conversion and an atomic per lane), at (45, 43) 0.95 ms
-                        // where the staged form's stores, 8 bytes apart by Dx, took 1.82.
+                        // At (45, 43) X1 takes 0.95 ms a launch where the staged
+                        // form's stores, 8 bytes apart by Dx, took 1.82.
                         // The warp's 32 columns are the same for every lane: lane j
                         // loads column j's exponent, offset and consumer-row offset once
                         // and the loop takes them by shuffle, so no global load waits
@@ -615,6 +644,44 @@ k_split_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                         const bool one_row = __match_any_sync(0xffffffffu, cm0) == 0xffffffffu;
                         const int ncol = min(CPT, g.N - nt);
                         int cur = -1, cur_max = 0;
+                        if constexpr (MODE == EPI_SHORT) {
+                            // Columns of one consumer row, exponents in range
+                            // (checked afterwards; the general loop below rewrites
+                            // them otherwise): no branch between the results, so
+                            // that their conversions overlap, and the exponent is
+                            // added to the high word.  Bound by the instructions
+                            // per result.  X1 at D = 64 (K = 64): 1.46 ms a launch
+                            // in the general form, 1.26 with the conversions above,
+                            // 1.09 with the exponent added, 0.78 without branches;
+                            // D = 48 1.30 -> 0.85, D = 32 0.168 -> 0.106.  With many
+                            // chunks the products hide all of it, and the registers
+                            // it takes cost more (X2 at D = 64: 12.0 -> 12.5 ms).
+                            const int cn0 = __shfl_sync(0xffffffffu, cn_l, 0);
+                            if (__all_sync(0xffffffffu, !col_in || cn_l == cn0) && ncol > 0) {
+                                int hi_f = 0, lo_f = 2046;
+#pragma unroll
+                                for (int j = 0; j < CPT; ++j) {
+                                    const int e2 = ea + __shfl_sync(0xffffffffu, eb_l, j);
+                                    const long long co = __shfl_sync(0xffffffffu, co_l, j);
+                                    const double d = (double)J[j];
+                                    const int hi = __double2hiint(d), f = (hi >> 20) & 0x7FF;
+                                    const bool in = row_ok && j < ncol;
+                                    if (in && f) hi_f = max(hi_f, f + e2), lo_f = min(lo_f, f + e2);
+                                    if (in) cp[co] = __hiloint2double(f ? hi + (e2 << 20) : 0, __double2loint(d));
+                                }
+                                if (__all_sync(0xffffffffu, hi_f <= 2046 && lo_f >= 1)) {
+                                    if (g.cons_ef) {
+                                        if (one_row) {
+                                            const unsigned mx = __reduce_max_sync(0xffffffffu, (unsigned)hi_f);
+                                            if (lane == 0 && mx && cm0 >= 0) atomicMax(&g.cons_ef[cm0 + cn0], (int)mx);
+                                        } else if (cm0 >= 0 && hi_f) {
+                                            atomicMax(&g.cons_ef[cm0 + cn0], hi_f);
+                                        }
+                                    }
+                                    continue;
+                                }
+                            }
+                        }
                         auto record = [&]() {
                             if (one_row) {
                                 const unsigned mx = __reduce_max_sync(0xffffffffu, (unsigned)cur_max);
@@ -887,7 +954,8 @@ void launch_mma_k(Ctx& ctx, const CUtensorMap& ta, const CUtensorMap& tb, const 
 
 template <int S, int CG>
 void launch_mma(Ctx& ctx, const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& tbh, const MmaArgs& a) {
-    if (a.c_rows_fast) launch_mma_k<S, CG, EPI_DIRECT>(ctx, ta, tb, tbh, a);
+    if (a.c_rows_fast && a.Kp <= CHUNK_STAGES * BK && a.ksplit == 1) launch_mma_k<S, CG, EPI_SHORT>(ctx, ta, tb, tbh, a);
+    else if (a.c_rows_fast) launch_mma_k<S, CG, EPI_DIRECT>(ctx, ta, tb, tbh, a);
     else if (a.ksplit > 1) launch_mma_k<S, CG, EPI_KSPLIT>(ctx, ta, tb, tbh, a);
     else launch_mma_k<S, CG, EPI_STAGED>(ctx, ta, tb, tbh, a);
 }
