@@ -51,7 +51,7 @@ def parse():
                     help="bound of the contraction workspace (0 = the library default, 4 GiB: 16 values of j "
                          "per D^7 launch at Dcut 64)")
     ap.add_argument("--fused-slices", type=int, default=1, choices=[0, 1, 2],
-                    help="slice hand-over between contraction products: none (0), D^7 -> last (1), all (2)")
+                    help="accepted, without effect: the contraction's products hand over FP64")
     ap.add_argument("--mma-pairs", type=int, default=1, choices=[0, 1],
                     help="split products on CTA pairs (1) or one CTA per tile (0)")
     ap.add_argument("--shard", action="store_true",
@@ -256,10 +256,10 @@ SPLIT_MMA_TRAFFIC = {"sha256": "bb6c8ac231f7fc9b99737c0477f6b0d4aa10d3225d283afe
                      "bytes_per_launch": 1.5233e10}
 # Algorithmic bytes of one X2 launch at Dcut 64, S = 4: read the A slices
 # (S x 65536 x 4096 BF16) and the B slices (S x 4096 x 4096 BF16), write the
-# next product's A slices (S x 65536 x 4096 BF16) and row exponents.
+# FP64 result and the exponent fields of the next product's rows.
 def x2_algorithmic_bytes(slices: int, d: int = DCUT, jb: int = 16) -> float:
     rows = jb * d * d
-    return float(slices * rows * d * d * 2 + slices * d * d * d * d * 2 + slices * rows * d * d * 2 + rows * 8)
+    return float(slices * rows * d * d * 2 + slices * d * d * d * d * 2 + rows * d * d * 8 + rows * 4)
 
 
 def split_mma_traffic():
@@ -459,12 +459,13 @@ def run_native(args):
         per_launch = x2["flops"] / max(1, x2["calls"])
         t_launch = x2["ms"] / max(1, x2["calls"]) / 1e3
         achieved = per_launch / t_launch / 1e12
-        # FP64 FMA units: 2 FMA/clk/SM x 152 SMs x 2 flop x max SM clock (nominal 1.25 TF/s)
-        sm_mhz = peaks.get("sm_max_mhz", 2070.0)
-        peak = 152 * 2 * 2 * sm_mhz * 1e6 / 1e12
-        roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
-                "traffic": None, "kernel": "k_gemm_f64 (X2 = X1.t, D^7)",
-                "peak_source": "derived: 152 SMs x 2 FP64 FMA/clk x 2 flop x max SM clock"}
+        # FP64-equivalent FLOPs of the whole X2 phase (cutting included), against
+        # the tensor rate over the fewest digit products (45; 120 where the
+        # tensor's weak couplings need fifteen digits)
+        peak = peaks.get("bf16_tflops_sustained", 1713.4) / 45.0
+        roof = {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
+                "traffic": None, "kernel": "k_exact_mma (X2 = X1.t, D^7)",
+                "peak_source": "MEASURED_PEAKS.json bf16_tflops_sustained / 45 digit products"}
     else:
         # the X2 product's tensor-core launches alone (events around each launch)
         mx = ph["mma_x2"]
@@ -478,7 +479,7 @@ def run_native(args):
         alg = x2_algorithmic_bytes(args.slices)
         roof = {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                 "frac": achieved / peak, "traffic": traffic,
-                "kernel": "k_split_mma<%d,%d,EPI_FUSED> (X2 = X1.t, the D^7 product%s)" % (
+                "kernel": "k_split_mma<%d,%d,EPI_DIRECT> (X2 = X1.t, the D^7 product%s)" % (
                     args.slices, 2 if args.mma_pairs else 1, ", CTA pairs" if args.mma_pairs else ""),
                 "launches_per_step": mx["calls"] / steps, "ms_per_launch": t_launch * 1e3,
                 "fp64_equiv_tflops": mx["flops"] / calls / t_launch / 1e12 if t_launch > 0 else 0.0,
