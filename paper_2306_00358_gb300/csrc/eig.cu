@@ -672,6 +672,8 @@ __global__ void __launch_bounds__(256) k_lowdin(const double* P, const double* P
     }
 }
 
+__device__ __forceinline__ double rank_key(double x) { return isnan(x) ? -INFINITY : x; }
+
 // Step 3 of the Rayleigh-Ritz solve: H = (G + G^T) / 2, FP64 sweeps from
 // W = Win (accumulated in shared memory), then theta and W sorted by
 // descending theta (ties keep index order) into Wout (may alias Win).
@@ -697,12 +699,14 @@ __global__ void __launch_bounds__(512) k_rr_fp64(const double* G, int m, double 
     // (skipped for a rough Rayleigh-Ritz far from convergence: then theta is
     // the diagonal of H' and W the re-orthonormalised W32)
     const int s64 = fp64_sweeps ? jacobi_sweeps<double>(H, ld, Ws, m, tol, max_sweeps, cs64, rot, pq) : 0;
-    // rank of each diagonal value, descending; ties by index
+    // rank of each diagonal value, descending; ties by index.  A NaN ranks as
+    // -infinity: compared as it is, it would share its rank with others and
+    // leave entries of perm unwritten, which are indices below.
     for (int i = threadIdx.x; i < m; i += blockDim.x) {
-        const double hi = H[i * ld + i];
+        const double hi = rank_key(H[i * ld + i]);
         int r = 0;
         for (int j = 0; j < m; ++j) {
-            const double hj = H[j * ld + j];
+            const double hj = rank_key(H[j * ld + j]);
             r += (hj > hi || (hj == hi && j < i)) ? 1 : 0;
         }
         perm[r] = i;
