@@ -140,13 +140,14 @@ int trg_set_stream(trg_ctx* ctx, void* stream);
  * called before the first allocation (right after trg_create). */
 int trg_set_allocator(trg_ctx* ctx, trg_alloc_fn alloc, trg_free_fn free_fn, void* user);
 
-/* Limit, in ns, of one bounded device wait of the split products: the
- * epilogue's wait for a finished accumulator chunk (0 = the default, 2 s).
- * Every other wait keeps its 2 s limit.  When a wait runs out, the kernel
- * records a timeout, stops issuing, waits (bounded) for its own copies and
- * tensor-core work in flight, frees its tensor memory and returns; the call
- * that launched it returns TRG_ETIMEOUT (trg_gemm clears the flag at its
- * next call).  A limit below the time of one 512-deep chunk of products
+/* Limit, in ns, of one bounded device wait of the tensor-core products (split
+ * ones, and the digit products of TRG_FP64): the epilogue's wait for finished
+ * accumulators (0 = the default, 2 s).  Every other wait keeps its 2 s limit.
+ * When a wait runs out, the kernel records a timeout, stops issuing, waits
+ * (bounded) for its own copies and tensor-core work in flight, frees its tensor
+ * memory and returns; the call that launched it returns TRG_ETIMEOUT and clears
+ * the record.  Outputs are then undefined, and a half-step that timed out has
+ * not been taken.  A limit below the time of one run of products
  * (microseconds) makes that path run; it exists for tests of it. */
 int trg_set_wait_limit(trg_ctx* ctx, uint64_t acc_wait_ns);
 

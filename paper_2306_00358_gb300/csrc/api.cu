@@ -180,6 +180,7 @@ static void half_step_finish(Ctx& ctx, HalfPlan& p) {
         ctx.region_end(tok, 0.0, 0.0);
     }
     const int st = read_status(ctx);
+    check_timeout(ctx, st);
     if (st & ST_BAD_NORM) fail(TRG_ENUMERIC, "non-positive or non-finite norm at half-step " + std::to_string(p.k));
     std::swap(ctx.T, ctx.Tnext);
     if (ctx.have_impure) std::swap(ctx.Timp, ctx.Timp_next);
@@ -244,8 +245,7 @@ using trg::Error;
 #define TRG_GUARD_END(ctxp)                                                      \
     }                                                                            \
     catch (const Error& e) {                                                     \
-        if (ctxp) (ctxp)->last_error = e.msg;                                    \
-        return e.status;                                                         \
+        return report(ctxp, e);                                                  \
     }                                                                            \
     catch (const std::bad_alloc&) {                                              \
         if (ctxp) (ctxp)->last_error = "host allocation failed";                \
@@ -255,6 +255,28 @@ using trg::Error;
         if (ctxp) (ctxp)->last_error = e.what();                                 \
         return TRG_ECUDA;                                                        \
     }
+
+// What a call that failed with e returns.  A product whose wait ran out leaves
+// numbers that fail the checks after it: the timeout is then the cause.
+static int report(trg_ctx* ctx, const Error& e) {
+    if (!ctx) return e.status;
+    ctx->last_error = e.msg;
+    if (e.status == TRG_ETIMEOUT) return e.status;
+    try {
+        trg::check_timeout(*ctx, trg::read_status(*ctx));
+    } catch (const Error& t) {
+        if (t.status == TRG_ETIMEOUT && e.status == TRG_ENUMERIC) {
+            ctx->last_error = t.msg;
+            return t.status;
+        }
+    }
+    return e.status;
+}
+
+// A component call's own status: cleared before its first product, read after
+// its last one.
+static void begin_component(Ctx& ctx) { TRG_CUDA(cudaMemsetAsync(ctx.status.p, 0, sizeof(int), ctx.stream)); }
+static void end_component(Ctx& ctx) { trg::check_timeout(ctx, trg::read_status(ctx)); }
 
 static int bad(trg_ctx* ctx, int status, const char* msg) {
     if (ctx) ctx->last_error = msg;
@@ -554,6 +576,8 @@ int trg_shard_begin(trg_ctx* ctx, int Dcut, int j_begin, int j_end, double* slab
         o.s[0] = dn * ry; o.s[1] = dn * dn * ry; o.s[2] = ry; o.s[3] = 1;
         trg::contract(*ctx, p.r, p.r, ctx->U.as<double>(), dn, o, p.precision, j_begin, j_end, j_begin);
     }
+    // the slab goes to the other ranks: a timeout is this call's to report
+    trg::check_timeout(*ctx, trg::read_status(*ctx));
     ctx->shard = std::move(p);
     ctx->shard_pending = true;
     *dn_out = (int)dn;
@@ -636,7 +660,9 @@ int trg_solve3d(trg_ctx* ctx, int model, double beta, double h, int Dcut, int ns
         const int64_t kx = kept.first, ky = kept.second;
         c.phase = TRG_PHASE_NORM;
         trg::launch_normalise(c, c.Tnext.as<double>(), kx * kx * ky * ky * Dz * Dz, k, false);
-        if (trg::read_status(c) & trg::ST_BAD_NORM)
+        const int st = trg::read_status(c);
+        trg::check_timeout(c, st);
+        if (st & trg::ST_BAD_NORM)
             return bad(ctx, TRG_ENUMERIC, ("non-positive or non-finite norm at step " + std::to_string(k)).c_str());
         std::swap(c.T, c.Tnext);
         // the next axis to block into the z slot: a rotation of the view
@@ -704,8 +730,9 @@ int trg_environment(trg_ctx* ctx, const double* t_dev, int Dx, int Dy, double* M
     TRG_CUDA(cudaSetDevice(ctx->device));
     trg::View4 t = trg::contiguous_view(const_cast<double*>(t_dev), Dx, Dy, Dx, Dy);
     ctx->phase = TRG_PHASE_ENV;
+    begin_component(*ctx);
     trg::environment(*ctx, t, M_dev, ctx->cfg.precision);
-    TRG_CUDA(cudaStreamSynchronize(ctx->stream));
+    end_component(*ctx);
     return TRG_OK;
     TRG_GUARD_END(ctx)
 }
@@ -716,6 +743,7 @@ int trg_isometry(trg_ctx* ctx, const double* M_dev, int n, int Dcut, double* U_d
     TRG_GUARD_BEGIN
     TRG_CUDA(cudaSetDevice(ctx->device));
     const int dn_max = std::min(n, Dcut);
+    begin_component(*ctx);
     if (dn_max == n) {
         trg::launch_identity(*ctx, U_dev, n);
         *dn_out = n;
@@ -727,7 +755,7 @@ int trg_isometry(trg_ctx* ctx, const double* M_dev, int n, int Dcut, double* U_d
         *dn_out = dn;
         if (lam_host) std::memcpy(lam_host, lam.data(), sizeof(double) * (size_t)dn);
     }
-    TRG_CUDA(cudaStreamSynchronize(ctx->stream));
+    TRG_CUDA(cudaStreamSynchronize(ctx->stream));   // (the isometry has read the status after its last product)
     return TRG_OK;
     TRG_GUARD_END(ctx)
 }
@@ -741,8 +769,9 @@ int trg_contract(trg_ctx* ctx, const double* t_dev, const double* U_dev, int Dx,
     trg::View4 t = trg::contiguous_view(const_cast<double*>(t_dev), Dx, Dy, Dx, Dy);
     trg::View4 o = trg::contiguous_view(Tx_dev, Dn, Dy, Dn, Dy);
     ctx->phase = TRG_PHASE_X1;
+    begin_component(*ctx);
     trg::contract(*ctx, t, t, U_dev, Dn, o, ctx->cfg.precision);
-    TRG_CUDA(cudaStreamSynchronize(ctx->stream));
+    end_component(*ctx);
     return TRG_OK;
     TRG_GUARD_END(ctx)
 }
@@ -761,11 +790,9 @@ int trg_gemm(trg_ctx* ctx, int M, int N, int K, const double* A, int lda, const 
     g.B.base = B; g.B.off_r = ctx->table({{K, ldb}}); g.B.off_c = ctx->table({{N, 1}}); g.B.c_fast = true;
     g.C = C; g.c_m = ctx->table({{M, ldc}}); g.c_n = ctx->table({{N, 1}}); g.beta = 0.0;
     ctx->phase = TRG_PHASE_X2;
-    // a status left by an earlier call is not this product's
-    TRG_CUDA(cudaMemsetAsync(ctx->status.p, 0, sizeof(int), ctx->stream));
+    begin_component(*ctx);
     trg::gemm(*ctx, g, ctx->cfg.precision);
-    TRG_CUDA(cudaStreamSynchronize(ctx->stream));
-    if (trg::read_status(*ctx) & trg::ST_TIMEOUT) return bad(ctx, TRG_ETIMEOUT, "gemm: device wait timed out");
+    end_component(*ctx);
     return TRG_OK;
     TRG_GUARD_END(ctx)
 }

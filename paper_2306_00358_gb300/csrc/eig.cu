@@ -1121,6 +1121,7 @@ int isometry(Ctx& ctx, const double* M, int64_t n, int dcut, double* U, std::vec
         ctx.counters[1] += 1;
         ctx.counters[2] += (uint64_t)hsw[0];
         ctx.counters[3] += (uint64_t)hsw[1];
+        check_timeout(ctx, st);
         if (st & ST_EIG_NOCONV) fail(TRG_ENUMERIC, "Rayleigh-Ritz Jacobi did not converge");
         if (!(th[0] > 0.0) || !std::isfinite(th[0])) fail(TRG_ENUMERIC, "environment has no positive eigenvalue");
         if ((res <= tol && full) || m == n) {

@@ -151,6 +151,7 @@ struct XArgs {
     const int64_t* c_m1;
     const int64_t* c_n1;
     int* status;
+    unsigned long long acc_wait_ns;   // limit of the epilogue's waits (trg_set_wait_limit)
 };
 
 // The int64 sums of an element, each in units of its last D, as FP64 times
@@ -338,7 +339,7 @@ k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             if constexpr (S == 1) {
                 // the sums of |a||b|: is any of them small?
                 int w_ok = 1;
-                if (lane == 0) w_ok = mbar_wait(&acc_full[1], run_no & 1, abort_flag, g.status) ? 1 : 0;
+                if (lane == 0) w_ok = mbar_wait(&acc_full[1], run_no & 1, abort_flag, g.status, g.acc_wait_ns) ? 1 : 0;
                 ok = __shfl_sync(0xffffffffu, w_ok, 0) != 0;
                 if (!ok) break;
                 tc_fence_after();
@@ -367,7 +368,7 @@ k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
 #pragma unroll
                 for (int grp = 1; grp >= 0; --grp) {
                     int w_ok = 1;
-                    if (lane == 0) w_ok = mbar_wait(&acc_full[grp], run_no & 1, abort_flag, g.status) ? 1 : 0;
+                    if (lane == 0) w_ok = mbar_wait(&acc_full[grp], run_no & 1, abort_flag, g.status, g.acc_wait_ns) ? 1 : 0;
                     ok = __shfl_sync(0xffffffffu, w_ok, 0) != 0;
                     if (!ok) break;
                     tc_fence_after();
@@ -594,6 +595,7 @@ void launch_exact(Ctx& ctx, const uint16_t* sa, int64_t mp, const uint16_t* sb, 
     const CUtensorMap tb = digit_map(sb, first, S, np, a.Kp, XT<S>::N, XT<S>::K);
     const int tiles_m = (a.M + XM - 1) / XM, tiles_n = (a.N + XT<S>::N - 1) / XT<S>::N;
     int tiles = tiles_m * tiles_n;
+    a.acc_wait_ns = ctx.acc_wait_ns ? ctx.acc_wait_ns : WAIT_NS;
     a.tile_list = nullptr;
     a.n_list = 0;
     if (a.sym) {

@@ -78,8 +78,8 @@ struct Ctx {
     void* alloc_user = nullptr;
     std::string last_error;
     uint64_t launches = 0;
-    // split products: limit of the epilogue's wait for a finished accumulator
-    // chunk in ns (0 = the kernel's default of 2 s); see trg_set_wait_limit
+    // tensor-core products: limit of the epilogue's wait for finished accumulators
+    // in ns (0 = the kernels' default of 2 s); see trg_set_wait_limit
     unsigned long long acc_wait_ns = 0;
     bool no_exact = false;   // FP64 products stay on the FP64 pipe (no room for their digits)
 
@@ -299,6 +299,9 @@ std::pair<int64_t, int64_t> step3(Ctx& ctx, const View6& t, int dcut, int step, 
                                   std::vector<double>& lam_x, std::vector<double>& lam_y);
 
 int read_status(Ctx& ctx);  // synchronises the stream
+// Throws TRG_ETIMEOUT, with the status word cleared for the next call, if the
+// status st that was read says that a bounded device wait ran out.
+void check_timeout(Ctx& ctx, int st);
 void trim_buffers(Ctx& ctx);  // free every solve buffer (engine.cu)
 
 }  // namespace trg

@@ -341,4 +341,10 @@ int read_status(Ctx& ctx) {
     return st;
 }
 
+void check_timeout(Ctx& ctx, int st) {
+    if (!(st & ST_TIMEOUT)) return;
+    TRG_CUDA(cudaMemsetAsync(ctx.status.p, 0, sizeof(int), ctx.stream));
+    fail(TRG_ETIMEOUT, "device wait timed out");
+}
+
 }  // namespace trg

@@ -108,7 +108,7 @@ class Solver:
         self._check(self._lib.trg_set_stream(self._h, ctypes.c_void_p(raw)), "trg_set_stream")
 
     def set_wait_limit(self, acc_wait_ns: int = 0):
-        """Limit of the split products' accumulator wait (0 = 2 s); see trg_set_wait_limit."""
+        """Limit of the tensor-core products' accumulator wait (0 = 2 s); see trg_set_wait_limit."""
         self._check(self._lib.trg_set_wait_limit(self._h, int(acc_wait_ns)), "trg_set_wait_limit")
 
     def set_precision(self, precision, split_slices: int = 4, split_from_step: int = 0):
