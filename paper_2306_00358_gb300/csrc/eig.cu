@@ -16,7 +16,6 @@
 #include <chrono>
 #include <cmath>
 #include <cstring>
-#include <mutex>
 
 #include "internal.h"
 #include "jacobi32.cuh"
@@ -836,10 +835,11 @@ static void gram(Ctx& ctx, const double* A, const double* B, int64_t n, int m, d
     const int nparts = (int)((n + rows_c - 1) / rows_c);
     ctx.ensure(ctx.f64_partial, (size_t)nparts * m * m * sizeof(double));
     const size_t smem = (size_t)rows_c * m * 2 * sizeof(double);
-    static std::once_flag once;
-    std::call_once(once, [] {
+    static PerDevice prepared;
+    prepared.get(ctx.device, [] {
         TRG_CUDA(cudaFuncSetAttribute((const void*)k_gram_partial, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       100 * 1024));
+        return 0;
     });
     launch_chained_if(chain_wide(ctx, n), ctx, k_gram_partial, nparts, 256, smem, A, B, n, m, rows_c, ctx.f64_partial.as<double>(), A == B ? 1 : 0);
     TRG_LAUNCHED(ctx);
@@ -903,13 +903,14 @@ int isometry(Ctx& ctx, const double* M, int64_t n, int dcut, double* U, std::vec
     if (dn_paper >= MAX_M && dn_paper < n)
         fail(TRG_ENOTSUP, "isometry: Dcut above the supported block (111 kept vectors)");
     const int m = (int)std::min<int64_t>({n, (int64_t)dn_paper + std::max(1, ctx.cfg.oversample), (int64_t)MAX_M});
-    static std::once_flag once;
-    std::call_once(once, [] {
+    static PerDevice prepared;
+    prepared.get(ctx.device, [] {
         set_smem((const void*)k_chol_trsm<8>, chol_smem(MAX_M, 8));
         set_smem((const void*)k_chol_trsm<16>, chol_smem(MAX_M, 16));
         set_smem((const void*)k_chol_trsm<32>, chol_smem(MAX_M, 32));
         set_smem((const void*)k_rr_fp32, std::max(rr32_smem(MAX_M), rr32_smem(JAC_PIPE_M)));
         set_smem((const void*)k_rr_fp64, rr64_smem(MAX_M));
+        return 0;
     });
     // buffers: Q, Y, Z, QW (n x m each); G, L, W (m x m); theta (m)
     ctx.ensure(ctx.eig, (size_t)(4 * n * m) * sizeof(double));

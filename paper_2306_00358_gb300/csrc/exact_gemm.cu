@@ -587,9 +587,10 @@ namespace {
 template <int S>
 void launch_exact(Ctx& ctx, const uint16_t* sa, int64_t mp, const uint16_t* sb, int64_t np, XArgs a) {
     constexpr int first = S == 1 ? 15 : 0;
-    static std::once_flag once;
-    std::call_once(once, [] {
+    static PerDevice prepared;
+    prepared.get(ctx.device, [] {
         TRG_CUDA(cudaFuncSetAttribute(k_exact_mma<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, XT<S>::SMEM));
+        return 0;
     });
     const CUtensorMap ta = digit_map(sa, first, S, mp, a.Kp, XM, XT<S>::K);
     const CUtensorMap tb = digit_map(sb, first, S, np, a.Kp, XT<S>::N, XT<S>::K);

@@ -9,6 +9,7 @@
 #include <utility>
 #include <vector>
 
+#include "per_device.h"
 #include "trg.h"
 
 namespace trg {

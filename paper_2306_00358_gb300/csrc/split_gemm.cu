@@ -896,9 +896,9 @@ template <int S, int CG, int MODE>
 void launch_mma_k(Ctx& ctx, const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& tbh,
                   const MmaArgs& a0) {
     MmaArgs a = a0;
-    static std::once_flag once;
-    static int max_clusters = 0;
-    std::call_once(once, [&ctx] {
+    static PerDevice prepared;
+    const int max_clusters = prepared.get(ctx.device, [&ctx] {
+        int pairs = 0;
         TRG_CUDA(cudaFuncSetAttribute(k_split_mma<S, CG, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       smem_bytes_for(S, CG, MODE)));
         if (CG == 2) {
@@ -912,8 +912,9 @@ void launch_mma_k(Ctx& ctx, const CUtensorMap& ta, const CUtensorMap& tb, const 
             cfg.dynamicSmemBytes = smem_bytes_for(S, CG, MODE);
             cfg.attrs = attr;
             cfg.numAttrs = 1;
-            TRG_CUDA(cudaOccupancyMaxActiveClusters(&max_clusters, k_split_mma<S, CG, MODE>, &cfg));
+            TRG_CUDA(cudaOccupancyMaxActiveClusters(&pairs, k_split_mma<S, CG, MODE>, &cfg));
         }
+        return pairs;
     });
     const int tiles_m = (a.M + BM * CG - 1) / (BM * CG), tiles_n = (a.N + BN - 1) / BN;
     const int tiles = (a.tile_list ? a.n_list : tiles_m * tiles_n) * a.ksplit;   // units of work
