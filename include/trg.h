@@ -58,10 +58,12 @@ typedef enum trg_precision {
     TRG_FP64 = 0,        /* FP64.  trg_gemm runs on the FP64 pipe.  The products of a solve and of
                             the component calls do too while they are small; larger ones are
                             computed from exact BF16 digit products on the tensor cores and
-                            brought to FP64, off by at most 2^-51 |C| + 16 K 2^-118 times the
-                            largest entries of the row and the column (an FP64 sum of K products
-                            is off by up to K 2^-53 |A||B|).  Operands with infinities, NaN or
-                            rows outside 2^-400 .. 2^400 stay on the FP64 pipe. */
+                            brought to FP64, off by at most 2^-51 |C| + K 2^-55 |A||B| element by
+                            element (an FP64 sum of K products is off by up to K 2^-53 |A||B|).
+                            Elements that the digits do not reach, with |A||B| below 2^-60 of the
+                            largest entries of their row and column, or in a row or column with
+                            infinities, NaN or its largest entry outside 2^-400 .. 2^400, are
+                            computed on the FP64 pipe. */
     TRG_SPLIT_BF16 = 1   /* FP64 operands cut into BF16 slices, exact FP32
                             partial sums on tcgen05 tensor cores, summed wide */
 } trg_precision;

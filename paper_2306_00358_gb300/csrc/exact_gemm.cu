@@ -17,29 +17,35 @@
 // How many digits: S leave out less than (S + 2) K 2^(-8 S) 2^(ea + eb).  The
 // result has to be as accurate as an FP64 sum element by element, relative to
 // its own sum |a||b| (the method feeds the couplings between nearly decoupled
-// sectors of a tensor back, so small elements count):
-//  - 15 digits do that down to sums |a||b| of 2^-60 2^(ea + eb) (120 digit
-//    products); products too small for a choice always take them;
-//  - 9 digits (45 digit products) do if no sum |a||b| lies between 0 and 2^-8
+// sectors of a tensor back, so small elements count).  So every form comes with
+// that sum, taken from one more BF16 plane of each operand, |x| cut off:
+//  - 15 digits (120 digit products) do it down to sums |a||b| of 2^-60 2^(ea +
+//    eb): they leave out less than K 2^-55 |a||b|, where an FP64 sum's roundings
+//    amount to up to K 2^-53 |a||b|; products too small for a choice always take
+//    them.  The sum is one more accumulator of the same kernel, which marks the
+//    elements below 2^-60, and those of rows or columns whose largest entry lies
+//    outside 2^-400 .. 2^400 or that hold an infinity or a NaN.  A kernel queued
+//    behind it computes the marked elements on the FP64 pipe (k_weak_f64; it
+//    returns at once if there is none).  In FP64 solves at the critical point no
+//    sum lies below 2^-54; far from it, once the tensor has flowed to a fixed
+//    point, 2 to 40 % of them do;
+//  - 9 digits (45 digit products) do it if no sum |a||b| lies between 0 and 2^-8
 //    2^(ea + eb): they leave out less than K 2^-60 |a||b| then, which is also
 //    below what the roundings of an FP64 sum amount to when their signs are
-//    random.  A kernel takes |A||B| from one BF16 plane of each operand and
-//    raises a flag where 9 do not suffice; the two product kernels read it,
-//    and the one that is not wanted returns at once.
-// Rows or columns whose largest entry lies outside 2^-400 .. 2^400, or that hold
-// an infinity or a NaN, raise another flag: then the FP64 pipe kernel that is
-// queued last, idle otherwise, computes the product.
+//    random.  A kernel takes all of |A||B| first and raises a flag where 9 do
+//    not suffice; the two product kernels read it, and the one that is not
+//    wanted returns at once.
 //
 // What bounds it: the tensor pipe (9 digits in a long product: active 62 % of
 // the time, with MMA instructions of N = 48 .. 240; a tenth goes to drains that
 // nothing covers).  128 x 32 output tile with 15 digits, 128 x 48 with 9, one
-// persistent CTA per SM: the S accumulators D_d of the tile's columns fill
-// tensor memory.  A stage is 16 (32) K of both operands, one TMA box each, two
+// persistent CTA per SM: the S accumulators D_d of the tile's columns (and with 15
+// digits the sums) fill tensor memory.  A stage is 16 (32) K of both operands, one TMA box each, two
 // stages; the cut stores the digits in the order of a stage, so that a box is
 // made of 4 KB pieces (as [p][r][k] planes its rows are pieces of 32 or 64
 // bytes, and the TMA unit's requests hold the products up: 72 -> 68.6 us a
-// product of an environment at (24, 22)).  The products of one A digit with
-// adjacent B digits land in adjacent accumulators, so 23 (13) instructions of up
+// product of an environment at (24, 22), without the sums).  The products of one A digit with
+// adjacent B digits land in adjacent accumulators, so 24 (13) instructions of up
 // to N = 256 cover the products of a 16-deep step.  They are issued in two
 // groups, the one that lands in the higher D_d (84 of 120, 35 of 45 products)
 // before the other: a run's drain of the higher D_d runs under the other group's
@@ -74,7 +80,11 @@ struct XT {
     static constexpr int THREADS = 64 + 32 * EPI;
     static constexpr int KB = K / 16;
     static constexpr int A_TILE = XM * 32, B_TILE = N * 32;        // bytes of 16 K of one digit's tiles
-    static constexpr int STAGE = KB * S * (A_TILE + B_TILE);       // 75, 99 and 24 KB
+    // 15 digits come with the |x| plane: its product, the sum of |a||b|, has
+    // accumulators of its own (SUM) and runs over the whole K
+    static constexpr bool SUM = S == 15;
+    static constexpr int P = S + (SUM ? 1 : 0);                    // planes staged
+    static constexpr int STAGE = KB * P * (A_TILE + B_TILE);       // 80, 99 and 24 KB
     static constexpr int STAGES = S == 1 ? 4 : 2;
     static constexpr int RUN = S == 1 ? 1 << 30 : S == 9 ? 3 : 4;  // stages of an exact run
     static constexpr int CPT = N / (EPI / 4);                      // columns per epilogue thread
@@ -84,7 +94,7 @@ struct XT {
     static constexpr int BYTES = STAGES * STAGE + STAGING + XBAR + 1024;
     static constexpr int SMEM = BYTES > 120 * 1024 ? BYTES : 120 * 1024;
     static_assert(SMEM <= 232448, "exact product shared memory");
-    static_assert(S * N <= 512 && (S == 1 || (double)S * RUN * K * (1 << 14) <= (1 << 24)), "accumulators");
+    static_assert(P * N <= 512 && (S == 1 || (double)S * RUN * K * (1 << 14) <= (1 << 24)), "accumulators");
 };
 
 // The digit products of one 16-deep step: A digit a times the n B digits from
@@ -142,7 +152,10 @@ struct XArgs {
     const long long* tile_list;    // mb << 32 | nb, or nullptr for all
     int n_list;
     int group_n;                   // tile order: column blocks per group
-    int* flags;                    // [0] an operand is outside the digits' range, [1] nine digits do not suffice
+    int* flags;                    // [0] some element is left to the FP64 pipe, [1] nine digits do not suffice
+    uint32_t* weak;                // the elements left to it: bit n % 32 of weak[(n / 32) weak_rows + m]
+    int* weak_tile;                // ... does the 128 x 32 tile (m / 128) words + n / 32 hold one
+    int weak_rows, words;
     int nine;                      // the nine-digit form has been tried
     // a second Gram product of the same size: its rows are those from half on
     // (0: none), its tiles are in tile_list too
@@ -187,14 +200,25 @@ __device__ __forceinline__ void tmem_arrived(uint32_t (&r)[N]) {
 
 constexpr int XNINE_K = 16384;                    // the nine-digit sums fit in int64 up to this K
 static_assert(5.0 * XNINE_K * (1 << 14) * 4294967296.0 * 1.01 < 9.2e18, "nine-digit sums");
-constexpr float SUM_MIN = 0.00390625f;           // 2^-8
+// Sums |a||b| as the |x| planes give them, at which 9 and 15 digits suffice: 2^-8
+// and 2^-60 of 2^(ea + eb).
+constexpr float two_to(int e) { return e == 0 ? 1.0f : e > 0 ? 2.0f * two_to(e - 1) : 0.5f * two_to(e + 1); }
+constexpr float SUM9_MIN = two_to(2 * SIZE_SHIFT - 8), SUM15_MIN = two_to(2 * SIZE_SHIFT - 60);
+__device__ __forceinline__ bool sum_below(uint32_t bits, float least) {
+    const float s = __uint_as_float(bits);
+    return s > 0.0f && s < least;
+}
+// Largest exponent field of a row that the digits do not reach (2^-400 .. 2^400,
+// infinities and NaN).
+__device__ __forceinline__ bool field_outside(int f) { return f && (f < 1023 - 400 || f > 1023 + 400); }
 
 template <int S>
 __global__ void __launch_bounds__(XT<S>::THREADS, 1)
 k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const XArgs g) {
     constexpr int XN = XT<S>::N, XK = XT<S>::K, XL = XT<S>::L, XSTAGES = XT<S>::STAGES, XSTAGE = XT<S>::STAGE;
     constexpr int XA_TILE = XT<S>::A_TILE, XKB = XT<S>::KB, XB_TILE = XT<S>::B_TILE, XRUN = XT<S>::RUN, XCPT = XT<S>::CPT;
-    if (g.flags[0] || (S == 9 && g.flags[1]) || (S == 15 && g.nine && !g.flags[1])) return;
+    if ((S == 9 && g.flags[1]) || (S == 15 && g.nine && !g.flags[1])) return;
+    constexpr int XP = XT<S>::P;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint64_t* full = (uint64_t*)(smem + XSTAGES * XSTAGE + XT<S>::STAGING);
@@ -259,7 +283,7 @@ k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                     uint8_t* st = smem + stage * XSTAGE;
                     mbar_expect_tx(&full[stage], XSTAGE);
                     tma_load_4d(st, &tmA, 0, mb * (XM / 4), 0, kb * XKB, &full[stage]);
-                    tma_load_4d(st + XKB * S * XA_TILE, &tmB, 0, nb * (XN / 4), 0, kb * XKB, &full[stage]);
+                    tma_load_4d(st + XKB * XP * XA_TILE, &tmB, 0, nb * (XN / 4), 0, kb * XKB, &full[stage]);
 #pragma unroll
                     for (int s = 0; s < XSTAGES; ++s)
                         if (s == stage) issued[s] = (int)phase;
@@ -294,12 +318,16 @@ k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                                 const XIns in = xins<S>(t);
                                 if (in.group != group) continue;
                                 const uint32_t acc = ((t == 0 || t == S) && run_start && kk == 0) ? 0u : 1u;
-                                const uint64_t da = dbase + (uint64_t)(((kk * S + in.a) * XA_TILE) >> 4);
+                                const uint64_t da = dbase + (uint64_t)(((kk * XP + in.a) * XA_TILE) >> 4);
                                 const uint64_t db =
-                                    dbase + (uint64_t)((XKB * S * XA_TILE + (kk * S + in.b) * XB_TILE) >> 4);
+                                    dbase + (uint64_t)((XKB * XP * XA_TILE + (kk * XP + in.b) * XB_TILE) >> 4);
                                 mma_bf16<1>(tmem + (uint32_t)((in.a + in.b) * XN), da, db, idesc_bf16(XM, in.n * XN),
                                             acc);
                             }
+                            if (XT<S>::SUM && group == 1)
+                                mma_bf16<1>(tmem + (uint32_t)(S * XN), dbase + (uint64_t)(((kk * XP + S) * XA_TILE) >> 4),
+                                            dbase + (uint64_t)((XKB * XP * XA_TILE + (kk * XP + S) * XB_TILE) >> 4),
+                                            idesc_bf16(XM, XN), (kb == 0 && kk == 0) ? 0u : 1u);
                         }
                     };
                     if (run_start && run_no > 0) {
@@ -337,13 +365,19 @@ k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             int mb, nb;
             coords(tile, mb, nb);
             if constexpr (S == 1) {
-                // the sums of |a||b|: is any of them small?
+                // the sums of |a||b|: is any of them small, or outside the digits' range?
                 int w_ok = 1;
                 if (lane == 0) w_ok = mbar_wait(&acc_full[1], run_no & 1, abort_flag, g.status, g.acc_wait_ns) ? 1 : 0;
                 ok = __shfl_sync(0xffffffffu, w_ok, 0) != 0;
                 if (!ok) break;
                 tc_fence_after();
-                bool small = false;
+                const int row = mb * XM + quad * 32 + lane;
+                bool small = row < g.M && field_outside(g.fa[row]);
+#pragma unroll
+                for (int h = 0; h < XCPT / 32; ++h) {
+                    const int col = nb * XN + colq * XCPT + h * 32 + lane;
+                    small |= col < g.N && field_outside(g.fb[col]);
+                }
 #pragma unroll
                 for (int h = 0; h < XCPT / 8; ++h) {
                     uint32_t r[8];
@@ -351,7 +385,7 @@ k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                     tmem_wait_ld();
                     tmem_arrived(r);
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) small |= __uint_as_float(r[j]) > 0.0f && __uint_as_float(r[j]) < SUM_MIN;
+                    for (int j = 0; j < 8; ++j) small |= sum_below(r[j], SUM9_MIN);
                 }
                 tc_fence_before();
                 if (__any_sync(0xffffffffu, small) && lane == 0) g.flags[1] = 1;
@@ -364,6 +398,7 @@ k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             for (int j = 0; j < XCPT; ++j)
 #pragma unroll
                 for (int q = 0; q < XT<S>::LIMBS; ++q) w[j][q] = 0;
+            unsigned weak = 0;      // columns of this thread's row that 15 digits do not suffice for
             for (int c = 0; c < nruns && ok; ++c, ++run_no) {
 #pragma unroll
                 for (int grp = 1; grp >= 0; --grp) {
@@ -396,6 +431,16 @@ k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                                 w[j][q] += (long long)x * (1ll << (8 * (last - d))) + (long long)y * (1ll << (8 * (last - d - 1)));
                         }
                     }
+                    if constexpr (XT<S>::SUM) {
+                        if (grp == 1 && c == nruns - 1) {
+                            uint32_t r[XCPT];
+                            tmem_ldn(tmem + lane_base + (uint32_t)(S * XN + colq * XCPT), r);
+                            tmem_wait_ld();
+                            tmem_arrived(r);
+#pragma unroll
+                            for (int j = 0; j < XCPT; ++j) weak |= sum_below(r[j], SUM15_MIN) ? 1u << j : 0u;
+                        }
+                    }
                     tc_fence_before();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&acc_empty[grp]);
@@ -415,7 +460,19 @@ k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             const bool col_in = lane < XCPT && nt + lane < g.N;
             const int fb = col_in ? g.fb[nt + lane + r0] : 0;
             const long long cn_l = col_in ? (long long)c_n[nt + lane] : 0;
-            const int ea = row_ok ? max(g.fa[m + r0], 1) - 1022 : 0;
+            const int fa = row_ok ? g.fa[m + r0] : 0;
+            const int ea = max(fa, 1) - 1022;
+            if constexpr (XT<S>::SUM) {
+                weak |= __ballot_sync(0xffffffffu, field_outside(fb));
+                if (field_outside(fa)) weak = ~0u;
+                // of the elements that are stored
+                if (!row_ok) weak = 0;
+                weak &= (1u << max(0, min(XCPT, g.N - nt))) - 1u;
+                if (g.sym) weak &= ~0u << max(0, min(XCPT, m - nt));
+                static_assert(!XT<S>::SUM || (XN == 32 && XCPT == 8), "a byte of a word per thread");
+                ((uint8_t*)g.weak)[((size_t)nb * g.weak_rows + mb * XM + quad * 32 + lane) * 4 + colq] = (uint8_t)weak;
+                if (__any_sync(0xffffffffu, weak != 0) && lane == 0) g.weak_tile[mb * g.words + nb] = g.flags[0] = 1;
+            }
             const int eb_l = max(fb, 1) - 1022 - 14 - 8 * (S - 1);
             if (g.rows_fast) {
                 // lanes are adjacent rows, adjacent in C
@@ -476,6 +533,104 @@ k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     }
 }
 
+// ---------------------------------------------- elements left to the pipe ---
+// C(m, n) of the elements that the digit product marked weak, as FP64 sums in
+// order of k, the bits of k_gemm_f64.  A block takes 128 x 32 elements at a time,
+// those of a word column of the marks, lists the marked ones, and gives each
+// thread up to sixteen of them, so its time follows their number; operands are
+// staged as in k_gemm_f64.  Bound by the FP64 pipe: one FMA of a warp takes 16
+// clocks there, the two operands from shared memory about four.
+struct WeakArgs {
+    int M, N, K, sym, half;
+    const double* A[2]; const int64_t* a_m[2]; const int64_t* a_k[2]; int a_kfast[2];
+    const double* B[2]; const int64_t* b_k[2]; const int64_t* b_n[2]; int b_nfast[2];
+    double* C[2]; const int64_t* c_m[2]; const int64_t* c_n[2];
+    const int* any;
+    const int* tile;           // [tiles_m][words]
+    const uint32_t* weak;      // [words][rows]
+    int tiles_m, words, rows;
+};
+constexpr int WK = 16, WN = 32, WT = 256;       // K per stage, columns, threads
+constexpr int WE = XM * WN / WT;                // elements a thread can be given
+__global__ void __launch_bounds__(WT, 2) k_weak_f64(const WeakArgs g) {
+    if (*g.any == 0) return;
+    __shared__ double As[WK][XM + 1];
+    __shared__ double Bs[WK][WN + 1];
+    __shared__ uint16_t list[XM * WN];          // row << 5 | column
+    __shared__ int count;
+    const int tid = threadIdx.x;
+    for (int t = blockIdx.x; t < g.tiles_m * g.words; t += gridDim.x) {
+        if (!g.tile[t]) continue;
+        const int mb = t / g.words, w = t - mb * g.words;
+        const int q = g.half && mb * XM >= g.half ? 1 : 0;
+        const int m0 = mb * XM - (q ? g.half : 0), n0 = w * WN - (q ? g.half : 0);
+        __syncthreads();                        // the previous tile's list has been used
+        if (tid == 0) count = 0;
+        __syncthreads();
+        if (tid < XM) {
+            uint32_t bits = m0 + tid < g.M ? g.weak[(size_t)w * g.rows + mb * XM + tid] : 0u;
+            const int cols = g.N - n0;
+            if (cols < WN) bits &= (1u << max(cols, 0)) - 1u;
+            int at = atomicAdd(&count, __popc(bits));
+            for (; bits; bits &= bits - 1) list[at++] = (uint16_t)(tid << 5 | (__ffs((int)bits) - 1));
+        }
+        __syncthreads();
+        const int n = count;
+        int el[WE];
+        double acc[WE];
+#pragma unroll
+        for (int e = 0; e < WE; ++e) {
+            el[e] = tid + e * WT < n ? list[tid + e * WT] : 0;
+            acc[e] = 0.0;
+        }
+        double ra[XM * WK / WT], rb[WN * WK / WT];
+        auto load = [&](int k0) {
+#pragma unroll
+            for (int i = 0; i < XM * WK / WT; ++i) {
+                const int e = tid + i * WT;
+                const int r = g.a_kfast[q] ? e / WK : e % XM, k = k0 + (g.a_kfast[q] ? e % WK : e / XM);
+                ra[i] = m0 + r < g.M && k < g.K ? g.A[q][g.a_m[q][m0 + r] + g.a_k[q][k]] : 0.0;
+            }
+#pragma unroll
+            for (int i = 0; i < WN * WK / WT; ++i) {
+                const int e = tid + i * WT;
+                const int c = g.b_nfast[q] ? e % WN : e / WK, k = k0 + (g.b_nfast[q] ? e / WN : e % WK);
+                rb[i] = n0 + c < g.N && k < g.K ? g.B[q][g.b_k[q][k] + g.b_n[q][n0 + c]] : 0.0;
+            }
+        };
+        load(0);
+        for (int k0 = 0; k0 < g.K; k0 += WK) {
+            __syncthreads();
+#pragma unroll
+            for (int i = 0; i < XM * WK / WT; ++i) {
+                const int e = tid + i * WT;
+                if (g.a_kfast[q]) As[e % WK][e / WK] = ra[i]; else As[e / XM][e % XM] = ra[i];
+            }
+#pragma unroll
+            for (int i = 0; i < WN * WK / WT; ++i) {
+                const int e = tid + i * WT;
+                if (g.b_nfast[q]) Bs[e / WN][e % WN] = rb[i]; else Bs[e % WK][e / WK] = rb[i];
+            }
+            __syncthreads();
+            if (k0 + WK < g.K) load(k0 + WK);
+#pragma unroll
+            for (int e = 0; e < WE; ++e) {
+                if ((tid & ~31) + e * WT >= n) break;       // (the same for the warp)
+                const int r = el[e] >> 5, c = el[e] & 31;
+#pragma unroll
+                for (int kk = 0; kk < WK; ++kk) acc[e] = fma(As[kk][r], Bs[kk][c], acc[e]);
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < WE; ++e) {
+            if (tid + e * WT >= n) break;
+            const int m = m0 + (el[e] >> 5), c = n0 + (el[e] & 31);
+            g.C[q][g.c_m[q][m] + g.c_n[q][c]] = acc[e];
+            if (g.sym && c > m) g.C[q][g.c_m[q][c] + g.c_n[q][m]] = acc[e];
+        }
+    }
+}
+
 // ------------------------------------------------------------- host side ---
 // `count` planes from plane `first` on of the digits [kp / 16][XPLANES][rows][16]
 // (their order in a stage: no swizzle here), four rows to a 128-byte line,
@@ -498,16 +653,16 @@ inline int64_t up(int64_t v, int64_t q) { return (v + q - 1) / q * q; }
 
 // Exponent fields and digits of rows [0, R) of an operand, as rows of an array
 // of Rs.
-void digits(Ctx& ctx, const Gather& g, int R, int K, int Rp, int Kp, int* ef, uint16_t* out, int* bad, int Rs) {
+void digits(Ctx& ctx, const Gather& g, int R, int K, int Rp, int Kp, int* ef, uint16_t* out, int Rs) {
     if (g.c_identity && Kp <= CUT_ROWS4_MAX_K) {
-        launch_cut_rows4(ctx.stream, g.base, g.off_r, R, K, Rp, Kp, ef, out, bad, Rs);
+        launch_cut_rows4(ctx.stream, g.base, g.off_r, R, K, Rp, Kp, ef, out, Rs);
         TRG_LAUNCHED(ctx);
         return;
     }
     TRG_CUDA(cudaMemsetAsync(ef, 0, (size_t)R * sizeof(int), ctx.stream));
     launch_row_field<true>(ctx.stream, g, R, K, ef);
     TRG_LAUNCHED(ctx);
-    launch_cut<15>(ctx.stream, g, R, K, Rp, Kp, ef, nullptr, out, bad, Rs);
+    launch_cut<15>(ctx.stream, g, R, K, Rp, Kp, ef, nullptr, out, Rs);
     TRG_LAUNCHED(ctx);
 }
 
@@ -535,26 +690,34 @@ const long long* diagonal_tiles(Ctx& ctx, int tiles_m, int tiles_n, int xn, int 
     return it->second.as<long long>();
 }
 
-// Rows of an operand whose digits are held at a time: at most XCAP bytes of
-// them (a multiple of the tile).
-constexpr int64_t XCAP = (int64_t)1 << 30;
-constexpr int64_t XNP = 64;                      // B's rows are padded to this
-int64_t block_rows(int64_t rows, int64_t kp, int64_t tile) {
-    const int64_t most = std::max<int64_t>(tile, XCAP / (2 * XPLANES * kp) / tile * tile);
-    return std::min(up(rows, tile), most);
+// Rows of the operands whose digits are held at a time: at most XCAP bytes of
+// them each, and a weak bit for at most XBITS elements of C (multiples of the
+// tile; B's rows of XNP).
+constexpr int64_t XCAP = (int64_t)1 << 30, XBITS = (int64_t)1 << 28;
+constexpr int64_t XNP = 64;
+struct XBlock { int64_t a, b; };
+XBlock block_rows(int64_t M, int64_t N, int64_t kp) {
+    const int64_t most = XCAP / (2 * XPLANES * kp);
+    XBlock x;
+    x.a = std::min(up(M, XM), std::max<int64_t>(XM, most / XM * XM));
+    x.b = std::min(up(N, XNP), std::max<int64_t>(XNP, std::min(most, XBITS / x.a) / XNP * XNP));
+    return x;
 }
+// Bytes of the flags, the weak tiles and the weak bits of an a x b block.
+int64_t flag_bytes(int64_t a, int64_t b) { return up(256 + 4 * (a / XM) * (up(b, 32) / 32), 256); }
+int64_t weak_bytes(int64_t a, int64_t b) { return 4 * a * (up(b, 32) / 32); }
 
 }  // namespace
 
 int64_t exact_scratch_bytes(int64_t M, int64_t N, int64_t K) {
     const int64_t kp = up(std::max<int64_t>(K, 1), XKP);
-    const int64_t ra = block_rows(M, kp, XM), rb = block_rows(N, kp, XNP);
-    return 2 * XPLANES * kp * (ra + rb) + 4 * (ra + rb) + 2048;
+    const XBlock x = block_rows(M, N, kp);
+    return 2 * XPLANES * kp * (x.a + x.b) + 4 * (x.a + x.b) + flag_bytes(x.a, x.b) + weak_bytes(x.a, x.b) + 2048;
 }
 
 int64_t exact_pair_scratch_bytes(int64_t M, int64_t K) {
     const int64_t kp = up(std::max<int64_t>(K, 1), XKP), rows = 2 * up(M, XM);
-    return 2 * XPLANES * kp * rows + 4 * rows + 2048;
+    return 2 * XPLANES * kp * rows + 4 * rows + flag_bytes(rows, rows) + weak_bytes(rows, rows) + 2048;
 }
 
 namespace {
@@ -592,8 +755,8 @@ void launch_exact(Ctx& ctx, const uint16_t* sa, int64_t mp, const uint16_t* sb, 
         TRG_CUDA(cudaFuncSetAttribute(k_exact_mma<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, XT<S>::SMEM));
         return 0;
     });
-    const CUtensorMap ta = digit_map(sa, first, S, mp, a.Kp, XM, XT<S>::K);
-    const CUtensorMap tb = digit_map(sb, first, S, np, a.Kp, XT<S>::N, XT<S>::K);
+    const CUtensorMap ta = digit_map(sa, first, XT<S>::P, mp, a.Kp, XM, XT<S>::K);
+    const CUtensorMap tb = digit_map(sb, first, XT<S>::P, np, a.Kp, XT<S>::N, XT<S>::K);
     const int tiles_m = (a.M + XM - 1) / XM, tiles_n = (a.N + XT<S>::N - 1) / XT<S>::N;
     int tiles = tiles_m * tiles_n;
     a.acc_wait_ns = ctx.acc_wait_ns ? ctx.acc_wait_ns : WAIT_NS;
@@ -609,27 +772,43 @@ void launch_exact(Ctx& ctx, const uint16_t* sa, int64_t mp, const uint16_t* sb, 
     TRG_LAUNCHED(ctx);
 }
 
+// The weak elements of the block at (m0, n0) of d0 (and of d1, for a pair).
+void launch_weak(Ctx& ctx, const GemmDesc& d0, const GemmDesc& d1, int64_t m0, int64_t n0, const XArgs& a) {
+    WeakArgs w;
+    w.M = a.M; w.N = a.N; w.K = (int)d0.K; w.sym = a.sym; w.half = a.half;
+    const GemmDesc* d[2] = {&d0, &d1};
+    for (int q = 0; q < 2; ++q) {
+        w.A[q] = d[q]->A.base; w.a_m[q] = d[q]->A.off_r + m0; w.a_k[q] = d[q]->A.off_c; w.a_kfast[q] = d[q]->A.c_fast;
+        w.B[q] = d[q]->B.base; w.b_k[q] = d[q]->B.off_r; w.b_n[q] = d[q]->B.off_c + n0; w.b_nfast[q] = d[q]->B.c_fast;
+        w.C[q] = d[q]->C; w.c_m[q] = d[q]->c_m + m0; w.c_n[q] = d[q]->c_n + n0;
+    }
+    w.any = a.flags; w.tile = a.weak_tile; w.weak = a.weak;
+    w.tiles_m = (a.half + a.M + XM - 1) / XM; w.words = a.words; w.rows = a.weak_rows;
+    k_weak_f64<<<std::min(w.tiles_m * w.words, 4 * ctx.sm_count), WT, 0, ctx.stream>>>(w);
+    TRG_LAUNCHED(ctx);
+}
+
 }  // namespace
 
 bool gemm_exact(Ctx& ctx, const GemmDesc& d) {
     const int K = (int)std::max<int64_t>(d.K, 1), Kp = (int)up(K, XKP);
-    const int64_t ra = block_rows(d.M, Kp, XM), rb = block_rows(d.N, Kp, XNP);
-    const bool sym = d.gram && d.M == d.N && ra >= d.M;
+    const XBlock blk = block_rows(d.M, d.N, Kp);
+    const int64_t ra = blk.a, rb = blk.b;
+    const bool sym = d.gram && d.M == d.N && ra >= d.M && rb >= d.N;
     try {
-        ctx.ensure(ctx.split_ws, (size_t)exact_scratch_bytes(d.M, sym ? 1 : d.N, K));
+        ctx.ensure(ctx.split_ws, (size_t)exact_scratch_bytes(d.M, d.N, K));
     } catch (const Error& e) {
         if (e.status == TRG_ENOMEM) return false;    // no room for the digits: the FP64 pipe needs none
         throw;
     }
     uint8_t* p = ctx.split_ws.as<uint8_t>();
     auto take = [&](size_t bytes) { uint8_t* q = p; p += (bytes + 255) & ~(size_t)255; return q; };
-    int* flags = (int*)take(2 * sizeof(int));
-    int* bad = flags;
+    int* flags = (int*)take((size_t)flag_bytes(ra, rb));
+    uint32_t* weak = (uint32_t*)take((size_t)weak_bytes(ra, rb));
     int* fa = (int*)take((size_t)ra * 4);
     int* fb = sym ? fa : (int*)take((size_t)rb * 4);
     uint16_t* sa = (uint16_t*)take((size_t)(2 * XPLANES) * ra * Kp);
     uint16_t* sb = sym ? sa : (uint16_t*)take((size_t)(2 * XPLANES) * rb * Kp);
-    TRG_CUDA(cudaMemsetAsync(flags, 0, 2 * sizeof(int), ctx.stream));
 
     // B as rows n, columns k
     const Gather bt = transposed(d.B);
@@ -637,13 +816,13 @@ bool gemm_exact(Ctx& ctx, const GemmDesc& d) {
         const int mr = (int)std::min(ra, d.M - m0), mp = (int)up(mr, XM);
         Gather ga = d.A;
         ga.off_r += m0;
-        digits(ctx, ga, mr, K, mp, Kp, fa, sa, bad, mp);
+        digits(ctx, ga, mr, K, mp, Kp, fa, sa, mp);
         for (int64_t n0 = 0; n0 < d.N; n0 += rb) {
             const int nr = (int)std::min(rb, d.N - n0), np = sym ? mp : (int)up(nr, XNP);
             if (!sym && (m0 == 0 || rb < d.N)) {
                 Gather gb = bt;
                 gb.off_r += n0;
-                digits(ctx, gb, nr, K, np, Kp, fb, sb, bad, np);
+                digits(ctx, gb, nr, K, np, Kp, fb, sb, np);
             }
             XArgs a;
             a.M = mr; a.N = sym ? mr : nr; a.Kp = Kp;
@@ -652,22 +831,22 @@ bool gemm_exact(Ctx& ctx, const GemmDesc& d) {
             a.rows_fast = d.c_m_fast && !sym ? 1 : 0;
             a.sym = sym ? 1 : 0;
             a.flags = flags; a.status = ctx.status.as<int>();
+            a.weak = weak; a.weak_tile = flags + 64; a.weak_rows = mp; a.words = (a.N + 31) / 32;
+            TRG_CUDA(cudaMemsetAsync(flags, 0, (size_t)flag_bytes(mp, a.N), ctx.stream));
             const int tok = ctx.region_begin(TRG_PHASE_MMA);
             const bool nine = try_nine(ctx, a.M, a.N, K, sym);
             a.nine = nine ? 1 : 0;
             a.half = 0;
             if (nine) {
-                // (each block decides for itself; an operand out of range stays so)
-                if (m0 + n0 > 0) TRG_CUDA(cudaMemsetAsync(flags + 1, 0, sizeof(int), ctx.stream));
                 launch_exact<1>(ctx, sa, mp, sb, np, a);
                 launch_exact<9>(ctx, sa, mp, sb, np, a);
             }
             launch_exact<15>(ctx, sa, mp, sb, np, a);
             ctx.region_end(tok, 2.0 * (double)mr * nr * K, (nine ? 45.0 : 120.0) * 2.0 * (double)mr * nr * Kp);   // 120 also if nine do not suffice
+            launch_weak(ctx, d, d, m0, n0, a);
             if (sym) break;
         }
     }
-    gemm_f64(ctx, d, bad);    // computes the product if an operand was out of range, else returns at once
     return true;
 }
 
@@ -688,12 +867,14 @@ bool gemm_exact_pair(Ctx& ctx, const GemmDesc& d0, const GemmDesc& d1) {
     }
     const int phase = ctx.region_begin(ctx.phase);
     uint8_t* p = ctx.split_ws.as<uint8_t>();
-    int* flags = (int*)p;
-    int* f = (int*)(p + 256);
-    uint16_t* s = (uint16_t*)(p + 256 + up((int64_t)2 * mp * 4, 256));
-    TRG_CUDA(cudaMemsetAsync(flags, 0, 2 * sizeof(int), ctx.stream));
-    digits(ctx, d0.A, (int)M, (int)K, mp, Kp, f, s, flags, 2 * mp);
-    digits(ctx, d1.A, (int)M, (int)K, mp, Kp, f + mp, s + (size_t)mp * 16, flags, 2 * mp);
+    auto take = [&](int64_t bytes) { uint8_t* q = p; p += up(bytes, 256); return q; };
+    int* flags = (int*)take(flag_bytes(2 * mp, 2 * mp));
+    uint32_t* weak = (uint32_t*)take(weak_bytes(2 * mp, 2 * mp));
+    int* f = (int*)take((int64_t)2 * mp * 4);
+    uint16_t* s = (uint16_t*)p;
+    TRG_CUDA(cudaMemsetAsync(flags, 0, (size_t)flag_bytes(2 * mp, 2 * mp), ctx.stream));
+    digits(ctx, d0.A, (int)M, (int)K, mp, Kp, f, s, 2 * mp);
+    digits(ctx, d1.A, (int)M, (int)K, mp, Kp, f + mp, s + (size_t)mp * 16, 2 * mp);
     XArgs a;
     a.M = (int)M; a.N = (int)M; a.Kp = Kp;
     a.fa = f; a.fb = f;
@@ -704,11 +885,11 @@ bool gemm_exact_pair(Ctx& ctx, const GemmDesc& d0, const GemmDesc& d1) {
     a.half = mp;
     a.nine = 0;
     a.flags = flags; a.status = ctx.status.as<int>();
+    a.weak = weak; a.weak_tile = flags + 64; a.weak_rows = 2 * mp; a.words = 2 * mp / 32;
     const int tok = ctx.region_begin(TRG_PHASE_MMA);
     launch_exact<15>(ctx, s, 2 * mp, s, 2 * mp, a);
     ctx.region_end(tok, 4.0 * (double)M * M * K, 120.0 * 4.0 * (double)M * M * Kp);
-    gemm_f64(ctx, d0, flags);
-    gemm_f64(ctx, d1, flags);
+    launch_weak(ctx, d0, d1, 0, 0, a);
     ctx.region_end(phase, 4.0 * (double)M * M * K, 0.0);
     return true;
 }

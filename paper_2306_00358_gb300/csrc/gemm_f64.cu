@@ -37,7 +37,6 @@ struct GemmArgs {
     double beta;
     int64_t tiles_n, tiles;
     int sym;               // C = A A^T: tiles below the diagonal are mirrors of those above
-    const int* only_if;    // device flag: compute only if it is set
 };
 
 // T x T outputs per block, R x R per thread (stride T / R), BK deep stages.
@@ -46,7 +45,6 @@ __global__ void __launch_bounds__(NT) k_gemm_f64(const GemmArgs g) {
     constexpr int W = T / R;                  // threads along a tile side
     constexpr int E = T * BK / NT;            // elements a thread stages per operand
     static_assert(W * W == NT && E * NT == T * BK, "tile shape");
-    if (g.only_if && *g.only_if == 0) return;
     __shared__ double As[BK][T + 1];
     __shared__ double Bs[BK][T + 1];
     const int tid = threadIdx.x;
@@ -133,8 +131,7 @@ __global__ void __launch_bounds__(NT) k_gemm_f64(const GemmArgs g) {
 
 // C = beta C + sum_z P[z], summed in z order (deterministic).
 __global__ void k_reduce_partials(const double* __restrict__ P, int nz, int64_t M, int64_t N, double* C,
-                                  const int64_t* c_m, const int64_t* c_n, double beta, const int* only_if) {
-    if (only_if && *only_if == 0) return;
+                                  const int64_t* c_m, const int64_t* c_n, double beta) {
     const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (e >= M * N) return;
     double s = 0.0;
@@ -178,15 +175,13 @@ void launch(Ctx& ctx, GemmArgs g, int64_t nz) {
         ctx.ensure(ctx.f64_partial, (size_t)(parts * g.M * g.N) * sizeof(double));
         g.partial = ctx.f64_partial.as<double>();
     }
-    // a conditional product that is normally skipped launches few blocks
-    const int64_t most = g.only_if ? 8 * ctx.sm_count : 1 << 30;
-    dim3 grid((unsigned)std::min<int64_t>(g.tiles, most), 1, (unsigned)parts);
+    dim3 grid((unsigned)std::min<int64_t>(g.tiles, 1 << 30), 1, (unsigned)parts);
     k_gemm_f64<T, R, BK, NT><<<grid, NT, 0, ctx.stream>>>(g);
     TRG_LAUNCHED(ctx);
     if (parts > 1) {
         const int64_t tot = g.M * g.N;
         k_reduce_partials<<<(unsigned)((tot + 255) / 256), 256, 0, ctx.stream>>>(g.partial, (int)parts, g.M, g.N, g.C,
-                                                                              g.c_m, g.c_n, g.beta, g.only_if);
+                                                                              g.c_m, g.c_n, g.beta);
         TRG_LAUNCHED(ctx);
     }
 }
@@ -197,13 +192,12 @@ double f64_us(const Ctx& ctx, int64_t M, int64_t N, int64_t K, bool sym) {
     return choose_shape(M, N, std::max<int64_t>(K, 1), ctx.sm_count, sym).clocks / 1900.0 + 3.0;
 }
 
-void gemm_f64(Ctx& ctx, const GemmDesc& d, const int* only_if) {
+void gemm_f64(Ctx& ctx, const GemmDesc& d) {
     if (d.M <= 0 || d.N <= 0) return;
     GemmArgs g;
     g.M = d.M; g.N = d.N; g.K = d.K;
     g.kper = std::max<int64_t>(d.K, 1);
     g.partial = nullptr;
-    g.only_if = only_if;
     g.A = d.A.base; g.a_m = d.A.off_r; g.a_k = d.A.off_c; g.a_kfast = d.A.c_fast ? 1 : 0;
     g.B = d.B.base; g.b_k = d.B.off_r; g.b_n = d.B.off_c; g.b_nfast = d.B.c_fast ? 1 : 0;
     g.C = d.C; g.c_m = d.c_m; g.c_n = d.c_n; g.beta = d.beta;

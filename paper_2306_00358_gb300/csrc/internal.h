@@ -235,8 +235,7 @@ void split_slice_operand(Ctx& ctx, const Gather& A, int64_t M, int64_t K, uint16
 void split_slice_b(Ctx& ctx, const Gather& B, int64_t K, int64_t N, uint16_t* slices, int* e);
 int64_t split_cols_padded(int64_t N);
 void gemm(Ctx& ctx, const GemmDesc& g, int precision);
-// only_if: device flag; the product is computed only if it is set.
-void gemm_f64(Ctx& ctx, const GemmDesc& g, const int* only_if = nullptr);
+void gemm_f64(Ctx& ctx, const GemmDesc& g);
 double f64_us(const Ctx& ctx, int64_t M, int64_t N, int64_t K, bool sym);   // modelled time of gemm_f64
 // FP64 product from exact BF16 digit products (exact_gemm.cu); false if its
 // scratch cannot be had (nothing computed).

@@ -44,9 +44,13 @@ __device__ __forceinline__ unsigned exponent_field(double x) {
 // Scale exponent of a row from its largest field (-1022 for a zero row).
 __device__ __forceinline__ int row_exponent(int f) { return f ? f - 1022 : -1022; }
 
-// Planes stored for S digits: 15 digits are followed by |x| 2^-e itself, cut off
-// to BF16 (the operands of the product's |A||B|, see exact_gemm.cu).
+// Planes stored for S digits: 15 digits are followed by |x| 2^(SIZE_SHIFT - e),
+// cut off to BF16 (the operands of the product's |A||B|, see exact_gemm.cu).
+// The shift keeps sums of up to 2^17 products of two of them below 2^127, and
+// the floor, 2^-63 for any x that is not zero, keeps every product normal in
+// FP32: such a sum is zero only if every |a||b| of it is.
 __host__ __device__ constexpr int planes(int S) { return S == 15 ? 16 : S; }
+constexpr int SIZE_SHIFT = 54, SIZE_FLOOR = -63;
 
 // The digits of x in a row of largest field f, as the FP32 values to store
 // (exact in BF16: their upper halves).
@@ -72,9 +76,9 @@ __device__ __forceinline__ void cut(double x, int f, float (&d)[planes(S)]) {
             const int byte = 14 - p;
             d[p] = __uint_as_float(__byte_perm(q[byte >> 2], 0x4B000000u, 0x7440u | (unsigned)(byte & 3))) - 8388736.0f;   // 2^23 + 128
         }
-        // FP32 exponent field of |x| 2^-e, not below 2^-60: products stay normal
-        const int ea = max(ex - f + 126, 127 - 60);
-        d[15] = ex ? __uint_as_float(((unsigned)ea << 23) | (((unsigned)(m53 >> 45) & 0x7Fu) << 16)) : 0.0f;
+        // its FP32 exponent field: that of 1 is 127, |x| 2^-e = 1.mmm 2^(ex - f - 1)
+        const int ea = max(ex - f + 126 + SIZE_SHIFT, 127 + SIZE_FLOOR);
+        d[15] = (b << 1) ? __uint_as_float(((unsigned)ea << 23) | (((unsigned)(m53 >> 45) & 0x7Fu) << 16)) : 0.0f;
     } else {
         constexpr int F = 7 + 8 * (S - 1);
         constexpr unsigned BIAS = S == 2 ? 0x80u : S == 3 ? 0x8080u : S == 4 ? 0x808080u : 0x80808080u;
@@ -111,13 +115,6 @@ __device__ __forceinline__ void cut2(double x0, double x1, int f, uint32_t (&w)[
     cut<S>(x1, f, b);
 #pragma unroll
     for (int p = 0; p < planes(S); ++p) w[p] = __byte_perm(__float_as_uint(a[p]), __float_as_uint(b[p]), 0x7632);
-}
-
-// Rows of an exact product whose largest entry lies outside this range make
-// it take the FP64 pipe instead (exact_gemm.cu).
-constexpr int FIELD_LO = 1023 - 400, FIELD_HI = 1023 + 400;
-__device__ __forceinline__ void check_range(int f, int* bad) {
-    if (bad && f && (f < FIELD_LO || f > FIELD_HI)) *bad = 1;
 }
 
 // Largest exponent field of each row, maxima into ef (zeroed); a block takes 32
@@ -176,7 +173,7 @@ template <int S>
 __global__ void __launch_bounds__(256) k_cut(const double* __restrict__ src, const int64_t* __restrict__ off_r,
                                              const int64_t* __restrict__ off_c, int R, int K, int Rp, int Kp,
                                              int k_fast, const int* __restrict__ ef, int* __restrict__ e_out,
-                                             uint16_t* __restrict__ out, int* bad, int Rs) {
+                                             uint16_t* __restrict__ out, int Rs) {
     __shared__ double tile[XD_R * XD_LD];
     const int k0 = blockIdx.x * XD_K;
     const size_t plane = digit_stride<S>(Rs, Kp);
@@ -197,7 +194,6 @@ __global__ void __launch_bounds__(256) k_cut(const double* __restrict__ src, con
         const int r = r0 + rr, k = k0 + kg * 8;
         if (r >= Rp || k >= Kp) continue;
         const int f = r < R ? ef[r] : 0;
-        check_range(f, bad);
         if (e_out && blockIdx.x == 0 && kg == 0 && r < R) e_out[r] = row_exponent(f);
         const double* x = tile + rr * XD_LD + kg * 9;
         uint32_t w[4][planes(S)];
@@ -235,7 +231,7 @@ __device__ __forceinline__ void store4(const double (&v)[4], int f, uint16_t* o,
 template <int S>
 __global__ void __launch_bounds__(256) k_slice_contig(const double* __restrict__ src, const int64_t* __restrict__ off_r,
                                                       int R, int K, int Rp, int Kp, const int* __restrict__ ef,
-                                                      int* __restrict__ e_out, uint16_t* __restrict__ out, int* bad) {
+                                                      int* __restrict__ e_out, uint16_t* __restrict__ out) {
     const int lane = threadIdx.x & 31;
     const int r = blockIdx.x * 8 + (threadIdx.x >> 5);
     if (r >= Rp) return;
@@ -244,7 +240,6 @@ __global__ void __launch_bounds__(256) k_slice_contig(const double* __restrict__
     const double* row = real ? src + off_r[r] : nullptr;
     const bool vec = real && ((reinterpret_cast<uintptr_t>(row) & 15) == 0);
     const int f = real ? ef[r] : 0;
-    check_range(f, bad);
     if (e_out && lane == 0 && real) e_out[r] = row_exponent(f);
     for (int k = lane * 4; k < Kp; k += 128) {
         double v[4];
@@ -258,7 +253,7 @@ __global__ void __launch_bounds__(256) k_slice_contig(const double* __restrict__
 template <int S, int TPR, int NCH, bool SUB>
 __global__ void __launch_bounds__(256) k_cut_rows(const double* __restrict__ src, const int64_t* __restrict__ off_r,
                                                   int R, int K, int Rp, int Kp, int* __restrict__ ef_out,
-                                                  int* __restrict__ e_out, uint16_t* __restrict__ out, int* bad) {
+                                                  int* __restrict__ e_out, uint16_t* __restrict__ out) {
     __shared__ unsigned wmax[8];
     const int t = threadIdx.x % TPR;
     const int r = blockIdx.x * (256 / TPR) + threadIdx.x / TPR;
@@ -283,7 +278,6 @@ __global__ void __launch_bounds__(256) k_cut_rows(const double* __restrict__ src
         for (int w = 0; w < 8; ++w) fm = max(fm, wmax[w]);
     }
     const int f = (int)fm;
-    check_range(f, bad);
     if (t == 0 && real) {
         if (ef_out) ef_out[r] = f;
         if (e_out) e_out[r] = row_exponent(f);
@@ -298,13 +292,13 @@ __global__ void __launch_bounds__(256) k_cut_rows(const double* __restrict__ src
 constexpr int CUT_ROWS_MAX_K = 8192;
 template <int S, bool SUB>
 void launch_cut_rows(cudaStream_t stream, const double* src, const int64_t* off_r, int R, int K, int Rp, int Kp,
-                     int* ef_out, int* e_out, uint16_t* out, int* bad) {
+                     int* ef_out, int* e_out, uint16_t* out) {
     const unsigned gw = (unsigned)((Rp + 7) / 8), gb = (unsigned)Rp;
-    if (Kp <= 128) k_cut_rows<S, 32, 1, SUB><<<gw, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, e_out, out, bad);
-    else if (Kp <= 512) k_cut_rows<S, 32, 4, SUB><<<gw, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, e_out, out, bad);
-    else if (Kp <= 2048) k_cut_rows<S, 256, 2, SUB><<<gb, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, e_out, out, bad);
-    else if (Kp <= 4096) k_cut_rows<S, 256, 4, SUB><<<gb, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, e_out, out, bad);
-    else k_cut_rows<S, 256, 8, SUB><<<gb, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, e_out, out, bad);
+    if (Kp <= 128) k_cut_rows<S, 32, 1, SUB><<<gw, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, e_out, out);
+    else if (Kp <= 512) k_cut_rows<S, 32, 4, SUB><<<gw, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, e_out, out);
+    else if (Kp <= 2048) k_cut_rows<S, 256, 2, SUB><<<gb, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, e_out, out);
+    else if (Kp <= 4096) k_cut_rows<S, 256, 4, SUB><<<gb, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, e_out, out);
+    else k_cut_rows<S, 256, 8, SUB><<<gb, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, e_out, out);
 }
 
 // The same for 15 digits, K <= 256 NCH: a block holds four rows, and a warp
@@ -314,7 +308,7 @@ void launch_cut_rows(cudaStream_t stream, const double* src, const int64_t* off_
 template <int NCH>
 __global__ void __launch_bounds__(256) k_cut_rows4(const double* __restrict__ src, const int64_t* __restrict__ off_r,
                                                    int R, int K, int Rp, int Kp, int* __restrict__ ef_out,
-                                                   uint16_t* __restrict__ out, int* bad, int Rs) {
+                                                   uint16_t* __restrict__ out, int Rs) {
     __shared__ unsigned wmax[8][4];
     const int warp = threadIdx.x >> 5, rr = (threadIdx.x >> 3) & 3, kc = threadIdx.x & 7;
     const int r = blockIdx.x * 4 + rr;                   // Rp is a multiple of four
@@ -337,7 +331,6 @@ __global__ void __launch_bounds__(256) k_cut_rows4(const double* __restrict__ sr
 #pragma unroll
     for (int w = 0; w < 8; ++w) fm = max(fm, wmax[w][rr]);
     const int f = (int)fm;
-    check_range(f, bad);
     if (warp == 0 && kc == 0 && real) ef_out[r] = f;
 #pragma unroll
     for (int c = 0; c < NCH; ++c) {
@@ -348,14 +341,14 @@ __global__ void __launch_bounds__(256) k_cut_rows4(const double* __restrict__ sr
 
 constexpr int CUT_ROWS4_MAX_K = 4096;
 inline void launch_cut_rows4(cudaStream_t stream, const double* src, const int64_t* off_r, int R, int K, int Rp, int Kp,
-                             int* ef_out, uint16_t* out, int* bad, int Rs) {
+                             int* ef_out, uint16_t* out, int Rs) {
     const unsigned grid = (unsigned)(Rp / 4);
-    if (Kp <= 256) k_cut_rows4<1><<<grid, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, out, bad, Rs);
-    else if (Kp <= 512) k_cut_rows4<2><<<grid, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, out, bad, Rs);
-    else if (Kp <= 1024) k_cut_rows4<4><<<grid, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, out, bad, Rs);
-    else if (Kp <= 2048) k_cut_rows4<8><<<grid, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, out, bad, Rs);
-    else if (Kp <= 3072) k_cut_rows4<12><<<grid, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, out, bad, Rs);
-    else k_cut_rows4<16><<<grid, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, out, bad, Rs);
+    if (Kp <= 256) k_cut_rows4<1><<<grid, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, out, Rs);
+    else if (Kp <= 512) k_cut_rows4<2><<<grid, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, out, Rs);
+    else if (Kp <= 1024) k_cut_rows4<4><<<grid, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, out, Rs);
+    else if (Kp <= 2048) k_cut_rows4<8><<<grid, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, out, Rs);
+    else if (Kp <= 3072) k_cut_rows4<12><<<grid, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, out, Rs);
+    else k_cut_rows4<16><<<grid, 256, 0, stream>>>(src, off_r, R, K, Rp, Kp, ef_out, out, Rs);
 }
 
 template <bool SUB>
@@ -368,9 +361,9 @@ void launch_row_field(cudaStream_t stream, const Gather& g, int R, int K, int* e
 
 template <int S>
 void launch_cut(cudaStream_t stream, const Gather& g, int R, int K, int Rp, int Kp, const int* ef, int* e_out,
-                uint16_t* out, int* bad, int Rs = 0) {
+                uint16_t* out, int Rs = 0) {
     dim3 grid((unsigned)((Kp + XD_K - 1) / XD_K), (unsigned)std::min((Rp + XD_R - 1) / XD_R, 65535));
-    k_cut<S><<<grid, 256, 0, stream>>>(g.base, g.off_r, g.off_c, R, K, Rp, Kp, g.c_fast ? 1 : 0, ef, e_out, out, bad,
+    k_cut<S><<<grid, 256, 0, stream>>>(g.base, g.off_r, g.off_c, R, K, Rp, Kp, g.c_fast ? 1 : 0, ef, e_out, out,
                                          Rs ? Rs : Rp);
 }
 

@@ -970,10 +970,9 @@ constexpr int SLICE_ROWS_MAX = 256, SLICE_ROWS_MAX_K = 16384;
 template <int S>
 void slice_operand(Ctx& ctx, const Gather& g, int R, int K, int Rp, int Kp, const int* known, int* e, uint16_t* out) {
     if (g.c_identity && known) {
-        k_slice_contig<S><<<(unsigned)((Rp + 7) / 8), 256, 0, ctx.stream>>>(g.base, g.off_r, R, K, Rp, Kp, known, e, out,
-                                                                            nullptr);
+        k_slice_contig<S><<<(unsigned)((Rp + 7) / 8), 256, 0, ctx.stream>>>(g.base, g.off_r, R, K, Rp, Kp, known, e, out);
     } else if (g.c_identity && Kp <= CUT_ROWS_MAX_K) {
-        launch_cut_rows<S, false>(ctx.stream, g.base, g.off_r, R, K, Rp, Kp, nullptr, e, out, nullptr);
+        launch_cut_rows<S, false>(ctx.stream, g.base, g.off_r, R, K, Rp, Kp, nullptr, e, out);
     } else if (!known && Rp <= SLICE_ROWS_MAX && K <= SLICE_ROWS_MAX_K) {
         k_slice_rows<S><<<(unsigned)Rp, 256, 0, ctx.stream>>>(g.base, g.off_r, g.off_c, R, K, Rp, Kp, e, out);
     } else {
@@ -985,7 +984,7 @@ void slice_operand(Ctx& ctx, const Gather& g, int R, int K, int Rp, int Kp, cons
             TRG_LAUNCHED(ctx);
             known = f;
         }
-        launch_cut<S>(ctx.stream, g, R, K, Rp, Kp, known, e, out, nullptr);
+        launch_cut<S>(ctx.stream, g, R, K, Rp, Kp, known, e, out);
     }
     TRG_LAUNCHED(ctx);
 }
@@ -1326,14 +1325,14 @@ extern "C" int trg_gemm_noalloc(int M, int N, int K, const double* A, int lda, c
             launch_row_field<false>(stream, gb, N, K, eb);
             TRG_CUDA(cudaGetLastError());
             switch (S) {
-                case 2: launch_cut<2>(stream, ga, M, K, Mp, Kp, ea, nullptr, sa, nullptr);
-                        launch_cut<2>(stream, gb, N, K, Np, Kp, eb, nullptr, sb, nullptr); break;
-                case 3: launch_cut<3>(stream, ga, M, K, Mp, Kp, ea, nullptr, sa, nullptr);
-                        launch_cut<3>(stream, gb, N, K, Np, Kp, eb, nullptr, sb, nullptr); break;
-                case 4: launch_cut<4>(stream, ga, M, K, Mp, Kp, ea, nullptr, sa, nullptr);
-                        launch_cut<4>(stream, gb, N, K, Np, Kp, eb, nullptr, sb, nullptr); break;
-                default: launch_cut<5>(stream, ga, M, K, Mp, Kp, ea, nullptr, sa, nullptr);
-                         launch_cut<5>(stream, gb, N, K, Np, Kp, eb, nullptr, sb, nullptr); break;
+                case 2: launch_cut<2>(stream, ga, M, K, Mp, Kp, ea, nullptr, sa);
+                        launch_cut<2>(stream, gb, N, K, Np, Kp, eb, nullptr, sb); break;
+                case 3: launch_cut<3>(stream, ga, M, K, Mp, Kp, ea, nullptr, sa);
+                        launch_cut<3>(stream, gb, N, K, Np, Kp, eb, nullptr, sb); break;
+                case 4: launch_cut<4>(stream, ga, M, K, Mp, Kp, ea, nullptr, sa);
+                        launch_cut<4>(stream, gb, N, K, Np, Kp, eb, nullptr, sb); break;
+                default: launch_cut<5>(stream, ga, M, K, Mp, Kp, ea, nullptr, sa);
+                         launch_cut<5>(stream, gb, N, K, Np, Kp, eb, nullptr, sb); break;
             }
             TRG_CUDA(cudaGetLastError());
             k_exponent_finish<<<(unsigned)((M + 255) / 256), 256, 0, stream>>>(ea, M);
