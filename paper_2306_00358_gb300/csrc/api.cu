@@ -4,6 +4,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <stdexcept>
 
@@ -61,6 +62,45 @@ void Ctx::release(Buf& b) {
     raw_free(b.p, b.bytes);
     b.p = nullptr;
     b.bytes = 0;
+}
+
+// Mapped host memory costs tens of microseconds to get, more than a small call
+// takes, so contexts hand theirs on: at most HOST_SLOTS_KEPT are kept for the
+// next ones.  (Portable and, with unified addressing, at one address on every
+// device.)
+static std::mutex g_slot_mu;
+static std::vector<void*>& g_slots = *new std::vector<void*>();    // (contexts may outlive static destruction)
+constexpr size_t HOST_SLOTS_KEPT = 64;
+
+void Ctx::take_host_slot() {
+    void* p = nullptr;
+    {
+        std::lock_guard<std::mutex> lock(g_slot_mu);
+        if (!g_slots.empty()) {
+            p = g_slots.back();
+            g_slots.pop_back();
+        }
+    }
+    if (!p) TRG_CUDA(cudaHostAlloc(&p, HOST_SLOT_BYTES, cudaHostAllocMapped | cudaHostAllocPortable));
+    std::memset(p, 0, HOST_SLOT_BYTES);
+    gave_up = (int*)p;
+    box = (char*)p + HOST_SLOT_BOX;
+}
+
+// idle: no kernel can write the slot any more (else it is left alone for good).
+void Ctx::give_host_slot(bool idle) {
+    void* p = gave_up;
+    gave_up = nullptr;
+    box = nullptr;
+    if (!p || !idle) return;
+    {
+        std::lock_guard<std::mutex> lock(g_slot_mu);
+        if (g_slots.size() < HOST_SLOTS_KEPT) {
+            g_slots.push_back(p);
+            return;
+        }
+    }
+    cudaFreeHost(p);
 }
 
 cudaEvent_t Ctx::get_event() {
@@ -180,7 +220,7 @@ static void half_step_finish(Ctx& ctx, HalfPlan& p) {
         ctx.region_end(tok, 0.0, 0.0);
     }
     const int st = read_status(ctx);
-    check_timeout(ctx, st);
+    check_timeout(ctx);
     if (st & ST_BAD_NORM) fail(TRG_ENUMERIC, "non-positive or non-finite norm at half-step " + std::to_string(p.k));
     std::swap(ctx.T, ctx.Tnext);
     if (ctx.have_impure) std::swap(ctx.Timp, ctx.Timp_next);
@@ -261,9 +301,10 @@ using trg::Error;
 static int report(trg_ctx* ctx, const Error& e) {
     if (!ctx) return e.status;
     ctx->last_error = e.msg;
-    if (e.status == TRG_ETIMEOUT) return e.status;
+    if (e.status == TRG_ETIMEOUT) return e.status;   // (cleared already)
     try {
-        trg::check_timeout(*ctx, trg::read_status(*ctx));
+        TRG_CUDA(cudaStreamSynchronize(ctx->stream));
+        trg::check_timeout(*ctx);
     } catch (const Error& t) {
         if (t.status == TRG_ETIMEOUT && e.status == TRG_ENUMERIC) {
             ctx->last_error = t.msg;
@@ -273,10 +314,11 @@ static int report(trg_ctx* ctx, const Error& e) {
     return e.status;
 }
 
-// A component call's own status: cleared before its first product, read after
-// its last one.
-static void begin_component(Ctx& ctx) { TRG_CUDA(cudaMemsetAsync(ctx.status.p, 0, sizeof(int), ctx.stream)); }
-static void end_component(Ctx& ctx) { trg::check_timeout(ctx, trg::read_status(ctx)); }
+// The end of a component call: its products have run, and none gave up waiting.
+static void end_component(Ctx& ctx) {
+    TRG_CUDA(cudaStreamSynchronize(ctx.stream));
+    trg::check_timeout(ctx);
+}
 
 static int bad(trg_ctx* ctx, int status, const char* msg) {
     if (ctx) ctx->last_error = msg;
@@ -349,6 +391,7 @@ int trg_create(trg_ctx** out, int device, const trg_config* cfg) {
     ctx->ensure(ctx->status, 64);
     TRG_CUDA(cudaMemset(ctx->scal.p, 0, trg::SC_COUNT * sizeof(double)));
     TRG_CUDA(cudaMemset(ctx->status.p, 0, 64));
+    ctx->take_host_slot();
     *out = ctx;
     return TRG_OK;
     }
@@ -362,7 +405,7 @@ int trg_create(trg_ctx** out, int device, const trg_config* cfg) {
 int trg_destroy(trg_ctx* ctx) {
     if (!ctx) return TRG_OK;
     cudaSetDevice(ctx->device);
-    cudaStreamSynchronize(ctx->stream);
+    const bool idle = cudaStreamSynchronize(ctx->stream) == cudaSuccess;
     Ctx& c = *ctx;
     for (trg::Buf* b : {&c.T, &c.Tnext, &c.M, &c.U, &c.scal, &c.status, &c.ws, &c.envP, &c.envQ, &c.eig,
                         &c.eig_small, &c.flags, &c.split_ws, &c.f64_partial, &c.ksplit_ws, &c.bslices, &c.cons_ef, &c.field_ws, &c.Timp, &c.Timp_next,
@@ -373,7 +416,7 @@ int trg_destroy(trg_ctx* ctx) {
     for (auto& kv : c.lists) c.release(kv.second);
     c.tables.clear();
     c.lists.clear();
-    if (c.box) cudaFreeHost(c.box);
+    c.give_host_slot(idle);
     try {
         c.collect_timings();   // a context whose stream has failed still frees its resources
     } catch (const trg::Error&) {
@@ -577,7 +620,7 @@ int trg_shard_begin(trg_ctx* ctx, int Dcut, int j_begin, int j_end, double* slab
         trg::contract(*ctx, p.r, p.r, ctx->U.as<double>(), dn, o, p.precision, j_begin, j_end, j_begin);
     }
     // the slab goes to the other ranks: a timeout is this call's to report
-    trg::check_timeout(*ctx, trg::read_status(*ctx));
+    end_component(*ctx);
     ctx->shard = std::move(p);
     ctx->shard_pending = true;
     *dn_out = (int)dn;
@@ -661,7 +704,7 @@ int trg_solve3d(trg_ctx* ctx, int model, double beta, double h, int Dcut, int ns
         c.phase = TRG_PHASE_NORM;
         trg::launch_normalise(c, c.Tnext.as<double>(), kx * kx * ky * ky * Dz * Dz, k, false);
         const int st = trg::read_status(c);
-        trg::check_timeout(c, st);
+        trg::check_timeout(c);
         if (st & trg::ST_BAD_NORM)
             return bad(ctx, TRG_ENUMERIC, ("non-positive or non-finite norm at step " + std::to_string(k)).c_str());
         std::swap(c.T, c.Tnext);
@@ -730,7 +773,6 @@ int trg_environment(trg_ctx* ctx, const double* t_dev, int Dx, int Dy, double* M
     TRG_CUDA(cudaSetDevice(ctx->device));
     trg::View4 t = trg::contiguous_view(const_cast<double*>(t_dev), Dx, Dy, Dx, Dy);
     ctx->phase = TRG_PHASE_ENV;
-    begin_component(*ctx);
     trg::environment(*ctx, t, M_dev, ctx->cfg.precision);
     end_component(*ctx);
     return TRG_OK;
@@ -743,7 +785,6 @@ int trg_isometry(trg_ctx* ctx, const double* M_dev, int n, int Dcut, double* U_d
     TRG_GUARD_BEGIN
     TRG_CUDA(cudaSetDevice(ctx->device));
     const int dn_max = std::min(n, Dcut);
-    begin_component(*ctx);
     if (dn_max == n) {
         trg::launch_identity(*ctx, U_dev, n);
         *dn_out = n;
@@ -755,7 +796,7 @@ int trg_isometry(trg_ctx* ctx, const double* M_dev, int n, int Dcut, double* U_d
         *dn_out = dn;
         if (lam_host) std::memcpy(lam_host, lam.data(), sizeof(double) * (size_t)dn);
     }
-    TRG_CUDA(cudaStreamSynchronize(ctx->stream));   // (the isometry has read the status after its last product)
+    end_component(*ctx);
     return TRG_OK;
     TRG_GUARD_END(ctx)
 }
@@ -769,7 +810,6 @@ int trg_contract(trg_ctx* ctx, const double* t_dev, const double* U_dev, int Dx,
     trg::View4 t = trg::contiguous_view(const_cast<double*>(t_dev), Dx, Dy, Dx, Dy);
     trg::View4 o = trg::contiguous_view(Tx_dev, Dn, Dy, Dn, Dy);
     ctx->phase = TRG_PHASE_X1;
-    begin_component(*ctx);
     trg::contract(*ctx, t, t, U_dev, Dn, o, ctx->cfg.precision);
     end_component(*ctx);
     return TRG_OK;
@@ -790,7 +830,6 @@ int trg_gemm(trg_ctx* ctx, int M, int N, int K, const double* A, int lda, const 
     g.B.base = B; g.B.off_r = ctx->table({{K, ldb}}); g.B.off_c = ctx->table({{N, 1}}); g.B.c_fast = true;
     g.C = C; g.c_m = ctx->table({{M, ldc}}); g.c_n = ctx->table({{N, 1}}); g.beta = 0.0;
     ctx->phase = TRG_PHASE_X2;
-    begin_component(*ctx);
     trg::gemm(*ctx, g, ctx->cfg.precision);
     end_component(*ctx);
     return TRG_OK;

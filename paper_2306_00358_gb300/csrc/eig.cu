@@ -876,7 +876,7 @@ static void orthonormalise(Ctx& ctx, double* Y, int64_t n, int m, double* G, int
             TRG_LAUNCHED(ctx);
             gram(ctx, Y, Y, n, m, G, TRG_FP64);
             const unsigned long long seq = ++ctx.box_seq;
-            chol_trsm(ctx, G, Y, n, m, pass == 0 ? 1e-8 : 1e-12, false, flags, (EigBox*)ctx.box_dev, seq);
+            chol_trsm(ctx, G, Y, n, m, pass == 0 ? 1e-8 : 1e-12, false, flags, (EigBox*)ctx.box, seq);
             const EigBox& box = wait_box(ctx, seq);
             pm = box.pivmin;
             const int hb = box.nbad;
@@ -932,11 +932,7 @@ int isometry(Ctx& ctx, const double* M, int64_t n, int dcut, double* U, std::vec
     int* flags = ctx.flags.as<int>();
     int* sweeps = flags + m + 2;   // [0] FP32 sweeps, [1] FP64 sweeps of the last Rayleigh-Ritz
 
-    if (!ctx.box) {
-        TRG_CUDA(cudaHostAlloc(&ctx.box, sizeof(EigBox), cudaHostAllocMapped | cudaHostAllocPortable));
-        std::memset(ctx.box, 0, sizeof(EigBox));
-        TRG_CUDA(cudaHostGetDevicePointer(&ctx.box_dev, ctx.box, 0));
-    }
+    static_assert(HOST_SLOT_BOX + sizeof(EigBox) <= HOST_SLOT_BYTES, "isometry answers");
     int* status = ctx.status.as<int>();
     double* res_slot = ctx.scal.as<double>() + SC_RES;
     const uint64_t seed = ctx.cfg.seed ^ (0xA24BAED4963EE407ull * (uint64_t)step);
@@ -1111,7 +1107,7 @@ int isometry(Ctx& ctx, const double* M, int64_t n, int dcut, double* U, std::vec
         launch_chained(ctx, k_residual, dn_paper, 256, 0, Z, QW, theta, n, (unsigned long long*)res_slot);
         TRG_LAUNCHED(ctx);
         const unsigned long long seq = ++ctx.box_seq;
-        launch_chained(ctx, k_tell, 1, 128, 0, theta, res_slot, sweeps, status, m, (EigBox*)ctx.box_dev, seq);
+        launch_chained(ctx, k_tell, 1, 128, 0, theta, res_slot, sweeps, status, m, (EigBox*)ctx.box, seq);
         TRG_LAUNCHED(ctx);
         const EigBox& box = wait_box(ctx, seq);
         std::copy(box.theta, box.theta + m, th.begin());
@@ -1122,7 +1118,7 @@ int isometry(Ctx& ctx, const double* M, int64_t n, int dcut, double* U, std::vec
         ctx.counters[1] += 1;
         ctx.counters[2] += (uint64_t)hsw[0];
         ctx.counters[3] += (uint64_t)hsw[1];
-        check_timeout(ctx, st);
+        check_timeout(ctx);
         if (st & ST_EIG_NOCONV) fail(TRG_ENUMERIC, "Rayleigh-Ritz Jacobi did not converge");
         if (!(th[0] > 0.0) || !std::isfinite(th[0])) fail(TRG_ENUMERIC, "environment has no positive eigenvalue");
         if ((res <= tol && full) || m == n) {

@@ -830,7 +830,7 @@ bool gemm_exact(Ctx& ctx, const GemmDesc& d) {
             a.C = d.C; a.c_m = d.c_m + m0; a.c_n = d.c_n + n0;
             a.rows_fast = d.c_m_fast && !sym ? 1 : 0;
             a.sym = sym ? 1 : 0;
-            a.flags = flags; a.status = ctx.status.as<int>();
+            a.flags = flags; a.status = ctx.gave_up;
             a.weak = weak; a.weak_tile = flags + 64; a.weak_rows = mp; a.words = (a.N + 31) / 32;
             TRG_CUDA(cudaMemsetAsync(flags, 0, (size_t)flag_bytes(mp, a.N), ctx.stream));
             const int tok = ctx.region_begin(TRG_PHASE_MMA);
@@ -884,7 +884,7 @@ bool gemm_exact_pair(Ctx& ctx, const GemmDesc& d0, const GemmDesc& d1) {
     a.sym = 1;
     a.half = mp;
     a.nine = 0;
-    a.flags = flags; a.status = ctx.status.as<int>();
+    a.flags = flags; a.status = ctx.gave_up;
     a.weak = weak; a.weak_tile = flags + 64; a.weak_rows = 2 * mp; a.words = 2 * mp / 32;
     const int tok = ctx.region_begin(TRG_PHASE_MMA);
     launch_exact<15>(ctx, s, 2 * mp, s, 2 * mp, a);

@@ -32,7 +32,7 @@ enum : int {
     ST_BAD_TRACE = 2,      // trace <= 0 or NaN
     ST_EIG_NOCONV = 4,     // Jacobi sweeps exhausted
     ST_CHOL_BREAK = 8,     // Cholesky pivot could not be repaired
-    ST_TIMEOUT = 16,       // a bounded device wait ran out
+    ST_TIMEOUT = 16,       // a bounded device wait ran out (in Ctx::gave_up)
     ST_BOUNDS = 32         // a checked index fell outside its buffer (skipped)
 };
 
@@ -102,6 +102,11 @@ struct Ctx {
     Buf U;                 // isometry (n x Dn row-major)
     Buf scal;              // device scalars, see SC_* below
     Buf status;            // device status word (int)
+    // Mapped host memory that kernels write and the host reads without a copy
+    // (host_slot, api.cu): set by a product whose bounded device wait ran out
+    // (check_timeout), and the isometry's answers (EigBox, eig.cu).
+    int* gave_up = nullptr;
+    void* box = nullptr;
     std::vector<std::vector<double>> spectra;
 
     // ---- scratch
@@ -140,11 +145,10 @@ struct Ctx {
     // predecessor needed and that solve's smallest Ritz value theta_m
     struct EigHint { int64_t n = -1; int m = -1; int precision = -1; int products = 0; double theta_m = 0.0; };
     EigHint eig_hint[2];
-    // mapped host memory the isometry's kernels answer to (EigBox, eig.cu)
-    void* box = nullptr;
-    void* box_dev = nullptr;
     unsigned long long box_seq = 0;
     cudaEvent_t get_event();
+    void take_host_slot();
+    void give_host_slot(bool idle);
     // Record the start of a timed region of phase p (no-op unless profiling).
     int region_begin(int p);
     void region_end(int token, double flops, double mma_flops);
@@ -156,6 +160,7 @@ struct Ctx {
     void release(Buf& b);
     const int64_t* table(const std::vector<std::pair<int64_t, int64_t>>& modes);
 };
+constexpr size_t HOST_SLOT_BYTES = 2048, HOST_SLOT_BOX = 64;    // bytes of a slot; the box's offset
 
 // Device scalar slots (doubles) in Ctx::scal.
 enum : int {
@@ -299,9 +304,9 @@ std::pair<int64_t, int64_t> step3(Ctx& ctx, const View6& t, int dcut, int step, 
                                   std::vector<double>& lam_x, std::vector<double>& lam_y);
 
 int read_status(Ctx& ctx);  // synchronises the stream
-// Throws TRG_ETIMEOUT, with the status word cleared for the next call, if the
-// status st that was read says that a bounded device wait ran out.
-void check_timeout(Ctx& ctx, int st);
+// Throws TRG_ETIMEOUT, with the word cleared for the next call, if a bounded
+// device wait ran out (the stream has been synchronised).
+void check_timeout(Ctx& ctx);
 void trim_buffers(Ctx& ctx);  // free every solve buffer (engine.cu)
 
 }  // namespace trg

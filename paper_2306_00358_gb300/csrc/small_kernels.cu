@@ -341,9 +341,9 @@ int read_status(Ctx& ctx) {
     return st;
 }
 
-void check_timeout(Ctx& ctx, int st) {
-    if (!(st & ST_TIMEOUT)) return;
-    TRG_CUDA(cudaMemsetAsync(ctx.status.p, 0, sizeof(int), ctx.stream));
+void check_timeout(Ctx& ctx) {
+    if (!__atomic_load_n(ctx.gave_up, __ATOMIC_ACQUIRE)) return;
+    *ctx.gave_up = 0;
     fail(TRG_ETIMEOUT, "device wait timed out");
 }
 

@@ -1129,7 +1129,7 @@ void gemm_split(Ctx& ctx, const GemmDesc& d) {
     MmaArgs a;
     a.M = M; a.N = N; a.Kp = Kp; a.Mp = Mp; a.Np = Np; a.S = S;
     a.ea = ea; a.eb = eb; a.C = d.C; a.c_m = d.c_m; a.c_n = d.c_n;
-    a.status = ctx.status.as<int>();
+    a.status = ctx.gave_up;
     a.acc_wait_ns = ctx.acc_wait_ns ? ctx.acc_wait_ns : WAIT_NS;
     a.cons_ef = d.cons_ef; a.cons_m = d.cons_m; a.cons_n = d.cons_n;
     a.c_rows_fast = d.c_m_fast ? 1 : 0;
