@@ -29,12 +29,17 @@
 //    returns at once if there is none).  In FP64 solves at the critical point no
 //    sum lies below 2^-54; far from it, once the tensor has flowed to a fixed
 //    point, 2 to 40 % of them do;
-//  - 9 digits (45 digit products) do it if no sum |a||b| lies between 0 and 2^-8
-//    2^(ea + eb): they leave out less than K 2^-60 |a||b| then, which is also
-//    below what the roundings of an FP64 sum amount to when their signs are
-//    random.  A kernel takes all of |A||B| first and raises a flag where 9 do
-//    not suffice; the two product kernels read it, and the one that is not
-//    wanted returns at once.
+//  - 9 digits (45 digit products) do it if the sum |a||b| does not lie between 0
+//    and 2^-8 2^(ea + eb): they leave out less than K 2^-60 |a||b| then, which is
+//    also below what the roundings of an FP64 sum amount to when their signs are
+//    random.  A kernel takes all of |A||B| first and marks the rows with a sum
+//    for which 9 do not suffice (the columns, where the product is a slab of
+//    columns; the whole of a Gram product).  The nine-digit kernel stores the
+//    others, the fifteen-digit kernel these, and each leaves out the tiles that
+//    hold none of its own.  A row's decision is its own, so an element has the
+//    same bits whatever slab or block of the product it is computed in.  (By
+//    tiles there would be less to compute twice, but tiles begin where a slab
+//    does.)
 //
 // What bounds it: the tensor pipe (9 digits in a long product: active 62 % of
 // the time, with MMA instructions of N = 48 .. 240; a tenth goes to drains that
@@ -140,6 +145,7 @@ __device__ __forceinline__ uint64_t smem_desc32(uint32_t addr) {
     return d;
 }
 
+enum Scope { NONE = 0, ROWS = 1, COLUMNS = 2, WHOLE = 3 };
 struct XArgs {
     int M, N, Kp;
     const int* fa;                 // largest exponent field of each A row
@@ -152,11 +158,16 @@ struct XArgs {
     const long long* tile_list;    // mb << 32 | nb, or nullptr for all
     int n_list;
     int group_n;                   // tile order: column blocks per group
-    int* flags;                    // [0] some element is left to the FP64 pipe, [1] nine digits do not suffice
+    int* flags;                    // [0] some element is left to the FP64 pipe, [1] / [2] some need / do not need 15 digits
+    // Which elements need 15 digits, if nine are tried: those of the rows (ROWS),
+    // of the columns (COLUMNS) or of the product (WHOLE) with need[] set; state[]
+    // says it for the tiles, 1: some do, 2: some do not.
+    int scope;
+    int* need;
+    const int* state;
     uint32_t* weak;                // the elements left to it: bit n % 32 of weak[(n / 32) weak_rows + m]
     int* weak_tile;                // ... does the 128 x 32 tile (m / 128) words + n / 32 hold one
     int weak_rows, words;
-    int nine;                      // the nine-digit form has been tried
     // a second Gram product of the same size: its rows are those from half on
     // (0: none), its tiles are in tile_list too
     int half;
@@ -217,7 +228,7 @@ __global__ void __launch_bounds__(XT<S>::THREADS, 1)
 k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const XArgs g) {
     constexpr int XN = XT<S>::N, XK = XT<S>::K, XL = XT<S>::L, XSTAGES = XT<S>::STAGES, XSTAGE = XT<S>::STAGE;
     constexpr int XA_TILE = XT<S>::A_TILE, XKB = XT<S>::KB, XB_TILE = XT<S>::B_TILE, XRUN = XT<S>::RUN, XCPT = XT<S>::CPT;
-    if ((S == 9 && g.flags[1]) || (S == 15 && g.nine && !g.flags[1])) return;
+    if ((S == 9 && !g.flags[2]) || (S == 15 && g.scope && !g.flags[1])) return;
     constexpr int XP = XT<S>::P;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -248,6 +259,17 @@ k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         }
     };
 
+    // What the tile holds (state[]): this kernel computes those with the bit MINE.
+    // Its roles ask for the next tile while they work on the present one.
+    constexpr int MINE = S == 9 ? 2 : 1;
+    const bool mixed = S != 1 && g.scope && g.flags[1] && g.flags[2];     // (else every tile is this kernel's)
+    auto state_of = [&](int tile) {
+        if (!mixed || tile >= num_tiles) return MINE;
+        int mb, nb;
+        coords(tile, mb, nb);
+        return g.state[g.scope == ROWS ? mb : g.scope == COLUMNS ? nb : 0];
+    };
+
     if (threadIdx.x == 0) {
         for (int s = 0; s < XSTAGES; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
         for (int q = 0; q < 2; ++q) { mbar_init(&acc_full[q], 1); mbar_init(&acc_empty[q], XT<S>::EPI); }
@@ -274,7 +296,11 @@ k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
 #pragma unroll
             for (int s = 0; s < XSTAGES; ++s) issued[s] = -1;
             bool ok = true;
+            int ahead = state_of(blockIdx.x);
             for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
+                const int now = ahead;
+                ahead = state_of(tile + gridDim.x);
+                if (!(now & MINE)) continue;
                 int mb, nb;
                 coords(tile, mb, nb);
                 for (int kb = 0; kb < num_kb; ++kb) {
@@ -302,7 +328,11 @@ k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             uint32_t phase = 0;
             uint32_t run_no = 0;        // runs begun so far (all tiles)
             bool ok = true;
+            int ahead = state_of(blockIdx.x);
             for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
+                const int now = ahead;
+                ahead = state_of(tile + gridDim.x);
+                if (!(now & MINE)) continue;
                 for (int kb = 0; kb < num_kb; ++kb) {
                     const bool run_start = kb % XRUN == 0;
                     const bool run_end = (kb + 1) % XRUN == 0 || kb + 1 == num_kb;
@@ -362,33 +392,53 @@ k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         uint32_t run_no = 0;
         bool ok = true;
         for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
+            // (read under the tile's first run of products)
+            const int now = state_of(tile);
+            if (!(now & MINE)) continue;
             int mb, nb;
             coords(tile, mb, nb);
             if constexpr (S == 1) {
-                // the sums of |a||b|: is any of them small, or outside the digits' range?
+                // the sums of |a||b|: which are small, or outside the digits' range?
+                const int row = mb * XM + quad * 32 + lane, col0 = nb * XN + colq * XCPT;
+                const bool row_out = row < g.M && field_outside(g.fa[row]);
+                unsigned col_out = 0;        // bit h: column col0 + 32 h + lane
+#pragma unroll
+                for (int h = 0; h < XCPT / 32; ++h)
+                    if (col0 + h * 32 + lane < g.N && field_outside(g.fb[col0 + h * 32 + lane])) col_out |= 1u << h;
                 int w_ok = 1;
                 if (lane == 0) w_ok = mbar_wait(&acc_full[1], run_no & 1, abort_flag, g.status, g.acc_wait_ns) ? 1 : 0;
                 ok = __shfl_sync(0xffffffffu, w_ok, 0) != 0;
                 if (!ok) break;
                 tc_fence_after();
-                const int row = mb * XM + quad * 32 + lane;
-                bool small = row < g.M && field_outside(g.fa[row]);
-#pragma unroll
-                for (int h = 0; h < XCPT / 32; ++h) {
-                    const int col = nb * XN + colq * XCPT + h * 32 + lane;
-                    small |= col < g.N && field_outside(g.fb[col]);
-                }
+                bool small = row_out;
 #pragma unroll
                 for (int h = 0; h < XCPT / 8; ++h) {
                     uint32_t r[8];
                     tmem_ld8(tmem + lane_base + (uint32_t)(colq * XCPT + h * 8), r);
                     tmem_wait_ld();
                     tmem_arrived(r);
+                    if (g.scope == COLUMNS) {
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) small |= sum_below(r[j], SUM9_MIN);
+                        for (int j = 0; j < 8; ++j)
+                            if (__any_sync(0xffffffffu, row_out || sum_below(r[j], SUM9_MIN)) && lane == j &&
+                                col0 + h * 8 + j < g.N)
+                                g.need[col0 + h * 8 + j] = 1;
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) small |= sum_below(r[j], SUM9_MIN);
+                    }
                 }
                 tc_fence_before();
-                if (__any_sync(0xffffffffu, small) && lane == 0) g.flags[1] = 1;
+                if (g.scope == COLUMNS) {
+#pragma unroll
+                    for (int h = 0; h < XCPT / 32; ++h)
+                        if (col_out >> h & 1u) g.need[col0 + h * 32 + lane] = 1;
+                } else {
+                    small |= __any_sync(0xffffffffu, col_out != 0);    // (every row meets that column)
+                }
+                if (g.scope == ROWS && small && row < g.M) g.need[row] = 1;
+                if (g.scope == WHOLE && small) g.need[0] = 1;
+                __syncwarp();
                 if (lane == 0) mbar_arrive(&acc_empty[1]);
                 ++run_no;
             } else {
@@ -398,6 +448,19 @@ k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             for (int j = 0; j < XCPT; ++j)
 #pragma unroll
                 for (int q = 0; q < XT<S>::LIMBS; ++q) w[j][q] = 0;
+            // The columns of this thread's row that this kernel stores, kept in the
+            // store staging until they are needed: the sums take the registers.
+            uint32_t* const keep_slot = (uint32_t*)(staging + ew * (32 * 8)) + lane;
+            if (mixed) {
+                unsigned k = ~0u;
+                const int i = g.scope == ROWS ? mb * XM + quad * 32 + lane : nb * XN + colq * XCPT + lane;
+                const bool in = g.scope == ROWS ? i < g.M : lane < XCPT && i < g.N;
+                if (now != MINE && g.scope != WHOLE) {
+                    const bool mine = in && (g.need[i] != 0) == (S == 15);
+                    k = g.scope == ROWS ? (mine ? ~0u : 0u) : __ballot_sync(0xffffffffu, mine);
+                }
+                *keep_slot = k;
+            }
             unsigned weak = 0;      // columns of this thread's row that 15 digits do not suffice for
             for (int c = 0; c < nruns && ok; ++c, ++run_no) {
 #pragma unroll
@@ -460,13 +523,15 @@ k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             const bool col_in = lane < XCPT && nt + lane < g.N;
             const int fb = col_in ? g.fb[nt + lane + r0] : 0;
             const long long cn_l = col_in ? (long long)c_n[nt + lane] : 0;
+            const unsigned keep = mixed ? *(volatile uint32_t*)keep_slot : ~0u;
+            __syncwarp();            // (the staging is written below)
             const int fa = row_ok ? g.fa[m + r0] : 0;
             const int ea = max(fa, 1) - 1022;
             if constexpr (XT<S>::SUM) {
                 weak |= __ballot_sync(0xffffffffu, field_outside(fb));
                 if (field_outside(fa)) weak = ~0u;
                 // of the elements that are stored
-                if (!row_ok) weak = 0;
+                weak = row_ok ? weak & keep : 0u;
                 weak &= (1u << max(0, min(XCPT, g.N - nt))) - 1u;
                 if (g.sym) weak &= ~0u << max(0, min(XCPT, m - nt));
                 static_assert(!XT<S>::SUM || (XN == 32 && XCPT == 8), "a byte of a word per thread");
@@ -481,7 +546,7 @@ k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                 for (int j = 0; j < XCPT; ++j) {
                     const int e2 = ea + __shfl_sync(0xffffffffu, eb_l, j);
                     const long long cn = __shfl_sync(0xffffffffu, cn_l, j);
-                    if (row_ok && nt + j < g.N) cp[cn] = wide_to_double(w[j], e2);
+                    if (row_ok && nt + j < g.N && (keep >> j & 1u)) cp[cn] = wide_to_double(w[j], e2);
                 }
                 continue;
             }
@@ -497,7 +562,7 @@ k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
 #pragma unroll
                 for (int j = 0; j < XCPT; ++j) {
                     const int n = nt + j;
-                    if (n < g.N && n > m) C[c_m[n] + cm_mirror] = v[j];
+                    if (n < g.N && n > m && (keep >> j & 1u)) C[c_m[n] + cm_mirror] = v[j];
                 }
             }
             // columns adjacent in C: through the warp's 32 x 8 staging tile, so
@@ -515,7 +580,8 @@ k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                 for (int q = 0; q < 8; ++q) {
                     const int rr = 4 * q + quarter;
                     const int mr = mb * XM + quad * 32 + rr - r0;
-                    if (mr < g.M && n < g.N && (!g.sym || n >= mr))
+                    const unsigned kr = __shfl_sync(0xffffffffu, keep, rr);
+                    if (mr < g.M && n < g.N && (!g.sym || n >= mr) && (kr >> (pass * 8 + cl) & 1u))
                         C[c_m[mr] + cn] = stg[rr * 8 + (cl ^ ((rr >> 1) & 7))];
                 }
                 __syncwarp();
@@ -631,6 +697,27 @@ __global__ void __launch_bounds__(WT, 2) k_weak_f64(const WeakArgs g) {
     }
 }
 
+// Which tiles hold rows (columns) that need 15 digits (1) and which hold others
+// (2): out9 for the tiles of the nine-digit kernel, t9 rows (columns) long, out15
+// for the other's; flags[1] and flags[2] for all of them.
+__global__ void __launch_bounds__(256) k_need_tiles(const int* need, int count, int t9, int* out9, int t15, int* out15,
+                                                    int* flags) {
+    const int t = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;      // a warp per tile
+    auto state = [&](int side) {
+        unsigned s = 0;
+        for (int i = t * side + lane; i < min(count, (t + 1) * side); i += 32) s |= need[i] ? 1u : 2u;
+        return (int)__reduce_or_sync(0xffffffffu, s);
+    };
+    const int s9 = state(t9), s15 = state(t15);
+    if (lane != 0) return;
+    if (t * t9 < count) out9[t] = s9;
+    if (t * t15 < count) {
+        out15[t] = s15;
+        if (s15 & 1) flags[1] = 1;
+        if (s15 & 2) flags[2] = 1;
+    }
+}
+
 // ------------------------------------------------------------- host side ---
 // `count` planes from plane `first` on of the digits [kp / 16][XPLANES][rows][16]
 // (their order in a stage: no swizzle here), four rows to a 128-byte line,
@@ -706,13 +793,17 @@ XBlock block_rows(int64_t M, int64_t N, int64_t kp) {
 // Bytes of the flags, the weak tiles and the weak bits of an a x b block.
 int64_t flag_bytes(int64_t a, int64_t b) { return up(256 + 4 * (a / XM) * (up(b, 32) / 32), 256); }
 int64_t weak_bytes(int64_t a, int64_t b) { return 4 * a * (up(b, 32) / 32); }
+// ... and of need[] and state[] of a product of M x N in such blocks.
+int64_t need_bytes(int64_t M, int64_t N) { return 4 * std::max(M, N); }
+int64_t state_bytes(int64_t a, int64_t b) { return 4 * (std::max(a, b) / 32 + 1); }
 
 }  // namespace
 
 int64_t exact_scratch_bytes(int64_t M, int64_t N, int64_t K) {
     const int64_t kp = up(std::max<int64_t>(K, 1), XKP);
     const XBlock x = block_rows(M, N, kp);
-    return 2 * XPLANES * kp * (x.a + x.b) + 4 * (x.a + x.b) + flag_bytes(x.a, x.b) + weak_bytes(x.a, x.b) + 2048;
+    return 2 * XPLANES * kp * (x.a + x.b) + 4 * (x.a + x.b) + flag_bytes(x.a, x.b) + weak_bytes(x.a, x.b) +
+           need_bytes(M, N) + 2 * state_bytes(x.a, x.b) + 4096;
 }
 
 int64_t exact_pair_scratch_bytes(int64_t M, int64_t K) {
@@ -728,7 +819,7 @@ double tiles_of(int64_t M, int64_t N, int xn, bool sym) {
 double us15(const Ctx& ctx, int64_t M, int64_t N, int64_t K, bool sym) {
     return std::ceil(tiles_of(M, N, XT<15>::N, sym) / ctx.sm_count) * (std::ceil((double)K / 64.0) * 4.4 + 3.0);
 }
-// Whether to look for the nine-digit form: the check and the two more launches
+// Whether to look for the nine-digit form: the check and the three more launches
 // have to be made good.
 bool try_nine(const Ctx& ctx, int64_t M, int64_t N, int64_t K, bool sym) {
     if (K > XNINE_K) return false;
@@ -804,49 +895,73 @@ bool gemm_exact(Ctx& ctx, const GemmDesc& d) {
     uint8_t* p = ctx.split_ws.as<uint8_t>();
     auto take = [&](size_t bytes) { uint8_t* q = p; p += (bytes + 255) & ~(size_t)255; return q; };
     int* flags = (int*)take((size_t)flag_bytes(ra, rb));
+    int* need = (int*)take((size_t)need_bytes(d.M, d.N));     // (cleared with the flags)
     uint32_t* weak = (uint32_t*)take((size_t)weak_bytes(ra, rb));
     int* fa = (int*)take((size_t)ra * 4);
     int* fb = sym ? fa : (int*)take((size_t)rb * 4);
+    int* state9 = (int*)take((size_t)state_bytes(ra, rb));
+    int* state15 = (int*)take((size_t)state_bytes(ra, rb));
     uint16_t* sa = (uint16_t*)take((size_t)(2 * XPLANES) * ra * Kp);
     uint16_t* sb = sym ? sa : (uint16_t*)take((size_t)(2 * XPLANES) * rb * Kp);
 
+    // Nine digits or fifteen: one decision for a row (a column, if the product is
+    // a slab of columns), so that it is the same from every slab and block; one
+    // for all of a Gram product, which is symmetric.
+    const int scope = !try_nine(ctx, d.choice_m(), d.choice_n(), K, d.gram) ? NONE : d.gram ? WHOLE : d.whole_n ? COLUMNS : ROWS;
+    TRG_CUDA(cudaMemsetAsync(flags, 0, (size_t)(flag_bytes(ra, rb) + (scope ? need_bytes(d.M, d.N) : 0)), ctx.stream));
+    bool cleared = true;      // the flags, for the next block
+    const bool one_a = ra >= d.M, one_b = rb >= d.N;      // (an operand cut once)
+    const bool check_first = scope && !(one_a && one_b) && !(scope == ROWS && one_b) && !(scope == COLUMNS && one_a);
     // B as rows n, columns k
     const Gather bt = transposed(d.B);
-    for (int64_t m0 = 0; m0 < d.M; m0 += ra) {
-        const int mr = (int)std::min(ra, d.M - m0), mp = (int)up(mr, XM);
-        Gather ga = d.A;
-        ga.off_r += m0;
-        digits(ctx, ga, mr, K, mp, Kp, fa, sa, mp);
-        for (int64_t n0 = 0; n0 < d.N; n0 += rb) {
-            const int nr = (int)std::min(rb, d.N - n0), np = sym ? mp : (int)up(nr, XNP);
-            if (!sym && (m0 == 0 || rb < d.N)) {
-                Gather gb = bt;
-                gb.off_r += n0;
-                digits(ctx, gb, nr, K, np, Kp, fb, sb, np);
+    auto blocks = [&](bool check, bool products) {
+        for (int64_t m0 = 0; m0 < d.M; m0 += ra) {
+            const int mr = (int)std::min(ra, d.M - m0), mp = (int)up(mr, XM);
+            Gather ga = d.A;
+            ga.off_r += m0;
+            digits(ctx, ga, mr, K, mp, Kp, fa, sa, mp);
+            for (int64_t n0 = 0; n0 < d.N; n0 += rb) {
+                const int nr = (int)std::min(rb, d.N - n0), np = sym ? mp : (int)up(nr, XNP);
+                if (!sym && (m0 == 0 || !one_b)) {
+                    Gather gb = bt;
+                    gb.off_r += n0;
+                    digits(ctx, gb, nr, K, np, Kp, fb, sb, np);
+                }
+                XArgs a;
+                a.M = mr; a.N = sym ? mr : nr; a.Kp = Kp;
+                a.fa = fa; a.fb = fb;
+                a.C = d.C; a.c_m = d.c_m + m0; a.c_n = d.c_n + n0;
+                a.rows_fast = d.c_m_fast && !sym ? 1 : 0;
+                a.sym = sym ? 1 : 0;
+                a.half = 0;
+                a.flags = flags; a.status = ctx.gave_up;
+                a.weak = weak; a.weak_tile = flags + 64; a.weak_rows = mp; a.words = (a.N + 31) / 32;
+                a.scope = scope;
+                a.need = need + (scope == ROWS ? m0 : scope == COLUMNS ? n0 : 0);
+                a.state = nullptr;
+                if (check) launch_exact<1>(ctx, sa, mp, sb, np, a);
+                if (!products) continue;
+                if (!cleared) TRG_CUDA(cudaMemsetAsync(flags, 0, (size_t)flag_bytes(mp, a.N), ctx.stream));
+                cleared = false;
+                const int tok = ctx.region_begin(TRG_PHASE_MMA);
+                if (scope) {
+                    const int count = scope == ROWS ? mr : scope == COLUMNS ? nr : 1;
+                    const int t9 = scope == COLUMNS ? XT<9>::N : XM, t15 = scope == COLUMNS ? XT<15>::N : XM;
+                    const int tiles = (count + t15 - 1) / t15;
+                    k_need_tiles<<<(tiles + 7) / 8, 256, 0, ctx.stream>>>(a.need, count, t9, state9, t15, state15, flags);
+                    TRG_LAUNCHED(ctx);
+                    a.state = state9;
+                    launch_exact<9>(ctx, sa, mp, sb, np, a);
+                    a.state = state15;
+                }
+                launch_exact<15>(ctx, sa, mp, sb, np, a);
+                ctx.region_end(tok, 2.0 * (double)mr * nr * K, (scope ? 45.0 : 120.0) * 2.0 * (double)mr * nr * Kp);   // 120 also if nine do not suffice
+                launch_weak(ctx, d, d, m0, n0, a);
             }
-            XArgs a;
-            a.M = mr; a.N = sym ? mr : nr; a.Kp = Kp;
-            a.fa = fa; a.fb = fb;
-            a.C = d.C; a.c_m = d.c_m + m0; a.c_n = d.c_n + n0;
-            a.rows_fast = d.c_m_fast && !sym ? 1 : 0;
-            a.sym = sym ? 1 : 0;
-            a.flags = flags; a.status = ctx.gave_up;
-            a.weak = weak; a.weak_tile = flags + 64; a.weak_rows = mp; a.words = (a.N + 31) / 32;
-            TRG_CUDA(cudaMemsetAsync(flags, 0, (size_t)flag_bytes(mp, a.N), ctx.stream));
-            const int tok = ctx.region_begin(TRG_PHASE_MMA);
-            const bool nine = try_nine(ctx, a.M, a.N, K, sym);
-            a.nine = nine ? 1 : 0;
-            a.half = 0;
-            if (nine) {
-                launch_exact<1>(ctx, sa, mp, sb, np, a);
-                launch_exact<9>(ctx, sa, mp, sb, np, a);
-            }
-            launch_exact<15>(ctx, sa, mp, sb, np, a);
-            ctx.region_end(tok, 2.0 * (double)mr * nr * K, (nine ? 45.0 : 120.0) * 2.0 * (double)mr * nr * Kp);   // 120 also if nine do not suffice
-            launch_weak(ctx, d, d, m0, n0, a);
-            if (sym) break;
         }
-    }
+    };
+    if (check_first) blocks(true, false);
+    blocks(scope && !check_first, true);
     return true;
 }
 
@@ -883,7 +998,9 @@ bool gemm_exact_pair(Ctx& ctx, const GemmDesc& d0, const GemmDesc& d1) {
     a.rows_fast = 0;
     a.sym = 1;
     a.half = mp;
-    a.nine = 0;
+    a.scope = NONE;
+    a.need = nullptr;
+    a.state = nullptr;
     a.flags = flags; a.status = ctx.gave_up;
     a.weak = weak; a.weak_tile = flags + 64; a.weak_rows = 2 * mp; a.words = 2 * mp / 32;
     const int tok = ctx.region_begin(TRG_PHASE_MMA);

@@ -146,14 +146,14 @@ __global__ void k_reduce_partials(const double* __restrict__ P, int nz, int64_t 
 // dealt evenly over the SMs, each K stage costs the latency of its loads
 // unless several blocks share the SM, and split K adds a second launch.
 struct Shape { int T; int64_t nz; double clocks; };
-Shape choose_shape(int64_t M, int64_t N, int64_t K, int sms, bool sym) {
+Shape choose_shape(int64_t M, int64_t N, int64_t K, int sms, bool sym, int64_t max_nz = 64) {
     Shape best{64, 1, 0.0};
     double best_t = 1e300;
     for (int T : {64, 32, 16, 8}) {
         const int bk = T == 64 ? 16 : T == 8 ? 64 : 32;
         const int64_t gx = (N + T - 1) / T, gy = (M + T - 1) / T;
         const double tiles = sym ? 0.5 * (double)gx * (double)(gx + 1) : (double)gx * (double)gy;
-        for (int64_t nz = 1; nz <= 64; nz *= 2) {
+        for (int64_t nz = 1; nz <= max_nz; nz *= 2) {
             if (nz > 1 && (K / nz < 128 || (double)nz * M * N * 8 > (double)(4 << 20))) break;
             const double kper = std::ceil((double)K / nz / bk) * bk;
             const double per_sm = std::ceil(tiles * nz / sms);
@@ -204,7 +204,12 @@ void gemm_f64(Ctx& ctx, const GemmDesc& d) {
     // a Gram product's C(n, m) sums the products of C(m, n) in the same order
     g.sym = (d.gram && d.M == d.N && d.beta == 0.0) ? 1 : 0;
     if ((d.M + 63) / 64 > 65535) fail(TRG_EINVAL, "gemm_f64: too many row tiles");
-    const Shape s = choose_shape(d.M, d.N, std::max<int64_t>(d.K, 1), ctx.sm_count, g.sym != 0);
+    // The K parts (whose length follows the tile) change bits, the tile alone
+    // does not: a slab takes the parts of its whole product, and without any the
+    // tile of its own size.
+    const int64_t k = std::max<int64_t>(d.K, 1);
+    Shape s = choose_shape(d.choice_m(), d.choice_n(), k, ctx.sm_count, g.sym != 0);
+    if (s.nz == 1) s = choose_shape(d.M, d.N, k, ctx.sm_count, g.sym != 0, 1);
     switch (s.T) {
         case 64: launch<64, 4, 16, 256>(ctx, g, s.nz); break;
         case 32: launch<32, 2, 32, 256>(ctx, g, s.nz); break;

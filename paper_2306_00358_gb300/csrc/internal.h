@@ -200,6 +200,14 @@ struct GemmDesc {
     // FP64 mode: the product may run on the tensor cores when it is large
     // enough (gemm_exact).
     bool allow_exact = false;
+    // The product is a slab, some rows (whole_m > 0) or columns (whole_n > 0), of
+    // one with so many: a slice of j's of a contraction, whose extent depends on
+    // the workspace and on the rank.  Choices that change bits (digits or pipe,
+    // nine or fifteen of them, split K) are those of the whole product, so that
+    // an element comes out the same from every slab.
+    int64_t whole_m = 0, whole_n = 0;
+    int64_t choice_m() const { return whole_m ? whole_m : M; }
+    int64_t choice_n() const { return whole_n ? whole_n : N; }
     // consecutive rows are (mostly) adjacent in C: the epilogues store row-wise,
     // without staging.  The consumer rows cons_m + cons_n are below 2^31.
     bool c_m_fast = false;

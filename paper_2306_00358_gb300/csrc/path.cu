@@ -79,8 +79,9 @@ void gemm_split(Ctx& ctx, const GemmDesc& g);  // split_gemm.cu
 // against more than 30.
 static bool takes_exact(const Ctx& ctx, const GemmDesc& g) {
     const bool sym = g.gram && g.M == g.N;
+    const int64_t M = g.choice_m(), N = g.choice_n();
     return g.allow_exact && !ctx.no_exact && g.beta == 0.0 && g.M > 0 && g.N > 0 &&
-           exact_us(ctx, g.M, g.N, g.K, sym) < 0.8 * f64_us(ctx, g.M, g.N, g.K, sym);
+           exact_us(ctx, M, N, g.K, sym) < 0.8 * f64_us(ctx, M, N, g.K, sym);
 }
 
 void gemm(Ctx& ctx, const GemmDesc& g, int precision) {
@@ -244,6 +245,7 @@ void contract(Ctx& ctx, const View4& top, const View4& bottom, const double* U, 
             ctx.phase = TRG_PHASE_X1;
             GemmDesc g;
             g.M = Dx * Dn; g.N = jn * DD; g.K = Dx;
+            g.whole_n = Dy * DD;
             g.allow_exact = true;
             g.A = a1;
             g.a_slices = p1.s;
@@ -268,6 +270,7 @@ void contract(Ctx& ctx, const View4& top, const View4& bottom, const double* U, 
             GemmDesc g;
             g.allow_exact = true;
             g.M = M2; g.N = DD; g.K = DD;
+            g.whole_m = Dy * Dn * Dx;
             g.A = gather(ctx, X1, {{jb * Dn * Dx, DD}}, {{DD, 1}});
             g.B = b2;
             g.b_slices = p2.s;
@@ -292,6 +295,7 @@ void contract(Ctx& ctx, const View4& top, const View4& bottom, const double* U, 
             g.allow_exact = true;
             g.c_m_fast = o[3] == 1;
             g.M = M3; g.N = Dn; g.K = Dx * Dx;
+            g.whole_m = Dy * Dn * Dy;
             g.A = gather(ctx, X2, {{jb * Dn * Dy, Dx * Dx}}, {{Dx * Dx, 1}});
             g.B = b3;
             g.b_slices = p3.s;
