@@ -87,7 +87,10 @@ typedef struct trg_config {
                                 TRG_SPLIT_BF16 at least 2^-(8*S-10), S = the env slices) */
     int eig_max_iter;        /* subspace iterations before TRG_ENUMERIC (default 300) */
     uint64_t seed;           /* seed of the start block of the subspace iteration */
-    size_t workspace_bytes;  /* bound on the contraction workspace (0 = 4 GiB) */
+    size_t workspace_bytes;  /* bound on the contraction workspace (0 = 4 GiB).  TRG_FP64: the digits
+                                of a product that runs on the tensor cores take as much again, but
+                                256 MiB .. 2 GiB (2 GiB for 0), and less where that cannot be had;
+                                results do not depend on it */
     int mma_pairs;           /* TRG_SPLIT_BF16: 1 (default) runs products with more than 128
                                 rows on CTA pairs (256-row tiles, cta_group::2: every
                                 tensor-core instruction drives two SMs, each staging half

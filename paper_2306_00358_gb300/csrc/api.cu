@@ -54,7 +54,16 @@ void Ctx::ensure(Buf& b, size_t bytes) {
         b.bytes = 0;
     }
     const size_t sz = std::max<size_t>(bytes, 256);
-    b.p = raw_alloc(sz);
+    try {
+        b.p = raw_alloc(sz);
+    } catch (const Error& e) {
+        // the products' scratch is only kept for the next one, which makes do
+        // with less: it goes first
+        if (e.status != TRG_ENOMEM || &b == &split_ws || !split_ws.p || split_ws_users) throw;
+        TRG_CUDA(cudaStreamSynchronize(stream));
+        release(split_ws);
+        b.p = raw_alloc(sz);
+    }
     b.bytes = sz;
 }
 

@@ -34,8 +34,9 @@ double secs(Clock::time_point a, Clock::time_point b) { return std::chrono::dura
 // Device bytes one solve can hold at its largest half-step: tensors, the
 // environment and its two intermediates, isometry, subspace-iteration blocks,
 // the contraction workspace and the split-GEMM scratch.  An upper bound.
-// exact: FP64 products may run on the tensor cores (their digits count).
-size_t estimate_bytes(const trg_solve_spec& s, size_t workspace_cap, bool exact) {
+// digit_cap: bound on the digits of FP64 products that run on the tensor cores
+// (0: none do).
+size_t estimate_bytes(const trg_solve_spec& s, size_t workspace_cap, int64_t digit_cap) {
     const double d0 = (s.model == TRG_ISING) ? 2 : std::max(1, s.D0);
     const double D = std::max<double>(d0, std::min<double>(s.Dcut, std::max(d0 * d0, (double)s.Dcut)));
     const double D2 = D * D, D4 = D2 * D2;
@@ -62,16 +63,16 @@ size_t estimate_bytes(const trg_solve_spec& s, size_t workspace_cap, bool exact)
                  3 * (D2 + 256) * 4 + 3 * 256.0;            // their exponents, alignment
         // split-K parts of the isometry's products: at most 152 x 128 rows x m
         bytes += 152.0 * 128 * m * 8;
-    } else if (exact) {
+    } else if (digit_cap) {
         // the digits of the largest FP64 product: environment, U.T.T.U in
         // blocks of j, M.Q of the isometry
         const double jb = std::max(1.0, std::floor(ws / std::max(1.0, 2 * D * D * D2 * 8)));
         const int64_t d = (int64_t)D, d2 = d * d, rows = (int64_t)std::min(D, jb) * d2;
-        bytes += (double)std::max({trg::exact_scratch_bytes(d2, d2, d2), trg::exact_scratch_bytes(d2, rows, d),
+        auto scratch = [&](int64_t M, int64_t N, int64_t K) { return trg::exact_scratch_bytes(M, N, K, digit_cap); };
+        bytes += (double)std::max({scratch(d2, d2, d2), scratch(d2, rows, d),
                                    // (two Gram products share a launch up to 640 rows)
-                                   trg::exact_pair_scratch_bytes(std::min<int64_t>(d2, 640), d2),
-                                   trg::exact_scratch_bytes(rows, d2, d2), trg::exact_scratch_bytes(rows, d, d2),
-                                   trg::exact_scratch_bytes(d2, (int64_t)m, d2)});
+                                   std::min(digit_cap, trg::exact_pair_scratch_bytes(std::min<int64_t>(d2, 640), d2)),
+                                   scratch(rows, d2, d2), scratch(rows, d, d2), scratch(d2, (int64_t)m, d2)});
     }
     bytes += 64.0 * 1024 * 1024;               // tables, scalars, allocator slack
     return (size_t)bytes;
@@ -87,7 +88,8 @@ struct Request {
     uint64_t ticket = 0;
     trg_solve_spec spec{};
     size_t bytes = 0;
-    bool no_exact = false;   // see Ctx::no_exact
+    bool no_exact = false;   // see Ctx::no_exact, Ctx::digit_bytes
+    size_t digit_bytes = 0;
     double work = 0.0;
     Clock::time_point t_submit, t_start, t_end;
     enum { QUEUED, RUNNING, DONE, CANCELLED } state = QUEUED;
@@ -161,6 +163,7 @@ void trg_server::run_request(trg_ctx*& ctx, Request* r) {
     int st = trg_set_precision(ctx, s.precision, s.precision == TRG_SPLIT_BF16 ? s.split_slices : 4, 0);
     if (st == TRG_OK) {
         ctx->no_exact = r->no_exact;
+        ctx->digit_bytes = r->digit_bytes;
         ctx->cfg.trunc = s.trunc;
         ctx->cfg.seed = s.seed ? s.seed : 0x5EEDull;
         st = trg_init_tensor(ctx, s.model, s.beta, s.h, s.D0);
@@ -281,7 +284,8 @@ int trg_solve_spec_default(trg_solve_spec* s) {
 
 size_t trg_solve_bytes(const trg_solve_spec* spec, size_t workspace_bytes) {
     if (!spec) return 0;
-    return estimate_bytes(*spec, workspace_bytes ? workspace_bytes : ((size_t)1 << 30), true);
+    const size_t ws = workspace_bytes ? workspace_bytes : ((size_t)1 << 30);
+    return estimate_bytes(*spec, ws, trg::exact_cap(ws));
 }
 
 int trg_serve_create(trg_server** out, int device, const trg_server_config* cfg) {
@@ -326,10 +330,17 @@ int trg_serve_submit(trg_server* s, const trg_solve_spec* spec, uint64_t* ticket
     Request* r = new (std::nothrow) Request();
     if (!r) return TRG_ENOMEM;
     r->spec = *spec;
-    r->bytes = estimate_bytes(*spec, s->cfg.workspace_bytes, true);
-    if (r->bytes > s->cfg.hbm_budget_bytes) {   // no room for FP64 digits: such a solve takes the FP64 pipe
+    // FP64 digits are cut in smaller blocks until they fit the budget (the results
+    // are the same bit for bit); if not even a tile's do, the solve takes the FP64
+    // pipe
+    const size_t ws = s->cfg.workspace_bytes, budget = s->cfg.hbm_budget_bytes;
+    int64_t cap = trg::exact_cap(ws);
+    r->bytes = estimate_bytes(*spec, ws, cap);
+    for (; r->bytes > budget && cap > ((int64_t)1 << 20); cap /= 2) r->bytes = estimate_bytes(*spec, ws, cap / 2);
+    r->digit_bytes = (size_t)cap;
+    if (r->bytes > budget) {
         r->no_exact = true;
-        r->bytes = estimate_bytes(*spec, s->cfg.workspace_bytes, false);
+        r->bytes = estimate_bytes(*spec, ws, 0);
     }
     r->work = estimate_work(*spec);
     if (r->bytes > s->cfg.hbm_budget_bytes) {   // could never be admitted

@@ -777,17 +777,19 @@ const long long* diagonal_tiles(Ctx& ctx, int tiles_m, int tiles_n, int xn, int 
     return it->second.as<long long>();
 }
 
-// Rows of the operands whose digits are held at a time: at most XCAP bytes of
-// them each, and a weak bit for at most XBITS elements of C (multiples of the
-// tile; B's rows of XNP).
-constexpr int64_t XCAP = (int64_t)1 << 30, XBITS = (int64_t)1 << 28;
+// Rows of the operands whose digits are held at a time (multiples of the tile;
+// B's of XNP): at most cap bytes of them, half of it for either, and a weak bit
+// for an element of C in at most a 64th of that.  One tile of each is the least;
+// below XCAP_MIN the tiles of a block (256 at K = 4096) no longer fill the SMs, so
+// less is taken only where more cannot be had.
+constexpr int64_t XCAP = (int64_t)2 << 30, XCAP_MIN = (int64_t)256 << 20;
 constexpr int64_t XNP = 64;
 struct XBlock { int64_t a, b; };
-XBlock block_rows(int64_t M, int64_t N, int64_t kp) {
-    const int64_t most = XCAP / (2 * XPLANES * kp);
+XBlock block_rows(int64_t M, int64_t N, int64_t kp, int64_t cap) {
+    const int64_t most = cap / 2 / (2 * XPLANES * kp);
     XBlock x;
     x.a = std::min(up(M, XM), std::max<int64_t>(XM, most / XM * XM));
-    x.b = std::min(up(N, XNP), std::max<int64_t>(XNP, std::min(most, XBITS / x.a) / XNP * XNP));
+    x.b = std::min(up(N, XNP), std::max<int64_t>(XNP, std::min(most, cap / 8 / x.a) / XNP * XNP));
     return x;
 }
 // Bytes of the flags, the weak tiles and the weak bits of an a x b block.
@@ -799,9 +801,13 @@ int64_t state_bytes(int64_t a, int64_t b) { return 4 * (std::max(a, b) / 32 + 1)
 
 }  // namespace
 
-int64_t exact_scratch_bytes(int64_t M, int64_t N, int64_t K) {
+int64_t exact_cap(size_t workspace_bytes) {
+    return std::min(XCAP, std::max(XCAP_MIN, workspace_bytes ? (int64_t)workspace_bytes : XCAP));
+}
+
+int64_t exact_scratch_bytes(int64_t M, int64_t N, int64_t K, int64_t cap) {
     const int64_t kp = up(std::max<int64_t>(K, 1), XKP);
-    const XBlock x = block_rows(M, N, kp);
+    const XBlock x = block_rows(M, N, kp, cap);
     return 2 * XPLANES * kp * (x.a + x.b) + 4 * (x.a + x.b) + flag_bytes(x.a, x.b) + weak_bytes(x.a, x.b) +
            need_bytes(M, N) + 2 * state_bytes(x.a, x.b) + 4096;
 }
@@ -883,15 +889,21 @@ void launch_weak(Ctx& ctx, const GemmDesc& d0, const GemmDesc& d1, int64_t m0, i
 
 bool gemm_exact(Ctx& ctx, const GemmDesc& d) {
     const int K = (int)std::max<int64_t>(d.K, 1), Kp = (int)up(K, XKP);
-    const XBlock blk = block_rows(d.M, d.N, Kp);
+    const ScratchUse use(ctx);
+    // smaller blocks where there is no room for these (the bits are the same)
+    XBlock blk;
+    for (int64_t cap = ctx.digit_bytes ? (int64_t)ctx.digit_bytes : exact_cap(ctx.cfg.workspace_bytes);; cap /= 2) {
+        blk = block_rows(d.M, d.N, Kp, cap);
+        try {
+            ctx.ensure(ctx.split_ws, (size_t)exact_scratch_bytes(d.M, d.N, K, cap));
+            break;
+        } catch (const Error& e) {
+            if (e.status != TRG_ENOMEM) throw;
+            if (blk.a <= XM && blk.b <= XNP) return false;    // not even for a tile: the FP64 pipe needs none
+        }
+    }
     const int64_t ra = blk.a, rb = blk.b;
     const bool sym = d.gram && d.M == d.N && ra >= d.M && rb >= d.N;
-    try {
-        ctx.ensure(ctx.split_ws, (size_t)exact_scratch_bytes(d.M, d.N, K));
-    } catch (const Error& e) {
-        if (e.status == TRG_ENOMEM) return false;    // no room for the digits: the FP64 pipe needs none
-        throw;
-    }
     uint8_t* p = ctx.split_ws.as<uint8_t>();
     auto take = [&](size_t bytes) { uint8_t* q = p; p += (bytes + 255) & ~(size_t)255; return q; };
     int* flags = (int*)take((size_t)flag_bytes(ra, rb));
@@ -974,6 +986,8 @@ bool gemm_exact_pair(Ctx& ctx, const GemmDesc& d0, const GemmDesc& d1) {
     if (2 * tiles_of(M, M, XT<15>::N, true) > ctx.sm_count || try_nine(ctx, M, M, K, true)) return false;
     const int Kp = (int)up(K, XKP), mp = (int)up(M, XM);
     static_assert(XM % XT<15>::N == 0, "the second product starts on a column tile");
+    const ScratchUse use(ctx);
+    if (ctx.digit_bytes && exact_pair_scratch_bytes(M, K) > (int64_t)ctx.digit_bytes) return false;
     try {
         ctx.ensure(ctx.split_ws, (size_t)exact_pair_scratch_bytes(M, K));
     } catch (const Error& e) {

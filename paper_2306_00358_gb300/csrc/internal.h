@@ -83,6 +83,7 @@ struct Ctx {
     // in ns (0 = the kernels' default of 2 s); see trg_set_wait_limit
     unsigned long long acc_wait_ns = 0;
     bool no_exact = false;   // FP64 products stay on the FP64 pipe (no room for their digits)
+    size_t digit_bytes = 0;  // bound on the digits' scratch (0: exact_cap of the workspace)
 
     // ---- solve state
     bool have_tensor = false;
@@ -115,7 +116,8 @@ struct Ctx {
     Buf eig;               // subspace-iteration buffers
     Buf eig_small;         // m x m buffers
     Buf flags;             // per-column flags (int)
-    Buf split_ws;          // split GEMM: exponents and BF16 slices of both operands
+    Buf split_ws;          // tensor-core products: exponents and BF16 slices / digits of both operands
+    int split_ws_users = 0;   // a product holds pointers into it (ScratchUse)
     Buf f64_partial;       // FP64 GEMM: split-K partial sums
     Buf ksplit_ws;         // split GEMM: split-K partial fixed-point sums
     Buf bslices;           // contraction: the D^7 product's B slices, shared by its j-blocks
@@ -161,6 +163,15 @@ struct Ctx {
     const int64_t* table(const std::vector<std::pair<int64_t, int64_t>>& modes);
 };
 constexpr size_t HOST_SLOT_BYTES = 2048, HOST_SLOT_BOX = 64;    // bytes of a slot; the box's offset
+
+// While one lives, Ctx::ensure does not give split_ws up for another buffer.
+struct ScratchUse {
+    Ctx& ctx;
+    explicit ScratchUse(Ctx& c) : ctx(c) { ++ctx.split_ws_users; }
+    ~ScratchUse() { --ctx.split_ws_users; }
+    ScratchUse(const ScratchUse&) = delete;
+    ScratchUse& operator=(const ScratchUse&) = delete;
+};
 
 // Device scalar slots (doubles) in Ctx::scal.
 enum : int {
@@ -254,7 +265,11 @@ double f64_us(const Ctx& ctx, int64_t M, int64_t N, int64_t K, bool sym);   // m
 // scratch cannot be had (nothing computed).
 bool gemm_exact(Ctx& ctx, const GemmDesc& g);
 double exact_us(const Ctx& ctx, int64_t M, int64_t N, int64_t K, bool sym);
-int64_t exact_scratch_bytes(int64_t M, int64_t N, int64_t K);
+// Bound on the digits' scratch, as a rule: the workspace's, within 256 MiB .. 2 GiB
+// (2 GiB if it is not set).  How the operands are cut into blocks that fit changes
+// no bit.
+int64_t exact_cap(size_t workspace_bytes);
+int64_t exact_scratch_bytes(int64_t M, int64_t N, int64_t K, int64_t cap);
 // Two Gram products in one launch; false, with nothing computed, if they do not
 // fit the chip together or their scratch cannot be had.
 bool gemm_exact_pair(Ctx& ctx, const GemmDesc& d0, const GemmDesc& d1);

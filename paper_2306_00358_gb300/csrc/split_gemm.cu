@@ -1106,6 +1106,7 @@ void gemm_split(Ctx& ctx, const GemmDesc& d) {
     const bool gram_b = d.gram && Mp == Np;
     const bool pre_b = d.b_slices != nullptr || gram_b;   // B arrives sliced (shared by several products)
 
+    const ScratchUse use(ctx);
     // scratch: exponents + slices of A and B (unless given)
     const size_t bytes_e = (size_t)(Mp + Np) * sizeof(int);
     const size_t bytes_a = pre_a ? 0 : (size_t)S * Mp * Kp * 2, bytes_b = pre_b ? 0 : (size_t)S * Np * Kp * 2;
