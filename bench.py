@@ -460,12 +460,13 @@ def run_native(args):
         t_launch = x2["ms"] / max(1, x2["calls"]) / 1e3
         achieved = per_launch / t_launch / 1e12
         # FP64-equivalent FLOPs of the whole X2 phase (cutting included), against
-        # the tensor rate over the fewest digit products (45; 120 where the
-        # tensor's weak couplings need fifteen digits)
-        peak = peaks.get("bf16_tflops_sustained", 1713.4) / 45.0
+        # the tensor rate over the digit products that were computed for each
+        # (45, or 120 where the tensor's weak couplings need fifteen digits)
+        digits = ph["mma"]["mma_flops"] / max(1.0, ph["mma"]["flops"])
+        peak = peaks.get("bf16_tflops_sustained", 1713.4) / max(1.0, digits)
         roof = {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
                 "traffic": None, "kernel": "k_exact_mma (X2 = X1.t, D^7)",
-                "peak_source": "MEASURED_PEAKS.json bf16_tflops_sustained / 45 digit products"}
+                "peak_source": f"MEASURED_PEAKS.json bf16_tflops_sustained / {digits:.1f} digit products"}
     else:
         # the X2 product's tensor-core launches alone (events around each launch)
         mx = ph["mma_x2"]

@@ -481,7 +481,9 @@ typedef struct trg_phase_stats {
     double ms;          /* summed event time of the phase's timed regions */
     uint64_t calls;     /* timed regions (one per product / normalisation) */
     double flops;       /* algorithmic FLOPs: 2*M*N*K per product, FP64-equivalent */
-    double mma_flops;   /* tensor-core FLOPs issued (split mode: slice products x 2MNK) */
+    double mma_flops;   /* tensor-core FLOPs issued (split mode: slice products x 2MNK; TRG_FP64, phase
+                           TRG_PHASE_MMA only: the digit products of the tiles that were
+                           computed) */
 } trg_phase_stats;
 
 /* Enable (on != 0) or disable phase timing; enabling resets the counters.

@@ -139,8 +139,23 @@ void Ctx::region_end(int token, double flops, double mma_flops) {
     ph[token].mma_flops += mma_flops;
 }
 
+double* Ctx::device_flops() {
+    if (!prof) return nullptr;
+    if (!mma_flops.p) {
+        ensure(mma_flops, sizeof(double));
+        TRG_CUDA(cudaMemsetAsync(mma_flops.p, 0, sizeof(double), stream));
+    }
+    return mma_flops.as<double>();
+}
+
 void Ctx::collect_timings() {
     TRG_CUDA(cudaStreamSynchronize(stream));
+    if (mma_flops.p) {
+        double v = 0.0;
+        TRG_CUDA(cudaMemcpy(&v, mma_flops.p, sizeof(double), cudaMemcpyDeviceToHost));
+        TRG_CUDA(cudaMemset(mma_flops.p, 0, sizeof(double)));
+        ph[TRG_PHASE_MMA].mma_flops += v;
+    }
     for (auto& acc : ph) {
         for (auto& pr : acc.pending) {
             float ms = 0.f;
@@ -416,9 +431,13 @@ int trg_destroy(trg_ctx* ctx) {
     cudaSetDevice(ctx->device);
     const bool idle = cudaStreamSynchronize(ctx->stream) == cudaSuccess;
     Ctx& c = *ctx;
+    try {
+        c.collect_timings();   // a context whose stream has failed still frees its resources
+    } catch (const trg::Error&) {
+    }
     for (trg::Buf* b : {&c.T, &c.Tnext, &c.M, &c.U, &c.scal, &c.status, &c.ws, &c.envP, &c.envQ, &c.eig,
                         &c.eig_small, &c.flags, &c.split_ws, &c.f64_partial, &c.ksplit_ws, &c.bslices, &c.cons_ef, &c.field_ws, &c.Timp, &c.Timp_next,
-                        &c.Timp_tmp, &c.eig_slices})
+                        &c.Timp_tmp, &c.eig_slices, &c.mma_flops})
         c.release(*b);
     for (trg::Buf& b : c.s3) c.release(b);
     for (auto& kv : c.tables) c.release(kv.second);
@@ -426,10 +445,6 @@ int trg_destroy(trg_ctx* ctx) {
     c.tables.clear();
     c.lists.clear();
     c.give_host_slot(idle);
-    try {
-        c.collect_timings();   // a context whose stream has failed still frees its resources
-    } catch (const trg::Error&) {
-    }
     for (cudaEvent_t e : c.event_pool) cudaEventDestroy(e);
     delete ctx;
     return TRG_OK;

@@ -176,6 +176,8 @@ struct XArgs {
     const int64_t* c_n1;
     int* status;
     unsigned long long acc_wait_ns;   // limit of the epilogue's waits (trg_set_wait_limit)
+    double* flops;                 // profiling: the digit products of the tiles computed are added here
+    double tile_flops;
 };
 
 // The int64 sums of an element, each in units of its last D, as FP64 times
@@ -327,12 +329,14 @@ k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             int stage = 0;
             uint32_t phase = 0;
             uint32_t run_no = 0;        // runs begun so far (all tiles)
+            int done = 0;               // tiles
             bool ok = true;
             int ahead = state_of(blockIdx.x);
             for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
                 const int now = ahead;
                 ahead = state_of(tile + gridDim.x);
                 if (!(now & MINE)) continue;
+                ++done;
                 for (int kb = 0; kb < num_kb; ++kb) {
                     const bool run_start = kb % XRUN == 0;
                     const bool run_end = (kb + 1) % XRUN == 0 || kb + 1 == num_kb;
@@ -381,6 +385,7 @@ k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                     if (++stage == XSTAGES) { stage = 0; phase ^= 1; }
                 }
             }
+            if (S != 1 && g.flops && done) atomicAdd(g.flops, done * g.tile_flops);
             // every MMA issued has completed (also after an abort)
             mma_commit<1>(mma_done);
             volatile int never = 0;
@@ -863,6 +868,9 @@ void launch_exact(Ctx& ctx, const uint16_t* sa, int64_t mp, const uint16_t* sb, 
         a.tile_list = diagonal_tiles(ctx, tiles_m, tiles_n, XT<S>::N, a.half, a.n_list);
         tiles = a.n_list;
     }
+    // (which tiles are computed is decided on the device)
+    a.flops = ctx.device_flops();
+    a.tile_flops = S * (S + 1) / 2 * 2.0 * XM * XT<S>::N * a.Kp;
     // column blocks whose digits share L2 (about 40 MB of them)
     a.group_n = (int)std::max<int64_t>(1, std::min<int64_t>(tiles_n, (40ll << 20) / ((int64_t)XT<S>::N * a.Kp * 2 * S)));
     k_exact_mma<S><<<std::min(tiles, ctx.sm_count), XT<S>::THREADS, XT<S>::SMEM, ctx.stream>>>(ta, tb, a);
@@ -967,7 +975,7 @@ bool gemm_exact(Ctx& ctx, const GemmDesc& d) {
                     a.state = state15;
                 }
                 launch_exact<15>(ctx, sa, mp, sb, np, a);
-                ctx.region_end(tok, 2.0 * (double)mr * nr * K, (scope ? 45.0 : 120.0) * 2.0 * (double)mr * nr * Kp);   // 120 also if nine do not suffice
+                ctx.region_end(tok, 2.0 * (double)mr * nr * K, 0.0);    // (the kernels add their digit products)
                 launch_weak(ctx, d, d, m0, n0, a);
             }
         }
@@ -1019,7 +1027,7 @@ bool gemm_exact_pair(Ctx& ctx, const GemmDesc& d0, const GemmDesc& d1) {
     a.weak = weak; a.weak_tile = flags + 64; a.weak_rows = 2 * mp; a.words = 2 * mp / 32;
     const int tok = ctx.region_begin(TRG_PHASE_MMA);
     launch_exact<15>(ctx, s, 2 * mp, s, 2 * mp, a);
-    ctx.region_end(tok, 4.0 * (double)M * M * K, 120.0 * 4.0 * (double)M * M * Kp);
+    ctx.region_end(tok, 4.0 * (double)M * M * K, 0.0);
     launch_weak(ctx, d0, d1, 0, 0, a);
     ctx.region_end(phase, 4.0 * (double)M * M * K, 0.0);
     return true;

@@ -154,6 +154,10 @@ struct Ctx {
     // Record the start of a timed region of phase p (no-op unless profiling).
     int region_begin(int p);
     void region_end(int token, double flops, double mma_flops);
+    // Where kernels add tensor-core FLOPs that only they know (TRG_PHASE_MMA);
+    // null unless profiling.
+    double* device_flops();
+    Buf mma_flops;
     void collect_timings();
 
     void* raw_alloc(size_t bytes);
