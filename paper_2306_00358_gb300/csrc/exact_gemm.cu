@@ -606,11 +606,14 @@ k_exact_mma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
 
 // ---------------------------------------------- elements left to the pipe ---
 // C(m, n) of the elements that the digit product marked weak, as FP64 sums in
-// order of k, the bits of k_gemm_f64.  A block takes 128 x 32 elements at a time,
-// those of a word column of the marks, lists the marked ones, and gives each
-// thread up to sixteen of them, so its time follows their number; operands are
-// staged as in k_gemm_f64.  Bound by the FP64 pipe: one FMA of a warp takes 16
-// clocks there, the two operands from shared memory about four.
+// order of k, the bits of k_gemm_f64.  A block takes R x 32 elements at a time,
+// lists the marked ones and gives each thread up to sixteen (eight) of them, so
+// its time follows their number; operands are staged as in k_gemm_f64.  Bound by
+// the FP64 pipe: one FMA of a warp takes 16 clocks there, the two operands from
+// shared memory about four.  R = 128 where that gives every SM eight blocks'
+// worth, 32 for smaller products, whose marks lie unevenly: late in an off-critical
+// solve at Dcut 24 the D^7 product takes 1.99 ms with 128 and 2.25 with 32, P and Q
+// in one launch 0.35 and 0.22.
 struct WeakArgs {
     int M, N, K, sym, half;
     const double* A[2]; const int64_t* a_m[2]; const int64_t* a_k[2]; int a_kfast[2];
@@ -621,32 +624,49 @@ struct WeakArgs {
     const uint32_t* weak;      // [words][rows]
     int tiles_m, words, rows;
 };
-constexpr int WK = 16, WN = 32, WT = 256;       // K per stage, columns, threads
-constexpr int WE = XM * WN / WT;                // elements a thread can be given
-__global__ void __launch_bounds__(WT, 2) k_weak_f64(const WeakArgs g) {
+constexpr int WS = 32, WK = 16;                 // columns, K per stage
+template <int R>
+__global__ void __launch_bounds__(R == 32 ? 128 : 256, 2) k_weak_f64(const WeakArgs g) {
+    constexpr int WT = R == 32 ? 128 : 256;     // threads
+    constexpr int WE = R * WS / WT;             // elements a thread can be given
     if (*g.any == 0) return;
-    __shared__ double As[WK][XM + 1];
-    __shared__ double Bs[WK][WN + 1];
-    __shared__ uint16_t list[XM * WN];          // row << 5 | column
-    __shared__ int count;
+    __shared__ double As[WK][R + 1];
+    __shared__ double Bs[WK][WS + 1];
+    __shared__ uint16_t list[R * WS];           // row << 5 | column
+    __shared__ int warp_count[R / 32];
     const int tid = threadIdx.x;
-    for (int t = blockIdx.x; t < g.tiles_m * g.words; t += gridDim.x) {
-        if (!g.tile[t]) continue;
-        const int mb = t / g.words, w = t - mb * g.words;
-        const int q = g.half && mb * XM >= g.half ? 1 : 0;
-        const int m0 = mb * XM - (q ? g.half : 0), n0 = w * WN - (q ? g.half : 0);
-        __syncthreads();                        // the previous tile's list has been used
-        if (tid == 0) count = 0;
-        __syncthreads();
-        if (tid < XM) {
-            uint32_t bits = m0 + tid < g.M ? g.weak[(size_t)w * g.rows + mb * XM + tid] : 0u;
+    for (int t = blockIdx.x; t < g.tiles_m * g.words * (XM / R); t += gridDim.x) {
+        const int tile = t / (XM / R), row0 = tile / g.words * XM + t % (XM / R) * R, w = tile % g.words;
+        if (!g.tile[tile]) continue;
+        const int q = g.half && row0 >= g.half ? 1 : 0;
+        const int m0 = row0 - (q ? g.half : 0), n0 = w * WS - (q ? g.half : 0);
+        __syncthreads();                        // the previous list has been used
+        uint32_t bits = 0;
+        int at = 0;
+        if (tid < R) {
+            if (m0 + tid < g.M) bits = g.weak[(size_t)w * g.rows + row0 + tid];
             const int cols = g.N - n0;
-            if (cols < WN) bits &= (1u << max(cols, 0)) - 1u;
-            int at = atomicAdd(&count, __popc(bits));
-            for (; bits; bits &= bits - 1) list[at++] = (uint16_t)(tid << 5 | (__ffs((int)bits) - 1));
+            if (cols < WS) bits &= (1u << max(cols, 0)) - 1u;
+            // place of this row's elements in the list: first within the warp
+            at = __popc(bits);
+#pragma unroll
+            for (int o = 1; o < 32; o *= 2) {
+                const int v = __shfl_up_sync(0xffffffffu, at, o);
+                if ((tid & 31) >= o) at += v;
+            }
+            if ((tid & 31) == 31) warp_count[tid >> 5] = at;
+            at -= __popc(bits);
         }
         __syncthreads();
-        const int n = count;
+        int n = 0;
+#pragma unroll
+        for (int i = 0; i < R / 32; ++i) {
+            if (i < tid >> 5) at += warp_count[i];
+            n += warp_count[i];
+        }
+        for (; bits; bits &= bits - 1) list[at++] = (uint16_t)(tid << 5 | (__ffs((int)bits) - 1));
+        __syncthreads();
+        if (n == 0) continue;
         int el[WE];
         double acc[WE];
 #pragma unroll
@@ -654,18 +674,18 @@ __global__ void __launch_bounds__(WT, 2) k_weak_f64(const WeakArgs g) {
             el[e] = tid + e * WT < n ? list[tid + e * WT] : 0;
             acc[e] = 0.0;
         }
-        double ra[XM * WK / WT], rb[WN * WK / WT];
+        double ra[R * WK / WT], rb[WS * WK / WT];
         auto load = [&](int k0) {
 #pragma unroll
-            for (int i = 0; i < XM * WK / WT; ++i) {
+            for (int i = 0; i < R * WK / WT; ++i) {
                 const int e = tid + i * WT;
-                const int r = g.a_kfast[q] ? e / WK : e % XM, k = k0 + (g.a_kfast[q] ? e % WK : e / XM);
+                const int r = g.a_kfast[q] ? e / WK : e % R, k = k0 + (g.a_kfast[q] ? e % WK : e / R);
                 ra[i] = m0 + r < g.M && k < g.K ? g.A[q][g.a_m[q][m0 + r] + g.a_k[q][k]] : 0.0;
             }
 #pragma unroll
-            for (int i = 0; i < WN * WK / WT; ++i) {
+            for (int i = 0; i < WS * WK / WT; ++i) {
                 const int e = tid + i * WT;
-                const int c = g.b_nfast[q] ? e % WN : e / WK, k = k0 + (g.b_nfast[q] ? e / WN : e % WK);
+                const int c = g.b_nfast[q] ? e % WS : e / WK, k = k0 + (g.b_nfast[q] ? e / WS : e % WK);
                 rb[i] = n0 + c < g.N && k < g.K ? g.B[q][g.b_k[q][k] + g.b_n[q][n0 + c]] : 0.0;
             }
         };
@@ -673,14 +693,14 @@ __global__ void __launch_bounds__(WT, 2) k_weak_f64(const WeakArgs g) {
         for (int k0 = 0; k0 < g.K; k0 += WK) {
             __syncthreads();
 #pragma unroll
-            for (int i = 0; i < XM * WK / WT; ++i) {
+            for (int i = 0; i < R * WK / WT; ++i) {
                 const int e = tid + i * WT;
-                if (g.a_kfast[q]) As[e % WK][e / WK] = ra[i]; else As[e / XM][e % XM] = ra[i];
+                if (g.a_kfast[q]) As[e % WK][e / WK] = ra[i]; else As[e / R][e % R] = ra[i];
             }
 #pragma unroll
-            for (int i = 0; i < WN * WK / WT; ++i) {
+            for (int i = 0; i < WS * WK / WT; ++i) {
                 const int e = tid + i * WT;
-                if (g.b_nfast[q]) Bs[e / WN][e % WN] = rb[i]; else Bs[e % WK][e / WK] = rb[i];
+                if (g.b_nfast[q]) Bs[e / WS][e % WS] = rb[i]; else Bs[e % WK][e / WK] = rb[i];
             }
             __syncthreads();
             if (k0 + WK < g.K) load(k0 + WK);
@@ -889,7 +909,9 @@ void launch_weak(Ctx& ctx, const GemmDesc& d0, const GemmDesc& d1, int64_t m0, i
     }
     w.any = a.flags; w.tile = a.weak_tile; w.weak = a.weak;
     w.tiles_m = (a.half + a.M + XM - 1) / XM; w.words = a.words; w.rows = a.weak_rows;
-    k_weak_f64<<<std::min(w.tiles_m * w.words, 4 * ctx.sm_count), WT, 0, ctx.stream>>>(w);
+    const int tiles = w.tiles_m * w.words;
+    if (tiles >= 8 * ctx.sm_count) k_weak_f64<128><<<4 * ctx.sm_count, 256, 0, ctx.stream>>>(w);
+    else k_weak_f64<32><<<std::min(4 * tiles, 8 * ctx.sm_count), 128, 0, ctx.stream>>>(w);
     TRG_LAUNCHED(ctx);
 }
 
