@@ -854,7 +854,7 @@ static void times_small(Ctx& ctx, const double* A, const double* W, int64_t n, i
     g.C = C; g.c_m = ctx.table({{n, 1}}); g.c_n = ctx.table({{m, n}}); g.beta = 0.0;
     g.A.r_fast = true; g.A.r_identity = true;
     g.B.r_fast = true; g.B.r_identity = true;
-    g.allow_exact = precision == TRG_FP64;    // split mode: see k_chol_flag on the bits of Q
+    g.allow_exact = precision == TRG_FP64;    // split mode: see k_chol_trsm on the bits of Q
     g.c_m_fast = true;
     gemm(ctx, g, TRG_FP64);
 }

@@ -45,20 +45,22 @@
 // the time, with MMA instructions of N = 48 .. 240; a tenth goes to drains that
 // nothing covers).  128 x 32 output tile with 15 digits, 128 x 48 with 9, one
 // persistent CTA per SM: the S accumulators D_d of the tile's columns (and with 15
-// digits the sums) fill tensor memory.  A stage is 16 (32) K of both operands, one TMA box each, two
-// stages; the cut stores the digits in the order of a stage, so that a box is
-// made of 4 KB pieces (as [p][r][k] planes its rows are pieces of 32 or 64
-// bytes, and the TMA unit's requests hold the products up: 72 -> 68.6 us a
-// product of an environment at (24, 22), without the sums).  The products of one A digit with
-// adjacent B digits land in adjacent accumulators, so 24 (13) instructions of up
-// to N = 256 cover the products of a 16-deep step.  They are issued in two
+// digits the sums) fill tensor memory.  A stage is 16 (32) K of both operands, one
+// TMA box each, two stages; the cut stores the digits in the order of a stage, so
+// that a box is made of 4 KB pieces (as [p][r][k] planes its rows are pieces of 32
+// or 64 bytes, and the TMA unit's requests hold the products up: 72 -> 68.6 us a
+// product of an environment at (24, 22), both without the sums).  The products of
+// one A digit with adjacent B digits land in adjacent accumulators, so 24 (13)
+// instructions of up to N = 256 cover the products of a 16-deep step, the sums
+// among them (one instruction more with 15; the launches of a contraction at (6,
+// 37, 36) 149 -> 153 us with the marks).  They are issued in two
 // groups, the one that lands in the higher D_d (84 of 120, 35 of 45 products)
 // before the other: a run's drain of the higher D_d runs under the other group's
 // products, and the drain of the lower ones under the next run's first group.
 // Measured, contraction at Dx = Dy = Dn = 48 (1.22e12 FP64 FLOPs): 993 ms on
-// the FP64 pipe, 113.6 ms with 15 digits always, 45.3 ms with 9 where they
-// suffice (38.7 ms of it in this kernel, 1.5 ms in the |A||B| sums, 3.8 ms in
-// the cut); with operands that need 15, the sums are the only loss.
+// the FP64 pipe, 110.7 ms where every row needs 15 digits, 44.8 ms where 9 suffice
+// (39 ms of it in this kernel, 1.6 ms in the |A||B| sums, 3.8 ms in the cut), 619
+// ms where half of the elements are left to the pipe.
 #include <algorithm>
 #include <cmath>
 
